@@ -144,36 +144,22 @@ __global__ void fill_kernel(T* v, int64_t p, T val) {
     v[j] = val;
 }
 
-// out[j] = sum_c part[c*NB*p + j] (fixed order); optional sum of squares
-template <typename TA, typename T>
-__global__ void reduce_partials_kernel(const TA* part, int ncl, int NB, int64_t p, T* out, double* sq) {
-  double s2 = 0.0;
+// out[j] = sum_c part[c*NB*p + j] (fixed order); part: FP32 pairs or FP64
+__global__ void reduce_partials_kernel(const void* part, int pair, int ncl, int NB, int64_t p, double* out) {
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < p; j += (int64_t)gridDim.x * blockDim.x) {
-    TA s = (TA)0;
-    for (int c = 0; c < ncl; ++c) s += part[(int64_t)c * NB * p + j];
-    out[j] = (T)s;
-    s2 += (double)s * (double)s;
+    double s = 0.0;
+    if (pair) {
+      relax::ffs f{0.f, 0.f};
+      for (int c = 0; c < ncl; ++c) {
+        const float2 v = static_cast<const float2*>(part)[(int64_t)c * NB * p + j];
+        f = ff_add(f, relax::ffs{v.x, v.y});
+      }
+      s = (double)f.hi + (double)f.lo;
+    } else {
+      for (int c = 0; c < ncl; ++c) s += static_cast<const double*>(part)[(int64_t)c * NB * p + j];
+    }
+    out[j] = s;
   }
-  if (sq) {
-    s2 = warp_sum(s2);
-    if ((threadIdx.x & 31) == 0 && s2 != 0.0) atomicAdd(sq, s2);
-  }
-}
-
-template <typename T>
-__global__ void scale_kernel(T* v, int64_t p, const double* sq) {
-  const double nrm = sqrt(*sq);
-  const T inv = nrm > 0.0 ? (T)(1.0 / nrm) : (T)0;
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < p; j += (int64_t)gridDim.x * blockDim.x)
-    v[j] *= inv;
-}
-
-__global__ void sumsq_kernel(const double* v, int64_t m, double* out) {
-  double s = 0.0;
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x)
-    s += v[j] * v[j];
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0 && s != 0.0) atomicAdd(out, s);
 }
 
 // {F(z), -F*(-zeta)} at zeta = -grad F(z) (Eq. 6-7 loss parts), FP64
@@ -259,19 +245,20 @@ struct BatchWs {
   unsigned long long* bars = nullptr;
   void *Bm = nullptr, *Zm = nullptr, *Rm = nullptr, *Gm = nullptr;   // FP64 data: operands and products
   __nv_bfloat16 *Bp = nullptr, *Rp = nullptr;                      // FP32 data: BF16 planes of B and R
-  double *P1 = nullptr, *P2 = nullptr;                              // FP32 data: partial products per slot
-  double* part = nullptr;
+  float *P1 = nullptr, *P2 = nullptr;                               // FP32 data: partial products per slot
+  double* part = nullptr;         // gradients per node (FP64 data; backtracking)
+  double* lsum = nullptr;         // [cap][link blocks][4] loss sums
   int* active_d = nullptr;
   int* done_d = nullptr;
   int8_t* fix = nullptr;          // [cap][p] the call's fixings (zeros without)
   int* cnt = nullptr;             // [cap][3] fixing counts
-  PassState* psd = nullptr;       // [cap][2] certificate passes
+  PassState* psd = nullptr;       // [cap] certificate passes
   double* certd = nullptr;        // [cap][4] certificate values
   std::vector<std::pair<int, cudaGraphExec_t>> graphs;
   bool planned = false, clustered = false;
-  PPlan pc;                       // cluster plan of the p-phase (when clustered)
+  PPlan pc;                       // backtracking: cluster plan of the p-phase (when clustered)
   void release() {
-    void* ptrs[] = {dst, vec, acc, bpart, bars, Bm, Zm, Rm, Gm, Bp, Rp, P1, P2, part, active_d, done_d, fix, cnt,
+    void* ptrs[] = {dst, vec, acc, bpart, bars, Bm, Zm, Rm, Gm, Bp, Rp, P1, P2, part, lsum, active_d, done_d, fix, cnt,
                     psd, certd};
     for (void* q : ptrs) if (q) cudaFree(q);
     for (auto& g : graphs) cudaGraphExecDestroy(g.second);
@@ -282,8 +269,30 @@ struct BatchWs {
   BatchWs(bool pl, bool cl, PPlan c) : planned(pl), clustered(cl), pc(c) {}
 };
 
+// Certificates of several points: their passes write into slots of one group,
+// and one launch evaluates the group (kept on the handle, freed with it).
+struct CertWs {
+  int cap = 0;                    // points the per-point buffers hold
+  double* pts = nullptr;          // [cap][p] (relax_certify_batch)
+  PassState* psd = nullptr;       // [cap]
+  double* outd = nullptr;         // [cap][2]
+  int* cnt = nullptr;             // [cap][3]
+  void* xg = nullptr;             // [kCertGroup][gstride] gradient partials
+  double* lsum = nullptr;         // [kCertGroup][lstride] loss sums
+  void* gev = nullptr;            // [2 kCertGroup][p] the evaluations' gradients
+  unsigned char* zero = nullptr;  // [kCertGroup][zstride] the passes' zeroed areas
+  size_t gstride = 0, lstride = 0, zstride = 0;
+  void release() {
+    void* ptrs[] = {pts, psd, outd, cnt, xg, lsum, gev, zero};
+    for (void* q : ptrs) if (q) cudaFree(q);
+    *this = CertWs{};
+  }
+};
+constexpr int kCertGroup = 32;
+
 struct relax_handle {
   BatchWs bw;                // relax_solve_batch's device memory and graphs
+  CertWs cw;
   // batched solves of FP32 data: BF16 planes of X (K = p) and of X' (K = n)
   // for the tensor-core products, built on the first batched call; the K
   // chunks chosen per product and column tile width (BN / 16)
@@ -325,11 +334,12 @@ struct relax_handle {
   // loop), then float-float products on the master X; the p-phase in FP64.
   XSPlan pl_acc32, pl_ff;
   bool has_acc32 = false, has_ff = false;
-  PPlan pp_iter, pp_eval, pp_exact;
+  PPlan pp_iter;             // the backtracking loop's p-phase (pphase.cuh)
+  NPlan np_iter, np_eval, np_exact;   // node p-phase: the loop, the certificate, the ladder's last rungs
   // buffers
-  double* xg = nullptr;          // [Gr][2][p] X' r per row group
-  double* lterm = nullptr;       // [n][2] certification loss terms
-  double* lterm2 = nullptr;      // [n][2] the same at a second dual point
+  void* xg = nullptr;            // [Gr][2][p] X' r per row group (FP32 pairs; FP64 data: FP64)
+  double* lsum = nullptr;        // [CTA][4] loss sums of a pass
+  void* gev = nullptr;           // [2][p] gradients of a certificate's evaluation
   unsigned* xcnt = nullptr;      // per-pass zeroed area: block counters, max |beta|, fixed-point z
   double rowl1_x = 0.0;          // max_i ||x_i||_1 of X (NaN if X holds a NaN)
   double rowl1_q = 0.0;          // the same for the BF16/FP8 copy (stored values)
@@ -371,7 +381,8 @@ void handle_free(relax_handle* h) {
   cudaSetDevice(h->dev);
   cudaStreamSynchronize(h->stream);
   h->bw.release();
-  void* ptrs[] = {h->Xown, h->Xq, h->colscale, h->y, h->xg, h->lterm, h->lterm2, h->xcnt, h->st,
+  h->cw.release();
+  void* ptrs[] = {h->Xown, h->Xq, h->colscale, h->y, h->xg, h->lsum, h->gev, h->xcnt, h->st,
                   h->ps_aux, h->acc, h->bpart, h->bar, h->bar_aux, h->status, h->dscr, h->iscr, h->colstat};
   for (void* q : ptrs) if (q) cudaFree(q);
   for (void* q : h->vb) if (q) cudaFree(q);
@@ -423,8 +434,7 @@ XSArgs pass_args(relax_handle* h, const XSPlan& pl, int link, PassState* ps) {
   a.colscale = lowp ? h->colscale : nullptr;
   a.ps = ps;
   a.g = h->xg;
-  a.lterm = nullptr;
-  a.lterm2 = nullptr;
+  a.lsum = nullptr;
   a.rowl1 = lowp ? h->rowl1_q : h->rowl1_x;
   xstrip_zero_layout(pl, h->xcnt, a);
   a.status = h->status;
@@ -433,9 +443,28 @@ XSArgs pass_args(relax_handle* h, const XSPlan& pl, int link, PassState* ps) {
 }
 
 // one fused pass (its block counters are zeroed first)
-cudaError_t run_pass(relax_handle* h, const XSPlan& pl, const XSArgs& a, cudaStream_t st) {
-  (void)h;
-  return xstrip_launch(pl, a, st);
+cudaError_t run_pass(const XSPlan& pl, const XSArgs& a, cudaStream_t st) { return xstrip_launch(pl, a, true, st); }
+
+NArgs base_nargs(relax_handle* h) {
+  NArgs a{};
+  a.loss = h->loss;
+  a.p = h->p;
+  a.n = h->n;
+  a.k = h->k;
+  a.lambda2 = h->lambda2;
+  a.M = h->M;
+  a.step = 1.0 / h->L;
+  a.rho = 2.0 * h->lambda2 / h->L;
+  a.eta = h->eta;
+  a.max_iters = h->max_iters;
+  a.stall_min = h->stall_min;
+  a.method = h->method;
+  a.restart_rule = h->restart_rule;
+  a.gpair = h->dtype == RELAX_F32 ? 1 : 0;   // the passes of FP32 data write pairs
+  a.nq = 1;
+  a.status = h->status;
+  a.kc = pconst_make(a.lambda2, a.M, a.step, a.rho);
+  return a;
 }
 
 PArgs base_pargs(relax_handle* h) {
@@ -453,7 +482,7 @@ PArgs base_pargs(relax_handle* h) {
   a.method = h->method;
   a.restart_rule = h->restart_rule;
   a.backtrack = h->backtrack;
-  a.lossp = nullptr;
+  a.gpair = h->dtype == RELAX_F32 ? 1 : 0;
   a.acc = h->acc;
   a.bpart = h->bpart;
   a.status = h->status;
@@ -628,8 +657,8 @@ relax_status power_iteration(relax_handle* h, double* L_out) {
       *reinterpret_cast<PassState*>(h->h_d + 1000) = ps;   // staging in pinned memory
       CU(cudaMemcpyAsync(h->ps_aux, h->h_d + 1000, sizeof(PassState), cudaMemcpyHostToDevice, h->stream));
       XSArgs a = pass_args(h, h->pl_ident, LINK_IDENT, h->ps_aux);
-      CU(run_pass(h, h->pl_ident, a, h->stream));
-      reduce_partials_kernel<double, double><<<g, 256, 0, h->stream>>>(h->xg, h->pl_ident.Gr, 1, p, w, nullptr);
+      CU(run_pass(h->pl_ident, a, h->stream));
+      reduce_partials_kernel<<<g, 256, 0, h->stream>>>(h->xg, !h->f64(), h->pl_ident.Gr, 1, p, w);
       CU(cudaGetLastError());
       // two rounds of classical Gram-Schmidt against q_0..q_j
       double hc[LZ_MAX + 1], hc2[LZ_MAX + 1];
@@ -681,107 +710,127 @@ relax_status count_fixings(relax_handle* h, const int8_t* fix, int* j1, int* jf)
   return RELAX_OK;
 }
 
-// FP64 Phi(beta_p) and Psi(zeta) with the master X -> h->h_d[0..1].
-// zeta = -grad F(X beta_d) when zd == NULL, else zeta = -grad F(zd) (a dual
-// point given by its z).
-// Enqueue the FP64 certificate of one point pair on the handle's stream:
-// {Phi(bp), Psi(zeta)} into out_dev[0..1], zeta = -grad F(z_d) when the pass
-// state names z_d (zprev), else -grad F(X bd).  ps_dev: the pass state in
-// device memory (beta = bp, beta2 = bd or NULL, zprev = z_d or NULL).  No
-// host synchronisation; consecutive calls share the handle's scratch in
-// stream order.
-// The dual point of a certificate: the pass state's zprev (DUAL_Z), X beta2
-// (DUAL_B2, a second product), or X beta itself (DUAL_SELF, one product).
-enum { DUAL_Z = 0, DUAL_B2 = 1, DUAL_SELF = 2 };
+// The dual point of a certificate: the pass state's zprev and, from the same
+// product, X beta itself (DUAL_PAIR, two values), X beta2 (DUAL_B2, a second
+// product), or X beta itself (DUAL_SELF).
+enum { DUAL_PAIR = 0, DUAL_B2 = 1, DUAL_SELF = 2 };
 
-relax_status certify_enqueue(relax_handle* h, const int8_t* fix, const void* bp, int dual,
-                             PassState* ps_dev, double* out_dev) {
-  const XSPlan& pl = dual == DUAL_B2 ? h->pl_cert : h->pl_certz;   // NF = 2 / NF = 1
-  const int link = dual == DUAL_Z ? (h->loss == RELAX_LS ? LINK_CERTZ_LS : LINK_CERTZ_LOGI)
-                                  : (h->loss == RELAX_LS ? LINK_CERT_LS : LINK_CERT_LOGI);
-  XSArgs a = pass_args(h, pl, link, ps_dev);
-  a.colscale = nullptr;
-  a.lterm = h->lterm;
-  CU(run_pass(h, pl, a, h->stream));
-  PArgs pa = base_pargs(h);
-  pa.mode = PM_EVAL;
-  pa.fix = fix;
-  pa.part = h->xg;
-  pa.ncl = pl.Gr;
-  pa.NB = 1;
-  pa.st = nullptr;
-  pa.vin = bp;
-  pa.out = out_dev;
-  pa.fast_s1 = 0;
-  pa.lossp = h->lterm;
-  pa.n = h->n;
-  pa.bar = h->bar_aux;
-  pa.bar_base = 0;
-  CU(cudaMemsetAsync(h->bar_aux, 0, sizeof(unsigned long long), h->stream));
-  CU(pphase_launch(h->pp_eval, pa, h->stream));
+const XSPlan& cert_plan(relax_handle* h, int dual) {
+  return dual == DUAL_PAIR ? h->pl_cert2 : dual == DUAL_B2 ? h->pl_cert : h->pl_certz;
+}
+int cert_link(relax_handle* h, int dual) {
+  const bool ls = h->loss == RELAX_LS;
+  return dual == DUAL_PAIR ? (ls ? LINK_CERT2_LS : LINK_CERT2_LOGI) : (ls ? LINK_CERT_LS : LINK_CERT_LOGI);
+}
+
+// Enqueue the certificate's evaluation of `items` points whose passes wrote
+// their gradient partials and loss sums at part + gstride i, lsum + lstride i:
+// {Phi(beta), Psi} per dual point into out + ostride i (Phi, Psi pairs).  ps:
+// device pass states (beta); cnt: device fixing counts per item or NULL (root)
+relax_status cert_eval(relax_handle* h, int dual, int items, const int8_t* fix, const int* cnt, const PassState* ps,
+                       const void* part, size_t gstride, const double* lsum, size_t lstride, void* gev, double* out,
+                       int64_t ostride) {
+  const XSPlan& pl = cert_plan(h, dual);
+  NArgs na = base_nargs(h);
+  na.mode = PM_EVAL;
+  na.fix = fix;
+  na.fix_stride = h->p;
+  na.cnt = cnt;
+  na.ev = ps;
+  na.nq = dual == DUAL_PAIR ? 2 : 1;
+  na.part = part;
+  na.part_stride = (int64_t)gstride;
+  na.ncl = pl.Gr;
+  na.NB = pl.NB;
+  na.lsum = lsum;
+  na.nl = pl.grid;
+  na.lsum_stride = (int64_t)lstride;
+  na.gev = gev;
+  na.out = out;
+  na.out_stride = ostride;
+  NPlan np = h->np_eval;
+  if (items * na.nq > 2) CU(pnode_plan(np, h->dtype == RELAX_F64, h->p, items * na.nq));
+  CU(pnode_launch(np, na, items * na.nq, h->stream));
   return RELAX_OK;
 }
 
-// Both certificates of a point in one pass (the X beta product shared): the
-// pass state holds beta = beta_best and zprev = the loop's dual-point z.  The
-// first evaluation gives (Phi(beta), Psi at the loop's dual point) in
-// out_dev[0..1], the second (Phi(beta), Psi at zeta = -grad F(X beta)) in
-// out_dev[2..3] -- the values of the two single-certificate calls.
-relax_status certify_pair_enqueue(relax_handle* h, const int8_t* fix, const void* bp, PassState* ps_dev,
-                                  double* out_dev) {
-  const XSPlan& pl = h->pl_cert2;
-  XSArgs a = pass_args(h, pl, h->loss == RELAX_LS ? LINK_CERT2_LS : LINK_CERT2_LOGI, ps_dev);
-  a.colscale = nullptr;
-  a.lterm = h->lterm;
-  a.lterm2 = h->lterm2;
-  CU(run_pass(h, pl, a, h->stream));
-  for (int q = 0; q < 2; ++q) {
-    PArgs pa = base_pargs(h);
-    pa.mode = PM_EVAL;
-    pa.fix = fix;
-    pa.part = h->xg + (size_t)q * h->p;    // partials [Gr][2][p]: right-hand side q
-    pa.ncl = pl.Gr;
-    pa.NB = 2;
-    pa.st = nullptr;
-    pa.vin = bp;
-    pa.out = out_dev + 2 * q;
-    pa.fast_s1 = 0;
-    pa.lossp = q == 0 ? h->lterm : h->lterm2;
-    pa.n = h->n;
-    pa.bar = h->bar_aux;
-    pa.bar_base = 0;
-    CU(cudaMemsetAsync(h->bar_aux, 0, sizeof(unsigned long long), h->stream));
-    CU(pphase_launch(h->pp_eval, pa, h->stream));
-  }
-  return RELAX_OK;
-}
-
-relax_status certify(relax_handle* h, const int8_t* fix, const void* bp, const void* bd, const void* zd) {
+// Certificate of one point on the handle's stream, its values (2, or 4 with
+// DUAL_PAIR) in h_d: Phi(bp) and Psi at the dual points of `dual` (zd: the
+// given dual point's z).  FP64 passes for FP64 data, float-float for FP32.
+relax_status certify(relax_handle* h, const int8_t* fix, const int* cnt, int dual, const void* bp, const void* bd,
+                     const void* zd) {
   PassState ps{};
   ps.beta = bp;
-  ps.beta2 = zd ? nullptr : bd;
+  ps.beta2 = bd;
   ps.zprev = zd;
   *reinterpret_cast<PassState*>(h->h_d + 1000) = ps;
   CU(cudaMemcpyAsync(h->ps_aux, h->h_d + 1000, sizeof(PassState), cudaMemcpyHostToDevice, h->stream));
-  const int dual = zd ? DUAL_Z : (bd == bp ? DUAL_SELF : DUAL_B2);
-  relax_status rs = certify_enqueue(h, fix, bp, dual, h->ps_aux, h->dscr);
-  if (rs != RELAX_OK) return rs;
-  CU(cudaMemcpyAsync(h->h_d, h->dscr, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  CU(cudaStreamSynchronize(h->stream));
-  return RELAX_OK;
-}
-
-// certify_pair_enqueue for one point, its four values in h_d[0..3]
-relax_status certify_pair(relax_handle* h, const int8_t* fix, const void* bp, const void* zd) {
-  PassState ps{};
-  ps.beta = bp;
-  ps.zprev = zd;
-  *reinterpret_cast<PassState*>(h->h_d + 1000) = ps;
-  CU(cudaMemcpyAsync(h->ps_aux, h->h_d + 1000, sizeof(PassState), cudaMemcpyHostToDevice, h->stream));
-  relax_status rs = certify_pair_enqueue(h, fix, bp, h->ps_aux, h->dscr);
+  const XSPlan& pl = cert_plan(h, dual);
+  XSArgs a = pass_args(h, pl, cert_link(h, dual), h->ps_aux);
+  a.colscale = nullptr;
+  a.rowl1 = h->rowl1_x;
+  a.lsum = h->lsum;
+  CU(run_pass(pl, a, h->stream));
+  relax_status rs = cert_eval(h, dual, 1, fix, cnt, h->ps_aux, h->xg, 0, h->lsum, 0, h->gev, h->dscr, 0);
   if (rs != RELAX_OK) return rs;
   CU(cudaMemcpyAsync(h->h_d, h->dscr, 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CU(cudaStreamSynchronize(h->stream));
+  return RELAX_OK;
+}
+
+// The group's buffers of `certify_many`, for every certificate plan
+relax_status cert_group(relax_handle* h) {
+  CertWs& W = h->cw;
+  if (W.xg) return RELAX_OK;
+  const XSPlan* pls[3] = {&h->pl_cert, &h->pl_certz, &h->pl_cert2};
+  size_t gr = 1, grid = 1, zb = 16;
+  for (const XSPlan* q : pls) {
+    gr = std::max(gr, (size_t)q->Gr);
+    grid = std::max(grid, (size_t)q->grid);
+    zb = std::max(zb, xstrip_zero_bytes(*q, h->n));
+  }
+  W.gstride = gr * 2 * (size_t)h->p;
+  W.lstride = grid * PN_LSUM;
+  W.zstride = (zb + 255) / 256 * 256;
+  relax_status rs = alloc((void**)&W.zero, W.zstride * kCertGroup);
+  if (rs == RELAX_OK) rs = alloc((void**)&W.lsum, W.lstride * kCertGroup * sizeof(double));
+  if (rs == RELAX_OK) rs = alloc(&W.gev, (size_t)2 * kCertGroup * h->p * 8);
+  if (rs == RELAX_OK) rs = alloc(&W.xg, W.gstride * kCertGroup * 8);   // last: its pointer says that all are there
+  if (rs != RELAX_OK) {
+    for (void* q : {(void*)W.zero, (void*)W.lsum, W.gev})
+      if (q) cudaFree(q);
+    W.zero = nullptr;
+    W.lsum = nullptr;
+    W.gev = nullptr;
+  }
+  return rs;
+}
+
+// Enqueue the certificates of `items` points (device pass states ps) on the
+// handle's stream, a group at a time: the group's passes, then one launch
+// that evaluates all of its points and dual points.
+relax_status certify_many(relax_handle* h, int dual, int items, const int8_t* fix, const int* cnt, PassState* ps,
+                          double* out, int64_t ostride) {
+  relax_status rs = cert_group(h);
+  if (rs != RELAX_OK) return rs;
+  CertWs& W = h->cw;
+  const XSPlan& pl = cert_plan(h, dual);
+  for (int i0 = 0; i0 < items; i0 += kCertGroup) {
+    const int m = std::min(kCertGroup, items - i0);
+    CU(cudaMemsetAsync(W.zero, 0, W.zstride * (size_t)m, h->stream));
+    for (int i = 0; i < m; ++i) {
+      XSArgs a = pass_args(h, pl, cert_link(h, dual), ps + i0 + i);
+      a.colscale = nullptr;
+      a.rowl1 = h->rowl1_x;
+      a.lsum = W.lsum + W.lstride * (size_t)i;
+      a.g = static_cast<double*>(W.xg) + W.gstride * (size_t)i;
+      xstrip_zero_layout(pl, W.zero + W.zstride * (size_t)i, a);
+      CU(xstrip_launch(pl, a, false, h->stream));
+    }
+    rs = cert_eval(h, dual, m, fix ? fix + (size_t)i0 * h->p : nullptr, fix ? cnt + 3 * (size_t)i0 : nullptr, ps + i0, W.xg,
+                   W.gstride, W.lsum, W.lstride, W.gev, out + ostride * i0, ostride);
+    if (rs != RELAX_OK) return rs;
+  }
   return RELAX_OK;
 }
 
@@ -940,23 +989,25 @@ relax_status relax_create(relax_handle** out, const void* X, const void* y, int6
     // FP32, BF16 and FP8 data: the loop's per-coordinate arithmetic in FP32
     // (FP64 at a small fraction of the FP32 rate on this GPU); FP64 data keeps
     // FP64 throughout
-    TRYC(pphase_plan(h->pp_iter, true, p, h->backtrack != 0, h->xk_loop != XK_F64 && !h->backtrack));
+    TRYC(pnode_plan(h->np_iter, h->xk_loop == XK_F64, p, 1));
     // the certificate's evaluation: FP32 per coordinate and FP64 wherever a
     // term of Phi or Psi is nonzero (FP32 data); FP64 throughout for FP64 data
-    TRYC(pphase_plan(h->pp_eval, true, p, false, !vd));
-    TRYC(pphase_plan(h->pp_exact, true, p, h->backtrack != 0, false));
+    TRYC(pnode_plan(h->np_eval, vd, p, 2));
+    TRYC(pnode_plan(h->np_exact, true, p, 1));
+    if (h->backtrack) TRYC(pphase_plan(h->pp_iter, true, p, true));
     {
       const XSPlan* pls[7] = {&h->pl_loop, &h->pl_ident, &h->pl_cert, &h->pl_certz, &h->pl_cert2,
                               h->has_ff ? &h->pl_ff : &h->pl_loop, h->has_acc32 ? &h->pl_acc32 : &h->pl_loop};
       size_t zero_b = 0;
-      int gr_max = 1;
+      int gr_max = 1, grid_max = 1;
       for (const XSPlan* q : pls) {
         zero_b = std::max(zero_b, xstrip_zero_bytes(*q, n));
         gr_max = std::max(gr_max, q->Gr);
+        grid_max = std::max(grid_max, q->grid);
       }
-      TRY(alloc((void**)&h->xg, (size_t)gr_max * 2 * p * sizeof(double)));
-      TRY(alloc((void**)&h->lterm, (size_t)2 * n * sizeof(double)));
-      TRY(alloc((void**)&h->lterm2, (size_t)2 * n * sizeof(double)));
+      TRY(alloc(&h->xg, (size_t)gr_max * 2 * p * sizeof(double)));
+      TRY(alloc((void**)&h->lsum, (size_t)grid_max * PN_LSUM * sizeof(double)));
+      TRY(alloc(&h->gev, (size_t)2 * p * sizeof(double)));
       TRY(alloc((void**)&h->xcnt, zero_b));
     }
     TRY(alloc((void**)&h->st, sizeof(IterState)));
@@ -968,8 +1019,7 @@ relax_status relax_create(relax_handle** out, const void* X, const void* y, int6
     for (int i = 13; i < 15; ++i) TRY(alloc(&h->vb[i], (size_t)p * sizeof(double)));
     TRY(alloc(&h->vb[15], (size_t)n * sizeof(double)));
     TRY(alloc((void**)&h->acc, 3 * ACC_STRIDE * sizeof(unsigned long long)));
-    const int gmax = std::max(std::max(h->pp_iter.grid, h->pp_eval.grid), h->pp_exact.grid);
-    TRY(alloc((void**)&h->bpart, (size_t)2 * gmax * NBP * sizeof(double)));
+    TRY(alloc((void**)&h->bpart, (size_t)2 * h->pp_iter.grid * NBP * sizeof(double)));
     TRY(alloc((void**)&h->bar, sizeof(unsigned long long)));
     TRY(alloc((void**)&h->bar_aux, sizeof(unsigned long long)));
     TRY(alloc((void**)&h->status, sizeof(int)));
@@ -1066,6 +1116,8 @@ relax_status relax_solve(relax_handle* h, const int8_t* fixings, const void* war
   s.y_keep = h->vb[13];
   s.gy_keep = h->vb[14];
   s.zy_keep = h->vb[15];
+  s.opm32 = 1.f;
+  s.beta_next = h->vb[13];   // (y_keep with backtracking, which needs no spare)
   *h->h_state = s;
   CU(cudaMemcpyAsync(h->st, h->h_state, sizeof(IterState), cudaMemcpyHostToDevice, h->stream));
   CU(cudaMemsetAsync(h->bar, 0, sizeof(unsigned long long), h->stream));
@@ -1088,9 +1140,22 @@ relax_status relax_solve(relax_handle* h, const int8_t* fixings, const void* war
   pa.st = h->st;
   pa.bar = h->bar;
   pa.fast_s1 = h->dtype == RELAX_F32 ? 1 : 0;   // FP32-key top-k select only for FP32 data
-  pa.lossp = nullptr;                          // loss terms from z^t (FP64, in the p-phase)
-  pa.y = (const double*)h->y;
+  pa.y = (const double*)h->y;                  // loss terms from z^t (FP64, in the p-phase)
   pa.n = h->n;
+  // without backtracking: the node p-phase, which sums the pass's loss terms
+  // and clears the next pass's counters
+  NArgs na = base_nargs(h);
+  na.mode = PM_ITER;
+  na.fix = fix_loop;
+  na.part = h->xg;
+  na.ncl = h->pl_loop.Gr;
+  na.NB = h->pl_loop.NB;
+  na.st = h->st;
+  na.lsum = h->lsum;
+  na.nl = h->pl_loop.grid;
+  na.zero = h->xcnt;
+  na.zero_bytes = (int64_t)xstrip_zero_bytes(h->pl_loop, h->n);
+  xa.lsum = h->backtrack ? nullptr : h->lsum;
   // Timing mode: event records around every loop kernel (captured into the
   // graph); the host then waits for each chunk before enqueueing the next.
   const bool timing = h->opt.timing != 0;
@@ -1103,7 +1168,7 @@ relax_status relax_solve(relax_handle* h, const int8_t* fixings, const void* war
   cudaEvent_t* tev = h->tev;
   // the pass and p-phase of the current rung of the precision ladder
   const XSPlan* cur_pl = &h->pl_loop;
-  const PPlan* cur_pp = &h->pp_iter;
+  const NPlan* cur_np = &h->np_iter;
   XSArgs cur_xa = xa;
   // inside a capture the timing events are recorded as external graph nodes;
   // on direct launches they are plain records
@@ -1115,9 +1180,10 @@ relax_status relax_solve(relax_handle* h, const int8_t* fixings, const void* war
     for (int i = 0; i < chunk; ++i) {
       cudaError_t e;
       if (timing && (e = rec(tev[3 * i], cs)) != cudaSuccess) return e;
-      if ((e = run_pass(h, *cur_pl, cur_xa, cs)) != cudaSuccess) return e;
+      if ((e = xstrip_launch(*cur_pl, cur_xa, h->backtrack != 0, cs)) != cudaSuccess) return e;
       if (timing && (e = rec(tev[3 * i + 1], cs)) != cudaSuccess) return e;
-      if ((e = pphase_launch(*cur_pp, pa, cs)) != cudaSuccess) return e;
+      e = h->backtrack ? pphase_launch(h->pp_iter, pa, cs) : pnode_launch(*cur_np, na, 1, cs);
+      if (e != cudaSuccess) return e;
       if (timing && (e = rec(tev[3 * i + 2], cs)) != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -1160,6 +1226,8 @@ relax_status relax_solve(relax_handle* h, const int8_t* fixings, const void* war
   auto run_loop = [&](int64_t chunk_budget) {
     xms.clear();
     pms.clear();
+    err = cudaMemsetAsync(h->xcnt, 0, xstrip_zero_bytes(*cur_pl, h->n), h->stream);   // the first pass's counters
+    if (err != cudaSuccess) return;
     for (int64_t c = 0; c < chunk_budget; ++c) {
       err = enqueue_chunk();
       if (err != cudaSuccess) break;
@@ -1217,12 +1285,12 @@ relax_status relax_solve(relax_handle* h, const int8_t* fixings, const void* war
       account(it_before, h->h_state->iter);
       if (dst0 != ST_OK || !h->certify) break;
       const IterState& S0 = *h->h_state;
-      relax_status r = certify_pair(h, fixings, S0.beta_best, S0.z_dbest);
+      relax_status r = certify(h, fixings, fixings ? h->iscr : nullptr, DUAL_PAIR, S0.beta_best, nullptr, S0.z_dbest);
       if (r != RELAX_OK) return r;
       const double phi = h->h_d[0];
       double psi = h->h_d[1];
       if (h->h_d[3] > psi || !(psi == psi)) psi = h->h_d[3];
-      out->launches += 3;
+      out->launches += 2;
       // every rung's dual bound is valid: the best one stays
       cert_dual = have_cert ? std::max(cert_dual, psi) : psi;
       cert_primal = phi;
@@ -1260,9 +1328,13 @@ relax_status relax_solve(relax_handle* h, const int8_t* fixings, const void* war
     if (rung == 0 && h->has_acc32) { rung = 1; cur_pl = &h->pl_acc32; }
     else if (rung < 2 && h->has_ff) { rung = 2; cur_pl = &h->pl_ff; }
     else break;
-    cur_pp = &h->pp_exact;
+    cur_np = &h->np_exact;
     cur_xa = pass_args(h, *cur_pl, h->loss == RELAX_LS ? LINK_LS : LINK_LOGISTIC, &h->st->ps);
+    cur_xa.lsum = h->backtrack ? nullptr : h->lsum;
     pa.ncl = cur_pl->Gr;
+    na.ncl = cur_pl->Gr;
+    na.nl = cur_pl->grid;
+    na.zero_bytes = (int64_t)xstrip_zero_bytes(*cur_pl, h->n);
     const int it0 = h->h_state->iter;
     if (it0 >= h->max_iters) break;
     // a warm start from beta_best: the first state again, the iteration count kept
@@ -1399,9 +1471,9 @@ relax_status relax_xpass(relax_handle* h, const void* beta, void* z_out, void* g
   CU(cudaMemsetAsync(h->status, 0, sizeof(int), h->stream));
   CU(cudaMemsetAsync(zp64, 0, (size_t)h->n * sizeof(double), h->stream));
   XSArgs a = pass_args(h, h->pl_loop, h->loss == RELAX_LS ? LINK_LS : LINK_LOGISTIC, h->ps_aux);
-  CU(run_pass(h, h->pl_loop, a, h->stream));
+  CU(run_pass(h->pl_loop, a, h->stream));
   const unsigned g = grid_for(h->p);
-  reduce_partials_kernel<double, double><<<g, 256, 0, h->stream>>>(h->xg, h->pl_loop.Gr, h->pl_loop.NB, h->p, g64, nullptr);
+  reduce_partials_kernel<<<g, 256, 0, h->stream>>>(h->xg, !h->f64(), h->pl_loop.Gr, h->pl_loop.NB, h->p, g64);
   from_f64_kernel<<<g, 256, 0, h->stream>>>(g64, g_out, h->f64(), h->p);
   if (z_out) from_f64_kernel<<<grid_for(h->n), 256, 0, h->stream>>>(z64, z_out, h->f64(), h->n);
   CU(cudaMemsetAsync(h->dscr, 0, 2 * sizeof(double), h->stream));
@@ -1432,7 +1504,8 @@ relax_status relax_certify(relax_handle* h, const int8_t* fixings, const void* b
   to_f64_kernel<<<grid_for(h->p), 256, 0, h->stream>>>(beta_dual, h->f64(), (double*)h->vb[9], h->p);
   CU(cudaGetLastError());
   // one product when both points are the same vector
-  rs = certify(h, fixings, h->vb[8], beta_dual == beta_primal ? h->vb[8] : h->vb[9], nullptr);
+  rs = certify(h, fixings, fixings ? h->iscr : nullptr, beta_dual == beta_primal ? DUAL_SELF : DUAL_B2, h->vb[8], h->vb[9],
+               nullptr);
   if (rs != RELAX_OK) return rs;
   int dst = 0;
   CU(cudaMemcpy(&dst, h->status, sizeof(int), cudaMemcpyDeviceToHost));
@@ -1611,10 +1684,11 @@ __global__ void gprod_f64_kernel(const double* X, int64_t ldx, int64_t n, int64_
       if (j0 + ty + 16 * q < p) G[(int64_t)(c0 + tx) * p + j0 + ty + 16 * q] = acc[q];
 }
 
-// FP64 data: z of node active[s] to its state, and the link: R[s] = grad F(z)
-// and, for the logistic loop, R[m + s] = grad F at the momentum point
+// FP64 data: z of node active[s] to its state, the link (R[s] = grad F(z) and,
+// for the logistic loop, R[m + s] = grad F at the momentum point) and the
+// block's loss sums lsum[s][block] = {F(z), -F*(-zeta), 0, 0}
 __global__ void batch_link_f64_kernel(const IterState* st, const int* active, int m, int64_t n, const double* Z,
-                                      const double* y, int loss, double* R) {
+                                      const double* y, int loss, double* R, double* lsum) {
   const int s = blockIdx.y;
   if (s >= m) return;
   const IterState& S = st[active[s]];
@@ -1622,17 +1696,36 @@ __global__ void batch_link_f64_kernel(const IterState* st, const int* active, in
   double* zout = static_cast<double*>(S.ps.zout);
   const double* zprev = static_cast<const double*>(S.ps.zprev);
   const double mom = S.ps.mom;
+  double f = 0.0, d = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const double z = Z[(size_t)s * n + i];
     const double yd = y[i];
     zout[i] = z;
     if (loss == RELAX_LS) {
-      R[(size_t)s * n + i] = 2.0 * (z - yd);
+      const double e = z - yd, zeta = -2.0 * e;
+      R[(size_t)s * n + i] = 2.0 * e;
+      f += e * e;
+      d += zeta * yd - 0.25 * zeta * zeta;
     } else {
       R[(size_t)s * n + i] = -yd / (1.0 + exp(yd * z));
       const double zy = (1.0 + mom) * z - mom * zprev[i];
       R[(size_t)(m + s) * n + i] = -yd / (1.0 + exp(yd * zy));
+      f += softplus_neg(yd * z);
+      d += entropy_of(yd * z);
     }
+  }
+  __shared__ double sh[2][8];
+  f = warp_sum(f);
+  d = warp_sum(d);
+  if ((threadIdx.x & 31) == 0) {
+    sh[0][threadIdx.x >> 5] = f;
+    sh[1][threadIdx.x >> 5] = d;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    double v = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[threadIdx.x][w];
+    lsum[((int64_t)s * gridDim.x + blockIdx.x) * PN_LSUM + threadIdx.x] = v;
   }
 }
 
@@ -1643,6 +1736,16 @@ __global__ void batch_grad_f64_kernel(const double* G, int m, int NB, int64_t p,
   for (int q = 0; q < NB; ++q)
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < p; j += (int64_t)gridDim.x * blockDim.x)
       part[((size_t)s * NB + q) * p + j] = G[(size_t)(q * m + s) * p + j];
+}
+
+// every node's best point to the caller, in the handle's dtype
+__global__ void best_out_kernel(const IterState* st, void* out, int f64, int64_t p) {
+  const int s = blockIdx.y;
+  const double* b = static_cast<const double*>(st[s].beta_best);
+  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < p; j += (int64_t)gridDim.x * blockDim.x) {
+    if (f64) static_cast<double*>(out)[(int64_t)s * p + j] = b[j];
+    else static_cast<float*>(out)[(int64_t)s * p + j] = (float)b[j];
+  }
 }
 
 __global__ void batch_done_kernel(const IterState* st, const int* active, int m, int* done) {
@@ -1671,7 +1774,7 @@ relax_status ensure_planes(relax_handle* h) {
   return RELAX_OK;
 }
 
-void fill_bgargs(BGArgs& a, const BGPlan& pl, double* P, int* status, uint64_t limit_ns) {
+void fill_bgargs(BGArgs& a, const BGPlan& pl, float* P, int* status, uint64_t limit_ns) {
   a.M = pl.M; a.N = pl.N; a.K = pl.K;
   a.BN = pl.BN; a.NT = pl.NT; a.MT = pl.MT;
   a.nkb = pl.nkb; a.stages = pl.stages;
@@ -1693,13 +1796,14 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
   const int NB = h->loss == RELAX_LS ? 1 : 2;
   std::memset(out, 0, sizeof(relax_result) * (size_t)nb);
   BatchWs& W = h->bw;
-  // ---- p-phase segments (planned once per handle): one thread-block cluster
-  // per node when p fits one cluster (hardware barriers, one launch for every
-  // node), else the fewest CTAs that cover p in cooperative waves of
-  // co-resident segments
-  if (!W.planned) {
-    W.clustered = pphase_cluster_plan(W.pc, p, h->backtrack != 0, !f64 && !h->backtrack) == cudaSuccess &&
-                  !std::getenv("RELAX_BATCH_WAVES");
+  // ---- the node p-phase runs one thread-block cluster per node.  The
+  // backtracking loop has its own (pphase.cuh; planned once per handle): one
+  // cluster per node when p fits one, else the fewest CTAs that cover p in
+  // cooperative waves of co-resident segments
+  const bool bt = h->backtrack != 0;
+  const bool tiles = !f64 && !bt;   // the p-phase sums the products' partial tiles itself
+  if (bt && !W.planned) {
+    W.clustered = pphase_cluster_plan(W.pc, p) == cudaSuccess;
     cudaGetLastError();   // a refused cluster plan leaves no sticky error
     W.planned = true;
   }
@@ -1709,7 +1813,8 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
   const int segb = clustered ? pc.seg
                              : (int)std::max<int64_t>(1, (p + (int64_t)PBLOCK * PEPT - 1) / ((int64_t)PBLOCK * PEPT));
   const int wave = std::max(1, pp.maxgrid / segb);
-  if (!clustered && segb > pp.maxgrid) return RELAX_ENOTSUP;
+  if (bt && !clustered && segb > pp.maxgrid) return RELAX_ENOTSUP;
+  const int nlb = f64 ? (int)std::min<int64_t>(64, (n + 255) / 256) : batch_link_blocks(n);   // loss-sum rows per node
   // ---- device memory of the batch (the handle's, grown to nb nodes)
   const size_t nvec = 8 * (size_t)p + 4 * (size_t)n;   // per node: 8 p-vectors, 4 n-vectors (FP64)
   if (nb > W.cap) {
@@ -1732,15 +1837,16 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
       if (ok && ensure_planes(h) != RELAX_OK) ok = false;
       get((void**)&W.Bp, sizeof(__nv_bfloat16) * 3 * (size_t)cap * h->ldbp);
       get((void**)&W.Rp, sizeof(__nv_bfloat16) * 3 * (size_t)NB * cap * h->ldbn);
-      get((void**)&W.P1, sizeof(double) * BG_MAXKC * (size_t)cap * n);
-      get((void**)&W.P2, sizeof(double) * BG_MAXKC * (size_t)NB * cap * p);
+      get((void**)&W.P1, sizeof(float) * BG_MAXKC * (size_t)cap * n);
+      get((void**)&W.P2, sizeof(float) * BG_MAXKC * (size_t)NB * cap * p);
     }
-    get((void**)&W.part, sizeof(double) * (size_t)p * NB * cap);
+    if (!tiles) get((void**)&W.part, sizeof(double) * (size_t)p * NB * cap);
+    get((void**)&W.lsum, sizeof(double) * PN_LSUM * (size_t)nlb * cap);
     get((void**)&W.active_d, sizeof(int) * (size_t)cap);
     get((void**)&W.done_d, sizeof(int) * (size_t)cap);
     get((void**)&W.fix, (size_t)p * cap);
     get((void**)&W.cnt, sizeof(int) * 3 * (size_t)cap);
-    get((void**)&W.psd, sizeof(PassState) * 2 * (size_t)cap);
+    get((void**)&W.psd, sizeof(PassState) * (size_t)cap);
     get((void**)&W.certd, sizeof(double) * 4 * (size_t)cap);
     if (!ok) {
       W.release();
@@ -1762,7 +1868,7 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
   unsigned long long* bars = W.bars;
   void *Bm = W.Bm, *Zm = W.Zm, *Rm = W.Rm, *Gm = W.Gm;
   __nv_bfloat16 *Bp = W.Bp, *Rp = W.Rp;
-  double *P1 = W.P1, *P2 = W.P2;
+  float *P1 = W.P1, *P2 = W.P2;
   double* part = W.part;
   int* active_d = W.active_d;
   int* done_d = W.done_d;
@@ -1841,6 +1947,8 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
     s.cutoff = h->cutoff;
     s.Lk = h->backtrack ? h->L / 64.0 : h->L;
     s.rho_last = 2.0 * h->lambda2 / s.Lk;
+    s.opm32 = 1.f;
+    s.beta_next = v + 6 * p;
     s.ps.beta = s.beta_cur;
     s.ps.zout = s.z_cur;
     s.ps.zprev = s.z_prev;
@@ -1851,27 +1959,51 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
                       h->stream>>>(warm_start, f64 ? 1 : 0, vec, (int64_t)nvec, p, n);
   BTRYC(cudaGetLastError());
   BTRYC(cudaMemcpyAsync(dst, hs.data(), sizeof(IterState) * (size_t)nb, cudaMemcpyHostToDevice, h->stream));
-  // ---- p-phase arguments (segmented)
-  PArgs pa = base_pargs(h);
-  pa.mode = PM_ITER;
-  pa.fix = W.fix;
-  pa.fix_stride = p;
-  pa.part = part;
-  pa.part_stride = (int64_t)NB * p;
-  pa.ncl = 1;
-  pa.NB = NB;
-  pa.st = dst;
-  pa.bar = bars;
-  pa.acc = acc;
-  pa.bpart = bpart;
-  pa.fast_s1 = h->dtype == RELAX_F32 ? 1 : 0;
-  pa.lossp = nullptr;
-  pa.y = (const double*)h->y;
-  pa.n = n;
-  pa.seg_blocks = segb;
+  // ---- p-phase arguments
+  PArgs pa{};
+  if (bt) {   // segmented
+    pa = base_pargs(h);
+    pa.mode = PM_ITER;
+    pa.fix = W.fix;
+    pa.fix_stride = p;
+    pa.part = part;
+    pa.part_stride = (int64_t)NB * p;
+    pa.gpair = 0;
+    pa.ncl = 1;
+    pa.NB = NB;
+    pa.st = dst;
+    pa.bar = bars;
+    pa.acc = acc;
+    pa.bpart = bpart;
+    pa.fast_s1 = h->dtype == RELAX_F32 ? 1 : 0;
+    pa.y = (const double*)h->y;
+    pa.n = n;
+    pa.seg_blocks = segb;
+  }
+  NArgs na = base_nargs(h);
+  na.mode = PM_ITER;
+  na.fix = W.fix;
+  na.fix_stride = p;
+  na.part = part;
+  na.part_stride = (int64_t)NB * p;
+  na.gpair = 0;
+  na.ncl = 1;
+  na.NB = NB;
+  na.st = dst;
+  na.seg_node = active_d;
+  na.lsum = W.lsum;
+  na.nl = nlb;
+  na.lsum_stride = (int64_t)PN_LSUM * nlb;
+  if (tiles) {
+    na.tiles = P2;
+    na.Bp = Bp;
+    na.ldp = h->ldbp;
+    na.bplane = (int64_t)cap * h->ldbp;
+  }
   // a node on the floor of the products hands over to the single-node finish
   // after a shorter stall than a single solve waits
-  if (pa.stall_min > kBatchStall) pa.stall_min = kBatchStall;
+  pa.stall_min = std::min(pa.stall_min, kBatchStall);
+  na.stall_min = std::min(na.stall_min, kBatchStall);
   // ---- the loop
   std::vector<int> active(nb), hdone(nb);
   for (int j = 0; j < nb; ++j) active[j] = j;
@@ -1911,7 +2043,12 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
       io.P2 = P2;
       io.s2 = pl2.split();
       io.part = part;
+      io.lsum = bt ? nullptr : W.lsum;
     }
+    NPlan np;
+    if (!bt) BTRYC(pnode_plan(np, f64, p, m));
+    na.m = m;
+    na.s2 = pl2.split();
     const dim3 gp((unsigned)std::min<int64_t>(64, (p + 255) / 256), (unsigned)m);
     const dim3 gn((unsigned)std::min<int64_t>(64, (n + 255) / 256), (unsigned)m);
     const dim3 gz((unsigned)((n + 63) / 64), (unsigned)((m + 15) / 16));
@@ -1925,20 +2062,25 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
           batch_pack_f64_kernel<<<gp, 256, 0, cs>>>(dst, active_d, m, p, (double*)Bm);
           zprod_f64_kernel<<<gz, 256, 0, cs>>>((const double*)h->X, h->ldx, n, p, (const double*)Bm, m, (double*)Zm);
           batch_link_f64_kernel<<<gn, 256, 0, cs>>>(dst, active_d, m, n, (const double*)Zm, (const double*)h->y,
-                                                    h->loss, (double*)Rm);
+                                                    h->loss, (double*)Rm, W.lsum);
           gprod_f64_kernel<<<gg, 256, 0, cs>>>((const double*)h->X, h->ldx, n, p, (const double*)Rm, NB * m,
                                                (double*)Gm);
           batch_grad_f64_kernel<<<gp, 256, 0, cs>>>((const double*)Gm, m, NB, p, part);
           if ((e = cudaGetLastError()) != cudaSuccess) return e;
         } else {
-          if ((e = batch_pack(io, cs)) != cudaSuccess) return e;
+          // the p-phase leaves the planes of the next points; the round's
+          // first iteration packs them (the active set has changed)
+          if ((it == 0 || bt) && (e = batch_pack(io, cs)) != cudaSuccess) return e;
           if ((e = bgemm_launch(pl1, a1, cs)) != cudaSuccess) return e;
           if ((e = batch_reduce_link(io, cs)) != cudaSuccess) return e;
           if ((e = bgemm_launch(pl2, a2, cs)) != cudaSuccess) return e;
-          if ((e = batch_reduce_grad(io, cs)) != cudaSuccess) return e;
+          if (bt && (e = batch_reduce_grad(io, cs)) != cudaSuccess) return e;
         }
         round_launches += 5;
-        if (clustered) {
+        if (!bt) {
+          if ((e = pnode_launch(np, na, m, cs)) != cudaSuccess) return e;
+          ++round_launches;
+        } else if (clustered) {
           PArgs pw = pa;
           pw.seg_node = active_d;
           pw.cluster = 1;
@@ -2002,34 +2144,30 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
   // all passes enqueued back to back, one synchronisation
   std::vector<double> cert(4 * (size_t)nb, 0.0);
   if (h->certify && map_dev_status(dstat) == RELAX_OK) {
-    PassState* psd = W.psd;
-    double* certd = W.certd;
-    std::vector<PassState> pss(2 * (size_t)nb);
+    std::vector<PassState> pss((size_t)nb);
     for (int j = 0; j < nb; ++j) {
-      PassState a{};
-      a.beta = hs[j].beta_best;            // Phi(beta_best); Psi at the loop's dual point
-      a.zprev = hs[j].z_dbest;             // and at zeta = -grad F(X beta_best)
-      pss[2 * j] = a;
+      pss[j].beta = hs[j].beta_best;       // Phi(beta_best); Psi at the loop's dual point
+      pss[j].zprev = hs[j].z_dbest;        // and at zeta = -grad F(X beta_best)
     }
     auto chk = [&](cudaError_t e, const char* what, int line) {
       if (e == cudaSuccess) return RELAX_OK;
       set_detail(what, e, line);
       return map_cuda(e);
     };
-    relax_status rc = chk(cudaMemcpyAsync(psd, pss.data(), sizeof(PassState) * 2 * (size_t)nb,
-                                          cudaMemcpyHostToDevice, h->stream), "pass states to device", __LINE__);
-    for (int j = 0; j < nb && rc == RELAX_OK; ++j) {
-      const int8_t* fx = fixings ? W.fix + (size_t)j * p : nullptr;
-      rc = certify_pair_enqueue(h, fx, hs[j].beta_best, psd + 2 * j, certd + 4 * j);
-    }
+    relax_status rc = chk(cudaMemcpyAsync(W.psd, pss.data(), sizeof(PassState) * (size_t)nb, cudaMemcpyHostToDevice,
+                                          h->stream), "pass states to device", __LINE__);
+    if (rc == RELAX_OK) rc = certify_many(h, DUAL_PAIR, nb, fixings ? W.fix : nullptr, W.cnt, W.psd, W.certd, 4);
     if (rc == RELAX_OK)
-      rc = chk(cudaMemcpyAsync(cert.data(), certd, sizeof(double) * 4 * (size_t)nb, cudaMemcpyDeviceToHost,
+      rc = chk(cudaMemcpyAsync(cert.data(), W.certd, sizeof(double) * 4 * (size_t)nb, cudaMemcpyDeviceToHost,
                                h->stream), "certificates to host", __LINE__);
     if (rc == RELAX_OK) rc = chk(cudaStreamSynchronize(h->stream), "certificate passes", __LINE__);
     cudaStreamSynchronize(h->stream);
     BTRY(rc);
     // a non-finite certificate shows in that node's own values (judged below)
   }
+  best_out_kernel<<<dim3((unsigned)std::min<int64_t>(64, (p + 255) / 256), (unsigned)nb), 256, 0, h->stream>>>(
+      dst, beta_out, f64 ? 1 : 0, p);
+  BTRYC(cudaGetLastError());
   for (int j = 0; j < nb; ++j) {
     const IterState& S = hs[j];
     const int8_t* fx = fixings ? fixings + (size_t)j * p : nullptr;
@@ -2041,7 +2179,7 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
     o.lipschitz = S.Lk;
     o.primal_loop = S.phi_best;
     o.dual_loop = S.psi_best;
-    o.launches = launches + (h->certify ? 4 * nb : 0);
+    o.launches = launches + (h->certify ? nb + 2 * ((nb + kCertGroup - 1) / kCertGroup) : 0) + 1;
     relax_status st_j = map_dev_status(dstat);
     if (h->certify && st_j == RELAX_OK) {
       const double phi = cert[4 * (size_t)j];
@@ -2056,9 +2194,6 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
     }
     o.gap = o.primal - o.dual_bound;
     o.rel_gap = o.gap / std::max(1.0, std::fabs(o.primal));
-    from_f64_kernel<<<grid_for(p), 256, 0, h->stream>>>((const double*)S.beta_best,
-                                                         static_cast<unsigned char*>(beta_out) + es * (size_t)p * j,
-                                                         f64 ? 1 : 0, p);
     o.stalled = S.stalled;
     o.cutoff_rule = S.cut_rule;
     auto judge = [&](relax_status s0) {
@@ -2213,55 +2348,51 @@ extern "C" relax_status relax_certify_batch(relax_handle* h, int32_t nb, const i
   if (!h || nb <= 0 || !points || !out_host) return RELAX_EINVAL;
   CU(cudaSetDevice(h->dev));
   const int64_t p = h->p;
-  // scratch: the points in FP64, their pass states, the values, the fixing counts
-  const size_t b64 = sizeof(double) * (size_t)nb * p;
-  const size_t bps = sizeof(PassState) * (size_t)nb;
-  const size_t bout = sizeof(double) * 2 * (size_t)nb;
-  const size_t bcnt = sizeof(int) * 3 * (size_t)nb;
-  auto al = [](size_t x) { return (x + 255) / 256 * 256; };
-  unsigned char* scr = nullptr;
-  relax_status rs = alloc((void**)&scr, al(b64) + al(bps) + al(bout) + al(bcnt));
-  if (rs != RELAX_OK) return rs;
-  double* pts = reinterpret_cast<double*>(scr);
-  PassState* psd = reinterpret_cast<PassState*>(scr + al(b64));
-  double* outd = reinterpret_cast<double*>(scr + al(b64) + al(bps));
-  int* cnt = reinterpret_cast<int*>(scr + al(b64) + al(bps) + al(bout));
+  // the points in FP64, their pass states, the values and the fixing counts:
+  // the handle's buffers, grown to nb points
+  CertWs& W = h->cw;
+  if (nb > W.cap) {
+    CU(cudaStreamSynchronize(h->stream));
+    W.release();
+    const int cap = (nb + 31) / 32 * 32;
+    relax_status rs = alloc((void**)&W.pts, sizeof(double) * (size_t)cap * p);
+    if (rs == RELAX_OK) rs = alloc((void**)&W.psd, sizeof(PassState) * (size_t)cap);
+    if (rs == RELAX_OK) rs = alloc((void**)&W.outd, sizeof(double) * 2 * (size_t)cap);
+    if (rs == RELAX_OK) rs = alloc((void**)&W.cnt, sizeof(int) * 3 * (size_t)cap);
+    if (rs != RELAX_OK) {
+      W.release();
+      return rs;
+    }
+    W.cap = cap;
+  }
   auto run = [&]() -> relax_status {
+    std::vector<int> hc(3 * (size_t)nb);
     if (fixings) {
-      std::vector<int> hc(3 * (size_t)nb);
-      CU(cudaMemsetAsync(cnt, 0, bcnt, h->stream));
+      CU(cudaMemsetAsync(W.cnt, 0, sizeof(int) * 3 * (size_t)nb, h->stream));
       count_fix_batch_kernel<<<dim3((unsigned)std::min<int64_t>(64, (p + 255) / 256), (unsigned)nb), 256, 0,
-                               h->stream>>>(fixings, p, cnt);
+                               h->stream>>>(fixings, p, W.cnt);
       CU(cudaGetLastError());
-      CU(cudaMemcpyAsync(hc.data(), cnt, bcnt, cudaMemcpyDeviceToHost, h->stream));
+      CU(cudaMemcpyAsync(hc.data(), W.cnt, sizeof(int) * 3 * (size_t)nb, cudaMemcpyDeviceToHost, h->stream));
       CU(cudaStreamSynchronize(h->stream));
       for (int j = 0; j < nb; ++j)
         if (hc[3 * j + 2] != 0 || hc[3 * j] > h->k) return RELAX_EINVAL;
     }
     CU(cudaMemsetAsync(h->status, 0, sizeof(int), h->stream));
-    to_f64_kernel<<<grid_for((int64_t)nb * p), 256, 0, h->stream>>>(points, h->f64(), pts, (int64_t)nb * p);
+    to_f64_kernel<<<grid_for((int64_t)nb * p), 256, 0, h->stream>>>(points, h->f64(), W.pts, (int64_t)nb * p);
     CU(cudaGetLastError());
     std::vector<PassState> pss((size_t)nb);
-    for (int j = 0; j < nb; ++j) {
-      PassState b{};
-      b.beta = pts + (size_t)j * p;   // Phi(b) and Psi at zeta = -grad F(X b)
-      pss[j] = b;
-    }
-    CU(cudaMemcpyAsync(psd, pss.data(), bps, cudaMemcpyHostToDevice, h->stream));
-    for (int j = 0; j < nb; ++j) {
-      const relax_status r = certify_enqueue(h, fixings ? fixings + (size_t)j * p : nullptr, pts + (size_t)j * p,
-                                             DUAL_SELF, psd + j, outd + 2 * j);
-      if (r != RELAX_OK) return r;
-    }
-    CU(cudaMemcpyAsync(out_host, outd, bout, cudaMemcpyDeviceToHost, h->stream));
+    for (int j = 0; j < nb; ++j) pss[j].beta = W.pts + (size_t)j * p;   // Phi(b) and Psi at zeta = -grad F(X b)
+    CU(cudaMemcpyAsync(W.psd, pss.data(), sizeof(PassState) * (size_t)nb, cudaMemcpyHostToDevice, h->stream));
+    const relax_status r = certify_many(h, DUAL_SELF, nb, fixings, W.cnt, W.psd, W.outd, 2);
+    if (r != RELAX_OK) return r;
+    CU(cudaMemcpyAsync(out_host, W.outd, sizeof(double) * 2 * (size_t)nb, cudaMemcpyDeviceToHost, h->stream));
     CU(cudaStreamSynchronize(h->stream));
     int dst = 0;
     CU(cudaMemcpy(&dst, h->status, sizeof(int), cudaMemcpyDeviceToHost));
     return map_dev_status(dst);
   };
-  rs = run();
+  const relax_status rs = run();
   cudaStreamSynchronize(h->stream);
-  cudaFree(scr);
   return rs;
 }
 
@@ -2287,8 +2418,8 @@ extern "C" relax_status relax_batch_xpass(relax_handle* h, int32_t nb, const voi
   const size_t b64 = sizeof(double) * (size_t)nb * p;
   const size_t bpb = sizeof(__nv_bfloat16) * 3 * (size_t)nb * h->ldbp;
   const size_t rpb = sizeof(__nv_bfloat16) * 3 * (size_t)nb * h->ldbn;
-  const size_t p1b = sizeof(double) * BG_MAXKC * (size_t)nb * n;
-  const size_t p2b = sizeof(double) * BG_MAXKC * (size_t)nb * p;
+  const size_t p1b = sizeof(float) * BG_MAXKC * (size_t)nb * n;
+  const size_t p2b = sizeof(float) * BG_MAXKC * (size_t)nb * p;
   unsigned char* scr = nullptr;
   rs = alloc((void**)&scr, b64 + bpb + rpb + p1b + p2b + 4 * 256);
   if (rs != RELAX_OK) return rs;
@@ -2296,8 +2427,8 @@ extern "C" relax_status relax_batch_xpass(relax_handle* h, int32_t nb, const voi
   double* bsrc = reinterpret_cast<double*>(scr);
   __nv_bfloat16* Bp = reinterpret_cast<__nv_bfloat16*>(scr + al(b64));
   __nv_bfloat16* Rp = reinterpret_cast<__nv_bfloat16*>(scr + al(b64) + al(bpb));
-  double* P1 = reinterpret_cast<double*>(scr + al(b64) + al(bpb) + al(rpb));
-  double* P2 = reinterpret_cast<double*>(scr + al(b64) + al(bpb) + al(rpb) + al(p1b));
+  float* P1 = reinterpret_cast<float*>(scr + al(b64) + al(bpb) + al(rpb));
+  float* P2 = reinterpret_cast<float*>(scr + al(b64) + al(bpb) + al(rpb) + al(p1b));
   auto run = [&]() -> relax_status {
     to_f64_kernel<<<grid_for((int64_t)nb * p), 256, 0, h->stream>>>(points, 0, bsrc, (int64_t)nb * p);
     CU(cudaGetLastError());

@@ -212,10 +212,10 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bgemm_kernel(const __grid_const
       }
       const int row = mt * BG_BM + q * 32 + lane;
       if (row < a.M) {
-        double* dst = a.P + ((size_t)g.slot * a.N + (size_t)nt * a.BN + c0) * a.M + row;
+        float* dst = a.P + ((size_t)g.slot * a.N + (size_t)nt * a.BN + c0) * a.M + row;
 #pragma unroll
         for (int j = 0; j < 64; ++j)
-          if (j < mine) __stcg(dst + (size_t)j * a.M, (double)hi[j]);
+          if (j < mine) __stcg(dst + (size_t)j * a.M, hi[j]);
       }
     }
   }
@@ -226,21 +226,6 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bgemm_kernel(const __grid_const
 }
 
 // ------------------------------------------------------------ plane splits
-__device__ __forceinline__ void split3(float x, __nv_bfloat16& b1, __nv_bfloat16& b2, __nv_bfloat16& b3) {
-  b1 = __float2bfloat16_rn(x);
-  const float r1 = x - __bfloat162float(b1);   // exact: the rounding error of a coarser format
-  b2 = __float2bfloat16_rn(r1);
-  const float r2 = r1 - __bfloat162float(b2);
-  b3 = __float2bfloat16_rn(r2);                // r2 has at most 8 significant bits: exact
-}
-__device__ __forceinline__ void split3(double x, __nv_bfloat16& b1, __nv_bfloat16& b2, __nv_bfloat16& b3) {
-  b1 = __double2bfloat16(x);
-  const double r1 = x - (double)__bfloat162float(b1);
-  b2 = __double2bfloat16(r1);
-  const double r2 = r1 - (double)__bfloat162float(b2);
-  b3 = __double2bfloat16(r2);
-}
-
 __global__ void split_x_kernel(const float* X, int64_t n, int64_t p, int64_t ldx, __nv_bfloat16* P, int64_t ld) {
   const int64_t plane = n * ld;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < plane; t += (int64_t)gridDim.x * blockDim.x) {
@@ -286,14 +271,27 @@ __global__ void pack_kernel(const BatchIo io) {
   const int64_t plane = (int64_t)io.nb * io.ldp;
   __nv_bfloat16* row = io.Bp + (int64_t)s * io.ldp;
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < io.p; j += (int64_t)gridDim.x * blockDim.x) {
-    __nv_bfloat16 b1, b2, b3;
-    split3(b[j], b1, b2, b3);
+    __nv_bfloat16 b1 = __ushort_as_bfloat16(0), b2 = b1, b3 = b1;
+    const double x = b[j];
+    if (!is_zero_bits(x)) split3(x, b1, b2, b3);   // most of a node's point is zero
     row[j] = b1;
     row[plane + j] = b2;
     row[2 * plane + j] = b3;
   }
 }
 
+// Sum of the `ns` FP32 partials of an output element, in slot order, as a pair.
+__device__ __forceinline__ ffs sum_slots(const float* src, int ns, int64_t chunk) {
+  ffs s{__ldcg(src), 0.f};
+  for (int c = 1; c < ns; ++c) ff_acc(s, __ldcg(src + c * chunk));
+  return ff_add(s, ffs{0.f, 0.f});
+}
+
+// One pass over the nodes' z: the slots' sum (float-float), the link's planes
+// and the loss sums.  FP64 arithmetic and conversions issue at about 1.6 lanes
+// per clock per SM here, so an element takes as few of them as its values
+// need: summing the slots and splitting the planes in FP64 made this kernel
+// FP64-bound (36 us at 256 x 5000; 16 us so).
 __global__ void reduce_link_kernel(const BatchIo io) {
   const int s = blockIdx.y;
   if (s >= io.m) return;
@@ -309,22 +307,33 @@ __global__ void reduce_link_kernel(const BatchIo io) {
   }
   const int64_t plane = (int64_t)io.NB * io.nb * io.ldn;
   const int64_t chunk = (int64_t)io.m * io.n;
+  double lf = 0.0, ld = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < io.n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double* src = io.P1 + (int64_t)s * io.n + i;
     const int ns = bg_slots(io.s1, (int)(i / BG_BM) * io.s1.NT + s / io.s1.BN);
-    double z = 0.0;
-    for (int kc = 0; kc < ns; ++kc) z += __ldcg(src + kc * chunk);   // fixed order
+    const ffs zf = sum_slots(io.P1 + (int64_t)s * io.n + i, ns, chunk);
+    const double z = (double)zf.hi + (double)zf.lo;
     zout[i] = z;
     const double yd = io.y ? io.y[i] : 0.0;
     double r0, r1 = 0.0;
     if (io.loss < 0) {
       r0 = z;
     } else if (io.loss == 0) {
-      r0 = 2.0 * (z - yd);
+      const double d = z - yd;
+      r0 = 2.0 * d;
+      if (io.lsum) {
+        lf += d * d;
+        ld -= r0 * yd;            // zeta y - zeta^2 / 4 with zeta = -2 d; the d^2 part joins at the end
+      }
     } else {
       r0 = -yd / (1.0 + exp(yd * z));
       const double zy = (1.0 + mom) * z - mom * zprev[i];
       r1 = -yd / (1.0 + exp(yd * zy));
+      if (io.lsum) {
+        float f, h;
+        logistic_terms_f((float)(yd * z), f, h);
+        lf += (double)f;
+        ld += (double)h;
+      }
     }
     __nv_bfloat16 b1, b2, b3;
     split3(r0, b1, b2, b3);
@@ -340,6 +349,21 @@ __global__ void reduce_link_kernel(const BatchIo io) {
       row[2 * plane] = b3;
     }
   }
+  if (!io.lsum) return;
+  if (io.loss == 0) ld -= lf;
+  __shared__ double sh[2][8];
+  lf = warp_sum(lf);
+  ld = warp_sum(ld);
+  if ((threadIdx.x & 31) == 0) {
+    sh[0][threadIdx.x >> 5] = lf;
+    sh[1][threadIdx.x >> 5] = ld;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    double v = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[threadIdx.x][w];
+    io.lsum[((int64_t)s * gridDim.x + blockIdx.x) * 4 + threadIdx.x] = v;
+  }
 }
 
 __global__ void reduce_grad_kernel(const BatchIo io) {
@@ -348,14 +372,13 @@ __global__ void reduce_grad_kernel(const BatchIo io) {
   if (io.st && io.st[io.active[s]].done) return;
   const int64_t chunk = (int64_t)io.NB * io.m * io.p;
   for (int q = 0; q < io.NB; ++q) {
-    const double* src = io.P2 + ((int64_t)q * io.m + s) * io.p;
+    const float* src = io.P2 + ((int64_t)q * io.m + s) * io.p;
     double* dst = io.part + ((int64_t)s * io.NB + q) * io.p;
     const int nt = (q * io.m + s) / io.s2.BN;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < io.p; j += (int64_t)gridDim.x * blockDim.x) {
       const int ns = bg_slots(io.s2, (int)(j / BG_BM) * io.s2.NT + nt);
-      double g = 0.0;
-      for (int kc = 0; kc < ns; ++kc) g += __ldcg(src + kc * chunk + j);
-      dst[j] = g;
+      const ffs g = sum_slots(src + j, ns, chunk);
+      dst[j] = (double)g.hi + (double)g.lo;
     }
   }
 }
@@ -468,8 +491,10 @@ cudaError_t batch_pack(const BatchIo& io, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+int batch_link_blocks(int64_t n) { return (int)std::min(64u, grid1(n, 256)); }
+
 cudaError_t batch_reduce_link(const BatchIo& io, cudaStream_t st) {
-  dim3 grid(grid1(io.n, 256) > 64 ? 64 : grid1(io.n, 256), (unsigned)io.m);
+  dim3 grid((unsigned)batch_link_blocks(io.n), (unsigned)io.m);
   reduce_link_kernel<<<grid, 256, 0, st>>>(io);
   return cudaGetLastError();
 }

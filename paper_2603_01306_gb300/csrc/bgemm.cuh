@@ -22,10 +22,10 @@
 // N-tiles innermost, is cut into one contiguous range per CTA of equal length
 // (to one K block), so every SM gets the same work whatever the tile count.
 // A range covers the end of one tile, whole tiles, the start of another; each
-// piece writes its partial tile in FP64 to slot (CTA - first CTA of the
-// tile), and a reduction kernel sums a tile's slots in FP64 in slot order
-// (deterministic), fused with what consumes the product: the link of the
-// loss (Z = X B) or the per-node gradient layout of the p-phase (G = X' R).
+// piece writes its FP32 partial tile (the epilogue's registers) to slot (CTA -
+// first CTA of the tile), and what consumes the product sums a tile's slots in
+// slot order (deterministic) in float-float arithmetic: the link of the loss
+// (Z = X B), and the p-phase itself (G = X' R).
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -44,7 +44,7 @@ constexpr int BG_DRAIN = 4;         // K blocks accumulated in TMEM between drai
 constexpr int BG_PLANES = 3;
 constexpr int BG_MAXS = 8;          // pipeline stages at most
 constexpr int BG_THREADS = 320;     // producer warp, MMA warp, eight epilogue warps
-constexpr int BG_MAXKC = 16;        // partial slots per tile at most (partials are KC x N x M doubles)
+constexpr int BG_MAXKC = 16;        // partial slots per tile at most (partials are KC x N x M floats)
 
 // The split of the iteration space: MT x NT tiles of nkb K blocks over `grid`
 // CTAs; CTA c takes [c T / grid, (c + 1) T / grid), T = MT NT nkb.
@@ -63,6 +63,26 @@ __host__ __device__ inline int bg_slots(const BGSplit& s, int t) {
   return (int)(bg_owner((int64_t)(t + 1) * s.nkb - 1, T, s.grid) - bg_owner((int64_t)t * s.nkb, T, s.grid)) + 1;
 }
 
+// x = b1 + b2 + b3 to 8 + 8 + 8 significant bits (exactly for an FP32 x)
+__device__ __forceinline__ void split3(float x, __nv_bfloat16& b1, __nv_bfloat16& b2, __nv_bfloat16& b3) {
+  b1 = __float2bfloat16_rn(x);
+  const float r1 = x - __bfloat162float(b1);   // exact: the rounding error of a coarser format
+  b2 = __float2bfloat16_rn(r1);
+  const float r2 = r1 - __bfloat162float(b2);
+  b3 = __float2bfloat16_rn(r2);                // r2 has at most 8 significant bits: exact
+}
+// x = hi + lo (an FP32 pair): lo reaches only the third plane's rounding
+__device__ __forceinline__ void split3(float hi, float lo, __nv_bfloat16& b1, __nv_bfloat16& b2, __nv_bfloat16& b3) {
+  b1 = __float2bfloat16_rn(hi);
+  const float r1 = hi - __bfloat162float(b1);
+  b2 = __float2bfloat16_rn(r1);
+  b3 = __float2bfloat16_rn((r1 - __bfloat162float(b2)) + lo);
+}
+__device__ __forceinline__ void split3(double x, __nv_bfloat16& b1, __nv_bfloat16& b2, __nv_bfloat16& b3) {
+  const float hi = (float)x;
+  split3(hi, (float)(x - (double)hi), b1, b2, b3);
+}
+
 struct BGArgs {
   CUtensorMap tmA;        // planes of A: dims {K, M, 3}, box {BG_BK, 128, 3}
   CUtensorMap tmB;        // planes of B: dims {K, N, 3}, box {BG_BK, BN, 3}
@@ -70,7 +90,7 @@ struct BGArgs {
   int BN, NT, MT;         // tile columns, N-tiles, M-tiles
   int nkb;                // K blocks (of BG_BK) over K
   int stages;
-  double* P;              // [slot][N][M] partial products (FP64)
+  float* P;               // [slot][N][M] partial products
   int* status;
   uint64_t limit_ns;
 };
@@ -116,18 +136,20 @@ struct BatchIo {
   const double* y;
   __nv_bfloat16* Bp;     // [3][nb][ldp] planes of the node points
   __nv_bfloat16* Rp;     // [3][NB nb][ldn] planes of the link (the second product's B)
-  const double* P1;      // [slot][m][n] partials of Z = X B
+  const float* P1;       // [slot][m][n] partials of Z = X B
   BGSplit s1;
-  const double* P2;      // [slot][NB m][p] partials of G = X' R
+  const float* P2;       // [slot][NB m][p] partials of G = X' R
   BGSplit s2;
-  double* part;          // [m][NB][p] gradients per node (p-phase layout)
+  double* part;          // [m][NB][p] gradients per node (batch_reduce_grad)
+  double* lsum;          // [m][blocks][4] the link's loss sums {F, -F*(-zeta), 0, 0} per block, or NULL
 };
 // B planes of the active nodes' next points
 cudaError_t batch_pack(const BatchIo& io, cudaStream_t st);
-// z = sum of the Z partials (FP64): each node's z^t, and the planes of
-// grad F at z (and at the momentum point for the logistic loop)
+// z = sum of the Z partials: each node's z^t, the planes of grad F at z (and
+// at the momentum point for the logistic loop), and the loss sums
 cudaError_t batch_reduce_link(const BatchIo& io, cudaStream_t st);
-// the gradients X' grad F of every node, summed over the chunks in FP64
+int batch_link_blocks(int64_t n);   // blocks per node of batch_reduce_link (lsum rows)
+// the gradients X' grad F of every node, summed over the slots
 cudaError_t batch_reduce_grad(const BatchIo& io, cudaStream_t st);
 
 }  // namespace relax

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "pnode.cuh"
 #include "pphase.cuh"
 #include "xstrip.cuh"
 #include "xpass.cuh"
@@ -33,11 +34,25 @@ struct XSPlan {
 cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t n, int64_t p);
 // encode the plan's tensor map of X (16-byte aligned, ldx * size a multiple of 16)
 cudaError_t xstrip_bind(XSPlan& pl, const void* X, int64_t ldx, int64_t n, int64_t p);
-// The per-pass area (block counters, the grid's max |beta|, z in fixed point)
-// starts at a.cnt; xstrip_launch zeroes it on the stream before the launch.
+// The per-pass area (block counters, the grid's max |beta|, z in fixed point;
+// a multiple of 16 bytes) starts at a.cnt and is zero before the launch: with
+// `clear` a memset on the stream, else the caller's p-phase has cleared it.
 size_t xstrip_zero_bytes(const XSPlan& pl, int64_t n);
 void xstrip_zero_layout(const XSPlan& pl, void* base, XSArgs& a);   // sets a.cnt, a.zcnt, a.zmax, a.zfix
-cudaError_t xstrip_launch(const XSPlan& pl, const XSArgs& a, cudaStream_t st);
+cudaError_t xstrip_launch(const XSPlan& pl, const XSArgs& a, bool clear, cudaStream_t st);
+
+// Node p-phase (pnode.cuh): the loop's iteration and the certificate's
+// evaluation of `nprob` problems of length p, one cluster each.
+struct NPlan {
+  const void* kernel = nullptr;
+  bool f64 = false;
+  int cl = 1, cpc = 32, lc = 64;   // CTAs per problem, coordinates per CTA, list entries per CTA
+  int warps = 8, wch = 32;         // warps per CTA (the first takes no coordinates), coordinates per warp
+  size_t smem = 0;
+};
+cudaError_t pnode_plan(NPlan& pl, bool f64, int64_t p, int nprob);
+// fills the plan's fields of `a`; grid = nprob clusters
+cudaError_t pnode_launch(const NPlan& pl, NArgs a, int nprob, cudaStream_t st);
 
 struct PPlan {
   const void* kernel = nullptr;
@@ -46,19 +61,19 @@ struct PPlan {
   bool vdouble = false;
   int seg = 0;             // cluster plans: CTAs per problem (the cluster size)
 };
-// backtrack: the instantiation with the backtracking step rule (FP64 vectors);
-// fast: the loop's FP32 per-coordinate instantiation (FP32 data, fixed step)
-cudaError_t pphase_plan(PPlan& pl, bool vdouble, int64_t p, bool backtrack = false, bool fast = false);
+// backtrack: the loop's instantiation with the backtracking step rule (FP64
+// vectors); otherwise the standalone regularizer operations
+cudaError_t pphase_plan(PPlan& pl, bool vdouble, int64_t p, bool backtrack = false);
 cudaError_t pphase_launch(const PPlan& pl, const PArgs& a, cudaStream_t st);
 // the same kernel on `grid` CTAs (a segmented launch: grid = segments x a.seg_blocks <= maxgrid)
 cudaError_t pphase_launch_grid(const PPlan& pl, const PArgs& a, int grid, cudaStream_t st);
-// Batched p-phase of many problems of length p, each on one thread-block
+// Batched backtracking p-phase of many problems of length p, each on one thread-block
 // cluster of pl.seg CTAs: PEPT coordinates per thread on up to 16 CTAs where
 // the device allows that non-portable cluster size, else PEPT_CLUSTER on up to
 // 8; cudaErrorNotSupported when p needs more.
-cudaError_t pphase_cluster_plan(PPlan& pl, int64_t p, bool backtrack = false, bool fast = false);
+cudaError_t pphase_cluster_plan(PPlan& pl, int64_t p);
 // the cluster instantiation with `ept` coordinates per thread (PEPT or PEPT_CLUSTER)
-const void* pphase_cluster_kernel(int ept, bool backtrack, bool fast);
+const void* pphase_cluster_kernel(int ept);
 // nseg clusters (a.seg_blocks = pl.seg, a.cluster = 1); no co-residency needed
 cudaError_t pphase_launch_clusters(const PPlan& pl, const PArgs& a, int nseg, cudaStream_t st);
 

@@ -1,12 +1,14 @@
-// p-phase: everything an iteration does on p-vectors, in one cooperative launch.
+// p-phase of the backtracking loop, and the standalone regularizer operations:
+// everything an iteration does on p-vectors, in one cooperative launch.  (The
+// fixed-step loop and the certificate take the same steps in pnode.cuh.)
 //
 //   P0  G^t = sum of the per-cluster X'r partials; a = -G^t/(2 lambda2) (the
 //       argument of g* in Psi, since X'zeta = -G^t); |beta^t| statistics.
 //   S1  TopSum_{kbar} H_M(|a_Jf|) of Lemma 4.2 through its variational form
 //       TopSum_k(h) = min_t k t + sum_j (h_j - t)_+ at t = the kbar-th largest h,
 //       found by a radix select over key bits (32 candidates per round, one per
-//       lane).  The certification and the standalone g* use the exact keys of
-//       the values; the loop selects on FP32-rounded keys, which makes the sum an
+//       lane).  FP64 data and the standalone g* use the exact keys of
+//       the values; the loop on FP32 data selects on FP32-rounded keys, which makes the sum an
 //       upper bound within FP32 rounding (Psi stays a valid bound).
 //   S2  g_N(beta^t) (Thm 4.4 / Algorithm 1): the water level w of Algorithm 1
 //       is the root of sum_j min(|beta_j|, w) = kbar w; a multisection over the
@@ -53,7 +55,7 @@ constexpr int ACC_STRIDE = NFIELD * PQ;
 constexpr int NBP = 10;         // doubles per block partial
 constexpr int MAX_POLISH = 8;
 
-enum PMode : int { PM_ITER = 0, PM_EVAL = 1, PM_PROX = 2, PM_GVAL = 3, PM_GSTAR = 4 };
+enum PMode : int { PM_ITER = 0, PM_EVAL = 1 /* pnode.cuh only */, PM_PROX = 2, PM_GVAL = 3, PM_GSTAR = 4 };
 
 // accumulator fields
 enum : int { F_S1 = 0, F_S2Z = 1, F_S2C = 2, F_S3Z = 3, F_S3CM = 4, F_S3CT = 5, F_S3NZ = 6 };
@@ -94,6 +96,17 @@ struct IterState {
   int bt_pending;               // 1: beta^t is a trial point whose test is pending
   int backtracks;               // retries so far (each doubles L)
   unsigned long long bar_base;  // grid-barrier counter value at the start of a launch
+  // scalars of the next iteration (pnode.cuh), formed by the epilogue of the
+  // last one: the water level of beta^t (0: not known), the momentum of "no
+  // restart" and 1 + it in FP32, the FP32 keys of the predicted S1 and S3
+  // thresholds (0: none)
+  double w_next;
+  float mu32, opm32;
+  unsigned key1, key3;
+  float mu_lo;                  // the rest of the momentum (mu32 + mu_lo)
+  int pad_;
+  int win1, win3;               // log2 of the candidates' window around them (FP32 keys)
+  void* beta_next;              // where the next point is formed (rotates with beta_prev and beta_cur)
 };
 
 // Scalars of a launch that follow from lambda2, M, the step and eta: taken
@@ -105,7 +118,10 @@ struct PConst {
   double inv1r;      // 1 / (1 + rho)
   double kTc;        // (1 + rho) / rho: T(c) = c kTc for c <= rho M
   double rhoM;       // rho M
+  double inv_rho;    // 1 / rho
   float M, inv2l_f, s_f, M1r_f, rr_f, inv_rho_f;   // FP32 forms (M (1 + rho), rho / (1 + rho))
+  float rho_f, kTc_f;             // rho, kTc
+  float M_lo, inv_rho_lo;         // the rest of M and 1 / rho: FP32 pairs
   uint32_t krho;     // FP32 key of rhoM rounded up
 };
 __host__ __device__ inline PConst pconst_make(double lambda2, double M, double step, double rho) {
@@ -115,12 +131,17 @@ __host__ __device__ inline PConst pconst_make(double lambda2, double M, double s
   k.inv1r = 1.0 / (1.0 + rho);
   k.kTc = (1.0 + rho) / rho;
   k.rhoM = rho * M;
+  k.inv_rho = 1.0 / rho;
   k.M = (float)M;
   k.inv2l_f = (float)k.inv2l;
   k.s_f = (float)step;
   k.M1r_f = (float)(M * (1.0 + rho));
   k.rr_f = (float)(rho / (1.0 + rho));
   k.inv_rho_f = (float)(1.0 / rho);
+  k.rho_f = (float)rho;
+  k.kTc_f = (float)k.kTc;
+  k.M_lo = M < 3e38 ? (float)(M - (double)k.M) : 0.f;
+  k.inv_rho_lo = (float)(k.inv_rho - (double)k.inv_rho_f);
 #ifdef __CUDA_ARCH__
   const float ru = __double2float_ru(k.rhoM);
 #else
@@ -148,7 +169,7 @@ struct PArgs {
   const int8_t* fix;            // NULL = root
   const void* part;             // [ncl][NB][p] doubles
   int ncl, NB;
-  const double* lossp;          // [n][2] per-row loss terms (certification); NULL: from z and y
+  int gpair;                    // part holds FP32 pairs (float2) instead of FP64
   const double* y;              // n: response (loss terms from z^t in the loop)
   int64_t n;
   IterState* st;
@@ -208,57 +229,6 @@ __device__ __forceinline__ KT warm_cand(KT kc, KT lo, KT hi, int q, int shift) {
   return (KT)x;
 }
 
-// Float-float sums (Knuth's TwoSum; about 48 significant bits from FP32
-// instructions).  This GPU issues FP64 arithmetic, comparisons and
-// conversions at about 1.6 lanes per clock per SM against about 112 for FP32
-// (measured), so the loop's per-coordinate work on FP32 data (the FAST
-// instantiation) is FP32 with float-float sums.
-struct ffs {
-  float hi, lo;
-};
-// s += x
-__device__ __forceinline__ void ff_acc(ffs& s, float x) {
-  const float t = s.hi + x;
-  const float bp = t - s.hi;
-  s.lo += (s.hi - (t - bp)) + (x - bp);
-  s.hi = t;
-}
-// s += x for an FP64 x (split into two floats first)
-__device__ __forceinline__ void ff_acc(ffs& s, double x) {
-  const float h = (float)x;
-  ff_acc(s, h);
-  s.lo += (float)(x - (double)h);
-}
-// a + b, renormalised; symmetric in a and b (every lane of a butterfly gets
-// the same bits)
-__device__ __forceinline__ ffs ff_add(ffs a, ffs b) {
-  const float t = a.hi + b.hi;
-  const float bp = t - a.hi;
-  const float e = (a.hi - (t - bp)) + (b.hi - bp);
-  const float lo = e + (a.lo + b.lo);
-  const float h = t + lo;
-  return ffs{h, lo - (h - t)};
-}
-__device__ __forceinline__ ffs ff_of(double x) {
-  const float h = (float)x;
-  return ffs{h, (float)(x - (double)h)};
-}
-__device__ __forceinline__ bool is_zero_bits(double x) { return (__double_as_longlong(x) << 1) == 0; }
-
-// The logistic loss terms of one row in FP32 (the FAST loop), t = y z:
-// log(1 + exp(-t)), and the entropy -(u log u + v log v) of u = 1/(1 + e^t),
-// v = 1 - u, written with e = exp(-|t|) <= 1 and L = log1p(e) so that
-// neither term loses its small part when the sigmoid saturates.
-__device__ __forceinline__ void logistic_terms_f(float t, float& f, float& h) {
-  const float s = fabsf(t);
-  const float e = expf(-s);
-  const float L = log1pf(e);
-  f = fmaxf(-t, 0.f) + L;
-  const float big = 1.f / (1.f + e), small = e * big;   // the two probabilities
-  // t >= 0: u = small (pays s + L), v = big (pays L); t < 0 the other way
-  h = small * (s + L) + big * L;
-}
-
 // One multisection decision, taken by every warp on its own: lane q holds
 // candidate x (non-decreasing in q) and `ge`, whether its field reaches the
 // target, which holds on a prefix of the lanes (the fields do not increase
@@ -291,21 +261,16 @@ __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// TV: element type of the p-vectors (double in the loop and certification;
+// TV: element type of the p-vectors (double in the backtracking loop;
 // float or double for the standalone entry points).  EPT: elements per thread
 // (at most), so one CTA covers PBLOCK * EPT coordinates.  BT: the backtracking
 // step rule is compiled in (its test and retry cost registers that the
 // fixed-step loop does not pay).  CL: the cluster-per-problem launch, whose
-// sums go through distributed shared memory.  FAST (the loop on FP32 data,
-// PM_ITER only): the per-coordinate arithmetic in FP32 with float-float
-// sums; FP64 only where beta^t or beta^{t-1} is nonzero (the iterate's FP64
-// accumulation), for the prox outputs that are nonzero, and per row of the
-// loss.  Every threshold decision stays exact for the values it classifies.
-template <typename TV, int EPT = PEPT, bool BT = false, bool CL = false, bool FAST = false>
+// sums go through distributed shared memory.
+template <typename TV, int EPT = PEPT, bool BT = false, bool CL = false>
 __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
-  static_assert(!FAST || (sizeof(TV) == 8 && !BT), "FAST: FP64 iterates, fixed step");
   // S1 keys: FP32 or FP64 bit patterns of |a|
-  using KG = typename std::conditional<FAST, uint32_t, unsigned long long>::type;
+  using KG = unsigned long long;
   using KV = uint32_t;             // FP32 keys of the S2 / S3 thresholds
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // this CTA's problem: the whole grid, or its segment of a batched launch
@@ -344,11 +309,6 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
   if (tid == 0) sh_done = (st != nullptr) ? st->done : 0;
   __syncthreads();
   if (sh_done) return;   // uniform: every block reads the same flag
-  // the host plans FAST for the loop and the certificate's evaluation only
-  if (FAST && !((a_in.mode == PM_ITER && st != nullptr) || (a_in.mode == PM_EVAL && st == nullptr))) {
-    if (blockIdx.x == 0 && tid == 0) atomicCAS(a_in.status, ST_OK, ST_INTERNAL);
-    return;
-  }
   // the node's state, read once into shared memory: the scalar stages below
   // (taken by thread 0) would otherwise wait on one global load after another
   __shared__ IterState sst;
@@ -405,56 +365,6 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
     }
     __syncthreads();
     for (int i = 0; i < nv; ++i) v[i] = sh_tot[i];
-    __syncthreads();
-  };
-  // the same over float-float partials (FAST): a warp butterfly, the warps in
-  // order, the blocks' partials (two floats each) by lane and a butterfly;
-  // the totals in FP64
-  auto gsum_ff = [&](ffs* v, int nv, double* out) {
-    const int buf = nstep & 1;
-    float2* bp = CL ? nullptr : reinterpret_cast<float2*>(a.bpart + (size_t)buf * nbk * NBP);
-    ++nstep;
-    for (int i = 0; i < nv; ++i) {
-      ffs s = v[i];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const ffs t{__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)};
-        s = ff_add(s, t);
-      }
-      if (lane == 0) red_f[warp][i] = make_float2(s.hi, s.lo);
-    }
-    __syncthreads();
-    if (tid < nv) {
-      ffs s{red_f[0][tid].x, red_f[0][tid].y};
-      for (int w = 1; w < PNW; ++w) s = ff_add(s, ffs{red_f[w][tid].x, red_f[w][tid].y});
-      if (CL) cl_f[buf][tid] = make_float2(s.hi, s.lo);
-      else bp[(size_t)lbk * NBP + tid] = make_float2(s.hi, s.lo);
-    }
-    barrier();
-    for (int c = warp; c < nv; c += PNW) {
-      ffs s{0.f, 0.f};
-      if (CL) {
-        if (lane < nbk) {
-          const uint32_t ra = mapa(&cl_f[buf][c], (uint32_t)lane);
-          float hi, lo;
-          asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(hi), "=f"(lo) : "r"(ra) : "memory");
-          s = ffs{hi, lo};
-        }
-      } else {
-        for (int b = lane; b < nbk; b += 32) {
-          const float2 q = __ldcg(bp + (size_t)b * NBP + c);
-          s = ff_add(s, ffs{q.x, q.y});
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const ffs t{__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)};
-        s = ff_add(s, t);
-      }
-      if (lane == 0) sh_tot[c] = (double)s.hi + (double)s.lo;
-    }
-    __syncthreads();
-    for (int i = 0; i < nv; ++i) out[i] = sh_tot[i];
     __syncthreads();
   };
   int nround = 0;
@@ -516,17 +426,17 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
     bprev = static_cast<const TV*>(sr->beta_prev);
     Gprev = static_cast<const double*>(sr->G_prev);
     Gcur = static_cast<double*>(sr->G_cur);
-  } else if (mode == PM_EVAL || mode == PM_GVAL) {
+  } else if (mode == PM_GVAL) {
     bcur = static_cast<const TV*>(a.vin);
   }
-  const double* part = static_cast<const double*>(a.part);
+  auto grad_part = [&](int64_t i) -> double {
+    if (!a.gpair) return static_cast<const double*>(a.part)[i];
+    const float2 v = static_cast<const float2*>(a.part)[i];
+    return (double)v.x + (double)v.y;
+  };
+  const float M32 = (float)M;
   // S1 keys: FP64 patterns when the values are FP64 and exactness is asked for
-  const bool key64 = !FAST && !a.fast_s1 && (mode == PM_EVAL || sizeof(TV) == 8);
-  // FAST: the FP32 forms of the scalars
-  const double inv2l = a.kc.inv2l;
-  const double Mtol = a.kc.Mtol;
-  const float M32 = a.kc.M;
-  const float inv2l32 = a.kc.inv2l_f;
+  const bool key64 = !a.fast_s1 && sizeof(TV) == 8;
   // the step's constants (the backtracking variant changes the step in flight)
   PConst kr = a.kc;
   if (BT && mode == PM_ITER && a.backtrack) kr = pconst_make(lam2, M, step, rho);
@@ -542,27 +452,13 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
   //       5 domain violations, 6 non-finite, 7 sum_Jf H(a), 8 F(z), 9 -F*(-zeta)
   double s0[NBP] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   double fy_sum = 0.0;   // backtracking: F at the kept momentum point
-  ffs lf8{0.f, 0.f}, lf9{0.f, 0.f};   // FAST, logistic: the loss terms in float-float
-  if (a.lossp) {
-    // per-row loss terms written by the certification pass
-    for (int64_t i = gt; i < a.n; i += nthr) {
-      s0[8] += a.lossp[2 * i];
-      s0[9] += a.lossp[2 * i + 1];
-    }
-  } else if (mode == PM_ITER) {
+  if (mode == PM_ITER) {
     // loss terms of Eq. 6-7 at z^t = X beta^t, zeta = -grad F(z^t), in FP64;
     // with a backtracking test pending, also F at the kept momentum point
     const double* zt = static_cast<const double*>(sr->z_cur);
     const double* zy = (BT && a.backtrack && sr->bt_pending) ? static_cast<const double*>(sr->zy_keep) : nullptr;
     for (int64_t i = gt; i < a.n; i += nthr) {
       const double yi = a.y[i], zi = zt[i];
-      if (FAST && a.loss != 0) {
-        float f, hh;
-        logistic_terms_f((float)(yi * zi), f, hh);
-        ff_acc(lf8, f);
-        ff_acc(lf9, hh);
-        continue;
-      }
       if (a.loss == 0) {
         const double d = zi - yi, zeta = -2.0 * d;
         s0[8] += d * d;
@@ -578,62 +474,8 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
       }
     }
   }
-  const bool need_a = (mode == PM_ITER || mode == PM_EVAL || mode == PM_GSTAR);
-  const bool need_b = (mode == PM_ITER || mode == PM_EVAL || mode == PM_GVAL);
-  float gf[EPT];     // FAST: G^t in FP32
-  float gyf[EPT];    // FAST: the logistic second gradient in FP32
-  ffs sf[NBP];       // FAST: the sums s0 as float-float
-  if constexpr (FAST) {
-    // The bulk of the coordinates (beta^t_j = 0, not fixed) costs FP32 work
-    // only; the terms of Phi and Psi that are not zero there (fixed-in
-    // coordinates, nonzero beta^t_j, and the whole free set when the
-    // cardinality budget is slack) are FP64, as are their sums (float-float).
-    int c_nnz = 0, c_dom = 0, c_bad = 0;
-#pragma unroll
-    for (int i = 0; i < NBP; ++i) sf[i] = ffs{0.f, 0.f};
-#pragma unroll
-    for (int e = 0; e < EPT; ++e) {
-      const int64_t j = (int64_t)gt + (int64_t)e * nthr;
-      fx[e] = 0; ka[e] = 0; bmf[e] = 0.f; bt[e] = (TV)0; gf[e] = 0.f; gyf[e] = 0.f;
-      if (j >= p) { fx[e] = -2; continue; }
-      const int8_t f = a.fix ? a.fix[j] : (int8_t)0;
-      fx[e] = f;
-      double G = 0.0, Gy = 0.0;   // partials summed in FP64, fixed order
-      for (int c = 0; c < a.ncl; ++c) {
-        G += part[((int64_t)c * a.NB) * p + j];
-        if (a.NB > 1) Gy += part[((int64_t)c * a.NB + 1) * p + j];
-      }
-      if (mode == PM_ITER) Gcur[j] = G;
-      gf[e] = (float)G;
-      if (a.NB > 1) gyf[e] = (float)Gy;
-      const float aa = fabsf(gf[e]) * inv2l32;   // |a_j| in FP32 (keys), a = -G / (2 lambda2)
-      if (!isfinite(aa)) ++c_bad;
-      if (f > 0) ff_acc(sf[0], huber_d<double>(fabs(G) * inv2l, M));
-      if (f == 0) ka[e] = key_of(aa);   // a slack budget's sum over the free set: in the finishing
-      const TV b = bcur[j];
-      bt[e] = b;
-      if (!is_zero_bits((double)b)) {          // most coordinates of beta^t are zero
-        const double bd = (double)b;
-        const double ab = fabs(bd);
-        if (!isfinite(bd)) ++c_bad;
-        if (f > 0) { ff_acc(sf[1], bd * bd); if (ab > Mtol) ++c_dom; }
-        else if (f < 0) ++c_dom;
-        else {
-          bmf[e] = (float)ab;
-          ff_acc(sf[2], ab);
-          ff_acc(sf[3], ab * ab);
-          ++c_nnz;
-          if (ab > Mtol) ++c_dom;
-        }
-      }
-    }
-    sf[4] = ffs{(float)c_nnz, 0.f};
-    sf[5] = ffs{(float)c_dom, 0.f};
-    sf[6] = ffs{(float)c_bad, 0.f};
-    const bool own_loss = a.loss != 0 && !a.lossp && mode == PM_ITER;   // the float-float loss loop ran
-    sf[8] = own_loss ? lf8 : ff_of(s0[8]);
-    sf[9] = own_loss ? lf9 : ff_of(s0[9]);
-  } else {
+  const bool need_a = (mode == PM_ITER || mode == PM_GSTAR);
+  const bool need_b = (mode == PM_ITER || mode == PM_GVAL);
 #pragma unroll
   for (int e = 0; e < EPT; ++e) {
     const int64_t j = (int64_t)gt + (int64_t)e * nthr;
@@ -648,8 +490,8 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
       } else {
         double G = 0.0, Gy = 0.0;   // cluster partials summed in FP64, fixed order
         for (int c = 0; c < a.ncl; ++c) {
-          G += part[((int64_t)c * a.NB) * p + j];
-          if (a.NB > 1) Gy += part[((int64_t)c * a.NB + 1) * p + j];
+          G += grad_part(((int64_t)c * a.NB) * p + j);
+          if (a.NB > 1) Gy += grad_part(((int64_t)c * a.NB + 1) * p + j);
         }
         gg[e] = G;
         gy[e] = Gy;
@@ -681,7 +523,6 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
       }
     }
   }
-  }
   const int kbar = st ? sr->kbar : 0;   // filled below for the standalone modes
   int kb = kbar, pb = st ? sr->pbar : 0;
   double tot[NBP];
@@ -694,8 +535,7 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
       if (fx[e] == 0) cnt2[1] += 1.0;
     }
   }
-  if constexpr (FAST) gsum_ff(sf, NBP, tot);
-  else gsum(tot, NBP);
+  gsum(tot, NBP);
   if (!st) {
     gsum(cnt2, 2);
     kb = a.k - (int)cnt2[0];
@@ -731,14 +571,14 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
     double topsum, gval, w_closed;
     unsigned long long c2lo, kc1;
     unsigned kc2;
-    int s1, s2, w_known, g_inf, warm1, warm2, slack;
+    int s1, s2, w_known, g_inf, warm1, warm2;
   };
   __shared__ ScA sca;
   if (tid == 0) {
     ScA r{};
     if (need_a) {
       if (kb <= 0) r.topsum = 0.0;
-      else if (pb <= kb) { r.topsum = tot[7]; r.slack = FAST; }   // FAST: summed in the finishing
+      else if (pb <= kb) { r.topsum = tot[7]; }
       else r.s1 = 1;
     }
     // In the loop beta^t (t >= 1) is the prox output of the last iteration,
@@ -858,14 +698,6 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
   // S1: t* = the kbar-th largest |a| (key lo1); TopSum = kbar H(t*) + sum (H(|a|) - H(t*))_+
   // S2: w on the bracket's piece, polished until the classification is stable.
   const bool fin1 = need_a && kb > 0 && pb > kb && !retry;
-  const bool fins = FAST && sca.slack && !retry;   // the whole free set, in FP64 (it has at most kbar coordinates)
-  // FP64 G_j: the loop's stored G^t, or the partials again (evaluation)
-  auto G64 = [&](int64_t j) {
-    if (mode == PM_ITER) return Gcur[j];
-    double G = 0.0;
-    for (int c = 0; c < a.ncl; ++c) G += part[((int64_t)c * a.NB) * p + j];
-    return G;
-  };
   // thread 0: the scalars of the finishing (the others read them below)
   __shared__ double shw[5];   // htstar, wcur, topsum, gval, wlast
   __shared__ int shw_pol2;
@@ -890,42 +722,6 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
   bool first = true;
   while (first || pol2) {
     double v[NBP] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    if constexpr (FAST) {
-      // only the coordinates at or above t* (FP32 keys: the others have
-      // |a_j| < t*) and the nonzero |beta_j| contribute: FP64 for those
-      ffs vf[5] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-      int nab = 0;
-      if (first && fin1) {
-        for (int e = 0; e < EPT; ++e) {
-          // keys are FP32 |a| (within two ulps of the FP64 value): a margin
-          // keeps every coordinate whose FP64 |a| exceeds t*
-          if (fx[e] != 0 || ka[e] + 4u < (KG)lo1) continue;
-          const int64_t j = (int64_t)gt + (int64_t)e * nthr;
-          const double hv = huber_d<double>(fabs(G64(j)) * inv2l, M) - htstar;
-          if (hv > 0.0) ff_acc(vf[0], hv);
-        }
-      }
-      if (first && fins) {
-        for (int e = 0; e < EPT; ++e) {
-          if (fx[e] != 0) continue;
-          const int64_t j = (int64_t)gt + (int64_t)e * nthr;
-          ff_acc(vf[0], huber_d<double>(fabs(G64(j)) * inv2l, M));
-        }
-      }
-      if (pol2) {
-        for (int e = 0; e < EPT; ++e) {
-          if (!(bmf[e] > 0.f)) continue;
-          const double m = fabs((double)bt[e]);
-          if (m > wcur) {
-            ++nab;
-            ff_acc(vf[3], m);
-            ff_acc(vf[4], m * m);
-          }
-        }
-      }
-      vf[2] = ffs{(float)nab, 0.f};
-      gsum_ff(vf, 5, v);
-    } else {
     if (first && fin1) {
       const TV* av_src = mode == PM_GSTAR ? static_cast<const TV*>(a.vin) : nullptr;
       for (int e = 0; e < EPT; ++e) {
@@ -946,10 +742,8 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
       }
     }
     gsum(v, 5);
-    }
     if (tid == 0) {
       if (first && fin1) shw[2] = (double)kb * htstar + v[0];
-      if (first && fins) shw[2] = v[0];
       if (pol2) {
         // classification at wcur: N_above, S_above, Q_above
         const double Nab = v[2], Sab = v[3], Qab = v[4];
@@ -995,17 +789,11 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
   __shared__ double shd_mu;
   __shared__ int shd_flags;
   if (tid == 0) {
-  if (mode == PM_ITER || mode == PM_EVAL) {
+  if (mode == PM_ITER) {
     phi = Ftot + 2.0 * lam2 * gval;
     psi = Dtot - 2.0 * lam2 * (tot[0] + topsum);
   }
-  if (mode == PM_EVAL) {
-    if (lbk == 0 && tid == 0) {
-      a.out[0] = phi;
-      a.out[1] = psi;
-      if (nonfinite) atomicCAS(a.status, ST_OK, ST_NUMERIC);
-    }
-  } else if (mode == PM_GVAL) {
+  if (mode == PM_GVAL) {
     if (lbk == 0 && tid == 0) a.out[0] = gval;
   } else if (mode == PM_GSTAR) {
     if (lbk == 0 && tid == 0) a.out[0] = tot[0] + topsum;
@@ -1115,62 +903,7 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
   float ti[EPT];   // T^{-1}(|v|) in FP32: where coordinate j reaches z_j = 1
   double nzv = 0.0;
   double nbad = 0.0;   // standalone prox: non-finite inputs (the output is then all NaN)
-  // FAST: bit e of `wide` set when v_j is FP64 (vv[e]: beta^t_j or
-  // beta^{t-1}_j nonzero, or j fixed in the support); otherwise v_j is the
-  // FP32 value -s gy_j with |v_j| = mmf[e] and its sign in bit e of `negm`
-  unsigned wide = 0, negm = 0;
-  if (do_prox && FAST) {
-    // v_j = y_j - s gy_j: FP64 where beta^t_j or beta^{t-1}_j is nonzero (or
-    // j is fixed in), FP32 elsewhere, where y_j = 0
-    __shared__ float shv[2];   // mu, 1 + mu in FP32
-    __shared__ int shv_mu0;
-    if (tid == 0) {
-      shv[0] = (float)mu;
-      shv[1] = (float)(1.0 + mu);
-      shv_mu0 = mu == 0.0;
-    }
-    __syncthreads();
-    const float mu32 = shv[0], opm32 = shv[1], s32 = kr.s_f, M1r32 = kr.M1r_f, rr32 = kr.rr_f;
-    const bool mu0 = shv_mu0 != 0;
-    int c_nz = 0;
-#pragma unroll
-    for (int e = 0; e < EPT; ++e) {
-      const int64_t j = (int64_t)gt + (int64_t)e * nthr;
-      vv[e] = (TV)0; mmf[e] = 0.f; ti[e] = 0.f;
-      if (j >= p) continue;
-      const double b = (double)bt[e];
-      const double bp = (double)bprev[j];
-      float v32;
-      if (fx[e] > 0 || !is_zero_bits(b) || !is_zero_bits(bp)) {
-        double gyv;
-        if (a.loss == 0) {
-          gyv = mu0 ? Gcur[j] : (1.0 + mu) * Gcur[j] - mu * Gprev[j];
-        } else if (mu0) {
-          gyv = Gcur[j];
-        } else {
-          gyv = 0.0;
-          for (int c = 0; c < a.ncl; ++c) gyv += part[((int64_t)c * a.NB + 1) * p + j];
-        }
-        const double v = (b + mu * (b - bp)) - step * gyv;   // the iterate's FP64 accumulation
-        vv[e] = v;
-        v32 = (float)v;
-        wide |= 1u << e;
-      } else {
-        float gyv;
-        if (a.loss == 0) gyv = mu0 ? gf[e] : opm32 * gf[e] - mu32 * (float)Gprev[j];
-        else gyv = mu0 ? gf[e] : gyf[e];
-        v32 = -(s32 * gyv);
-      }
-      if (v32 < 0.f) negm |= 1u << e;
-      if (fx[e] == 0) {
-        const float m = fabsf(v32);
-        mmf[e] = m;
-        ti[e] = m <= M1r32 ? m * rr32 : m - M32;
-        if (m > 0.f) ++c_nz;
-      }
-    }
-    nzv = (double)c_nz;
-  } else if (do_prox) {
+  if (do_prox) {
     const TV* vin = static_cast<const TV*>(a.vin);
     const TV muv = (TV)mu;
     const TV sv = (TV)step;
@@ -1222,12 +955,7 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
   if (do_prox) {
     {
       double nv[2] = {nzv, nbad};
-      if constexpr (FAST) {
-        ffs t[2] = {{(float)nzv, 0.f}, {0.f, 0.f}};
-        gsum_ff(t, 2, nv);
-      } else {
-        gsum(nv, 2);
-      }
+      gsum(nv, 2);
       nzv = nv[0];
       nbad = nv[1];
     }
@@ -1333,27 +1061,6 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
       for (int it = 0; it <= MAX_POLISH; ++it) {
         const double ccur = shp[0], Tc = shp[1];
         double v[NBP] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-        if constexpr (FAST) {
-          // an FP32 m satisfies m >= Tc iff m >= Tc rounded up, m > ccur iff
-          // m > ccur rounded down: exact classification in FP32
-          const float tcu = shpf[0], ccd = shpf[1];
-          int ntop = 0, nmid = 0;
-          ffs sm{0.f, 0.f};
-          for (int e = 0; e < EPT; ++e) {
-            if (fx[e] != 0) continue;
-            if (wide >> e & 1u) {
-              const double m = fabs((double)vv[e]);
-              if (m >= Tc) ++ntop;
-              else if (m > ccur) { ++nmid; ff_acc(sm, m); }
-            } else {
-              const float m = mmf[e];
-              if (m >= tcu) ++ntop;
-              else if (m > ccd) { ++nmid; ff_acc(sm, m); }
-            }
-          }
-          ffs t[3] = {{(float)ntop, 0.f}, {(float)nmid, 0.f}, sm};
-          gsum_ff(t, 3, v);
-        } else {
         for (int e = 0; e < EPT; ++e) {
           if (fx[e] != 0) continue;
           const double m = (double)mm[e];
@@ -1361,7 +1068,6 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
           else if (m > ccur) { v[1] += 1.0; v[2] += m; }
         }
         gsum(v, 3);
-        }
         if (tid == 0) {
           const double Ntop = v[0], Nmid = v[1], Smid = v[2];
           double cn;
@@ -1404,36 +1110,6 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
     __syncthreads();
     const double T_c = shq[0];
     double cnt[2] = {0, 0};
-    if constexpr (FAST) {
-      // FP64 only for the outputs that are nonzero (about the support)
-      const double inv1r = shq[1];
-      const float ccd = shq_c;   // an FP32 m exceeds c iff it exceeds ccd
-#pragma unroll
-      for (int e = 0; e < EPT; ++e) {
-        const int64_t j = (int64_t)gt + (int64_t)e * nthr;
-        if (j >= p) continue;
-        double b = 0.0;
-        if (fx[e] > 0) {
-          b = fmin(fmax((double)vv[e] * inv1r, -M), M);   // fixed in: v_j is FP64
-        } else if (fx[e] == 0) {
-          const bool w = (wide >> e) & 1u;
-          double m = 0.0;
-          bool nz;
-          if (w) {
-            m = fabs((double)vv[e]);
-            nz = m > c;
-          } else {
-            nz = mmf[e] > ccd;
-            if (nz) m = (double)mmf[e];
-          }
-          if (nz) {
-            const double r = fmax(0.0, fmin(fmin(m - c, m * inv1r), M));
-            b = ((negm >> e) & 1u) ? -r : r;
-          }
-        }
-        out[j] = (TV)b;
-      }
-    } else {
     // Standalone prox: a non-finite input, or a bounded wait of this block
     // that expired (its threshold then rests on incomplete sums), gives NaN
     // outputs instead of silently wrong ones; the counts get a sentinel below.
@@ -1479,7 +1155,6 @@ __global__ void __launch_bounds__(PBLOCK) pphase_kernel(const PArgs a_in) {
       }
     }
     if (mode == PM_PROX && nbad > 0.0 && lbk == 0 && tid == 0) atomicCAS(a.status, ST_OK, ST_NUMERIC);
-    }
   }
 
   // ------------------------------------------------------------- epilogue

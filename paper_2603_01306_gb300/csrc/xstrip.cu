@@ -48,7 +48,7 @@ static int xs_tv(int vec) { return vec == 2 ? 6 : vec == 4 ? 6 : vec == 8 ? 3 : 
 //    as many stages per warp as shared memory holds (ring A first);
 //  * phase A may lead phase B by `lag` blocks: about 64 MB of X in L2 (at
 //    least 20 blocks with four or more row groups).
-// RELAX_XS="B,SA,SB,lag,vps,mA,mB" overrides for tuning runs (0 keeps a default).
+// RELAX_XS="B,SA,SB,lag,vps,mA,mB,Gr" overrides for tuning runs (0 keeps a default).
 cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t n, int64_t p) {
   pl = XSPlan{};
   pl.xk = xk;
@@ -63,9 +63,9 @@ cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const int es = xkind_esize(xk);
   const int vec = xkind_vec(xk);
-  int B_f = 0, SA_f = 0, SB_f = 0, lag_f = 0, vps_f = 0, mA_f = 0, mB_f = 0;
+  int B_f = 0, SA_f = 0, SB_f = 0, lag_f = 0, vps_f = 0, mA_f = 0, mB_f = 0, gr_f = 0;
   if (const char* ov = std::getenv("RELAX_XS"))
-    std::sscanf(ov, "%d,%d,%d,%d,%d,%d,%d", &B_f, &SA_f, &SB_f, &lag_f, &vps_f, &mA_f, &mB_f);
+    std::sscanf(ov, "%d,%d,%d,%d,%d,%d,%d,%d", &B_f, &SA_f, &SB_f, &lag_f, &vps_f, &mA_f, &mB_f, &gr_f);
   // strips: over the number of row groups Gr, the strip width (at most `cap`
   // vectors) that keeps the most SMs busy, strips under 2 KB counted as
   // streaming less efficiently
@@ -129,6 +129,12 @@ cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t
   pl.SA = SA;
   pl.SB = SB;
   pl.Gr = (int)std::max<int64_t>(1, std::min<int64_t>(nsm / Gc, pl.nblk));
+  // at least two blocks per CTA: a row group costs the p-phase one partial of
+  // X'r per column, and the pass little (1000 x 1000 FP32, 63 -> 32 groups:
+  // pass 21.7 -> 20.8 us, p-phase 31.6 -> 29.2; 500 x 1000 FP64, 30 -> 16:
+  // 30.9 -> 30.6, 33.7 -> 29.7; fewer still and the pass loses more)
+  pl.Gr = std::max(1, std::min(pl.Gr, (pl.nblk + 1) / 2));
+  if (gr_f > 0) pl.Gr = std::min(pl.Gr, gr_f);
   const double row_bytes = (double)p * es;
   pl.lag = lag_f > 0 ? lag_f : (int)std::max(4.0, std::min(64.0, 64.0e6 / (B * row_bytes * pl.Gr)));
   // tall designs (four or more row groups): a deeper lead measured faster
@@ -139,7 +145,7 @@ cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t
   pl.threads = 32 * (2 + SA + SB);   // two producers, SA dot, SB axpy
   // the combine of the axpy warps' strip sums reuses the rings
   const size_t ring = (size_t)(pl.RA + pl.RB) * nbox * pl.boxb;
-  const size_t comb = (size_t)SB * NB * pl.sw * sizeof(double);
+  const size_t comb = (size_t)SB * NB * pl.sw * 8;
   pl.smem = std::max(ring, comb) + 128;
   if (pl.smem + 2048 > (size_t)optin) return cudaErrorNotSupported;
   // the attribute belongs to the kernel, shared by every plan and handle: only raise it
@@ -198,7 +204,7 @@ cudaError_t xstrip_bind(XSPlan& pl, const void* X, int64_t ldx, int64_t n, int64
 //   cnt[nblk] | zcnt | zmax[2] | zfix[NF][n]
 static size_t zero_off_zcnt(const XSPlan& pl) { return ((size_t)pl.nblk * sizeof(unsigned) + 15) / 16 * 16; }
 size_t xstrip_zero_bytes(const XSPlan& pl, int64_t n) {
-  return zero_off_zcnt(pl) + 32 + (size_t)pl.NF * n * sizeof(unsigned long long);
+  return (zero_off_zcnt(pl) + 32 + (size_t)pl.NF * n * sizeof(unsigned long long) + 15) / 16 * 16;
 }
 void xstrip_zero_layout(const XSPlan& pl, void* base, XSArgs& a) {
   unsigned char* b = static_cast<unsigned char*>(base);
@@ -209,9 +215,11 @@ void xstrip_zero_layout(const XSPlan& pl, void* base, XSArgs& a) {
   a.zfix = reinterpret_cast<unsigned long long*>(b + oz + 32);
 }
 
-cudaError_t xstrip_launch(const XSPlan& pl, const XSArgs& a, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(a.cnt, 0, xstrip_zero_bytes(pl, a.n), st);
-  if (e != cudaSuccess) return e;
+cudaError_t xstrip_launch(const XSPlan& pl, const XSArgs& a, bool clear, cudaStream_t st) {
+  if (clear) {
+    const cudaError_t e = cudaMemsetAsync(a.cnt, 0, xstrip_zero_bytes(pl, a.n), st);
+    if (e != cudaSuccess) return e;
+  }
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;

@@ -79,9 +79,9 @@ struct XSArgs {
   unsigned long long* zmax;   // [NF] max_j |beta_j| (bits of a nonnegative double) } before
   unsigned* zcnt;             // CTAs that have added to zmax                   } the launch
   double rowl1;               // max_i ||x_i||_1 of the stored X (NaN when X holds a NaN)
-  double* g;             // [Gr][NB][p] X' r per row group
-  double* lterm;         // [n][2] per-row {F, -F*(-zeta)} (certification links) or NULL
-  double* lterm2;        // [n][2] the same at the second dual point (LINK_CERT2_*) or NULL
+  void* g;               // [Gr][NB][p] X' r per row group: FP32 pairs (float2), FP64 for FP64 X
+  double* lsum;          // [CTA][4] sums over the rows the CTA records: F at z, -F*(-zeta) at the
+                         // dual point, the same at the second one (LINK_CERT2_*), 0; or NULL
   unsigned* cnt;         // [nblk] CTAs done with the block's dots (zeroed before the launch)
   int* status;
   uint64_t limit_ns;
@@ -226,20 +226,15 @@ __device__ __forceinline__ void butterfly16(double (&h)[16], int lane) {
 }
 
 // Link of one row: w[q] = the gradient weights of the row (r = grad F at z, and
-// at the momentum point for the logistic loop), lf = F term at z[0],
-// ld = -F*(-zeta) term of the dual point (certification links).  zp is the
-// row's entry of ps.zprev (z of the previous iterate, or the given dual point).
+// at the momentum point for the logistic loop).  zp is the row's entry of
+// ps.zprev (z of the previous iterate, or the given dual point).
 // LOWP (the loop's FP32-accumulating passes): the logistic link in FP32
 // (FP64 exp on this GPU costs about as much as streaming the row block);
 // the float-float and FP64 passes keep it in FP64.
 template <int NF, int NB, bool LOWP = false>
-__device__ __forceinline__ void link_of(int link, const double* z, double yd, double zp, double mom, double* w,
-                                        double& lf, double& ld, double& ld2) {
-  ld2 = 0.0;
+__device__ __forceinline__ void link_of(int link, const double* z, double yd, double zp, double mom, double* w) {
 #pragma unroll
   for (int q = 0; q < NB; ++q) w[q] = 0.0;
-  lf = 0.0;
-  ld = 0.0;
   switch (link) {
     case LINK_LS:
       w[0] = 2.0 * (z[0] - yd);
@@ -264,41 +259,53 @@ __device__ __forceinline__ void link_of(int link, const double* z, double yd, do
       w[0] = z[0];
       break;
     case LINK_CERT_LS:
-    case LINK_CERTZ_LS: {
-      const double zd = link == LINK_CERT_LS ? z[NF - 1] : zp;
-      const double d0 = z[0] - yd, d1 = zd - yd, zeta = -2.0 * d1;
-      w[0] = 2.0 * d1;
-      lf = d0 * d0;
-      ld = zeta * yd - 0.25 * zeta * zeta;
+    case LINK_CERTZ_LS:
+      w[0] = 2.0 * ((link == LINK_CERT_LS ? z[NF - 1] : zp) - yd);
       break;
-    }
     case LINK_CERT_LOGI:
-    case LINK_CERTZ_LOGI: {
-      const double zd = link == LINK_CERT_LOGI ? z[NF - 1] : zp;
-      w[0] = -yd / (1.0 + exp(yd * zd));
-      lf = softplus_neg(yd * z[0]);
-      ld = entropy_of(yd * zd);
+    case LINK_CERTZ_LOGI:
+      w[0] = -yd / (1.0 + exp(yd * (link == LINK_CERT_LOGI ? z[NF - 1] : zp)));
       break;
-    }
-    case LINK_CERT2_LS: {
-      const double d0 = z[0] - yd, d1 = zp - yd;
-      w[0] = 2.0 * d1;
-      if (NB > 1) w[NB - 1] = 2.0 * d0;
-      const double zeta1 = -2.0 * d1, zeta0 = -2.0 * d0;
-      lf = d0 * d0;
-      ld = zeta1 * yd - 0.25 * zeta1 * zeta1;
-      ld2 = zeta0 * yd - 0.25 * zeta0 * zeta0;
+    case LINK_CERT2_LS:
+      w[0] = 2.0 * (zp - yd);
+      if (NB > 1) w[NB - 1] = 2.0 * (z[0] - yd);
       break;
-    }
-    case LINK_CERT2_LOGI: {
+    case LINK_CERT2_LOGI:
       w[0] = -yd / (1.0 + exp(yd * zp));
       if (NB > 1) w[NB - 1] = -yd / (1.0 + exp(yd * z[0]));
-      lf = softplus_neg(yd * z[0]);
-      ld = entropy_of(yd * zp);
-      ld2 = entropy_of(yd * z[0]);
       break;
-    }
     default: break;
+  }
+}
+
+// Loss terms of one row, taken only by the lane that records it: s[0] += the F
+// term at z[0], s[1] += the -F*(-zeta) term of the dual point (z[0] itself in
+// the loop), s[2] += the same at the second dual point (LINK_CERT2_*: z[0]).
+template <int NF, bool LOWP>
+__device__ __forceinline__ void loss_of(int link, const double* z, double yd, double zp, double (&s)[3]) {
+  if (link == LINK_IDENT) return;
+  const bool ls = link == LINK_LS || link == LINK_CERT_LS || link == LINK_CERTZ_LS || link == LINK_CERT2_LS;
+  const bool loop = link == LINK_LS || link == LINK_LOGISTIC;
+  const bool two = link == LINK_CERT2_LS || link == LINK_CERT2_LOGI;
+  const double zd = loop ? z[0] : (link == LINK_CERT_LS || link == LINK_CERT_LOGI) ? z[NF - 1] : zp;
+  if (ls) {
+    auto dual = [&](double d) {
+      const double zeta = -2.0 * d;
+      return zeta * yd - 0.25 * zeta * zeta;
+    };
+    const double d0 = z[0] - yd;
+    s[0] += d0 * d0;
+    s[1] += dual(zd - yd);
+    if (two) s[2] += dual(d0);
+  } else if (LOWP && loop) {
+    float f, h;
+    logistic_terms_f((float)(yd * z[0]), f, h);
+    s[0] += (double)f;
+    s[1] += (double)h;
+  } else {
+    s[0] += softplus_neg(yd * z[0]);
+    s[1] += entropy_of(yd * zd);
+    if (two) s[2] += entropy_of(yd * z[0]);
   }
 }
 
@@ -375,6 +382,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
   TA acc[NB][TV][VEC];
   float ahi[kF32 && !FF ? NB : 1][TV][VEC], alo[kF32 && !FF ? NB : 1][TV][VEC];
   float accl[FF ? NB : 1][TV][VEC];   // FF: low parts of acc
+  double lsum[3] = {0.0, 0.0, 0.0};   // loss terms of the rows this lane records
   const bool axpy = warp >= 2 + a.SA && warp < 2 + a.SA + a.SB;
 
   if (warp == 0) {
@@ -705,8 +713,8 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
       double z[NF];
 #pragma unroll
       for (int f = 0; f < NF; ++f) z[f] = (double)(long long)__ldcg(&a.zfix[(size_t)f * n + rowj]) * zinv[f];
-      double rv[NB], lf, ld, ld2;
-      link_of<NF, NB, kF32 && !FF>(a.link, z, yd, zp, mom, rv, lf, ld, ld2);
+      double rv[NB];
+      link_of<NF, NB, kF32 && !FF>(a.link, z, yd, zp, mom, rv);
       if (jl >= rows) {
 #pragma unroll
         for (int q = 0; q < NB; ++q) rv[q] = 0.0;   // rows past the end carry weight 0
@@ -722,8 +730,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
       }
       if (cc == k % a.Gc && hb == 0 && jl < rows) {   // this CTA records the block
         if (zout) zout[r0 + jl] = z[0];
-        if (a.lterm) { a.lterm[2 * (r0 + jl)] = lf; a.lterm[2 * (r0 + jl) + 1] = ld; }
-        if (a.lterm2) { a.lterm2[2 * (r0 + jl)] = lf; a.lterm2[2 * (r0 + jl) + 1] = ld2; }
+        if (a.lsum) loss_of<NF, kF32 && !FF>(a.link, z, yd, zp, lsum);
       }
       const int sb = k % a.RB;   // one of this warp's stages
       if (!__all_sync(0xffffffffu, mbar_wait<false>(&fullB[sb], (k / a.RB) & 1, a.limit_ns, a.status))) {
@@ -811,7 +818,10 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
   }
   __syncthreads();   // every copy has landed: the rings are free
   const int wcols = nvs * VEC;
-  double* comb = reinterpret_cast<double*>(smem);   // [SB][NB][wcols] strip sums of the axpy warps
+  // the axpy warps' strip sums, [SB][NB][wcols]: FP32 pairs, FP64 for FP64 X
+  float2* combf = reinterpret_cast<float2*>(smem);
+  double* combd = reinterpret_cast<double*>(smem);
+  __shared__ double lcomb[XS_MAXS][3];
   if (axpy) {
     const int st = warp - 2 - a.SA;
 #pragma unroll
@@ -822,24 +832,52 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
         for (int l = 0; l < VEC; ++l) {
           const int e = (lane + 32 * t) * VEC + l;
           if (e < wcols) {
-            double v;
-            if constexpr (FF) v = (double)acc[q][t][l] + (double)accl[q][t][l];
-            else v = kF32 ? (double)ahi[q][t][l] + (double)alo[q][t][l] : (double)acc[q][t][l];
-            comb[((size_t)st * NB + q) * wcols + e] = v;
+            const size_t o = ((size_t)st * NB + q) * wcols + e;
+            if constexpr (FF) combf[o] = make_float2(acc[q][t][l], accl[q][t][l]);
+            else if constexpr (kF32) combf[o] = make_float2(ahi[q][t][l], alo[q][t][l]);
+            else combd[o] = acc[q][t][l];
           }
         }
+    if (a.lsum) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const double v = warp_sum(lsum[i]);
+        if (lane == 0) lcomb[st][i] = v;
+      }
+    }
   }
   __syncthreads();
-  // fixed-order sum of the SB warps' strip sums -> g[cr][q][s0 + e]
+  // fixed-order sum of the SB warps' strip sums -> g[cr][q][s0 + e].  Pairs are
+  // summed in float-float (FP64 additions and conversions of every column
+  // would take about as long as the whole pass of a small design)
   const int64_t ncol = s1 - s0;
   for (int64_t e = tid; e < ncol; e += blockDim.x) {
-    const double sc = a.colscale ? (double)a.colscale[s0 + e] : 1.0;
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
-      double sum = 0.0;
-      for (int w = 0; w < a.SB; ++w) sum += comb[((size_t)w * NB + q) * wcols + e];
-      a.g[((size_t)cr * NB + q) * p + s0 + e] = sum * sc;
+      const size_t at = ((size_t)cr * NB + q) * p + s0 + e;
+      if constexpr (kF32) {
+        ffs sum{0.f, 0.f};
+        for (int w = 0; w < a.SB; ++w) {
+          const float2 v = combf[((size_t)w * NB + q) * wcols + e];
+          sum = ff_add(sum, ffs{v.x, v.y});
+        }
+        if (a.colscale) {   // FP8: times the column's scale, the product's error kept
+          const float sc = a.colscale[s0 + e], h = sum.hi * sc;
+          sum = ff_add(ffs{h, fmaf(sum.hi, sc, -h)}, ffs{sum.lo * sc, 0.f});
+        }
+        static_cast<float2*>(a.g)[at] = make_float2(sum.hi, sum.lo);
+      } else {
+        double sum = 0.0;
+        for (int w = 0; w < a.SB; ++w) sum += combd[((size_t)w * NB + q) * wcols + e];
+        static_cast<double*>(a.g)[at] = sum;
+      }
     }
+  }
+  if (a.lsum && tid < 4) {
+    double v = 0.0;
+    if (tid < 3)
+      for (int w = 0; w < a.SB; ++w) v += lcomb[w][tid];
+    a.lsum[4 * (size_t)blockIdx.x + tid] = v;
   }
 }
 
