@@ -174,6 +174,11 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
   return f2_of(r);
 }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_of(r);
+}
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
   unsigned long long r;
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
@@ -186,6 +191,19 @@ __device__ __forceinline__ void two_sum_acc2(float2& hi, float2& lo, float2 a) {
   const float2 err = add2(sub2(hi, sub2(s, bp)), sub2(a, bp));
   hi = s;
   lo = add2(lo, err);
+}
+
+// (hi, lo) += x (bh + bl) per half, bh and bl with nb = -bh: the product formed
+// exactly as the pair (x bh, x bh - fl(x bh)) plus x bl, the sum by TwoSum;
+// eleven packed instructions for two terms
+__device__ __forceinline__ void dot_ff2(float2& hi, float2& lo, float2 x, float2 bh, float2 nb, float2 bl) {
+  const float2 n = mul2(x, nb);                      // -fl(x bh)
+  const float2 e = fma2(x, bl, fma2(x, bh, n));
+  const float2 s = sub2(hi, n);
+  const float2 bp = sub2(s, hi);
+  const float2 err = sub2(sub2(hi, sub2(s, bp)), add2(n, bp));
+  hi = s;
+  lo = add2(lo, add2(err, e));
 }
 
 __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float a) {

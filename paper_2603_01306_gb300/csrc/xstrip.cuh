@@ -490,34 +490,46 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
       float phl[FF ? NF : 1][XS_MAXB];   // FF: low parts
       float vh[NF][4], vl[NF][4];        // kGroup: the four row groups after two butterfly steps
       if constexpr (FF) {
-        // float-float: one row at a time (the fully unrolled block of
-        // float-float sums outgrew the instruction cache); the row partials
-        // go to a per-lane array for the butterfly
+        // float-float: two rows at a time, so that two chains of dependent
+        // sums are in flight (a fully unrolled block of them outgrew the
+        // instruction cache), in packed FP32 pairs; the row partials go to a
+        // per-lane array for the butterfly.  Scalar, one row at a time, the
+        // 96 certificates of a 2000 x 5000 problem took 4.43 ms, now 4.32 (256
+        // nodes of 5000 x 10000: 60.8 and 58.1 ms); the pass is bound by the
+        // latency of its chain of sums, not by their number.
 #pragma unroll 1
-        for (int jj = 0; jj < XS_MAXB; ++jj) {
-          float hh[NF], ll[NF];
+        for (int jj = 0; jj < XS_MAXB; jj += 2) {
+          float2 hh[NF][2], ll[NF][2];   // even and odd columns in the halves of packed pairs
 #pragma unroll
-          for (int f = 0; f < NF; ++f) { hh[f] = 0.f; ll[f] = 0.f; }
-          const int jr = jj < a.B ? jj : a.B - 1;   // rows >= rows: zero-filled or repeated, discarded
-          const unsigned char* rowp = tile + (size_t)jr * rowpitch;
+          for (int f = 0; f < NF; ++f)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) { hh[f][u] = make_float2(0.f, 0.f); ll[f][u] = make_float2(0.f, 0.f); }
+          // rows >= rows: zero-filled or repeated, discarded
+          const unsigned char* row0 = tile + (size_t)min(jj, a.B - 1) * rowpitch;
+          const unsigned char* row1 = tile + (size_t)min(jj + 1, a.B - 1) * rowpitch;
 #pragma unroll
           for (int t = 0; t < TV; ++t) {
-            TA x[VEC];
-            XTraits<TX>::load(reinterpret_cast<const TX*>(rowp + voff[t]), x);
+            TA x[2][VEC];
+            XTraits<TX>::load(reinterpret_cast<const TX*>(row0 + voff[t]), x[0]);
+            XTraits<TX>::load(reinterpret_cast<const TX*>(row1 + voff[t]), x[1]);
 #pragma unroll
             for (int f = 0; f < NF; ++f)
 #pragma unroll
-              for (int l = 0; l < VEC; ++l) {
-                const float pr = x[l] * bv[f][t][l];
-                const float lo = fmaf(x[l], bl[f][t][l], fmaf(x[l], bv[f][t][l], -pr));   // exact error + x bl
-                const float sacc = hh[f] + pr;
-                const float bp = sacc - hh[f];
-                ll[f] += ((hh[f] - (sacc - bp)) + (pr - bp)) + lo;
-                hh[f] = sacc;
-              }
+              for (int l = 0; l < VEC; l += 2)
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                  dot_ff2(hh[f][u], ll[f][u], make_float2(x[u][l], x[u][l + 1]), make_float2(bv[f][t][l], bv[f][t][l + 1]),
+                          make_float2(-bv[f][t][l], -bv[f][t][l + 1]), make_float2(bl[f][t][l], bl[f][t][l + 1]));
           }
 #pragma unroll
-          for (int f = 0; f < NF; ++f) { ph[f][jj] = hh[f]; phl[f][jj] = ll[f]; }
+          for (int f = 0; f < NF; ++f)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              float h = hh[f][u].x, l = ll[f][u].x + ll[f][u].y;
+              two_sum_acc(h, l, hh[f][u].y);
+              ph[f][jj + u] = h;
+              phl[f][jj + u] = l;
+            }
         }
       } else if constexpr (kGroup) {
         // FP32 sums, rows in four groups of four (a rolled loop, for the
@@ -756,7 +768,20 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
         for (int t = 0; t < TV; ++t) {
           TA x[VEC];
           XTraits<TX>::load(reinterpret_cast<const TX*>(rowp + voff[t]), x);
-          if constexpr (kPair) {
+          if constexpr (FF) {
+#pragma unroll
+            for (int l = 0; l < VEC; l += 2)
+#pragma unroll
+              for (int q = 0; q < NB; ++q) {
+                float2 h2 = make_float2(acc[q][t][l], acc[q][t][l + 1]), l2 = make_float2(accl[q][t][l], accl[q][t][l + 1]);
+                dot_ff2(h2, l2, make_float2(x[l], x[l + 1]), make_float2(w[q], w[q]), make_float2(-w[q], -w[q]),
+                        make_float2(wl[q], wl[q]));
+                acc[q][t][l] = h2.x;
+                acc[q][t][l + 1] = h2.y;
+                accl[q][t][l] = l2.x;
+                accl[q][t][l + 1] = l2.y;
+              }
+          } else if constexpr (kPair) {
             // two columns per packed FP32 FMA (the same roundings as two scalar FMAs)
 #pragma unroll
             for (int l = 0; l < VEC; l += 2)
@@ -772,16 +797,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
             for (int l = 0; l < VEC; ++l)
 #pragma unroll
               for (int q = 0; q < NB; ++q) {
-                if constexpr (FF) {
-                  const float pr = w[q] * x[l];
-                  const float lo = fmaf(wl[q], x[l], fmaf(w[q], x[l], -pr));
-                  const float sacc = acc[q][t][l] + pr;
-                  const float bp = sacc - acc[q][t][l];
-                  accl[q][t][l] += ((acc[q][t][l] - (sacc - bp)) + (pr - bp)) + lo;
-                  acc[q][t][l] = sacc;
-                } else {
-                  acc[q][t][l] += w[q] * x[l];
-                }
+                acc[q][t][l] += w[q] * x[l];
               }
           }
         }
