@@ -27,11 +27,16 @@ struct XSPlan {
   int B = 1, nblk = 1;     // rows per block, blocks
   int SA = 3, SB = 3, lag = 4;
   int RA = 3, RB = 3;       // ring stages, multiples of SA / SB
+  bool mma = false;         // the tensor-core pass (BF16 / FP8, xmma.cuh)
+  int vpb = 1, spb = 1, steps = 1;   // its vectors and steps per box, steps per strip
   int grid = 1, threads = 32;
   size_t smem = 0;
   const void* kernel = nullptr;
 };
 cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t n, int64_t p);
+// the BF16 / FP8 plans (xmma.cu; xstrip_plan and xstrip_launch go there)
+cudaError_t xmma_plan(XSPlan& pl, int xk, int NB, int64_t n, int64_t p);
+cudaError_t xmma_launch(const XSPlan& pl, const XSArgs& a, cudaStream_t st);
 // encode the plan's tensor map of X (16-byte aligned, ldx * size a multiple of 16)
 cudaError_t xstrip_bind(XSPlan& pl, const void* X, int64_t ldx, int64_t n, int64_t p);
 // The per-pass area (block counters, the grid's max |beta|, z in fixed point;

@@ -56,36 +56,6 @@ template <> struct XTraits<float> {
   template <typename TA> __device__ static void load_global(const float* p, TA* o) { cvt(__ldcg(reinterpret_cast<const float4*>(p)), o); }
   template <typename TA> __device__ static void load_global_last(const float* p, TA* o) { cvt(__ldcs(reinterpret_cast<const float4*>(p)), o); }
 };
-template <> struct XTraits<__nv_bfloat16> {
-  static constexpr int VEC = 8;
-  template <typename TA> __device__ static void cvt(const uint4 v, TA* o) {
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float2 f = __bfloat1622float2(h[i]);
-      o[2 * i] = (TA)f.x; o[2 * i + 1] = (TA)f.y;
-    }
-  }
-  template <typename TA> __device__ static void load(const __nv_bfloat16* p, TA* o) { cvt(*reinterpret_cast<const uint4*>(p), o); }
-  template <typename TA> __device__ static void load_global(const __nv_bfloat16* p, TA* o) { cvt(__ldcg(reinterpret_cast<const uint4*>(p)), o); }
-  template <typename TA> __device__ static void load_global_last(const __nv_bfloat16* p, TA* o) { cvt(__ldcs(reinterpret_cast<const uint4*>(p)), o); }
-};
-template <> struct XTraits<__nv_fp8_e4m3> {
-  static constexpr int VEC = 16;
-  template <typename TA> __device__ static void cvt(const uint4 v, TA* o) {
-    const __nv_fp8x2_storage_t* h = reinterpret_cast<const __nv_fp8x2_storage_t*>(&v);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      __half2_raw hr = __nv_cvt_fp8x2_to_halfraw2(h[i], __NV_E4M3);
-      float2 f = __half22float2(*reinterpret_cast<__half2*>(&hr));
-      o[2 * i] = (TA)f.x; o[2 * i + 1] = (TA)f.y;
-    }
-  }
-  template <typename TA> __device__ static void load(const __nv_fp8_e4m3* p, TA* o) { cvt(*reinterpret_cast<const uint4*>(p), o); }
-  template <typename TA> __device__ static void load_global(const __nv_fp8_e4m3* p, TA* o) { cvt(__ldcg(reinterpret_cast<const uint4*>(p)), o); }
-  template <typename TA> __device__ static void load_global_last(const __nv_fp8_e4m3* p, TA* o) { cvt(__ldcs(reinterpret_cast<const uint4*>(p)), o); }
-};
-
 // Float-float sums (Knuth's TwoSum; about 48 significant bits from FP32
 // instructions).  This GPU issues FP64 arithmetic, comparisons and
 // conversions at about 1.6 lanes per clock per SM against about 112 for FP32

@@ -19,8 +19,6 @@ static const void* xstrip_ptr(int xk, bool f64acc, int NF, int NB) {
     if (xk == XK_F64) return kptr<double, double, 1, 1>();
     // FP32 X: the certificate / power-iteration pass in float-float arithmetic
     if (xk == XK_F32) return f64acc ? kptr<float, float, 1, 1, true>() : kptr<float, float, 1, 1>();
-    if (xk == XK_BF16 && !f64acc) return kptr<__nv_bfloat16, float, 1, 1>();
-    if (xk == XK_FP8 && !f64acc) return kptr<__nv_fp8_e4m3, float, 1, 1>();
   } else if (NF == 1 && NB == 2 && f64acc) {
     // the logistic loop's float-float pass; the two-dual-point certificate
     if (xk == XK_F32) return kptr<float, float, 1, 2, true>();
@@ -28,8 +26,6 @@ static const void* xstrip_ptr(int xk, bool f64acc, int NF, int NB) {
   } else if (NF == 1 && NB == 2 && !f64acc) {
     if (xk == XK_F64) return kptr<double, double, 1, 2>();
     if (xk == XK_F32) return kptr<float, float, 1, 2>();
-    if (xk == XK_BF16) return kptr<__nv_bfloat16, float, 1, 2>();
-    if (xk == XK_FP8) return kptr<__nv_fp8_e4m3, float, 1, 2>();
   } else if (NF == 2 && NB == 1) {
     if (xk == XK_F64) return kptr<double, double, 2, 1>();
     if (xk == XK_F32 && f64acc) return kptr<float, float, 2, 1, true>();
@@ -37,7 +33,7 @@ static const void* xstrip_ptr(int xk, bool f64acc, int NF, int NB) {
   return nullptr;
 }
 
-static int xs_tv(int vec) { return vec == 2 ? 6 : vec == 4 ? 6 : vec == 8 ? 3 : 2; }   // XSShape<VEC>::TV
+static int xs_tv(int vec) { return vec == 2 ? XSShape<2>::TV : XSShape<4>::TV; }
 
 // Shape of the pass for an n x p design.
 //  * strips of a row of at most 32*TV vectors (the registers of one lane
@@ -50,6 +46,7 @@ static int xs_tv(int vec) { return vec == 2 ? 6 : vec == 4 ? 6 : vec == 8 ? 3 : 
 //    least 20 blocks with four or more row groups).
 // RELAX_XS="B,SA,SB,lag,vps,mA,mB,Gr" overrides for tuning runs (0 keeps a default).
 cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t n, int64_t p) {
+  if ((xk == XK_BF16 || xk == XK_FP8) && !f64acc && NF == 1) return xmma_plan(pl, xk, NB, n, p);
   pl = XSPlan{};
   pl.xk = xk;
   pl.cert = f64acc;
@@ -220,6 +217,7 @@ cudaError_t xstrip_launch(const XSPlan& pl, const XSArgs& a, bool clear, cudaStr
     const cudaError_t e = cudaMemsetAsync(a.cnt, 0, xstrip_zero_bytes(pl, a.n), st);
     if (e != cudaSuccess) return e;
   }
+  if (pl.mma) return xmma_launch(pl, a, st);
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;

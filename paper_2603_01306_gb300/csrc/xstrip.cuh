@@ -56,9 +56,9 @@ constexpr int XS_MAXR = 12;       // stages per ring at most
 constexpr int XS_MAXB = 16;       // rows per block at most (one butterfly group)
 constexpr int XS_MAXT = 256;      // 2 + SA + SB warps: at most two per scheduler
 // 16-byte vectors of the strip per lane: a lane holds the same number of
-// accumulators (24 FP32 or 12 FP64 columns, 24/32 for 16/8-bit X) for every type
+// accumulators (24 FP32 or 12 FP64 columns)
 template <int VEC> struct XSShape {
-  static constexpr int TV = VEC == 2 ? 6 : VEC == 4 ? 6 : VEC == 8 ? 3 : 2;
+  static constexpr int TV = 6;
 };
 
 struct XSArgs {
@@ -73,7 +73,7 @@ struct XSArgs {
   int RA, RB;            // ring stages (multiples of SA / SB)
   int link;
   const double* y;
-  const float* colscale;
+  const float* colscale; // FP8 storage (xmma.cuh): the columns' scales
   PassState* ps;
   unsigned long long* zfix;   // [NF][n] z in fixed point (two's complement)   } zeroed
   unsigned long long* zmax;   // [NF] max_j |beta_j| (bits of a nonnegative double) } before
@@ -165,28 +165,6 @@ __device__ __forceinline__ void pair_add(float& h, float& l, float rh, float rl)
   two_sum_acc(s, e, rh);
   h = s;
   l = l + rl + e;
-}
-
-// Steps of a transposed butterfly over N = 2^m rows, at lane strides o0,
-// o0/2, ...: each step sends half of the remaining rows to the partner lane
-// and keeps the other half (the upper half on lanes with the stride's bit
-// set); afterwards h[0], l[0] hold the sum over those m lane bits of the row
-// whose index bits, high to low, are the lane's bits o0, o0/2, ...
-template <int N>
-__device__ __forceinline__ void bfly_steps(float (&h)[N], float (&l)[N], int lane, int o0) {
-#pragma unroll
-  for (int half = N / 2, o = o0; half >= 1; half >>= 1, o >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < half; ++i) {
-      const float sh = up ? h[i] : h[i + half], sl = up ? l[i] : l[i + half];
-      const float kh = up ? h[i + half] : h[i], kl = up ? l[i + half] : l[i];
-      const float rh = __shfl_xor_sync(0xffffffffu, sh, o), rl = __shfl_xor_sync(0xffffffffu, sl, o);
-      h[i] = kh;
-      l[i] = kl;
-      pair_add(h[i], l[i], rh, rl);
-    }
-  }
 }
 
 // Transposed butterfly over 16 rows: on entry lane L holds its partial of
@@ -321,12 +299,9 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
   constexpr int TV = XSShape<VEC>::TV;
   constexpr bool kF32 = sizeof(TA) == 4;
   // FP32 sums on packed pairs (f32x2): measured faster wherever the pass does
-  // more than one FMA per 4 bytes of X (two right-hand sides, BF16 / FP8
-  // elements); the one-right-hand-side FP32 pass ran 10% slower on pairs
-  constexpr bool kPair = kF32 && !FF && !(sizeof(TX) == 4 && NB == 1);
-  // FP8 (16 elements per vector): the dot warps' rows in a rolled loop of
-  // four-row groups (measured faster there, slower for FP32 and BF16)
-  constexpr bool kGroup = kPair && sizeof(TX) == 1;
+  // more than one FMA per 4 bytes of X (two right-hand sides); the
+  // one-right-hand-side FP32 pass ran 10% slower on pairs
+  constexpr bool kPair = kF32 && !FF && NB == 2;
   static_assert(!FF || (sizeof(TX) == 4 && kF32), "float-float: FP32 X and FP32 pairs");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t fullA[XS_MAXR], emptyA[XS_MAXR], fullB[XS_MAXR], emptyB[XS_MAXR];
@@ -436,10 +411,9 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
       for (int l = 0; l < VEC; ++l) {
         const int64_t col = s0 + (int64_t)v * VEC + l;
         const bool in = v < nvs && col < p;
-        const double sc = (in && a.colscale) ? (double)a.colscale[col] : 1.0;
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
-          const double bd = in ? static_cast<const double*>(f == 0 ? a.ps->beta : a.ps->beta2)[col] * sc : 0.0;
+          const double bd = in ? static_cast<const double*>(f == 0 ? a.ps->beta : a.ps->beta2)[col] : 0.0;
           bv[f][t][l] = (TA)bd;
           if constexpr (FF) bl[f][t][l] = (float)(bd - (double)bv[f][t][l]);
         }
@@ -488,7 +462,6 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
       // columns), then one transposed butterfly per forward vector
       TA ph[NF][XS_MAXB];
       float phl[FF ? NF : 1][XS_MAXB];   // FF: low parts
-      float vh[NF][4], vl[NF][4];        // kGroup: the four row groups after two butterfly steps
       if constexpr (FF) {
         // float-float: two rows at a time, so that two chains of dependent
         // sums are in flight (a fully unrolled block of them outgrew the
@@ -530,61 +503,6 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
               ph[f][jj + u] = h;
               phl[f][jj + u] = l;
             }
-        }
-      } else if constexpr (kGroup) {
-        // FP32 sums, rows in four groups of four (a rolled loop, for the
-        // schedulers' instruction caches): group g holds rows g, g+4, g+8,
-        // g+12, whose partials take the butterfly's first two steps (lane
-        // strides 16, 8) in the group and the last ones (4, 2, 1) after the
-        // loop -- the additions of the 16-row butterfly, in its order
-#pragma unroll 1
-        for (int g = 0; g < 4; ++g) {
-          float gh[NF][4], gl[NF][4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int jj = g + 4 * i;
-            const int jr = jj < a.B ? jj : a.B - 1;   // rows >= rows: zero-filled or repeated, discarded
-            const unsigned char* rowp = tile + (size_t)jr * rowpitch;
-            if constexpr (kPair) {
-              // even and odd columns in the two halves of a packed pair
-              float2 p2[NF];
-#pragma unroll
-              for (int f = 0; f < NF; ++f) p2[f] = make_float2(0.f, 0.f);
-#pragma unroll
-              for (int t = 0; t < TV; ++t) {
-                TA x[VEC];
-                XTraits<TX>::load(reinterpret_cast<const TX*>(rowp + voff[t]), x);
-#pragma unroll
-                for (int f = 0; f < NF; ++f)
-#pragma unroll
-                  for (int l = 0; l < VEC; l += 2)
-                    p2[f] = fma2(make_float2(x[l], x[l + 1]), make_float2(bv[f][t][l], bv[f][t][l + 1]), p2[f]);
-              }
-#pragma unroll
-              for (int f = 0; f < NF; ++f) gh[f][i] = p2[f].x + p2[f].y;
-            } else {
-#pragma unroll
-              for (int f = 0; f < NF; ++f) gh[f][i] = 0.f;
-#pragma unroll
-              for (int t = 0; t < TV; ++t) {
-                TA x[VEC];
-                XTraits<TX>::load(reinterpret_cast<const TX*>(rowp + voff[t]), x);
-#pragma unroll
-                for (int f = 0; f < NF; ++f)
-#pragma unroll
-                  for (int l = 0; l < VEC; ++l) gh[f][i] += x[l] * bv[f][t][l];
-              }
-            }
-#pragma unroll
-            for (int f = 0; f < NF; ++f) gl[f][i] = 0.f;
-          }
-#pragma unroll
-          for (int f = 0; f < NF; ++f) {
-            bfly_steps<4>(gh[f], gl[f], lane, 16);
-#pragma unroll
-            for (int gg = 0; gg < 4; ++gg)   // registers, not an indexed array
-              if (gg == g) { vh[f][gg] = gh[f][0]; vl[f][gg] = gl[f][0]; }
-          }
         }
       } else {
 #pragma unroll
@@ -635,12 +553,6 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
           butterfly16(ph[f], phl[f], lane);
           mh[f] = ph[f][0];
           ml[f] = phl[f][0];
-        } else if constexpr (kGroup) {
-          bfly_steps<4>(vh[f], vl[f], lane, 4);
-          const float rh = __shfl_xor_sync(0xffffffffu, vh[f][0], 1), rl = __shfl_xor_sync(0xffffffffu, vl[f][0], 1);
-          pair_add(vh[f][0], vl[f][0], rh, rl);
-          mh[f] = vh[f][0];
-          ml[f] = vl[f][0];
         } else if constexpr (kF32) {
           float pl[XS_MAXB];
 #pragma unroll
@@ -876,10 +788,6 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
         for (int w = 0; w < a.SB; ++w) {
           const float2 v = combf[((size_t)w * NB + q) * wcols + e];
           sum = ff_add(sum, ffs{v.x, v.y});
-        }
-        if (a.colscale) {   // FP8: times the column's scale, the product's error kept
-          const float sc = a.colscale[s0 + e], h = sum.hi * sc;
-          sum = ff_add(ffs{h, fmaf(sum.hi, sc, -h)}, ffs{sum.lo * sc, 0.f});
         }
         static_cast<float2*>(a.g)[at] = make_float2(sum.hi, sum.lo);
       } else {
