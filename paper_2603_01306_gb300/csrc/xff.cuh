@@ -1,0 +1,376 @@
+// Fused pass over FP32 X in float-float arithmetic (the certificates, the power
+// iteration, the last digits of FP32 solves): z = X beta, r = link(z),
+// g = X' r, X read from HBM once.
+//
+// Strips x row groups, tiles kept in a ring from their dot products until
+// their axpy, the rows' words of z with their own arrival counts, link warps of
+// their own: as in xmma.cuh.  Each product x b, b = bh + bl, is formed exactly
+// as the FMA pair plus x bl and summed by TwoSum, in packed FP32 pairs
+// (dot_ff2: eleven instructions for two terms, about 48 significant bits).
+//
+// The sums are what bounds it: 5.5 packed instructions per element and
+// product, 22 us of the FP32 pipes for 5000 x 10000 at two cycles each, against
+// 30 us for X from HBM.  Hence twelve warps of them, three per scheduler, six
+// per product, in the registers of 512 threads:
+//  * a dot warp holds the strip of beta (hi, lo) and takes two rows of a block
+//    at a time;
+//  * an axpy warp owns 32 vectors of the strip and takes all rows, the weights
+//    read as ready operand pairs from shared memory.
+// 2000 x 5000, 96 certificates: 45 us each on the rows-and-columns kernel of
+// xstrip.cuh (one right-hand side; six summing warps, two per scheduler at most)
+// and 29 here; 5000 x 10000, two right-hand sides: 171 and 99 us.  What is left
+// over the pipes' 45 to 67 us is the depth of the ring (four blocks of 46 KB
+// between HBM and the end of their agreement) and, in small problems, filling
+// it.  Blocks of 8 rows: certificates 3% slower.
+// z in fixed point, two 64-bit words per row (8 bits of count each; the second
+// holds 44 further bits), converted by shifts: FP64 conversions of two lanes
+// per row pair would have taken as long as the sums.
+#pragma once
+#include "xmma.cuh"
+
+namespace relax {
+
+constexpr int XF_SA = 6, XF_SB = 6, XF_NL = 3;   // dot, axpy and link warps
+constexpr int XF_T = 32 * (1 + XF_SA + XF_SB + XF_NL);
+constexpr int XF_TV = XF_SB;                     // vectors of the strip per lane of a dot warp
+constexpr int XF_B = 16;                          // rows of a block
+constexpr int XF_LB = 16 / XF_B;                 // blocks a link warp takes at a time
+constexpr int XF_RW = 2 * XF_LB * XF_NL;         // blocks of weights in shared memory
+constexpr int XF_MAXR = 16;                      // ring stages at most
+constexpr int XF_LO = 44;                        // bits of the second word below the first's unit
+
+// m 2^sh as hi + lo 2^-XF_LO, in two's complement (|m 2^sh| < 2^54)
+__device__ __forceinline__ void fixed_words(float m, int sh, long long& hi, long long& lo) {
+  const uint32_t b = __float_as_uint(m);
+  const int ex = (int)((b >> 23) & 255u);
+  const unsigned long long mant = ex ? (b & 0x7fffffu) | 0x800000u : b & 0x7fffffu;
+  const int k = min((ex ? ex : 1) - 150 + sh, 38);   // |m| 2^sh = mant 2^k
+  long long h = 0, l = 0;
+  if (k >= 0) {
+    h = (long long)(mant << k);
+  } else {
+    const unsigned long long rem = k > -24 ? mant & ((1ull << -k) - 1ull) : mant;
+    if (k > -24) h = (long long)(mant >> -k);
+    const int s = k + XF_LO;
+    l = s >= 0 ? (long long)(rem << s) : s > -32 ? (long long)((rem + (1ull << (-s - 1))) >> -s) : 0ll;
+  }
+  const bool neg = (b >> 31) != 0u;
+  hi += neg ? -h : h;
+  lo += neg ? -l : l;
+}
+
+// bounded wait until the low eight bits of both words of a row count `want` arrivals
+__device__ __forceinline__ bool wait_row2(const unsigned long long* p, unsigned want, unsigned long long& h, unsigned long long& l,
+                                          uint64_t limit_ns, int* status) {
+  uint64_t t0 = 0;
+  for (uint32_t it = 0;; ++it) {
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(h), "=l"(l) : "l"(p) : "memory");
+    if ((unsigned)(h & 255ull) == want && (unsigned)(l & 255ull) == want) return true;
+    if ((it & 15u) == 0u) {
+      const uint64_t t = globaltimer_ns();
+      if (it == 0) t0 = t;
+      else if (t - t0 > limit_ns) {
+        atomicCAS(status, ST_OK, ST_TIMEOUT);
+        return false;
+      }
+    }
+  }
+}
+
+template <int NB>
+__global__ void __launch_bounds__(XF_T, 1) xff_kernel(const __grid_constant__ XSArgs a) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t full[XF_MAXR], empty[XF_MAXR], wfull[XF_RW], wempty[XF_RW];
+  __shared__ __align__(16) float wts[XF_RW][XF_B][NB][8];   // wh wh -wh -wh wl wl
+  __shared__ volatile int tmo;
+  __shared__ int skip;
+  __shared__ double lcomb[XF_NL][3];
+  __shared__ __align__(16) float bsh[2][32 * XF_TV * 4];   // the strip of beta, hi and lo
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    tmo = 0;
+    skip = a.ps->done;
+    for (int s = 0; s < a.RA; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], XF_SB); }
+    for (int s = 0; s < XF_RW; ++s) { mbar_init(&wfull[s], 1); mbar_init(&wempty[s], XF_SB); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  if (skip) return;   // uniform (same flag everywhere)
+
+  unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
+  const int cc = blockIdx.x % a.Gc, cr = blockIdx.x / a.Gc;
+  const int64_t n = a.n, p = a.p;
+  const int64_t s0 = (int64_t)cc * a.sw;
+  const int nvs = (int)((min(s0 + a.sw, p) - s0 + 3) / 4);   // vectors of the strip
+  const uint32_t rowpitch = (uint32_t)a.inner * 4u;
+  const uint32_t tilebytes = (uint32_t)a.nbox * XF_B * rowpitch;   // whole boxes, out-of-range parts zero-filled
+  const int kloc = (cr < a.nblk) ? (a.nblk - cr + a.Gr - 1) / a.Gr : 0;
+  const size_t stage = (size_t)a.nbox * a.boxb;
+  const int vpb = a.inner / 4;
+  // byte offset of a vector in row 0 of a tile (vectors past the strip read its
+  // last one: their beta is zero and their sums are never written)
+  auto voffset = [&](int v) {
+    v = min(v, nvs - 1);
+    return (uint32_t)((v / vpb) * a.boxb + (v % vpb) * 16);
+  };
+
+  if (warp == 0) {
+    // ------------------------------------------------ producer: HBM -> ring
+    if (lane == 0) {
+      const uint64_t pol = policy_evict_first();
+      int issued = 0;
+      for (int k = 0; k < kloc; ++k) {
+        const int s = k % a.RA;
+        if (tmo) break;
+        if (k >= a.RA && !mbar_wait<false>(&empty[s], ((k / a.RA) - 1) & 1, a.limit_ns, a.status)) { tmo = 1; break; }
+        const int y0 = (cr + k * a.Gr) * XF_B;
+        mbar_arrive_expect_tx(&full[s], tilebytes);
+        for (int i = 0; i < a.nbox; ++i)
+          tma_load_2d(smem + s * stage + (size_t)i * a.boxb, &a.tm, (int)s0 + i * a.inner, y0, &full[s], pol);
+        issued = k + 1;
+      }
+      // let every copy in flight land before the CTA may exit
+      for (int k = (issued > a.RA ? issued - a.RA : 0); k < issued; ++k)
+        mbar_wait<false>(&full[k % a.RA], (k / a.RA) & 1, a.limit_ns, a.status);
+    }
+    __syncwarp();
+  } else if (warp < 1 + XF_SA) {
+    // ------------------------------------------------ phase A: strip dot products
+    const int st = warp - 1;
+    // the strip of beta as pairs, split once for all dot warps
+    unsigned long long mb = 0ull;
+    for (int c = tid - 32; c < 32 * XF_TV * 4; c += 32 * XF_SA) {
+      const int64_t col = s0 + c;
+      const double bd = c < (int)a.sw && col < p ? static_cast<const double*>(a.ps->beta)[col] : 0.0;
+      const float h = (float)bd;
+      bsh[0][c] = h;
+      bsh[1][c] = (float)(bd - (double)h);
+      unsigned long long bits = (unsigned long long)__double_as_longlong(bd) & ~(1ull << 63);
+      if (!(fabsf(h) < INFINITY) && bits < 0x7ff0000000000000ull) bits = 0x7ff0000000000000ull;   // beyond FP32
+      mb = bits > mb ? bits : mb;
+    }
+    // this CTA's max |beta_j| (NaN dominates: its bits compare above +Inf)
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long ob = __shfl_xor_sync(0xffffffffu, mb, o);
+      mb = ob > mb ? ob : mb;
+    }
+    if (lane == 0 && mb) atomicMax(&a.zmax[0], mb);
+    if (lane == 0) __threadfence();
+    named_sync(1, 32 * XF_SA);
+    if (st == 0 && lane == 0) {
+      __threadfence();
+      atomicAdd(a.zcnt, 1u);
+    }
+    float2 bh[XF_TV][2], nb[XF_TV][2], bl[XF_TV][2];
+    uint32_t voff[XF_TV];
+#pragma unroll
+    for (int t = 0; t < XF_TV; ++t) {
+      const int v = lane + 32 * t;
+      voff[t] = voffset(v);
+      const float4 h = *reinterpret_cast<const float4*>(&bsh[0][4 * v]), l = *reinterpret_cast<const float4*>(&bsh[1][4 * v]);
+      bh[t][0] = make_float2(h.x, h.y);
+      bh[t][1] = make_float2(h.z, h.w);
+      nb[t][0] = make_float2(-h.x, -h.y);
+      nb[t][1] = make_float2(-h.z, -h.w);
+      bl[t][0] = make_float2(l.x, l.y);
+      bl[t][1] = make_float2(l.z, l.w);
+    }
+    int zs = 0;
+    bool have_scale = false;
+    constexpr int UB = XF_B / 2;   // row pairs of a block
+    const int units = kloc * UB;
+#pragma unroll 1
+    for (int i = st; i < units; i += XF_SA) {
+      if (tmo) break;
+      const int k = i / UB, pr = i % UB;
+      const int sa = k % a.RA;
+      if (!__all_sync(0xffffffffu, mbar_wait<false>(&full[sa], (k / a.RA) & 1, a.limit_ns, a.status))) {
+        tmo = 1;
+        break;
+      }
+      const int64_t r0 = (int64_t)(cr + k * a.Gr) * XF_B + 2 * pr;
+      const unsigned char* row0 = smem + sa * stage + (size_t)(2 * pr) * rowpitch;
+      float2 hh[2], ll[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) { hh[u] = make_float2(0.f, 0.f); ll[u] = make_float2(0.f, 0.f); }
+#pragma unroll
+      for (int t = 0; t < XF_TV; ++t) {
+        if (32 * t < nvs) {   // uniform
+          const float4 x0 = *reinterpret_cast<const float4*>(row0 + voff[t]);
+          const float4 x1 = *reinterpret_cast<const float4*>(row0 + rowpitch + voff[t]);
+          dot_ff2(hh[0], ll[0], make_float2(x0.x, x0.y), bh[t][0], nb[t][0], bl[t][0]);
+          dot_ff2(hh[1], ll[1], make_float2(x1.x, x1.y), bh[t][0], nb[t][0], bl[t][0]);
+          dot_ff2(hh[0], ll[0], make_float2(x0.z, x0.w), bh[t][1], nb[t][1], bl[t][1]);
+          dot_ff2(hh[1], ll[1], make_float2(x1.z, x1.w), bh[t][1], nb[t][1], bl[t][1]);
+        }
+      }
+      float h[2], l[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        h[u] = hh[u].x;
+        l[u] = ll[u].x + ll[u].y;
+        two_sum_acc(h[u], l[u], hh[u].y);
+      }
+      // the lower half warp sums row 0, the upper one row 1
+      const bool up = (lane & 16) != 0;
+      float zh = up ? h[1] : h[0], zl = up ? l[1] : l[0];
+      pair_add(zh, zl, __shfl_xor_sync(0xffffffffu, up ? h[0] : h[1], 16), __shfl_xor_sync(0xffffffffu, up ? l[0] : l[1], 16));
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1)
+        pair_add(zh, zl, __shfl_xor_sync(0xffffffffu, zh, o), __shfl_xor_sync(0xffffffffu, zl, o));
+      if (!have_scale) {
+        if (!__all_sync(0xffffffffu, wait_count(a.zcnt, gridDim.x, a.limit_ns, a.status))) {
+          tmo = 1;
+          break;
+        }
+        zs = fixed_scale(a.rowl1 * __longlong_as_double((long long)__ldcg(&a.zmax[0])));
+        have_scale = true;
+      }
+      const int64_t row = r0 + (lane >> 4);
+      if ((lane & 15) == 0 && row < n) {
+        long long qh = 0, ql = 0;
+        if (zs != INT_MIN) {
+          fixed_words(zh, zs - 8, qh, ql);
+          fixed_words(zl, zs - 8, qh, ql);
+        }
+        atomicAdd(&a.zfix[2 * row], ((unsigned long long)qh << 8) + 1ull);
+        atomicAdd(&a.zfix[2 * row + 1], ((unsigned long long)ql << 8) + 1ull);
+      }
+    }
+  } else if (warp < 1 + XF_SA + XF_SB) {
+    // ------------------------------------------------ phase B: X' r over the strip
+    const int e = warp - 1 - XF_SA;
+    const int v = 32 * e + lane;
+    const bool on = 32 * e < nvs;   // uniform
+    const uint32_t voff = voffset(v);
+    float2 hi[NB][2], lo[NB][2];
+#pragma unroll
+    for (int q = 0; q < NB; ++q)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) { hi[q][u] = make_float2(0.f, 0.f); lo[q][u] = make_float2(0.f, 0.f); }
+    for (int k = 0; k < kloc; ++k) {
+      if (tmo) break;
+      const int ws = k % XF_RW, sb = k % a.RA;
+      const bool ok = mbar_wait<false>(&full[sb], (k / a.RA) & 1, a.limit_ns, a.status) &&
+                      mbar_wait<false>(&wfull[ws], (k / XF_RW) & 1, a.limit_ns, a.status);
+      if (!__all_sync(0xffffffffu, ok)) {
+        tmo = 1;
+        break;
+      }
+      if (on) {
+        const unsigned char* col = smem + sb * stage + voff;
+#pragma unroll 4
+        for (int j = 0; j < XF_B; ++j) {
+          const float4 x = *reinterpret_cast<const float4*>(col + (size_t)j * rowpitch);
+#pragma unroll
+          for (int q = 0; q < NB; ++q) {
+            const float4 w = *reinterpret_cast<const float4*>(&wts[ws][j][q][0]);
+            const float2 wl = *reinterpret_cast<const float2*>(&wts[ws][j][q][4]);
+            dot_ff2(hi[q][0], lo[q][0], make_float2(x.x, x.y), make_float2(w.x, w.y), make_float2(w.z, w.w), wl);
+            dot_ff2(hi[q][1], lo[q][1], make_float2(x.z, x.w), make_float2(w.x, w.y), make_float2(w.z, w.w), wl);
+          }
+        }
+        // the low parts folded back, so that their own rounding stays small
+#pragma unroll
+        for (int q = 0; q < NB; ++q)
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const float2 s = add2(hi[q][u], lo[q][u]);
+            lo[q][u] = sub2(lo[q][u], sub2(s, hi[q][u]));
+            hi[q][u] = s;
+          }
+      }
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&empty[sb]);
+        mbar_arrive(&wempty[ws]);
+      }
+    }
+    // g[cr][q][column] as normalised pairs
+    float2* g = static_cast<float2*>(a.g);
+    if (v < nvs)
+#pragma unroll
+      for (int q = 0; q < NB; ++q)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int64_t colj = s0 + (int64_t)v * 4 + c;
+          const float2 h2 = hi[q][c >> 1], l2 = lo[q][c >> 1];
+          const ffs s = ff_add((c & 1) ? ffs{h2.y, l2.y} : ffs{h2.x, l2.x}, ffs{0.f, 0.f});
+          if (colj < p) g[((size_t)cr * NB + q) * p + colj] = make_float2(s.hi, s.lo);
+        }
+  } else {
+    // ------------------------------------------------ the link of the rows
+    const int st = warp - 1 - XF_SA - XF_SB;
+    const bool need_zp = a.link == LINK_CERTZ_LS || a.link == LINK_CERTZ_LOGI || a.link == LINK_CERT2_LS ||
+                         a.link == LINK_CERT2_LOGI || (a.link == LINK_LOGISTIC && NB > 1);
+    const double* zprev = static_cast<const double*>(a.ps->zprev);
+    double* zout = static_cast<double*>(a.ps->zout);
+    const double mom = a.ps->mom;
+    double uh = 0.0;   // value of the first word's unit
+    bool have_scale = false;
+    double lsum[3] = {0.0, 0.0, 0.0};
+    const int jl = lane % XF_B, hb = (lane / XF_B) % XF_LB;
+    for (int k0 = XF_LB * st; k0 < kloc; k0 += XF_LB * XF_NL) {
+      if (tmo) break;
+      const int k = k0 + hb;
+      const bool on = k < kloc && lane < 16;
+      const int64_t r0 = (int64_t)(cr + (k < kloc ? k : k0) * a.Gr) * XF_B;
+      const int rows = (int)((n - r0) < XF_B ? (n - r0) : XF_B);
+      const int64_t rowj = r0 + (jl < rows ? jl : rows - 1);
+      const double yd = a.y[rowj];
+      const double zp = need_zp ? zprev[rowj] : 0.0;
+      const int ws = k % XF_RW;
+      unsigned long long wh = 0ull, wl = 0ull;
+      const bool ok = (k >= kloc || k < XF_RW || mbar_wait<false>(&wempty[ws], ((k / XF_RW) - 1) & 1, a.limit_ns, a.status)) &&
+                      wait_row2(&a.zfix[2 * rowj], (unsigned)a.Gc, wh, wl, a.limit_ns, a.status);
+      if (!__all_sync(0xffffffffu, ok)) {
+        tmo = 1;
+        break;
+      }
+      if (!have_scale) {
+        if (!__all_sync(0xffffffffu, wait_count(a.zcnt, gridDim.x, a.limit_ns, a.status))) {
+          tmo = 1;
+          break;
+        }
+        const int zs = fixed_scale(a.rowl1 * __longlong_as_double((long long)__ldcg(&a.zmax[0])));
+        uh = zs == INT_MIN ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, 8 - zs);
+        have_scale = true;
+      }
+      double z[1];
+      z[0] = fma((double)((long long)wl >> 8), ldexp(uh, -XF_LO), (double)((long long)wh >> 8) * uh);
+      double rv[NB];
+      link_of<1, NB, false>(a.link, z, yd, zp, mom, rv);
+      if (on) {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+          const double r = jl < rows ? rv[q] : 0.0;   // rows past the end carry weight 0
+          const float h = (float)r, l = (float)(r - (double)h);
+          *reinterpret_cast<float4*>(&wts[ws][jl][q][0]) = make_float4(h, h, -h, -h);
+          *reinterpret_cast<float2*>(&wts[ws][jl][q][4]) = make_float2(l, l);
+        }
+      }
+      __syncwarp();
+      if (jl == 0 && on) mbar_arrive(&wfull[ws]);
+      if (on && cc == k % a.Gc && jl < rows) {   // this CTA records the block
+        if (zout) zout[r0 + jl] = z[0];
+        if (a.lsum) loss_of<1, false>(a.link, z, yd, zp, lsum);
+      }
+    }
+    if (a.lsum) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const double v = warp_sum(lsum[i]);
+        if (lane == 0) lcomb[st][i] = v;
+      }
+    }
+  }
+  __syncthreads();
+  if (a.lsum && tid < 4) {
+    double v = 0.0;
+    if (tid < 3)
+      for (int w = 0; w < XF_NL; ++w) v += lcomb[w][tid];
+    a.lsum[4 * (size_t)blockIdx.x + tid] = v;
+  }
+}
+
+}  // namespace relax

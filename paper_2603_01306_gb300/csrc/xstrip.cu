@@ -17,11 +17,9 @@ static const void* kptr() {
 static const void* xstrip_ptr(int xk, bool f64acc, int NF, int NB) {
   if (NF == 1 && NB == 1) {
     if (xk == XK_F64) return kptr<double, double, 1, 1>();
-    // FP32 X: the certificate / power-iteration pass in float-float arithmetic
-    if (xk == XK_F32) return f64acc ? kptr<float, float, 1, 1, true>() : kptr<float, float, 1, 1>();
+    if (xk == XK_F32) return kptr<float, float, 1, 1>();
   } else if (NF == 1 && NB == 2 && f64acc) {
-    // the logistic loop's float-float pass; the two-dual-point certificate
-    if (xk == XK_F32) return kptr<float, float, 1, 2, true>();
+    // the two-dual-point certificate
     if (xk == XK_F64) return kptr<double, double, 1, 2>();
   } else if (NF == 1 && NB == 2 && !f64acc) {
     if (xk == XK_F64) return kptr<double, double, 1, 2>();
@@ -47,10 +45,11 @@ static int xs_tv(int vec) { return vec == 2 ? XSShape<2>::TV : XSShape<4>::TV; }
 // RELAX_XS="B,SA,SB,lag,vps,mA,mB,Gr" overrides for tuning runs (0 keeps a default).
 cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t n, int64_t p) {
   if ((xk == XK_BF16 || xk == XK_FP8) && !f64acc && NF == 1) return xmma_plan(pl, xk, NB, n, p);
+  if (xk == XK_F32 && f64acc && NF == 1) return xff_plan(pl, NB, n, p);
   pl = XSPlan{};
   pl.xk = xk;
   pl.cert = f64acc;
-  pl.NF = NF;
+  pl.NF = pl.words = NF;
   pl.NB = NB;
   pl.kernel = xstrip_ptr(xk, f64acc, NF, NB);
   if (!pl.kernel || n < 1 || p < 1 || n > INT32_MAX || p > INT32_MAX) return cudaErrorNotSupported;
@@ -198,10 +197,10 @@ cudaError_t xstrip_bind(XSPlan& pl, const void* X, int64_t ldx, int64_t n, int64
 }
 
 // The per-pass area zeroed before every launch:
-//   cnt[nblk] | zcnt | zmax[2] | zfix[NF][n]
+//   cnt[nblk] | zcnt | zmax[2] | zfix[words of a row x n]
 static size_t zero_off_zcnt(const XSPlan& pl) { return ((size_t)pl.nblk * sizeof(unsigned) + 15) / 16 * 16; }
 size_t xstrip_zero_bytes(const XSPlan& pl, int64_t n) {
-  return (zero_off_zcnt(pl) + 32 + (size_t)pl.NF * n * sizeof(unsigned long long) + 15) / 16 * 16;
+  return (zero_off_zcnt(pl) + 32 + (size_t)pl.words * n * sizeof(unsigned long long) + 15) / 16 * 16;
 }
 void xstrip_zero_layout(const XSPlan& pl, void* base, XSArgs& a) {
   unsigned char* b = static_cast<unsigned char*>(base);

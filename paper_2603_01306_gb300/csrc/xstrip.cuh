@@ -463,13 +463,11 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
       TA ph[NF][XS_MAXB];
       float phl[FF ? NF : 1][XS_MAXB];   // FF: low parts
       if constexpr (FF) {
-        // float-float: two rows at a time, so that two chains of dependent
-        // sums are in flight (a fully unrolled block of them outgrew the
-        // instruction cache), in packed FP32 pairs; the row partials go to a
-        // per-lane array for the butterfly.  Scalar, one row at a time, the
-        // 96 certificates of a 2000 x 5000 problem took 4.43 ms, now 4.32 (256
-        // nodes of 5000 x 10000: 60.8 and 58.1 ms); the pass is bound by the
-        // latency of its chain of sums, not by their number.
+        // float-float, two forward vectors (one: xff.cuh): two rows at a time,
+        // so that two chains of dependent sums per vector are in flight (a
+        // fully unrolled block of them outgrew the instruction cache), in
+        // packed FP32 pairs; the row partials go to a per-lane array for the
+        // butterfly
 #pragma unroll 1
         for (int jj = 0; jj < XS_MAXB; jj += 2) {
           float2 hh[NF][2], ll[NF][2];   // even and odd columns in the halves of packed pairs
