@@ -401,6 +401,7 @@ void handle_free(relax_handle* h) {
     delete[] h->tev;
   }
   if (h->fixbuf) cudaFree(h->fixbuf);
+  pool_trim();
   delete h;
 }
 
@@ -1515,53 +1516,84 @@ relax_status relax_certify(relax_handle* h, const int8_t* fixings, const void* b
 }
 
 // ------------------------------------------------- standalone regularizer ops
+// One thread-block cluster where p fits its shared memory (pnode_plan), else the
+// cooperative grid.  p = 1000 FP32, prox, g and g*: 210 us on the grid (seven or
+// more grid barriers each, a scratch area zeroed per call), 119 on a cluster;
+// waited for after every round of the three, 421 and 138 (see pool.cu).
 static relax_status standalone(int mode, const void* vin, void* vout, int64_t p, double rho, int32_t k,
                                double lambda2, double M, const int8_t* fix, int32_t dtype, int32_t* counts,
                                double* out_host, cudaStream_t st) {
   if (!vin || p <= 0 || k < 0 || !(M > 0.0) || (dtype != RELAX_F64 && dtype != RELAX_F32)) return RELAX_EINVAL;
   const bool dbl = dtype == RELAX_F64;
+  NPlan np;
+  const bool cluster = pnode_plan(np, dbl, p, 1) == cudaSuccess;
   PPlan pl;
-  CU(pphase_plan(pl, dbl, p));
-  // scratch: round accumulators, block partials, barrier counter, status, output
-  const size_t acc_b = 3 * ACC_STRIDE * sizeof(unsigned long long);
-  const size_t bp_b = (size_t)2 * pl.grid * NBP * sizeof(double);
-  const size_t tot = acc_b + bp_b + 64;
+  if (!cluster) {
+    (void)cudaGetLastError();
+    CU(pphase_plan(pl, dbl, p));
+  }
+  // scratch: status and output; the grid's round accumulators, block partials
+  // and barrier counter (the cluster's prox needs none)
+  const size_t acc_b = cluster ? 0 : 3 * ACC_STRIDE * sizeof(unsigned long long);
+  const size_t bp_b = cluster ? 0 : (size_t)2 * pl.grid * NBP * sizeof(double);
+  const size_t tot = cluster && !out_host ? 0 : acc_b + bp_b + 64;
   unsigned char* scr = nullptr;
-  CU(cudaMallocAsync((void**)&scr, tot, st));
-  cudaError_t e = cudaMemsetAsync(scr, 0, tot, st);
-  PArgs a{};
-  a.mode = mode;
-  a.p = p;
-  a.k = k;
-  a.lambda2 = lambda2;
-  a.M = M;
-  a.rho = rho;
-  a.kc = pconst_make(lambda2, M, 0.0, rho);
-  a.fix = fix;
-  a.vin = vin;
-  a.vout = vout;
-  a.counts = counts;
-  a.acc = reinterpret_cast<unsigned long long*>(scr);
-  a.bpart = reinterpret_cast<double*>(scr + acc_b);
-  a.bar = reinterpret_cast<unsigned long long*>(scr + acc_b + bp_b);
-  a.status = reinterpret_cast<int*>(scr + acc_b + bp_b + 8);
-  a.out = reinterpret_cast<double*>(scr + acc_b + bp_b + 16);
-  a.bar_base = 0;
-  a.limit_ns = 4000000000ull;
-  if (e == cudaSuccess) e = pphase_launch(pl, a, st);
+  cudaError_t e = cudaSuccess;
+  if (tot) {
+    CU(pool_alloc((void**)&scr, tot, st));
+    e = cudaMemsetAsync(scr, 0, tot, st);
+  }
+  if (cluster) {
+    NArgs a{};
+    a.mode = mode;
+    a.p = p;
+    a.k = k;
+    a.lambda2 = lambda2;
+    a.M = M;
+    a.rho = rho;
+    a.kc = pconst_make(lambda2, M, 0.0, rho);
+    a.fix = fix;
+    a.vin = vin;
+    a.vout = vout;
+    a.counts = counts;
+    a.nq = 1;
+    a.out = reinterpret_cast<double*>(scr);
+    if (e == cudaSuccess) e = pnode_launch(np, a, 1, st);
+  } else {
+    PArgs a{};
+    a.mode = mode;
+    a.p = p;
+    a.k = k;
+    a.lambda2 = lambda2;
+    a.M = M;
+    a.rho = rho;
+    a.kc = pconst_make(lambda2, M, 0.0, rho);
+    a.fix = fix;
+    a.vin = vin;
+    a.vout = vout;
+    a.counts = counts;
+    a.out = reinterpret_cast<double*>(scr);
+    a.status = reinterpret_cast<int*>(scr + 8);
+    a.bar = reinterpret_cast<unsigned long long*>(scr + 16);
+    a.acc = reinterpret_cast<unsigned long long*>(scr + 64);
+    a.bpart = reinterpret_cast<double*>(scr + 64 + acc_b);
+    a.bar_base = 0;
+    a.limit_ns = 4000000000ull;
+    if (e == cudaSuccess) e = pphase_launch(pl, a, st);
+  }
   relax_status rs = RELAX_OK;
   if (e == cudaSuccess && out_host) {
-    double hv[3] = {0, 0, 0};
-    int dst = 0;
-    e = cudaMemcpyAsync(hv, a.out, sizeof(double), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&dst, a.status, sizeof(int), cudaMemcpyDeviceToHost, st);
+    double hv[2] = {0, 0};   // {value, status}
+    e = cudaMemcpyAsync(hv, scr, sizeof(hv), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e == cudaSuccess) {
+      int dst = 0;
+      std::memcpy(&dst, &hv[1], sizeof(dst));
       out_host[0] = hv[0];
       rs = map_dev_status(dst);
     }
   }
-  cudaFreeAsync(scr, st);
+  if (scr) cudaFreeAsync(scr, st);
   if (e != cudaSuccess) return map_cuda(e);
   return rs;
 }

@@ -180,6 +180,11 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long* counter, unsign
   return ok_sh != 0;
 }
 
+// Stream-ordered scratch from the library's own memory pool of the current
+// device (pool.cu); returned with cudaFreeAsync.
+cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t st);
+void pool_trim();   // gives what the current device's pool holds unused back to the driver
+
 // ------------------------------------------------------------ misc helpers
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {

@@ -506,7 +506,7 @@ relax_status relax_mlp_grad(const float* theta, int32_t bf16, const float* feat,
   const int64_t ntiles = (rows + tile - 1) / tile;
   const int nparts = (int)(ntiles < sms ? ntiles : sms);
   float* part = nullptr;
-  e = cudaMallocAsync((void**)&part, (size_t)nparts * (RELAX_MLP_NTRAIN + 1) * sizeof(float), st);
+  e = relax::pool_alloc((void**)&part, (size_t)nparts * (RELAX_MLP_NTRAIN + 1) * sizeof(float), st);
   if (e != cudaSuccess) return cuda_status(e);
   kernel<<<nparts, GRAD_T, smem, st>>>(theta, bf16 ? 1 : 0, feat, base, target, rows, part);
   e = cudaGetLastError();

@@ -256,7 +256,15 @@ __device__ __forceinline__ double pn_G64(int64_t j) {
   return (double)v.x + (double)v.y;
 }
 template <bool F64>
-__device__ __forceinline__ double pn_a64(int64_t j) { return fabs(pn_G64<F64>(j)) * pn().a.kc.inv2l; }
+__device__ __forceinline__ double pn_vin(int64_t j) {   // the standalone operations' input
+  const void* v = pn().a.vin;
+  return F64 ? static_cast<const double*>(v)[j] : (double)static_cast<const float*>(v)[j];
+}
+template <bool F64>
+__device__ __forceinline__ double pn_a64(int64_t j) {
+  if (pn().a.mode == PM_GSTAR) return fabs(pn_vin<F64>(j));
+  return fabs(pn_G64<F64>(j)) * pn().a.kc.inv2l;
+}
 
 // v_j of a wide coordinate, FP64 (on FP32 data the gradient at y, whose terms
 // are FP32 pairs, in float-float)
@@ -899,7 +907,7 @@ __device__ __noinline__ int pn_level(int nx) {
     for (int e = lane; e < nw; e += 32) {
       const int i = s.wl[w0 + e];
       if (!(s.fl[i] & 4)) continue;
-      const double ab = fabs(s.bcur[s.cb + i]);
+      const double ab = fabs(s.a.mode == PM_ITER ? s.bcur[s.cb + i] : s.vw[w0 + e]);
       if (ab > w) {
         ++na;
         v0.add(ab);
@@ -972,6 +980,14 @@ __device__ __noinline__ void pn_decisions() {
   const double phi = s.loss[0] + 2.0 * a.lambda2 * gval;
   const double psi = s.loss[1] - 2.0 * a.lambda2 * (s.tot[XS_J1H] + s.top);
   const bool nonfinite = s.bad > 0;
+  if (a.mode == PM_GVAL || a.mode == PM_GSTAR) {
+    if (s.rank == 0)
+      a.out[0] = a.mode == PM_GVAL                                            ? gval
+                 : nonfinite                                                 ? __longlong_as_double(0x7ff8000000000000ll)
+                 : s.nnz > 0 || (s.dom > 0 && s.kb > 0) ? INFINITY
+                                                        : s.tot[XS_J1H] + s.top;
+    return;
+  }
   if (a.mode != PM_ITER) {
     if (s.rank == 0) {
       double* o = a.out + (size_t)s.item * a.out_stride + 2 * s.q0;
@@ -1038,6 +1054,119 @@ __device__ __noinline__ void pn_decisions() {
   st->cut_rule = cut_rule;
 }
 
+// Stage 1 of the standalone operations over this warp's coordinates
+template <bool F64>
+__device__ __noinline__ void pn_load(Acc<F64> (&sum)[XS_NSUM], unsigned& nnz, unsigned& dom, unsigned& bad, unsigned& nzv,
+                                     unsigned& j1, unsigned& jf) {
+  PnSh& s = pn();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, mode = s.a.mode;
+  const int wch = s.a.wch, w0 = (warp - 1) * wch, w1 = min(s.cnt, w0 + wch);
+  int nw = 0;
+#pragma unroll 1
+  for (int i0 = w0; i0 < w0 + wch; i0 += 32) {
+    const int i = i0 + lane;
+    bool wide = false;
+    uint32_t key = 0;
+    float m = 0.f;
+    uint8_t f8 = 0;
+    double x = 0.0;
+    if (i < w1) {
+      const int64_t j = s.cb + i;
+      const int8_t f = s.fix ? s.fix[j] : (int8_t)0;
+      x = pn_vin<F64>(j);
+      f8 = f == 0 ? 4 : f > 0 ? 8 : 0;
+      j1 += f > 0;
+      jf += f == 0;
+      // (an FP64 value beyond FP32's range is finite all the same)
+      const bool inf_nan = (((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ffu) == 0x7ffu;
+      const float ax = fminf(fabsf((float)x), 3.4e38f);
+      if (inf_nan && (mode == PM_PROX || (x != x && f >= 0))) ++bad;
+      if (mode == PM_GSTAR) {   // an infinite value: dom on Jf, nnz on J1
+        if (f == 0) key = key_of(ax);
+        if (inf_nan && f == 0) ++dom;
+        if (f > 0) {
+          if (inf_nan) ++nnz;
+          else sum[XS_J1H].add(huber_d<double>(fabs(x), s.a.M));
+        }
+      } else if (mode == PM_PROX) {
+        wide = F64 ? f >= 0 : f > 0;
+        if (__double_as_longlong(x) < 0) f8 |= 1;
+        if (f == 0) {
+          m = ax;
+          nzv += !is_zero_bits(x);
+        }
+      } else if (!is_zero_bits(x)) {   // g's value
+        wide = true;
+        const double ab = fabs(x);
+        if (f < 0 || ab > s.a.kc.Mtol || (inf_nan && x == x)) ++dom;
+        if (f > 0) sum[XS_J1B2].add(ab * ab);
+        else if (f == 0) {
+          sum[XS_B].add(ab);
+          sum[XS_B2].add(ab * ab);
+          ++nnz;
+        }
+      }
+      if (wide) f8 |= 2;
+    }
+    s.ka[i] = key;
+    s.mv[i] = m;
+    s.fl[i] = f8;
+    const unsigned wm = __ballot_sync(0xffffffffu, wide);
+    if (wide) {
+      const int at = w0 + nw + __popc(wm & ((1u << lane) - 1u));
+      s.wl[at] = (uint16_t)i;
+      s.vw[at] = x;
+    }
+    nw += __popc(wm);
+  }
+  if (lane == 0) s.nw[warp] = nw;
+  j1 = __reduce_add_sync(0xffffffffu, j1);
+  jf = __reduce_add_sync(0xffffffffu, jf);
+  __syncwarp();
+}
+
+// The standalone prox's output and counts.  A non-finite input poisons them:
+// beta all NaN, counts -1.
+template <bool F64>
+__device__ __noinline__ void pn_prox_out(int nx, int kb, bool s3, unsigned bad) {
+  PnSh& s = pn();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int w0 = (warp - 1) * s.a.wch, w1 = warp ? min(s.cnt, w0 + s.a.wch) : w0, nw = s.nw[warp];
+  const double c = kb <= 0 ? INFINITY : s3 ? s.c : 0.0, T = pn_T(c), inv1r = s.a.kc.inv1r, M = s.a.M;
+  const float ccd = kb <= 0 ? INFINITY : s3 ? s.ccd : 0.f;   // an FP32 m exceeds c iff it exceeds c rounded down
+  unsigned ntop = 0, nnz = 0;
+#pragma unroll 1
+  for (int u = lane; u < (w1 - w0) + nw; u += 32) {
+    const bool narrow = u < w1 - w0;
+    const int e = w0 + u - (narrow ? 0 : w1 - w0);
+    const int i = narrow ? e : s.wl[e];
+    const uint8_t f8 = s.fl[i];
+    if (narrow && (f8 & 2)) continue;
+    double b = 0.0;
+    if (bad) b = __longlong_as_double(0x7ff8000000000000ll);
+    else if (f8 & 8) b = fmin(fmax(s.vw[e] * inv1r, -M), M);
+    else if ((f8 & 4) && (!narrow || s.mv[i] > ccd)) {
+      const double m = narrow ? (double)s.mv[i] : fabs(s.vw[e]);
+      const double r = fmax(0.0, fmin(fmin(m - c, m * inv1r), M));
+      if (r > 0.0) {
+        ++nnz;
+        ntop += m >= T;
+        b = (f8 & 1) ? -r : r;
+      }
+    }
+    if (F64) static_cast<double*>(s.a.vout)[s.cb + i] = b;
+    else static_cast<float*>(s.a.vout)[s.cb + i] = (float)b;
+  }
+  if (s.a.counts) {
+    const unsigned long long zero = Acc<F64>().word();
+    pn_small_sum<F64>(nx, zero, zero, ntop, nnz);
+    if (s.rank == 0 && threadIdx.x == 0) {
+      s.a.counts[0] = bad ? -1 : (int)s.cnt0;
+      s.a.counts[1] = bad ? -1 : (int)s.cnt1;
+    }
+  }
+}
+
 // ==================================================================== kernel
 template <bool F64>
 __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const __grid_constant__ NArgs args) {
@@ -1067,10 +1196,11 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
     if (tid == 0) {
       s.prob = prob;
       s.rank = (int)blockIdx.x - prob * S;
-      s.item = it ? node : prob / args.nq;
-      s.q0 = it ? 0 : prob % args.nq;
+      const bool ev = args.mode == PM_EVAL;
+      s.item = it ? node : ev ? prob / args.nq : 0;
+      s.q0 = ev ? prob % args.nq : 0;
       const size_t slot = it ? prob : s.item;
-      s.bcur = static_cast<const double*>(it ? s.st.beta_cur : args.ev[s.item].beta);
+      s.bcur = static_cast<const double*>(it ? s.st.beta_cur : ev ? args.ev[s.item].beta : nullptr);
       s.bprev = it ? static_cast<const double*>(s.st.beta_prev) : nullptr;
       s.fix = args.fix ? args.fix + (size_t)s.item * args.fix_stride : nullptr;
       s.part = static_cast<const double*>(args.part) + slot * args.part_stride + (size_t)s.q0 * args.p;   // 8-byte elements
@@ -1078,7 +1208,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
       s.Gcur = it ? s.st.G_cur : static_cast<double*>(args.gev) + (size_t)prob * args.p;
       s.kb = it ? s.st.kbar : args.k;
       s.pb = it ? s.st.pbar : (int)args.p;
-      if (!it && args.cnt) {
+      if (ev && args.cnt) {
         s.kb = args.k - args.cnt[3 * s.item];
         s.pb = args.cnt[3 * s.item + 1];
       }
@@ -1132,11 +1262,12 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
       __syncthreads();
     }
   }
-  const bool iter = s.a.mode == PM_ITER;
+  const int mode = s.a.mode;
+  const bool iter = mode == PM_ITER, alone = mode >= PM_PROX;
   const int64_t cb = s.cb;
   const int wch = s.a.wch, w0 = (warp - 1) * wch, w1 = warp ? min(s.cnt, w0 + wch) : w0;
   const PConst& kc = s.a.kc;
-  const int kb = s.kb;
+  int kb = s.kb;   // (standalone: known after exchange 1)
   const int t = iter ? s.st.iter : 0;
 
   // ----------------------------------------------------- stage 1, exchange 1
@@ -1146,8 +1277,10 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
   const bool w_known = !is_zero_bits(w_closed);
   const double mu = iter ? s.st.ps.mom : 0.0;
   A sum[XS_NSUM];
-  unsigned c_nnz = 0, c_dom = 0, c_bad = 0, c_nab = 0, c_nzv = 0;
-  if (warp == 0) {   // the loss sums of the pass, in FP64
+  unsigned c_nnz = 0, c_dom = 0, c_bad = 0, c_nab = 0, c_nzv = 0, c_j1 = 0, c_jf = 0;
+  if (alone) {
+    if (warp) pn_load<F64>(sum, c_nnz, c_dom, c_bad, c_nzv, c_j1, c_jf);
+  } else if (warp == 0) {   // the loss sums of the pass, in FP64
     const double* ls = s.a.lsum + (size_t)(iter ? s.prob : s.item) * s.a.lsum_stride;
     double f = 0.0, d = 0.0;
 #pragma unroll 4
@@ -1224,6 +1357,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
       const double b = s.bcur[j];
       const uint8_t f8 = s.fl[i];
       if (f8 & 8) sum[XS_J1H].add(huber_d<double>(pn_a64<F64>(j), s.a.M));
+      if (!iter) s.vw[w0 + e] = b;
       if (!is_zero_bits(b)) {
         const double ab = fabs(b);
         A a1, a2;   // |b| and b^2 (FP32 data: as pairs, one conversion for both)
@@ -1269,14 +1403,14 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
     }
     __syncwarp();
   }
-  const bool need1 = kb > 0 && s.pb > kb, can3 = iter && kb > 0;
+  bool need1 = alone ? mode == PM_GSTAR : kb > 0 && s.pb > kb, can3 = alone ? mode == PM_PROX : iter && kb > 0;
   const uint32_t k1 = iter ? s.st.key1 : 0u, k3 = iter ? s.st.key3 : 0u;
   uint32_t x1 = k1 ? pn_warm(k1, s.st.win1, 0u, kInfKey + 1, lane) : cand<uint32_t>(0u, kInfKey + 1, lane);
   uint32_t x3 = k3 ? pn_warm(k3, s.st.win3, 0u, kInfKey, lane) : cand<uint32_t>(0u, kInfKey, lane);
   pn_count(need1, can3, x1, x3);
   {
     unsigned long long* rw = s.red + warp * XW_WORDS;
-    if (s.nw[warp] > 0) {
+    if (s.nw[warp] > 0 || (alone && warp)) {
 #pragma unroll 1
       for (int o = 16; o > 0; o >>= 1)   // the six side by side
 #pragma unroll
@@ -1294,6 +1428,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
       rw[XW_INT] = pack2(c_nnz, c_dom);
       rw[XW_INT + 1] = pack2(c_bad, c_nzv);
       rw[XW_INT + 2] = c_nab;
+      rw[XW_INT + 3] = pack2(c_j1, c_jf);   // (per lane sums only in the standalone modes, reduced there)
     }
   }
   cluster_wait();   // every CTA of the cluster runs
@@ -1303,6 +1438,19 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
   // budget holds
   const unsigned long long bz = xcnt(nx, XW_INT + 1);
   const unsigned bad = (unsigned)bz, nzv = (unsigned)(bz >> 32);
+  if (alone) {
+    const unsigned long long jj = xcnt(nx, XW_INT + 3);
+    kb = s.a.k - (int)(unsigned)jj;
+    const int pb = (int)(jj >> 32);
+    if (tid == 0) {
+      s.kb = kb;
+      s.pb = pb;
+      s.c1lo = (unsigned)pb;
+    }
+    need1 = need1 && kb > 0 && pb > kb;
+    can3 = can3 && kb > 0;
+    __syncthreads();
+  }
   bool s3 = can3 && (int)nzv > kb && bad == 0;
   const bool s1 = need1 && bad == 0;
   if (warp == 2 % W) {
@@ -1322,10 +1470,11 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
   ++nx;
   if (s.more1 || s.more3) nx = pn_more_rounds<F64>(nx);
 
+  const bool need_b = iter || mode == PM_EVAL || mode == PM_GVAL;
   const bool check_dom = !iter || t == 0;
   const bool g_inf = check_dom && (s.dom > 0 || (kb > 0 && s.tot[XS_B] > s.a.M * (double)kb * (1.0 + 1e-6)) ||
                                    (kb <= 0 && s.tot[XS_B] > 0.0));
-  const bool level = !g_inf && kb > 0 && s.nnz > (unsigned)kb;   // a water level to find
+  const bool level = need_b && !g_inf && kb > 0 && s.nnz > (unsigned)kb;   // a water level to find
   if (level && !w_known) nx = pn_level<F64>(nx);
   // g, and FISTA's next t_k and momentum should this iteration not restart:
   // by warps that have nothing else to do while the searches end
@@ -1363,7 +1512,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
   ++nx;
   if ((s1 && (o1 || s.miss1)) || (s3 && (o3 || s.miss3)))
     nx = pn_repair<F64>(nx, s1 && (o1 || s.miss1), s3 && (o3 || s.miss3), o1, o3);
-  if (kb > 0 && s.pb <= kb) {   // a slack budget: the whole free set (at most kbar coordinates)
+  if (kb > 0 && s.pb <= kb && mode != PM_PROX && mode != PM_GVAL) {   // a slack budget: the whole free set (at most kbar coordinates)
     A v;
 #pragma unroll 1
     for (int i = w0 + lane; i < w1; i += 32)
@@ -1380,7 +1529,8 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
 
   // ---------------------------------------------------------------------- D
   if (!iter) {
-    if (tid == 0) pn_decisions();
+    if (mode == PM_PROX) pn_prox_out<F64>(nx, kb, s3, bad);
+    else if (tid == 0) pn_decisions();
     return;   // (every push to this CTA has been received: no exchange follows)
   }
   // Thread 0 decides while the other warps form the next point for "no

@@ -1,6 +1,6 @@
 // Node p-phase: everything an iteration does on p-vectors (the steps P0, S1,
-// S2, D, P1, S3, P2 of pphase.cuh), or the certificate's evaluation of Phi and
-// Psi, by one thread-block cluster per problem.
+// S2, D, P1, S3, P2 of pphase.cuh), the certificate's evaluation of Phi and Psi,
+// or a standalone prox, g or g*, by one thread-block cluster per problem.
 //
 // What bounds it is latency: the arithmetic is a few microseconds' worth of
 // one cluster, and every grid-wide sum of the iteration is a round trip
@@ -49,12 +49,12 @@ constexpr int PN_LSUM = 4;           // doubles per CTA of the pass's loss sums:
 
 // exchange words: [0, 32) S3 sums per candidate (float-float), then the sums
 // of Phi and Psi, then counts (packed pairs of 32-bit ones)
-enum : int { XW_S3 = 0, XW_SUM = 32, XW_N3 = 38, XW_N1 = 70, XW_INT = 102, XW_WORDS = 105 };
+enum : int { XW_S3 = 0, XW_SUM = 32, XW_N3 = 38, XW_N1 = 70, XW_INT = 102, XW_WORDS = 106 };
 enum : int { XS_J1H = 0, XS_J1B2 = 1, XS_B = 2, XS_B2 = 3, XS_SAB = 4, XS_QAB = 5, XS_NSUM = 6 };
 
 struct NArgs {
   PConst kc;
-  int mode;                     // PM_ITER or PM_EVAL
+  int mode;                     // PMode
   int loss, cl, cpc;            // CTAs per problem, coordinates per CTA
   int lc, wch;                  // list entries per CTA and search; coordinates per warp
   int64_t p, n;
@@ -87,8 +87,13 @@ struct NArgs {
   int nq;
   void* gev;                    // [problem][p] scratch: the summed gradients (8 bytes each)
   const int* cnt;               // [items][3] fixing counts {|J1|, |Jf|, .}; NULL: root
-  double* out;                  // item's values at out_stride item + 2 (s % nq)
+  double* out;                  // item's values at out_stride item + 2 (s % nq); PM_GVAL, PM_GSTAR: one value
   int64_t out_stride;
+  // the standalone operations, one problem on vectors of the kernel's type
+  // (F64: double, else float)
+  const void* vin;              // PM_PROX: v, PM_GVAL: beta, PM_GSTAR: alpha
+  void* vout;                   // PM_PROX
+  int* counts;                  // PM_PROX: {n_top, n_nz} or NULL
   int* status;
 };
 
