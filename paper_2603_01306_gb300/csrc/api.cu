@@ -162,22 +162,79 @@ __global__ void reduce_partials_kernel(const void* part, int pair, int ncl, int 
   }
 }
 
-// {F(z), -F*(-zeta)} at zeta = -grad F(z) (Eq. 6-7 loss parts), FP64
-__global__ void loss_terms_kernel(const double* z, const double* y, int64_t n, int loss, double* out) {
-  double f = 0.0, d = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    if (loss == RELAX_LS) {
-      const double r = z[i] - y[i], zeta = -2.0 * r;
-      f += r * r;
-      d += zeta * y[i] - 0.25 * zeta * zeta;
+// A standalone pass in three launches and one copy: everything the pass reads
+// (beta in FP64, the pass state, its zeroed area, the status), the pass, and
+// everything the caller gets.  (3001 x 7003 FP32 logistic: 129 us as six
+// kernels, six memsets and three copies, two of them waited for; 83 so, 70 with the loss
+// terms on warps of their own and the one-ring pass.)
+__global__ void xpass_prep_kernel(const void* beta, int f64, double* b64, int64_t p, PassState ps, PassState* psd, int* status,
+                                  double* res, uint4* zero, int64_t nzero) {
+  const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t j = t0; j < p; j += stride)
+    b64[j] = f64 ? static_cast<const double*>(beta)[j] : (double)static_cast<const float*>(beta)[j];
+  for (int64_t i = t0; i < nzero; i += stride) zero[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (t0 == 0) {
+    *psd = ps;
+    *status = ST_OK;
+    res[0] = res[1] = 0.0;
+  }
+}
+
+// z and g (the sum of the ncl row groups' partials, FP32 pairs or FP64, in
+// order) in the caller's type; res = {F(z), -F*(-zeta) at zeta = -grad F(z)
+// (Eq. 6-7 loss parts), the device status}
+__global__ void xpass_finish_kernel(const void* part, int pair, int ncl, int64_t p, void* g, const double* z, const double* y,
+                                    int64_t n, void* zo, int f64, int loss, int want_loss, const int* status, double* res) {
+  const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t j = t0; j < p; j += stride) {
+    double s = 0.0;
+    if (pair) {
+      relax::ffs f{0.f, 0.f};
+#pragma unroll 4
+      for (int c = 0; c < ncl; ++c) {
+        const float2 v = static_cast<const float2*>(part)[(int64_t)c * p + j];
+        f = ff_add(f, relax::ffs{v.x, v.y});
+      }
+      s = (double)f.hi + (double)f.lo;
     } else {
-      f += softplus_neg(y[i] * z[i]);
-      d += entropy_of(y[i] * z[i]);
+#pragma unroll 4
+      for (int c = 0; c < ncl; ++c) s += static_cast<const double*>(part)[(int64_t)c * p + j];
+    }
+    if (f64) static_cast<double*>(g)[j] = s;
+    else static_cast<float*>(g)[j] = (float)s;
+  }
+  // the two loss terms of a row on threads of their own: FP64 exp and log are
+  // latency here, and a warp per SM waits least (blocks of one warp)
+  double f = 0.0, d = 0.0;
+  for (int64_t t = t0; t < (want_loss ? 2 * n : n); t += stride) {
+    const bool first = t < n;
+    const int64_t i = first ? t : t - n;
+    const double zi = z[i];
+    if (first && zo) {
+      if (f64) static_cast<double*>(zo)[i] = zi;
+      else static_cast<float*>(zo)[i] = (float)zi;
+    }
+    if (!want_loss) continue;
+    const double yi = y[i];
+    if (loss == RELAX_LS) {
+      const double r = zi - yi, zeta = -2.0 * r;
+      if (first) f += r * r;
+      else d += zeta * yi - 0.25 * zeta * zeta;
+    } else if (first) {
+      f += softplus_neg(yi * zi);
+    } else {
+      d += entropy_of(yi * zi);
     }
   }
-  f = warp_sum(f);
-  d = warp_sum(d);
-  if ((threadIdx.x & 31) == 0) { atomicAdd(out, f); atomicAdd(out + 1, d); }
+  if (want_loss) {
+    f = warp_sum(f);
+    d = warp_sum(d);
+    if ((threadIdx.x & 31) == 0) {
+      if (f != 0.0) atomicAdd(res, f);
+      if (d != 0.0) atomicAdd(res + 1, d);
+    }
+  }
+  if (t0 == 0) res[2] = (double)*status;
 }
 
 __global__ void nnz_kernel(const double* v, int64_t p, int* out) {
@@ -1457,33 +1514,26 @@ relax_status relax_xpass(relax_handle* h, const void* beta, void* z_out, void* g
   if (!h || !beta || !g_out) return RELAX_EINVAL;
   CU(cudaSetDevice(h->dev));
   double* b64 = (double*)h->vb[8];
-  double* g64 = (double*)h->vb[9];
   double* z64 = (double*)h->vb[10];
-  double* zp64 = (double*)h->vb[11];
-  to_f64_kernel<<<grid_for(h->p), 256, 0, h->stream>>>(beta, h->f64(), b64, h->p);
-  CU(cudaGetLastError());
+  // one right-hand side: the plan of z = X beta, whichever link follows
+  const XSPlan& pl = h->pl_ident;
   PassState ps{};
   ps.beta = b64;
   ps.zout = z64;
-  ps.zprev = zp64;
-  ps.mom = 0.0;
-  *reinterpret_cast<PassState*>(h->h_d + 1000) = ps;
-  CU(cudaMemcpyAsync(h->ps_aux, h->h_d + 1000, sizeof(PassState), cudaMemcpyHostToDevice, h->stream));
-  CU(cudaMemsetAsync(h->status, 0, sizeof(int), h->stream));
-  CU(cudaMemsetAsync(zp64, 0, (size_t)h->n * sizeof(double), h->stream));
-  XSArgs a = pass_args(h, h->pl_loop, h->loss == RELAX_LS ? LINK_LS : LINK_LOGISTIC, h->ps_aux);
-  CU(run_pass(h->pl_loop, a, h->stream));
-  const unsigned g = grid_for(h->p);
-  reduce_partials_kernel<<<g, 256, 0, h->stream>>>(h->xg, !h->f64(), h->pl_loop.Gr, h->pl_loop.NB, h->p, g64);
-  from_f64_kernel<<<g, 256, 0, h->stream>>>(g64, g_out, h->f64(), h->p);
-  if (z_out) from_f64_kernel<<<grid_for(h->n), 256, 0, h->stream>>>(z64, z_out, h->f64(), h->n);
-  CU(cudaMemsetAsync(h->dscr, 0, 2 * sizeof(double), h->stream));
-  loss_terms_kernel<<<grid_for(h->n), 256, 0, h->stream>>>(z64, (const double*)h->y, h->n, h->loss, h->dscr);
+  XSArgs a = pass_args(h, pl, h->loss == RELAX_LS ? LINK_LS : LINK_LOGISTIC, h->ps_aux);
+  a.lsum = nullptr;   // the loss terms are taken in FP64 below
+  const int64_t nzero = (int64_t)(xstrip_zero_bytes(pl, h->n) / sizeof(uint4));
+  xpass_prep_kernel<<<grid_for(std::max(h->p, nzero)), 256, 0, h->stream>>>(
+      beta, h->f64(), b64, h->p, ps, h->ps_aux, h->status, h->dscr, reinterpret_cast<uint4*>(h->xcnt), nzero);
   CU(cudaGetLastError());
-  CU(cudaMemcpyAsync(h->h_d, h->dscr, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  CU(xstrip_launch(pl, a, false, h->stream));
+  xpass_finish_kernel<<<grid_for(std::max(h->p, 2 * h->n), 32), 32, 0, h->stream>>>(
+      h->xg, !h->f64(), pl.Gr, h->p, g_out, z64, (const double*)h->y, h->n, z_out, h->f64(), h->loss, loss_host != nullptr,
+      h->status, h->dscr);
+  CU(cudaGetLastError());
+  CU(cudaMemcpyAsync(h->h_d, h->dscr, 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CU(cudaStreamSynchronize(h->stream));
-  int dst = 0;
-  CU(cudaMemcpy(&dst, h->status, sizeof(int), cudaMemcpyDeviceToHost));
+  const int dst = (int)h->h_d[2];
   if (loss_host) {
     loss_host[0] = h->h_d[0];
     loss_host[1] = h->h_d[1];
