@@ -486,6 +486,7 @@ XSArgs pass_args(relax_handle* h, const XSPlan& pl, int link, PassState* ps) {
   a.SB = pl.SB;
   a.RA = pl.RA;
   a.RB = pl.RB;
+  a.keep = pl.keep;
   a.lag = pl.lag;
   a.link = link;
   a.y = (const double*)h->y;

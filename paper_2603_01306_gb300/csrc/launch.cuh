@@ -28,6 +28,7 @@ struct XSPlan {
   int SA = 3, SB = 3, lag = 4;
   int RA = 3, RB = 3;       // ring stages, multiples of SA / SB
   bool mma = false;         // the tensor-core pass (BF16 / FP8, xmma.cuh)
+  bool keep = false;        // X fits L2 beside the vectors
   int words = 1;            // 64-bit words of z per row
   int vpb = 1, spb = 1, steps = 1;   // its vectors and steps per box, steps per strip
   int grid = 1, threads = 32;
@@ -35,10 +36,11 @@ struct XSPlan {
   const void* kernel = nullptr;
 };
 cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t n, int64_t p);
+bool x_fits_l2(int xk, int64_t n, int64_t p);
 // the BF16 / FP8 plans (xmma.cu; xstrip_plan and xstrip_launch go there)
 cudaError_t xmma_plan(XSPlan& pl, int xk, int NB, int64_t n, int64_t p);
-// the float-float plans of FP32 X with one product z (xff.cu; xstrip_plan goes there)
-cudaError_t xff_plan(XSPlan& pl, int NB, int64_t n, int64_t p);
+// the plans of FP32 X with one product z (xf32.cu; xstrip_plan goes there)
+cudaError_t xf32_plan(XSPlan& pl, bool ff, int NB, int64_t n, int64_t p);
 cudaError_t xmma_launch(const XSPlan& pl, const XSArgs& a, cudaStream_t st);
 // encode the plan's tensor map of X (16-byte aligned, ldx * size a multiple of 16)
 cudaError_t xstrip_bind(XSPlan& pl, const void* X, int64_t ldx, int64_t n, int64_t p);

@@ -1,50 +1,58 @@
-// Plan of the float-float pass over FP32 X.
+// Plan of the passes over FP32 X with one product z.
 #include <algorithm>
+#include <cmath>
 
 #include "launch.cuh"
-#include "xff.cuh"
+#include "xf32.cuh"
 
 namespace relax {
 
-// Strips x row groups: the choice with the least work of the busiest CTA, a
-// block's six axpy warps taking as long as a dot warp with six vectors per lane.
-cudaError_t xff_plan(XSPlan& pl, int NB, int64_t n, int64_t p) {
+// Strips (at most 192 vectors: one per lane of the six axpy warps, six per lane
+// of a dot warp) x row groups (at least two blocks of 16 rows each).  The
+// float-float pass is bound by its sums: the choice with the least work of the
+// busiest CTA, a block's axpy taking as long as dot products with six vectors
+// per lane.  The FP32 pass is bound by X: the choice that keeps the most SMs
+// busy, strips under 2 KB counted as streaming less efficiently.
+cudaError_t xf32_plan(XSPlan& pl, bool ff, int NB, int64_t n, int64_t p) {
   pl = XSPlan{};
   pl.xk = XK_F32;
-  pl.cert = true;
+  pl.cert = ff;
   pl.NF = 1;
   pl.NB = NB;
-  pl.words = 2;
+  pl.words = ff ? 2 : 1;
+  pl.keep = x_fits_l2(XK_F32, n, p);
   if (NB < 1 || NB > 2 || n < 1 || p < 1 || n > INT32_MAX || p > INT32_MAX) return cudaErrorNotSupported;
-  pl.kernel = NB == 1 ? reinterpret_cast<const void*>(&xff_kernel<1>) : reinterpret_cast<const void*>(&xff_kernel<2>);
+  pl.kernel = ff ? (NB == 1 ? reinterpret_cast<const void*>(&xf32_kernel<1, true>) : reinterpret_cast<const void*>(&xf32_kernel<2, true>))
+                 : (NB == 1 ? reinterpret_cast<const void*>(&xf32_kernel<1, false>) : reinterpret_cast<const void*>(&xf32_kernel<2, false>));
   int dev = 0, nsm = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const int64_t nvec = (p + 3) / 4, cap = 32 * XF_TV;
-  pl.B = XF_B;
-  pl.nblk = (int)((n + XF_B - 1) / XF_B);
-  int64_t best = INT64_MAX;
+  pl.B = ff ? XF<true>::B : XF<false>::B;
+  pl.nblk = (int)((n + pl.B - 1) / pl.B);
+  const int64_t most = std::max<int64_t>(1, ((n + 15) / 16 + 1) / 2);
+  double best = 0.0;
   for (int64_t gc = (nvec + cap - 1) / cap; gc <= std::min<int64_t>({(int64_t)nsm, nvec, (int64_t)255}); ++gc) {
     const int64_t v = (nvec + gc - 1) / gc;
     const int64_t nbox = (v * 4 + 255) / 256, vpb = (v + nbox - 1) / nbox;
     const int64_t gcc = (nvec + nbox * vpb - 1) / (nbox * vpb);
     if (nbox * vpb > cap || gcc > nsm) continue;
-    const int64_t gr = std::max<int64_t>(1, std::min<int64_t>(nsm / gcc, (pl.nblk + 1) / 2));
-    const int64_t cost = (pl.nblk + gr - 1) / gr * (XF_TV + (nbox * vpb + 31) / 32);
-    if (cost >= best) continue;   // fewer strips where the cost is the same
-    best = cost;
+    const int64_t gr = std::max<int64_t>(1, std::min<int64_t>(nsm / gcc, most));
+    const double score = ff ? 1.0 / ((double)((pl.nblk + gr - 1) / gr) * (double)(XF_TV + (nbox * vpb + 31) / 32))
+                            : (double)(gcc * gr) * std::sqrt(std::min(1.0, (double)(v * 16) / 2048.0));
+    if (score <= best * 1.0001) continue;   // fewer strips where the score is the same
+    best = score;
     pl.nbox = (int)nbox;
     pl.inner = (int)(vpb * 4);
     pl.sw = nbox * pl.inner;
     pl.Gc = (int)gcc;
     pl.Gr = (int)gr;
   }
-  if (best == INT64_MAX) return cudaErrorNotSupported;   // p wider than nsm strips
-  pl.boxb = XF_B * pl.inner * 4;
-  pl.boxb = (pl.boxb + 127) / 128 * 128;
-  pl.SA = XF_SA;
-  pl.SB = XF_SB;
+  if (best == 0.0) return cudaErrorNotSupported;   // p wider than nsm strips
+  pl.boxb = (pl.B * pl.inner * 4 + 127) / 128 * 128;
+  pl.SA = ff ? XF<true>::SA : XF<false>::SA;
+  pl.SB = XF_TV;
   pl.grid = pl.Gc * pl.Gr;
   pl.threads = XF_T;
   const size_t stage = (size_t)pl.nbox * pl.boxb;

@@ -1,43 +1,51 @@
-// Fused pass over FP32 X in float-float arithmetic (the certificates, the power
-// iteration, the last digits of FP32 solves): z = X beta, r = link(z),
-// g = X' r, X read from HBM once.
+// Fused passes over FP32 X with one product z: z = X beta, r = link(z),
+// g = X' r, X read from HBM once.  FF = false: the loop's pass, FP32 sums in
+// compensated pairs.  FF = true: float-float arithmetic (the certificates, the
+// power iteration, the last digits of FP32 solves).
 //
 // Strips x row groups, tiles kept in a ring from their dot products until
 // their axpy, the rows' words of z with their own arrival counts, link warps of
-// their own: as in xmma.cuh.  Each product x b, b = bh + bl, is formed exactly
-// as the FMA pair plus x bl and summed by TwoSum, in packed FP32 pairs
-// (dot_ff2: eleven instructions for two terms, about 48 significant bits).
-//
-// The sums are what bounds it: 5.5 packed instructions per element and
-// product, 22 us of the FP32 pipes for 5000 x 10000 at two cycles each, against
-// 30 us for X from HBM.  Hence twelve warps of them, three per scheduler, six
-// per product, in the registers of 512 threads:
-//  * a dot warp holds the strip of beta (hi, lo) and takes two rows of a block
-//    at a time;
+// their own: as in xmma.cuh.  The twelve or so warps of sums:
+//  * a dot warp holds the strip of beta and takes R rows of a block at a time;
 //  * an axpy warp owns 32 vectors of the strip and takes all rows, the weights
 //    read as ready operand pairs from shared memory.
-// 2000 x 5000, 96 certificates: 45 us each on the rows-and-columns kernel of
-// xstrip.cuh (one right-hand side; six summing warps, two per scheduler at most)
-// and 29 here; 5000 x 10000, two right-hand sides: 171 and 99 us.  What is left
-// over the pipes' 45 to 67 us is the depth of the ring (four blocks of 46 KB
-// between HBM and the end of their agreement) and, in small problems, filling
-// it.  Blocks of 8 rows: certificates 3% slower.
-// z in fixed point, two 64-bit words per row (8 bits of count each; the second
-// holds 44 further bits), converted by shifts: FP64 conversions of two lanes
-// per row pair would have taken as long as the sums.
+// z in fixed point, 64-bit words with 8 bits of count (FF: a second word holds
+// 44 further bits), converted by shifts: FP64 conversions of two lanes per row
+// pair would take as long as the sums.
+//
+// FP32: bound by how much of X the rings hold (32 MB) against the round trip
+// from HBM to the end of a block's agreement, 5.2 TB/s for 20000 x 50000
+// (862 us on xstrip.cuh's kernel, which sent X through L2 twice, 772 now); small
+// designs by the fill of that pipeline (4000 x 4000 logistic 42 -> 29 us,
+// 1000 x 1000 24 -> 14.5).  Blocks of 8 rows: with 16 rows 817, 28 and 14.9 us.
+//
+// FF: each product x b, b = bh + bl, is formed exactly as the FMA pair plus
+// x bl and summed by TwoSum in packed pairs (dot_ff2: eleven instructions for
+// two terms, about 48 significant bits).  The sums are what bounds it: 22 us of
+// the FP32 pipes per product of 5000 x 10000 at two cycles each, against 30 us
+// for X from HBM.  Hence six warps per product, three of the twelve on each
+// scheduler.  96 certificates at 2000 x 5000: 45 us each on xstrip.cuh's kernel
+// (six summing warps, two per scheduler at most), 27.5 here; 5000 x 10000, two
+// right-hand sides: 171 and 99 us.  What is left is the depth of the ring (four
+// blocks of 46 KB) and, in small problems, filling it.  Blocks of 8 rows: 3%
+// slower.
 #pragma once
 #include "xmma.cuh"
 
 namespace relax {
 
-constexpr int XF_SA = 6, XF_SB = 6, XF_NL = 3;   // dot, axpy and link warps
-constexpr int XF_T = 32 * (1 + XF_SA + XF_SB + XF_NL);
-constexpr int XF_TV = XF_SB;                     // vectors of the strip per lane of a dot warp
-constexpr int XF_B = 16;                          // rows of a block
-constexpr int XF_LB = 16 / XF_B;                 // blocks a link warp takes at a time
-constexpr int XF_RW = 2 * XF_LB * XF_NL;         // blocks of weights in shared memory
-constexpr int XF_MAXR = 16;                      // ring stages at most
-constexpr int XF_LO = 44;                        // bits of the second word below the first's unit
+template <bool FF> struct XF {
+  static constexpr int SA = FF ? 6 : 4, SB = 6, NL = FF ? 3 : 5;   // dot, axpy and link warps
+  static constexpr int B = FF ? 16 : 8;     // rows of a block
+  static constexpr int R = FF ? 2 : 4;      // rows a dot warp takes at a time
+  static constexpr int RW = 4 * NL;         // blocks of weights in shared memory
+  static constexpr int WF = FF ? 8 : 2;     // floats of a weight there
+};
+constexpr int XF_T = 512;
+static_assert(32 * (1 + XF<true>::SA + XF<true>::SB + XF<true>::NL) == XF_T && 32 * (1 + XF<false>::SA + XF<false>::SB + XF<false>::NL) == XF_T);
+constexpr int XF_TV = 6;                    // vectors of the strip per lane of a dot warp = axpy warps
+constexpr int XF_MAXR = 16;                 // ring stages at most
+constexpr int XF_LO = 44;                   // bits of the second word below the first's unit
 
 // m 2^sh as hi + lo 2^-XF_LO, in two's complement (|m 2^sh| < 2^54)
 __device__ __forceinline__ void fixed_words(float m, int sh, long long& hi, long long& lo) {
@@ -77,15 +85,17 @@ __device__ __forceinline__ bool wait_row2(const unsigned long long* p, unsigned 
   }
 }
 
-template <int NB>
-__global__ void __launch_bounds__(XF_T, 1) xff_kernel(const __grid_constant__ XSArgs a) {
+template <int NB, bool FF>
+__global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ XSArgs a) {
+  constexpr int XF_SA = XF<FF>::SA, XF_SB = XF<FF>::SB, XF_NL = XF<FF>::NL, XF_B = XF<FF>::B, XF_RW = XF<FF>::RW;
+  constexpr int R = XF<FF>::R, WORDS = FF ? 2 : 1;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t full[XF_MAXR], empty[XF_MAXR], wfull[XF_RW], wempty[XF_RW];
-  __shared__ __align__(16) float wts[XF_RW][XF_B][NB][8];   // wh wh -wh -wh wl wl
+  __shared__ __align__(16) float wts[XF_RW][XF_B][NB][XF<FF>::WF];   // w w, or wh wh -wh -wh wl wl
   __shared__ volatile int tmo;
   __shared__ int skip;
   __shared__ double lcomb[XF_NL][3];
-  __shared__ __align__(16) float bsh[2][32 * XF_TV * 4];   // the strip of beta, hi and lo
+  __shared__ __align__(16) float bsh[WORDS][32 * XF_TV * 4];   // the strip of beta, hi and lo
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     tmo = 0;
@@ -117,7 +127,7 @@ __global__ void __launch_bounds__(XF_T, 1) xff_kernel(const __grid_constant__ XS
   if (warp == 0) {
     // ------------------------------------------------ producer: HBM -> ring
     if (lane == 0) {
-      const uint64_t pol = policy_evict_first();
+      const uint64_t pol = a.keep ? policy_evict_normal() : policy_evict_first();
       int issued = 0;
       for (int k = 0; k < kloc; ++k) {
         const int s = k % a.RA;
@@ -144,7 +154,7 @@ __global__ void __launch_bounds__(XF_T, 1) xff_kernel(const __grid_constant__ XS
       const double bd = c < (int)a.sw && col < p ? static_cast<const double*>(a.ps->beta)[col] : 0.0;
       const float h = (float)bd;
       bsh[0][c] = h;
-      bsh[1][c] = (float)(bd - (double)h);
+      if constexpr (FF) bsh[1][c] = (float)(bd - (double)h);
       unsigned long long bits = (unsigned long long)__double_as_longlong(bd) & ~(1ull << 63);
       if (!(fabsf(h) < INFINITY) && bits < 0x7ff0000000000000ull) bits = 0x7ff0000000000000ull;   // beyond FP32
       mb = bits > mb ? bits : mb;
@@ -161,23 +171,26 @@ __global__ void __launch_bounds__(XF_T, 1) xff_kernel(const __grid_constant__ XS
       __threadfence();
       atomicAdd(a.zcnt, 1u);
     }
-    float2 bh[XF_TV][2], nb[XF_TV][2], bl[XF_TV][2];
+    float2 bh[XF_TV][2], nb[FF ? XF_TV : 1][2], bl[FF ? XF_TV : 1][2];
     uint32_t voff[XF_TV];
 #pragma unroll
     for (int t = 0; t < XF_TV; ++t) {
       const int v = lane + 32 * t;
       voff[t] = voffset(v);
-      const float4 h = *reinterpret_cast<const float4*>(&bsh[0][4 * v]), l = *reinterpret_cast<const float4*>(&bsh[1][4 * v]);
+      const float4 h = *reinterpret_cast<const float4*>(&bsh[0][4 * v]);
       bh[t][0] = make_float2(h.x, h.y);
       bh[t][1] = make_float2(h.z, h.w);
-      nb[t][0] = make_float2(-h.x, -h.y);
-      nb[t][1] = make_float2(-h.z, -h.w);
-      bl[t][0] = make_float2(l.x, l.y);
-      bl[t][1] = make_float2(l.z, l.w);
+      if constexpr (FF) {
+        const float4 l = *reinterpret_cast<const float4*>(&bsh[1][4 * v]);
+        nb[t][0] = make_float2(-h.x, -h.y);
+        nb[t][1] = make_float2(-h.z, -h.w);
+        bl[t][0] = make_float2(l.x, l.y);
+        bl[t][1] = make_float2(l.z, l.w);
+      }
     }
     int zs = 0;
     bool have_scale = false;
-    constexpr int UB = XF_B / 2;   // row pairs of a block
+    constexpr int UB = XF_B / R;
     const int units = kloc * UB;
 #pragma unroll 1
     for (int i = st; i < units; i += XF_SA) {
@@ -188,36 +201,57 @@ __global__ void __launch_bounds__(XF_T, 1) xff_kernel(const __grid_constant__ XS
         tmo = 1;
         break;
       }
-      const int64_t r0 = (int64_t)(cr + k * a.Gr) * XF_B + 2 * pr;
-      const unsigned char* row0 = smem + sa * stage + (size_t)(2 * pr) * rowpitch;
-      float2 hh[2], ll[2];
+      const int64_t r0 = (int64_t)(cr + k * a.Gr) * XF_B + R * pr;
+      const unsigned char* row0 = smem + sa * stage + (size_t)(R * pr) * rowpitch;
+      float2 hh[R], ll[FF ? R : 1];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) { hh[u] = make_float2(0.f, 0.f); ll[u] = make_float2(0.f, 0.f); }
+      for (int u = 0; u < R; ++u) hh[u] = make_float2(0.f, 0.f);
+      if constexpr (FF)
+#pragma unroll
+        for (int u = 0; u < R; ++u) ll[u] = make_float2(0.f, 0.f);
 #pragma unroll
       for (int t = 0; t < XF_TV; ++t) {
         if (32 * t < nvs) {   // uniform
-          const float4 x0 = *reinterpret_cast<const float4*>(row0 + voff[t]);
-          const float4 x1 = *reinterpret_cast<const float4*>(row0 + rowpitch + voff[t]);
-          dot_ff2(hh[0], ll[0], make_float2(x0.x, x0.y), bh[t][0], nb[t][0], bl[t][0]);
-          dot_ff2(hh[1], ll[1], make_float2(x1.x, x1.y), bh[t][0], nb[t][0], bl[t][0]);
-          dot_ff2(hh[0], ll[0], make_float2(x0.z, x0.w), bh[t][1], nb[t][1], bl[t][1]);
-          dot_ff2(hh[1], ll[1], make_float2(x1.z, x1.w), bh[t][1], nb[t][1], bl[t][1]);
+          float4 x[R];
+#pragma unroll
+          for (int u = 0; u < R; ++u) x[u] = *reinterpret_cast<const float4*>(row0 + u * rowpitch + voff[t]);
+#pragma unroll
+          for (int u = 0; u < R; ++u) {
+            const float2 xa = make_float2(x[u].x, x[u].y), xb = make_float2(x[u].z, x[u].w);
+            if constexpr (FF) {
+              dot_ff2(hh[u], ll[u], xa, bh[t][0], nb[t][0], bl[t][0]);
+              dot_ff2(hh[u], ll[u], xb, bh[t][1], nb[t][1], bl[t][1]);
+            } else {
+              hh[u] = fma2(xa, bh[t][0], hh[u]);
+              hh[u] = fma2(xb, bh[t][1], hh[u]);
+            }
+          }
         }
       }
-      float h[2], l[2];
+      float h[R], l[R];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < R; ++u) {
         h[u] = hh[u].x;
-        l[u] = ll[u].x + ll[u].y;
+        l[u] = FF ? ll[FF ? u : 0].x + ll[FF ? u : 0].y : 0.f;
         two_sum_acc(h[u], l[u], hh[u].y);
       }
-      // the lower half warp sums row 0, the upper one row 1
-      const bool up = (lane & 16) != 0;
-      float zh = up ? h[1] : h[0], zl = up ? l[1] : l[0];
-      pair_add(zh, zl, __shfl_xor_sync(0xffffffffu, up ? h[0] : h[1], 16), __shfl_xor_sync(0xffffffffu, up ? l[0] : l[1], 16));
+      // the lanes' sums, half of the rows to each half warp (and quarter), then
+      // row lane / (32 / R) over its 32 / R lanes
+      int o = 16;
 #pragma unroll
-      for (int o = 8; o > 0; o >>= 1)
-        pair_add(zh, zl, __shfl_xor_sync(0xffffffffu, zh, o), __shfl_xor_sync(0xffffffffu, zl, o));
+      for (int half = R / 2; half >= 1; half >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int u = 0; u < half; ++u) {
+          const float sh = up ? h[u] : h[u + half], sl = up ? l[u] : l[u + half];
+          h[u] = up ? h[u + half] : h[u];
+          l[u] = up ? l[u + half] : l[u];
+          pair_add(h[u], l[u], __shfl_xor_sync(0xffffffffu, sh, o), __shfl_xor_sync(0xffffffffu, sl, o));
+        }
+      }
+#pragma unroll
+      for (o = 16 / R; o > 0; o >>= 1)
+        pair_add(h[0], l[0], __shfl_xor_sync(0xffffffffu, h[0], o), __shfl_xor_sync(0xffffffffu, l[0], o));
       if (!have_scale) {
         if (!__all_sync(0xffffffffu, wait_count(a.zcnt, gridDim.x, a.limit_ns, a.status))) {
           tmo = 1;
@@ -226,15 +260,15 @@ __global__ void __launch_bounds__(XF_T, 1) xff_kernel(const __grid_constant__ XS
         zs = fixed_scale(a.rowl1 * __longlong_as_double((long long)__ldcg(&a.zmax[0])));
         have_scale = true;
       }
-      const int64_t row = r0 + (lane >> 4);
-      if ((lane & 15) == 0 && row < n) {
+      const int64_t row = r0 + lane / (32 / R);
+      if (lane % (32 / R) == 0 && row < n) {
         long long qh = 0, ql = 0;
         if (zs != INT_MIN) {
-          fixed_words(zh, zs - 8, qh, ql);
-          fixed_words(zl, zs - 8, qh, ql);
+          fixed_words(h[0], zs - 8, qh, ql);
+          fixed_words(l[0], zs - 8, qh, ql);
         }
-        atomicAdd(&a.zfix[2 * row], ((unsigned long long)qh << 8) + 1ull);
-        atomicAdd(&a.zfix[2 * row + 1], ((unsigned long long)ql << 8) + 1ull);
+        atomicAdd(&a.zfix[WORDS * row], ((unsigned long long)qh << 8) + 1ull);
+        if constexpr (FF) atomicAdd(&a.zfix[WORDS * row + 1], ((unsigned long long)ql << 8) + 1ull);
       }
     }
   } else if (warp < 1 + XF_SA + XF_SB) {
@@ -259,26 +293,47 @@ __global__ void __launch_bounds__(XF_T, 1) xff_kernel(const __grid_constant__ XS
       }
       if (on) {
         const unsigned char* col = smem + sb * stage + voff;
+        if constexpr (FF) {
 #pragma unroll 4
-        for (int j = 0; j < XF_B; ++j) {
-          const float4 x = *reinterpret_cast<const float4*>(col + (size_t)j * rowpitch);
+          for (int j = 0; j < XF_B; ++j) {
+            const float4 x = *reinterpret_cast<const float4*>(col + (size_t)j * rowpitch);
 #pragma unroll
-          for (int q = 0; q < NB; ++q) {
-            const float4 w = *reinterpret_cast<const float4*>(&wts[ws][j][q][0]);
-            const float2 wl = *reinterpret_cast<const float2*>(&wts[ws][j][q][4]);
-            dot_ff2(hi[q][0], lo[q][0], make_float2(x.x, x.y), make_float2(w.x, w.y), make_float2(w.z, w.w), wl);
-            dot_ff2(hi[q][1], lo[q][1], make_float2(x.z, x.w), make_float2(w.x, w.y), make_float2(w.z, w.w), wl);
+            for (int q = 0; q < NB; ++q) {
+              const float4 w = *reinterpret_cast<const float4*>(&wts[ws][j][q][0]);
+              const float2 wl = *reinterpret_cast<const float2*>(&wts[ws][j][q][XF<FF>::WF / 2]);
+              dot_ff2(hi[q][0], lo[q][0], make_float2(x.x, x.y), make_float2(w.x, w.y), make_float2(w.z, w.w), wl);
+              dot_ff2(hi[q][1], lo[q][1], make_float2(x.z, x.w), make_float2(w.x, w.y), make_float2(w.z, w.w), wl);
+            }
           }
+          // the low parts folded back, so that their own rounding stays small
+#pragma unroll
+          for (int q = 0; q < NB; ++q)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const float2 s = add2(hi[q][u], lo[q][u]);
+              lo[q][u] = sub2(lo[q][u], sub2(s, hi[q][u]));
+              hi[q][u] = s;
+            }
+        } else {
+          // plain FP32 over the block's rows, the blocks' sums in pairs
+          float2 acc[NB][2];
+#pragma unroll
+          for (int q = 0; q < NB; ++q) acc[q][0] = acc[q][1] = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int j = 0; j < XF_B; ++j) {
+            const float4 x = *reinterpret_cast<const float4*>(col + (size_t)j * rowpitch);
+#pragma unroll
+            for (int q = 0; q < NB; ++q) {
+              const float2 w = *reinterpret_cast<const float2*>(&wts[ws][j][q][0]);
+              acc[q][0] = fma2(make_float2(x.x, x.y), w, acc[q][0]);
+              acc[q][1] = fma2(make_float2(x.z, x.w), w, acc[q][1]);
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < NB; ++q)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) two_sum_acc2(hi[q][u], lo[q][u], acc[q][u]);
         }
-        // the low parts folded back, so that their own rounding stays small
-#pragma unroll
-        for (int q = 0; q < NB; ++q)
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const float2 s = add2(hi[q][u], lo[q][u]);
-            lo[q][u] = sub2(lo[q][u], sub2(s, hi[q][u]));
-            hi[q][u] = s;
-          }
       }
       __syncwarp();
       if (lane == 0) {
@@ -306,23 +361,23 @@ __global__ void __launch_bounds__(XF_T, 1) xff_kernel(const __grid_constant__ XS
     const double* zprev = static_cast<const double*>(a.ps->zprev);
     double* zout = static_cast<double*>(a.ps->zout);
     const double mom = a.ps->mom;
-    double uh = 0.0;   // value of the first word's unit
+    double uh = 0.0, ul = 0.0;   // values of the words' units
     bool have_scale = false;
     double lsum[3] = {0.0, 0.0, 0.0};
-    const int jl = lane % XF_B, hb = (lane / XF_B) % XF_LB;
-    for (int k0 = XF_LB * st; k0 < kloc; k0 += XF_LB * XF_NL) {
+    const int jl = lane % XF_B;
+    for (int k = st; k < kloc; k += XF_NL) {
       if (tmo) break;
-      const int k = k0 + hb;
-      const bool on = k < kloc && lane < 16;
-      const int64_t r0 = (int64_t)(cr + (k < kloc ? k : k0) * a.Gr) * XF_B;
+      const bool on = lane < XF_B;
+      const int64_t r0 = (int64_t)(cr + k * a.Gr) * XF_B;
       const int rows = (int)((n - r0) < XF_B ? (n - r0) : XF_B);
       const int64_t rowj = r0 + (jl < rows ? jl : rows - 1);
       const double yd = a.y[rowj];
       const double zp = need_zp ? zprev[rowj] : 0.0;
       const int ws = k % XF_RW;
       unsigned long long wh = 0ull, wl = 0ull;
-      const bool ok = (k >= kloc || k < XF_RW || mbar_wait<false>(&wempty[ws], ((k / XF_RW) - 1) & 1, a.limit_ns, a.status)) &&
-                      wait_row2(&a.zfix[2 * rowj], (unsigned)a.Gc, wh, wl, a.limit_ns, a.status);
+      bool ok = k < XF_RW || mbar_wait<false>(&wempty[ws], ((k / XF_RW) - 1) & 1, a.limit_ns, a.status);
+      if constexpr (FF) ok = ok && wait_row2(&a.zfix[2 * rowj], (unsigned)a.Gc, wh, wl, a.limit_ns, a.status);
+      else ok = ok && wait_row(&a.zfix[rowj], (unsigned)a.Gc, wh, a.limit_ns, a.status);
       if (!__all_sync(0xffffffffu, ok)) {
         tmo = 1;
         break;
@@ -334,26 +389,33 @@ __global__ void __launch_bounds__(XF_T, 1) xff_kernel(const __grid_constant__ XS
         }
         const int zs = fixed_scale(a.rowl1 * __longlong_as_double((long long)__ldcg(&a.zmax[0])));
         uh = zs == INT_MIN ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, 8 - zs);
+        ul = ldexp(uh, -XF_LO);
         have_scale = true;
       }
       double z[1];
-      z[0] = fma((double)((long long)wl >> 8), ldexp(uh, -XF_LO), (double)((long long)wh >> 8) * uh);
+      z[0] = (double)((long long)wh >> 8) * uh;
+      if constexpr (FF) z[0] = fma((double)((long long)wl >> 8), ul, z[0]);
       double rv[NB];
-      link_of<1, NB, false>(a.link, z, yd, zp, mom, rv);
+      link_of<1, NB, !FF>(a.link, z, yd, zp, mom, rv);
       if (on) {
 #pragma unroll
         for (int q = 0; q < NB; ++q) {
           const double r = jl < rows ? rv[q] : 0.0;   // rows past the end carry weight 0
-          const float h = (float)r, l = (float)(r - (double)h);
-          *reinterpret_cast<float4*>(&wts[ws][jl][q][0]) = make_float4(h, h, -h, -h);
-          *reinterpret_cast<float2*>(&wts[ws][jl][q][4]) = make_float2(l, l);
+          const float h = (float)r;
+          if constexpr (FF) {
+            const float l = (float)(r - (double)h);
+            *reinterpret_cast<float4*>(&wts[ws][jl][q][0]) = make_float4(h, h, -h, -h);
+            *reinterpret_cast<float2*>(&wts[ws][jl][q][XF<FF>::WF / 2]) = make_float2(l, l);
+          } else {
+            *reinterpret_cast<float2*>(&wts[ws][jl][q][0]) = make_float2(h, h);
+          }
         }
       }
       __syncwarp();
       if (jl == 0 && on) mbar_arrive(&wfull[ws]);
       if (on && cc == k % a.Gc && jl < rows) {   // this CTA records the block
         if (zout) zout[r0 + jl] = z[0];
-        if (a.lsum) loss_of<1, false>(a.link, z, yd, zp, lsum);
+        if (a.lsum) loss_of<1, !FF>(a.link, z, yd, zp, lsum);
       }
     }
     if (a.lsum) {

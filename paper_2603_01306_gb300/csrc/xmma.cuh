@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
   if (warp == 0) {
     // ------------------------------------------------ producer: HBM -> ring
     if (lane == 0) {
-      const uint64_t pol = policy_evict_first();
+      const uint64_t pol = a.keep ? policy_evict_normal() : policy_evict_first();
       int issued = 0;
       for (int k = 0; k < kloc; ++k) {
         const int s = k % a.RA;

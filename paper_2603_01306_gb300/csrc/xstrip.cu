@@ -17,13 +17,11 @@ static const void* kptr() {
 static const void* xstrip_ptr(int xk, bool f64acc, int NF, int NB) {
   if (NF == 1 && NB == 1) {
     if (xk == XK_F64) return kptr<double, double, 1, 1>();
-    if (xk == XK_F32) return kptr<float, float, 1, 1>();
   } else if (NF == 1 && NB == 2 && f64acc) {
     // the two-dual-point certificate
     if (xk == XK_F64) return kptr<double, double, 1, 2>();
   } else if (NF == 1 && NB == 2 && !f64acc) {
     if (xk == XK_F64) return kptr<double, double, 1, 2>();
-    if (xk == XK_F32) return kptr<float, float, 1, 2>();
   } else if (NF == 2 && NB == 1) {
     if (xk == XK_F64) return kptr<double, double, 2, 1>();
     if (xk == XK_F32 && f64acc) return kptr<float, float, 2, 1, true>();
@@ -45,7 +43,7 @@ static int xs_tv(int vec) { return vec == 2 ? XSShape<2>::TV : XSShape<4>::TV; }
 // RELAX_XS="B,SA,SB,lag,vps,mA,mB,Gr" overrides for tuning runs (0 keeps a default).
 cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t n, int64_t p) {
   if ((xk == XK_BF16 || xk == XK_FP8) && !f64acc && NF == 1) return xmma_plan(pl, xk, NB, n, p);
-  if (xk == XK_F32 && f64acc && NF == 1) return xff_plan(pl, NB, n, p);
+  if (xk == XK_F32 && NF == 1) return xf32_plan(pl, f64acc, NB, n, p);
   pl = XSPlan{};
   pl.xk = xk;
   pl.cert = f64acc;
@@ -209,6 +207,16 @@ void xstrip_zero_layout(const XSPlan& pl, void* base, XSArgs& a) {
   a.zcnt = reinterpret_cast<unsigned*>(b + oz);
   a.zmax = reinterpret_cast<unsigned long long*>(b + oz + 16);
   a.zfix = reinterpret_cast<unsigned long long*>(b + oz + 32);
+}
+
+// Three quarters of L2: an X below that is found there by the next pass (4000 x
+// 4000 FP32 29.2 -> 29.0 us, certificates at 2000 x 5000 28.8 -> 27.5), a larger
+// one only pushes out the vectors that are (20000 x 50000: p-phase 57 -> 71 us).
+bool x_fits_l2(int xk, int64_t n, int64_t p) {
+  int dev = 0, l2 = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
+  return (double)n * (double)p * xkind_esize(xk) <= 0.75 * (double)l2;
 }
 
 cudaError_t xstrip_launch(const XSPlan& pl, const XSArgs& a, bool clear, cudaStream_t st) {

@@ -1,5 +1,7 @@
 // Fused pass over X, strip-stationary: z = X beta, r = link(z), g = X' r, with
-// X read from HBM once per pass.
+// X read from HBM once per pass.  FP64 X, and the two-vector certificate of FP32
+// X; the other passes over FP32 X are xf32.cuh's, those over BF16 and FP8
+// xmma.cuh's.
 //
 // This is the matrix-vector work that dominates the method (Sec. 5.2.3); the
 // induced dual point zeta = -grad F(X beta) (Sec. 3.3) comes out of it as -r.
@@ -35,8 +37,7 @@
 // barrier phase more than one ahead of the last one it saw (the reason the
 // ring depths are multiples of the warp counts).  A stage is held from its
 // TMA issue until its warp has read the block, so the stages per ring, not
-// the warps, set the bytes in flight: narrow element types, whose blocks are
-// small, take several stages per warp.  Phase A may lead
+// the warps, set the bytes in flight.  Phase A may lead
 // phase B by at most `lag` blocks of the CTA (L2 footprint).  Every wait is
 // bounded: on expiry the kernel records ST_TIMEOUT, stops issuing and waiting,
 // lets the copies in flight land and returns.
@@ -74,6 +75,7 @@ struct XSArgs {
   int link;
   const double* y;
   const float* colscale; // FP8 storage (xmma.cuh): the columns' scales
+  int keep;              // single-crossing passes: X stays in L2 from pass to pass
   PassState* ps;
   unsigned long long* zfix;   // [NF][n] z in fixed point (two's complement)   } zeroed
   unsigned long long* zmax;   // [NF] max_j |beta_j| (bits of a nonnegative double) } before
@@ -297,12 +299,7 @@ template <typename TX, typename TA, int NF, int NB, bool FF = false>
 __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constant__ XSArgs a) {
   constexpr int VEC = XTraits<TX>::VEC;
   constexpr int TV = XSShape<VEC>::TV;
-  constexpr bool kF32 = sizeof(TA) == 4;
-  // FP32 sums on packed pairs (f32x2): measured faster wherever the pass does
-  // more than one FMA per 4 bytes of X (two right-hand sides); the
-  // one-right-hand-side FP32 pass ran 10% slower on pairs
-  constexpr bool kPair = kF32 && !FF && NB == 2;
-  static_assert(!FF || (sizeof(TX) == 4 && kF32), "float-float: FP32 X and FP32 pairs");
+  static_assert(FF == (sizeof(TA) == 4) && (!FF || sizeof(TX) == 4), "FP64 X in FP64, FP32 X as FP32 pairs");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t fullA[XS_MAXR], emptyA[XS_MAXR], fullB[XS_MAXR], emptyB[XS_MAXR];
   __shared__ volatile int tmo;        // a bounded wait expired: stop issuing and waiting
@@ -355,7 +352,6 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
   }
   // phase-B accumulators (used by the axpy warps only)
   TA acc[NB][TV][VEC];
-  float ahi[kF32 && !FF ? NB : 1][TV][VEC], alo[kF32 && !FF ? NB : 1][TV][VEC];
   float accl[FF ? NB : 1][TV][VEC];   // FF: low parts of acc
   double lsum[3] = {0.0, 0.0, 0.0};   // loss terms of the rows this lane records
   const bool axpy = warp >= 2 + a.SA && warp < 2 + a.SA + a.SB;
@@ -509,24 +505,6 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
         for (int f = 0; f < NF; ++f) ph[f][jj] = (TA)0;
         const int jr = jj < a.B ? jj : a.B - 1;   // rows >= rows: zero-filled or repeated, discarded
         const unsigned char* rowp = tile + (size_t)jr * rowpitch;
-        if constexpr (kPair) {
-          // FP32: even and odd columns in the two halves of a packed pair
-          float2 p2[NF];
-#pragma unroll
-          for (int f = 0; f < NF; ++f) p2[f] = make_float2(0.f, 0.f);
-#pragma unroll
-          for (int t = 0; t < TV; ++t) {
-            TA x[VEC];
-            XTraits<TX>::load(reinterpret_cast<const TX*>(rowp + voff[t]), x);
-#pragma unroll
-            for (int f = 0; f < NF; ++f)
-#pragma unroll
-              for (int l = 0; l < VEC; l += 2)
-                p2[f] = fma2(make_float2(x[l], x[l + 1]), make_float2(bv[f][t][l], bv[f][t][l + 1]), p2[f]);
-          }
-#pragma unroll
-          for (int f = 0; f < NF; ++f) ph[f][jj] = p2[f].x + p2[f].y;
-        } else {
 #pragma unroll
           for (int t = 0; t < TV; ++t) {
             TA x[VEC];
@@ -536,7 +514,6 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
 #pragma unroll
               for (int l = 0; l < VEC; ++l) ph[f][jj] += x[l] * bv[f][t][l];
           }
-        }
       }
       }
       // every read of the stage is done (the partials are in registers):
@@ -551,13 +528,6 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
           butterfly16(ph[f], phl[f], lane);
           mh[f] = ph[f][0];
           ml[f] = phl[f][0];
-        } else if constexpr (kF32) {
-          float pl[XS_MAXB];
-#pragma unroll
-          for (int jj = 0; jj < XS_MAXB; ++jj) pl[jj] = 0.f;
-          butterfly16(ph[f], pl, lane);
-          mh[f] = ph[f][0];
-          ml[f] = pl[0];
         } else {
           butterfly16(ph[f], lane);
           mh[f] = ph[f][0];
@@ -602,7 +572,6 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
         for (int l = 0; l < VEC; ++l) {
           acc[q][t][l] = (TA)0;
           if constexpr (FF) accl[q][t][l] = 0.f;
-          else if constexpr (kF32) { ahi[q][t][l] = 0.f; alo[q][t][l] = 0.f; }
         }
     const bool need_zp = a.link == LINK_CERTZ_LS || a.link == LINK_CERTZ_LOGI || a.link == LINK_CERT2_LS ||
                          a.link == LINK_CERT2_LOGI || (a.link == LINK_LOGISTIC && NB > 1);
@@ -636,7 +605,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
 #pragma unroll
       for (int f = 0; f < NF; ++f) z[f] = (double)(long long)__ldcg(&a.zfix[(size_t)f * n + rowj]) * zinv[f];
       double rv[NB];
-      link_of<NF, NB, kF32 && !FF>(a.link, z, yd, zp, mom, rv);
+      link_of<NF, NB, false>(a.link, z, yd, zp, mom, rv);
       if (jl >= rows) {
 #pragma unroll
         for (int q = 0; q < NB; ++q) rv[q] = 0.0;   // rows past the end carry weight 0
@@ -652,7 +621,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
       }
       if (cc == k % a.Gc && hb == 0 && jl < rows) {   // this CTA records the block
         if (zout) zout[r0 + jl] = z[0];
-        if (a.lsum) loss_of<NF, kF32 && !FF>(a.link, z, yd, zp, lsum);
+        if (a.lsum) loss_of<NF, false>(a.link, z, yd, zp, lsum);
       }
       const int sb = k % a.RB;   // one of this warp's stages
       if (!__all_sync(0xffffffffu, mbar_wait<false>(&fullB[sb], (k / a.RB) & 1, a.limit_ns, a.status))) {
@@ -691,17 +660,6 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
                 accl[q][t][l] = l2.x;
                 accl[q][t][l + 1] = l2.y;
               }
-          } else if constexpr (kPair) {
-            // two columns per packed FP32 FMA (the same roundings as two scalar FMAs)
-#pragma unroll
-            for (int l = 0; l < VEC; l += 2)
-#pragma unroll
-              for (int q = 0; q < NB; ++q) {
-                const float2 r2 = fma2(make_float2(w[q], w[q]), make_float2(x[l], x[l + 1]),
-                                       make_float2(acc[q][t][l], acc[q][t][l + 1]));
-                acc[q][t][l] = r2.x;
-                acc[q][t][l + 1] = r2.y;
-              }
           } else {
 #pragma unroll
             for (int l = 0; l < VEC; ++l)
@@ -716,29 +674,6 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
       if (lane == 0) {
         mbar_arrive(&emptyB[sb]);
         atomicAdd((unsigned*)&bcnt, 1u);
-      }
-      if constexpr (kF32 && !FF) {   // fold the block's FP32 sums into the compensated pair
-#pragma unroll
-        for (int q = 0; q < NB; ++q)
-#pragma unroll
-          for (int t = 0; t < TV; ++t)
-#pragma unroll
-            for (int l = 0; l < VEC; l += 2) {
-              if constexpr (kPair) {
-                float2 h2 = make_float2(ahi[q][t][l], ahi[q][t][l + 1]);
-                float2 l2 = make_float2(alo[q][t][l], alo[q][t][l + 1]);
-                two_sum_acc2(h2, l2, make_float2((float)acc[q][t][l], (float)acc[q][t][l + 1]));
-                ahi[q][t][l] = h2.x;
-                ahi[q][t][l + 1] = h2.y;
-                alo[q][t][l] = l2.x;
-                alo[q][t][l + 1] = l2.y;
-              } else {
-                two_sum_acc(ahi[q][t][l], alo[q][t][l], (float)acc[q][t][l]);
-                two_sum_acc(ahi[q][t][l + 1], alo[q][t][l + 1], (float)acc[q][t][l + 1]);
-              }
-              acc[q][t][l] = (TA)0;
-              acc[q][t][l + 1] = (TA)0;
-            }
       }
     }
   }
@@ -760,7 +695,6 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
           if (e < wcols) {
             const size_t o = ((size_t)st * NB + q) * wcols + e;
             if constexpr (FF) combf[o] = make_float2(acc[q][t][l], accl[q][t][l]);
-            else if constexpr (kF32) combf[o] = make_float2(ahi[q][t][l], alo[q][t][l]);
             else combd[o] = acc[q][t][l];
           }
         }
@@ -781,7 +715,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       const size_t at = ((size_t)cr * NB + q) * p + s0 + e;
-      if constexpr (kF32) {
+      if constexpr (FF) {
         ffs sum{0.f, 0.f};
         for (int w = 0; w < a.SB; ++w) {
           const float2 v = combf[((size_t)w * NB + q) * wcols + e];
