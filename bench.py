@@ -74,7 +74,7 @@ def measured_peaks():
 
 def kernel_source_hash():
     h = hashlib.sha256()
-    for f in ("xstrip.cuh", "xpass.cuh", "common.cuh"):
+    for f in ("xring.cuh", "xmma.cuh", "xstrip.cuh", "xpass.cuh", "common.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2603_01306_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -298,7 +298,7 @@ def run_ours(args):
         "lipschitz": results[-1].lipschitz,
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
-                     "kernel": "xstrip_kernel (fused X beta / link / X' r)",
+                     "kernel": "xring_kernel (fused X beta / link / X' r)",
                      "avg_launch_ms": avg_ms, "launches_timed": xp_n,
                      "algorithmic_bytes_per_launch": alg_bytes,
                      "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if peaks

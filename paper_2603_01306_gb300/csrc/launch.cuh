@@ -39,8 +39,8 @@ cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t
 bool x_fits_l2(int xk, int64_t n, int64_t p);
 // the BF16 / FP8 plans (xmma.cu; xstrip_plan and xstrip_launch go there)
 cudaError_t xmma_plan(XSPlan& pl, int xk, int NB, int64_t n, int64_t p);
-// the plans of FP32 X with one product z (xf32.cu; xstrip_plan goes there)
-cudaError_t xf32_plan(XSPlan& pl, bool ff, int NB, int64_t n, int64_t p);
+// the plans of FP32 and FP64 X with one product z (xring.cu; xstrip_plan goes there)
+cudaError_t xring_plan(XSPlan& pl, int xk, bool f64acc, int NB, int64_t n, int64_t p);
 cudaError_t xmma_launch(const XSPlan& pl, const XSArgs& a, cudaStream_t st);
 // encode the plan's tensor map of X (16-byte aligned, ldx * size a multiple of 16)
 cudaError_t xstrip_bind(XSPlan& pl, const void* X, int64_t ldx, int64_t n, int64_t p);

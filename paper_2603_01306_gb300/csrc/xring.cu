@@ -1,9 +1,9 @@
-// Plan of the passes over FP32 X with one product z.
+// Plan of the passes over FP32 and FP64 X with one product z.
 #include <algorithm>
 #include <cmath>
 
 #include "launch.cuh"
-#include "xf32.cuh"
+#include "xring.cuh"
 
 namespace relax {
 
@@ -13,29 +13,35 @@ namespace relax {
 // busiest CTA, a block's axpy taking as long as dot products with six vectors
 // per lane.  The FP32 pass is bound by X: the choice that keeps the most SMs
 // busy, strips under 2 KB counted as streaming less efficiently.
-cudaError_t xf32_plan(XSPlan& pl, bool ff, int NB, int64_t n, int64_t p) {
+template <typename TX, bool FF>
+static const void* ring_ptr(int NB) {
+  return NB == 1 ? reinterpret_cast<const void*>(&xring_kernel<TX, 1, FF>) : reinterpret_cast<const void*>(&xring_kernel<TX, 2, FF>);
+}
+
+cudaError_t xring_plan(XSPlan& pl, int xk, bool f64acc, int NB, int64_t n, int64_t p) {
+  const bool dbl = xk == XK_F64, ff = f64acc && !dbl;
+  const int es = xkind_esize(xk), vec = xkind_vec(xk);
   pl = XSPlan{};
-  pl.xk = XK_F32;
-  pl.cert = ff;
+  pl.xk = xk;
+  pl.cert = f64acc;
   pl.NF = 1;
   pl.NB = NB;
-  pl.words = ff ? 2 : 1;
-  pl.keep = x_fits_l2(XK_F32, n, p);
+  pl.words = ff || dbl ? 2 : 1;
+  pl.keep = x_fits_l2(xk, n, p);
   if (NB < 1 || NB > 2 || n < 1 || p < 1 || n > INT32_MAX || p > INT32_MAX) return cudaErrorNotSupported;
-  pl.kernel = ff ? (NB == 1 ? reinterpret_cast<const void*>(&xf32_kernel<1, true>) : reinterpret_cast<const void*>(&xf32_kernel<2, true>))
-                 : (NB == 1 ? reinterpret_cast<const void*>(&xf32_kernel<1, false>) : reinterpret_cast<const void*>(&xf32_kernel<2, false>));
+  pl.kernel = dbl ? ring_ptr<double, false>(NB) : ff ? ring_ptr<float, true>(NB) : ring_ptr<float, false>(NB);
   int dev = 0, nsm = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const int64_t nvec = (p + 3) / 4, cap = 32 * XF_TV;
-  pl.B = ff ? XF<true>::B : XF<false>::B;
+  const int64_t nvec = (p + vec - 1) / vec, cap = 32 * XF_TV;
+  pl.B = dbl ? XF<double, false>::B : ff ? XF<float, true>::B : XF<float, false>::B;
   pl.nblk = (int)((n + pl.B - 1) / pl.B);
   const int64_t most = std::max<int64_t>(1, ((n + 15) / 16 + 1) / 2);
   double best = 0.0;
   for (int64_t gc = (nvec + cap - 1) / cap; gc <= std::min<int64_t>({(int64_t)nsm, nvec, (int64_t)255}); ++gc) {
     const int64_t v = (nvec + gc - 1) / gc;
-    const int64_t nbox = (v * 4 + 255) / 256, vpb = (v + nbox - 1) / nbox;
+    const int64_t nbox = (v * vec + 255) / 256, vpb = (v + nbox - 1) / nbox;
     const int64_t gcc = (nvec + nbox * vpb - 1) / (nbox * vpb);
     if (nbox * vpb > cap || gcc > nsm) continue;
     const int64_t gr = std::max<int64_t>(1, std::min<int64_t>(nsm / gcc, most));
@@ -44,14 +50,14 @@ cudaError_t xf32_plan(XSPlan& pl, bool ff, int NB, int64_t n, int64_t p) {
     if (score <= best * 1.0001) continue;   // fewer strips where the score is the same
     best = score;
     pl.nbox = (int)nbox;
-    pl.inner = (int)(vpb * 4);
+    pl.inner = (int)(vpb * vec);
     pl.sw = nbox * pl.inner;
     pl.Gc = (int)gcc;
     pl.Gr = (int)gr;
   }
   if (best == 0.0) return cudaErrorNotSupported;   // p wider than nsm strips
-  pl.boxb = (pl.B * pl.inner * 4 + 127) / 128 * 128;
-  pl.SA = ff ? XF<true>::SA : XF<false>::SA;
+  pl.boxb = (pl.B * pl.inner * es + 127) / 128 * 128;
+  pl.SA = ff ? XF<float, true>::SA : XF<float, false>::SA;
   pl.SB = XF_TV;
   pl.grid = pl.Gc * pl.Gr;
   pl.threads = XF_T;

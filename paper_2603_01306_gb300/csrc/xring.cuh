@@ -1,6 +1,6 @@
-// Fused passes over FP32 X with one product z: z = X beta, r = link(z),
-// g = X' r, X read from HBM once.  FF = false: the loop's pass, FP32 sums in
-// compensated pairs.  FF = true: float-float arithmetic (the certificates, the
+// Fused passes over FP32 or FP64 X with one product z: z = X beta, r = link(z),
+// g = X' r, X read from HBM once.  FP64 X: FP64 throughout.  FP32 X, FF = false:
+// the loop's pass, FP32 sums in compensated pairs.  FF = true: float-float arithmetic (the certificates, the
 // power iteration, the last digits of FP32 solves).
 //
 // Strips x row groups, tiles kept in a ring from their dot products until
@@ -9,8 +9,8 @@
 //  * a dot warp holds the strip of beta and takes R rows of a block at a time;
 //  * an axpy warp owns 32 vectors of the strip and takes all rows, the weights
 //    read as ready operand pairs from shared memory.
-// z in fixed point, 64-bit words with 8 bits of count (FF: a second word holds
-// 44 further bits), converted by shifts: FP64 conversions of two lanes per row
+// z in fixed point, 64-bit words with 8 bits of count (FF, FP64: a second word
+// holds 44 further bits), converted by shifts: FP64 conversions of two lanes per row
 // pair would take as long as the sums.
 //
 // FP32: bound by how much of X the rings hold (32 MB) against the round trip
@@ -18,6 +18,11 @@
 // (862 us on xstrip.cuh's kernel, which sent X through L2 twice, 772 now); small
 // designs by the fill of that pipeline (4000 x 4000 logistic 42 -> 29 us,
 // 1000 x 1000 24 -> 14.5).  Blocks of 8 rows: with 16 rows 817, 28 and 14.9 us.
+//
+// FP64: latency in small designs (500 x 1000: 30.4 -> 16.4 us; a dependent FP64
+// operation takes 64 cycles), the FP64 pipe in large ones (16 cycles per warp
+// instruction and SM).  Blocks of 16 rows, since every block costs the link warps
+// the same.
 //
 // FF: each product x b, b = bh + bl, is formed exactly as the FMA pair plus
 // x bl and summed by TwoSum in packed pairs (dot_ff2: eleven instructions for
@@ -34,15 +39,16 @@
 
 namespace relax {
 
-template <bool FF> struct XF {
+template <typename TX, bool FF> struct XF {
   static constexpr int SA = FF ? 6 : 4, SB = 6, NL = FF ? 3 : 5;   // dot, axpy and link warps
-  static constexpr int B = FF ? 16 : 8;     // rows of a block
+  static constexpr int B = FF || sizeof(TX) == 8 ? 16 : 8;     // rows of a block
   static constexpr int R = FF ? 2 : 4;      // rows a dot warp takes at a time
   static constexpr int RW = 4 * NL;         // blocks of weights in shared memory
-  static constexpr int WF = FF ? 8 : 2;     // floats of a weight there
+  static constexpr int WF = FF ? 8 : 2;     // words of 32 bits of a weight there
 };
 constexpr int XF_T = 512;
-static_assert(32 * (1 + XF<true>::SA + XF<true>::SB + XF<true>::NL) == XF_T && 32 * (1 + XF<false>::SA + XF<false>::SB + XF<false>::NL) == XF_T);
+static_assert(32 * (1 + XF<float, true>::SA + XF<float, true>::SB + XF<float, true>::NL) == XF_T &&
+              32 * (1 + XF<float, false>::SA + XF<float, false>::SB + XF<float, false>::NL) == XF_T);
 constexpr int XF_TV = 6;                    // vectors of the strip per lane of a dot warp = axpy warps
 constexpr int XF_MAXR = 16;                 // ring stages at most
 constexpr int XF_LO = 44;                   // bits of the second word below the first's unit
@@ -85,17 +91,20 @@ __device__ __forceinline__ bool wait_row2(const unsigned long long* p, unsigned 
   }
 }
 
-template <int NB, bool FF>
-__global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ XSArgs a) {
-  constexpr int XF_SA = XF<FF>::SA, XF_SB = XF<FF>::SB, XF_NL = XF<FF>::NL, XF_B = XF<FF>::B, XF_RW = XF<FF>::RW;
-  constexpr int R = XF<FF>::R, WORDS = FF ? 2 : 1;
+template <typename TX, int NB, bool FF>
+__global__ void __launch_bounds__(XF_T, 1) xring_kernel(const __grid_constant__ XSArgs a) {
+  using K = XF<TX, FF>;
+  constexpr int XF_SA = K::SA, XF_SB = K::SB, XF_NL = K::NL, XF_B = K::B, XF_RW = K::RW, R = K::R;
+  constexpr bool D = sizeof(TX) == 8;            // FP64 throughout
+  constexpr int VEC = 16 / (int)sizeof(TX), WORDS = FF || D ? 2 : 1;
+  static_assert(!(FF && D), "float-float: FP32 X");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t full[XF_MAXR], empty[XF_MAXR], wfull[XF_RW], wempty[XF_RW];
-  __shared__ __align__(16) float wts[XF_RW][XF_B][NB][XF<FF>::WF];   // w w, or wh wh -wh -wh wl wl
+  __shared__ __align__(16) float wts[XF_RW][XF_B][NB][K::WF];   // w w (FP64: w), or wh wh -wh -wh wl wl
   __shared__ volatile int tmo;
   __shared__ int skip;
   __shared__ double lcomb[XF_NL][3];
-  __shared__ __align__(16) float bsh[WORDS][32 * XF_TV * 4];   // the strip of beta, hi and lo
+  __shared__ __align__(16) float bsh[FF ? 2 : 1][D ? 4 : 32 * XF_TV * 4];   // the strip of beta, hi and lo
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     tmo = 0;
@@ -111,12 +120,12 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
   const int cc = blockIdx.x % a.Gc, cr = blockIdx.x / a.Gc;
   const int64_t n = a.n, p = a.p;
   const int64_t s0 = (int64_t)cc * a.sw;
-  const int nvs = (int)((min(s0 + a.sw, p) - s0 + 3) / 4);   // vectors of the strip
-  const uint32_t rowpitch = (uint32_t)a.inner * 4u;
+  const int nvs = (int)((min(s0 + a.sw, p) - s0 + VEC - 1) / VEC);   // vectors of the strip
+  const uint32_t rowpitch = (uint32_t)a.inner * (uint32_t)sizeof(TX);
   const uint32_t tilebytes = (uint32_t)a.nbox * XF_B * rowpitch;   // whole boxes, out-of-range parts zero-filled
   const int kloc = (cr < a.nblk) ? (a.nblk - cr + a.Gr - 1) / a.Gr : 0;
   const size_t stage = (size_t)a.nbox * a.boxb;
-  const int vpb = a.inner / 4;
+  const int vpb = a.inner / VEC;
   // byte offset of a vector in row 0 of a tile (vectors past the strip read its
   // last one: their beta is zero and their sums are never written)
   auto voffset = [&](int v) {
@@ -149,14 +158,16 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
     const int st = warp - 1;
     // the strip of beta as pairs, split once for all dot warps
     unsigned long long mb = 0ull;
-    for (int c = tid - 32; c < 32 * XF_TV * 4; c += 32 * XF_SA) {
+    for (int c = tid - 32; c < 32 * XF_TV * VEC; c += 32 * XF_SA) {
       const int64_t col = s0 + c;
       const double bd = c < (int)a.sw && col < p ? static_cast<const double*>(a.ps->beta)[col] : 0.0;
-      const float h = (float)bd;
-      bsh[0][c] = h;
-      if constexpr (FF) bsh[1][c] = (float)(bd - (double)h);
       unsigned long long bits = (unsigned long long)__double_as_longlong(bd) & ~(1ull << 63);
-      if (!(fabsf(h) < INFINITY) && bits < 0x7ff0000000000000ull) bits = 0x7ff0000000000000ull;   // beyond FP32
+      if constexpr (!D) {
+        const float h = (float)bd;
+        bsh[0][c] = h;
+        if constexpr (FF) bsh[1][c] = (float)(bd - (double)h);
+        if (!(fabsf(h) < INFINITY) && bits < 0x7ff0000000000000ull) bits = 0x7ff0000000000000ull;   // beyond FP32
+      }
       mb = bits > mb ? bits : mb;
     }
     // this CTA's max |beta_j| (NaN dominates: its bits compare above +Inf)
@@ -171,13 +182,22 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
       __threadfence();
       atomicAdd(a.zcnt, 1u);
     }
+    double bd[D ? XF_TV : 1][2];
     float2 bh[XF_TV][2], nb[FF ? XF_TV : 1][2], bl[FF ? XF_TV : 1][2];
     uint32_t voff[XF_TV];
 #pragma unroll
     for (int t = 0; t < XF_TV; ++t) {
       const int v = lane + 32 * t;
       voff[t] = voffset(v);
-      const float4 h = *reinterpret_cast<const float4*>(&bsh[0][4 * v]);
+      if constexpr (D) {
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const int64_t col = s0 + (int64_t)v * 2 + c;
+          bd[t][c] = v < nvs && col < p ? static_cast<const double*>(a.ps->beta)[col] : 0.0;
+        }
+        continue;
+      }
+      const float4 h = *reinterpret_cast<const float4*>(&bsh[0][D ? 0 : 4 * v]);
       bh[t][0] = make_float2(h.x, h.y);
       bh[t][1] = make_float2(h.z, h.w);
       if constexpr (FF) {
@@ -189,6 +209,7 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
       }
     }
     int zs = 0;
+    double zf = 0.0;   // FP64: 2^(zs - 8)
     bool have_scale = false;
     constexpr int UB = XF_B / R;
     const int units = kloc * UB;
@@ -203,6 +224,36 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
       }
       const int64_t r0 = (int64_t)(cr + k * a.Gr) * XF_B + R * pr;
       const unsigned char* row0 = smem + sa * stage + (size_t)(R * pr) * rowpitch;
+      double zd[R];
+      if constexpr (D) {
+#pragma unroll
+        for (int u = 0; u < R; ++u) zd[u] = 0.0;
+#pragma unroll
+        for (int t = 0; t < XF_TV; ++t) {
+          if (32 * t < nvs) {   // uniform
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+              const double2 x = *reinterpret_cast<const double2*>(row0 + u * rowpitch + voff[t]);
+              zd[u] = fma(x.x, bd[t][0], zd[u]);
+              zd[u] = fma(x.y, bd[t][1], zd[u]);
+            }
+          }
+        }
+        int o = 16;
+#pragma unroll
+        for (int half = R / 2; half >= 1; half >>= 1, o >>= 1) {
+          const bool up = (lane & o) != 0;
+#pragma unroll
+          for (int u = 0; u < half; ++u) {
+            const double s = up ? zd[u] : zd[u + half];
+            zd[u] = (up ? zd[u + half] : zd[u]) + __shfl_xor_sync(0xffffffffu, s, o);
+          }
+        }
+#pragma unroll
+        for (o = 16 / R; o > 0; o >>= 1) zd[0] += __shfl_xor_sync(0xffffffffu, zd[0], o);
+      }
+      float h[R], l[R];
+      if constexpr (!D) {
       float2 hh[R], ll[FF ? R : 1];
 #pragma unroll
       for (int u = 0; u < R; ++u) hh[u] = make_float2(0.f, 0.f);
@@ -228,7 +279,6 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
           }
         }
       }
-      float h[R], l[R];
 #pragma unroll
       for (int u = 0; u < R; ++u) {
         h[u] = hh[u].x;
@@ -252,23 +302,31 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
 #pragma unroll
       for (o = 16 / R; o > 0; o >>= 1)
         pair_add(h[0], l[0], __shfl_xor_sync(0xffffffffu, h[0], o), __shfl_xor_sync(0xffffffffu, l[0], o));
+      }
       if (!have_scale) {
         if (!__all_sync(0xffffffffu, wait_count(a.zcnt, gridDim.x, a.limit_ns, a.status))) {
           tmo = 1;
           break;
         }
         zs = fixed_scale(a.rowl1 * __longlong_as_double((long long)__ldcg(&a.zmax[0])));
+        zf = zs == INT_MIN ? 0.0 : ldexp(1.0, zs - 8);
         have_scale = true;
       }
       const int64_t row = r0 + lane / (32 / R);
       if (lane % (32 / R) == 0 && row < n) {
         long long qh = 0, ql = 0;
         if (zs != INT_MIN) {
-          fixed_words(h[0], zs - 8, qh, ql);
-          fixed_words(l[0], zs - 8, qh, ql);
+          if constexpr (D) {
+            const double v = zd[0] * zf, vi = rint(v);
+            qh = (long long)vi;
+            ql = __double2ll_rn((v - vi) * (double)(1ll << XF_LO));
+          } else {
+            fixed_words(h[0], zs - 8, qh, ql);
+            fixed_words(l[0], zs - 8, qh, ql);
+          }
         }
         atomicAdd(&a.zfix[WORDS * row], ((unsigned long long)qh << 8) + 1ull);
-        if constexpr (FF) atomicAdd(&a.zfix[WORDS * row + 1], ((unsigned long long)ql << 8) + 1ull);
+        if constexpr (WORDS == 2) atomicAdd(&a.zfix[WORDS * row + 1], ((unsigned long long)ql << 8) + 1ull);
       }
     }
   } else if (warp < 1 + XF_SA + XF_SB) {
@@ -277,11 +335,12 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
     const int v = 32 * e + lane;
     const bool on = 32 * e < nvs;   // uniform
     const uint32_t voff = voffset(v);
+    double ad[NB][2];
     float2 hi[NB][2], lo[NB][2];
 #pragma unroll
     for (int q = 0; q < NB; ++q)
 #pragma unroll
-      for (int u = 0; u < 2; ++u) { hi[q][u] = make_float2(0.f, 0.f); lo[q][u] = make_float2(0.f, 0.f); }
+      for (int u = 0; u < 2; ++u) { hi[q][u] = make_float2(0.f, 0.f); lo[q][u] = make_float2(0.f, 0.f); ad[q][u] = 0.0; }
     for (int k = 0; k < kloc; ++k) {
       if (tmo) break;
       const int ws = k % XF_RW, sb = k % a.RA;
@@ -293,14 +352,25 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
       }
       if (on) {
         const unsigned char* col = smem + sb * stage + voff;
-        if constexpr (FF) {
+        if constexpr (D) {
+#pragma unroll
+          for (int j = 0; j < XF_B; ++j) {
+            const double2 x = *reinterpret_cast<const double2*>(col + (size_t)j * rowpitch);
+#pragma unroll
+            for (int q = 0; q < NB; ++q) {
+              const double w = *reinterpret_cast<const double*>(&wts[ws][j][q][0]);
+              ad[q][0] = fma(x.x, w, ad[q][0]);
+              ad[q][1] = fma(x.y, w, ad[q][1]);
+            }
+          }
+        } else if constexpr (FF) {
 #pragma unroll 4
           for (int j = 0; j < XF_B; ++j) {
             const float4 x = *reinterpret_cast<const float4*>(col + (size_t)j * rowpitch);
 #pragma unroll
             for (int q = 0; q < NB; ++q) {
               const float4 w = *reinterpret_cast<const float4*>(&wts[ws][j][q][0]);
-              const float2 wl = *reinterpret_cast<const float2*>(&wts[ws][j][q][XF<FF>::WF / 2]);
+              const float2 wl = *reinterpret_cast<const float2*>(&wts[ws][j][q][K::WF / 2]);
               dot_ff2(hi[q][0], lo[q][0], make_float2(x.x, x.y), make_float2(w.x, w.y), make_float2(w.z, w.w), wl);
               dot_ff2(hi[q][1], lo[q][1], make_float2(x.z, x.w), make_float2(w.x, w.y), make_float2(w.z, w.w), wl);
             }
@@ -341,9 +411,17 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
         mbar_arrive(&wempty[ws]);
       }
     }
-    // g[cr][q][column] as normalised pairs
-    float2* g = static_cast<float2*>(a.g);
-    if (v < nvs)
+    // g[cr][q][column], FP32 data as normalised pairs
+    if constexpr (D) {
+      if (v < nvs)
+#pragma unroll
+        for (int q = 0; q < NB; ++q)
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const int64_t colj = s0 + (int64_t)v * 2 + c;
+            if (colj < p) static_cast<double*>(a.g)[((size_t)cr * NB + q) * p + colj] = ad[q][c];
+          }
+    } else if (v < nvs)
 #pragma unroll
       for (int q = 0; q < NB; ++q)
 #pragma unroll
@@ -351,7 +429,7 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
           const int64_t colj = s0 + (int64_t)v * 4 + c;
           const float2 h2 = hi[q][c >> 1], l2 = lo[q][c >> 1];
           const ffs s = ff_add((c & 1) ? ffs{h2.y, l2.y} : ffs{h2.x, l2.x}, ffs{0.f, 0.f});
-          if (colj < p) g[((size_t)cr * NB + q) * p + colj] = make_float2(s.hi, s.lo);
+          if (colj < p) static_cast<float2*>(a.g)[((size_t)cr * NB + q) * p + colj] = make_float2(s.hi, s.lo);
         }
   } else {
     // ------------------------------------------------ the link of the rows
@@ -376,7 +454,7 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
       const int ws = k % XF_RW;
       unsigned long long wh = 0ull, wl = 0ull;
       bool ok = k < XF_RW || mbar_wait<false>(&wempty[ws], ((k / XF_RW) - 1) & 1, a.limit_ns, a.status);
-      if constexpr (FF) ok = ok && wait_row2(&a.zfix[2 * rowj], (unsigned)a.Gc, wh, wl, a.limit_ns, a.status);
+      if constexpr (WORDS == 2) ok = ok && wait_row2(&a.zfix[2 * rowj], (unsigned)a.Gc, wh, wl, a.limit_ns, a.status);
       else ok = ok && wait_row(&a.zfix[rowj], (unsigned)a.Gc, wh, a.limit_ns, a.status);
       if (!__all_sync(0xffffffffu, ok)) {
         tmo = 1;
@@ -394,18 +472,20 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
       }
       double z[1];
       z[0] = (double)((long long)wh >> 8) * uh;
-      if constexpr (FF) z[0] = fma((double)((long long)wl >> 8), ul, z[0]);
+      if constexpr (WORDS == 2) z[0] = fma((double)((long long)wl >> 8), ul, z[0]);
       double rv[NB];
-      link_of<1, NB, !FF>(a.link, z, yd, zp, mom, rv);
+      link_of<1, NB, !FF && !D>(a.link, z, yd, zp, mom, rv);
       if (on) {
 #pragma unroll
         for (int q = 0; q < NB; ++q) {
           const double r = jl < rows ? rv[q] : 0.0;   // rows past the end carry weight 0
           const float h = (float)r;
-          if constexpr (FF) {
+          if constexpr (D) {
+            *reinterpret_cast<double*>(&wts[ws][jl][q][0]) = r;
+          } else if constexpr (FF) {
             const float l = (float)(r - (double)h);
             *reinterpret_cast<float4*>(&wts[ws][jl][q][0]) = make_float4(h, h, -h, -h);
-            *reinterpret_cast<float2*>(&wts[ws][jl][q][XF<FF>::WF / 2]) = make_float2(l, l);
+            *reinterpret_cast<float2*>(&wts[ws][jl][q][K::WF / 2]) = make_float2(l, l);
           } else {
             *reinterpret_cast<float2*>(&wts[ws][jl][q][0]) = make_float2(h, h);
           }
@@ -415,7 +495,7 @@ __global__ void __launch_bounds__(XF_T, 1) xf32_kernel(const __grid_constant__ X
       if (jl == 0 && on) mbar_arrive(&wfull[ws]);
       if (on && cc == k % a.Gc && jl < rows) {   // this CTA records the block
         if (zout) zout[r0 + jl] = z[0];
-        if (a.lsum) loss_of<1, !FF>(a.link, z, yd, zp, lsum);
+        if (a.lsum) loss_of<1, !FF && !D>(a.link, z, yd, zp, lsum);
       }
     }
     if (a.lsum) {

@@ -14,18 +14,11 @@ static const void* kptr() {
   return reinterpret_cast<const void*>(&xstrip_kernel<TX, TA, NF, NB, FF>);
 }
 
+// the certificate of two different vectors; FP32 X in float-float arithmetic
 static const void* xstrip_ptr(int xk, bool f64acc, int NF, int NB) {
-  if (NF == 1 && NB == 1) {
-    if (xk == XK_F64) return kptr<double, double, 1, 1>();
-  } else if (NF == 1 && NB == 2 && f64acc) {
-    // the two-dual-point certificate
-    if (xk == XK_F64) return kptr<double, double, 1, 2>();
-  } else if (NF == 1 && NB == 2 && !f64acc) {
-    if (xk == XK_F64) return kptr<double, double, 1, 2>();
-  } else if (NF == 2 && NB == 1) {
-    if (xk == XK_F64) return kptr<double, double, 2, 1>();
-    if (xk == XK_F32 && f64acc) return kptr<float, float, 2, 1, true>();
-  }
+  if (NF != 2 || NB != 1) return nullptr;
+  if (xk == XK_F64) return kptr<double, double, 2, 1>();
+  if (xk == XK_F32 && f64acc) return kptr<float, float, 2, 1, true>();
   return nullptr;
 }
 
@@ -43,7 +36,7 @@ static int xs_tv(int vec) { return vec == 2 ? XSShape<2>::TV : XSShape<4>::TV; }
 // RELAX_XS="B,SA,SB,lag,vps,mA,mB,Gr" overrides for tuning runs (0 keeps a default).
 cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t n, int64_t p) {
   if ((xk == XK_BF16 || xk == XK_FP8) && !f64acc && NF == 1) return xmma_plan(pl, xk, NB, n, p);
-  if (xk == XK_F32 && NF == 1) return xf32_plan(pl, f64acc, NB, n, p);
+  if ((xk == XK_F32 || xk == XK_F64) && NF == 1) return xring_plan(pl, xk, f64acc, NB, n, p);
   pl = XSPlan{};
   pl.xk = xk;
   pl.cert = f64acc;

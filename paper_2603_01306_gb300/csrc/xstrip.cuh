@@ -1,6 +1,6 @@
 // Fused pass over X, strip-stationary: z = X beta, r = link(z), g = X' r, with
-// X read from HBM once per pass.  FP64 X, and the two-vector certificate of FP32
-// X; the other passes over FP32 X are xf32.cuh's, those over BF16 and FP8
+// X read from HBM once per pass.  Left with the certificate of two different
+// vectors; the passes with one product are xring.cuh's, those over BF16 and FP8
 // xmma.cuh's.
 //
 // This is the matrix-vector work that dominates the method (Sec. 5.2.3); the
@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
       TA ph[NF][XS_MAXB];
       float phl[FF ? NF : 1][XS_MAXB];   // FF: low parts
       if constexpr (FF) {
-        // float-float, two forward vectors (one: xff.cuh): two rows at a time,
+        // float-float, two forward vectors (one: xring.cuh): two rows at a time,
         // so that two chains of dependent sums per vector are in flight (a
         // fully unrolled block of them outgrew the instruction cache), in
         // packed FP32 pairs; the row partials go to a per-lane array for the
