@@ -13,9 +13,10 @@ namespace relax {
 // busiest CTA, a block's axpy taking as long as dot products with six vectors
 // per lane.  The FP32 pass is bound by X: the choice that keeps the most SMs
 // busy, strips under 2 KB counted as streaming less efficiently.
-template <typename TX, bool FF>
+template <typename TX, bool FF, int ROWS>
 static const void* ring_ptr(int NB) {
-  return NB == 1 ? reinterpret_cast<const void*>(&xring_kernel<TX, 1, FF>) : reinterpret_cast<const void*>(&xring_kernel<TX, 2, FF>);
+  return NB == 1 ? reinterpret_cast<const void*>(&xring_kernel<TX, 1, FF, ROWS>)
+                 : reinterpret_cast<const void*>(&xring_kernel<TX, 2, FF, ROWS>);
 }
 
 cudaError_t xring_plan(XSPlan& pl, int xk, bool f64acc, int NB, int64_t n, int64_t p) {
@@ -29,13 +30,16 @@ cudaError_t xring_plan(XSPlan& pl, int xk, bool f64acc, int NB, int64_t n, int64
   pl.words = ff || dbl ? 2 : 1;
   pl.keep = x_fits_l2(xk, n, p);
   if (NB < 1 || NB > 2 || n < 1 || p < 1 || n > INT32_MAX || p > INT32_MAX) return cudaErrorNotSupported;
-  pl.kernel = dbl ? ring_ptr<double, false>(NB) : ff ? ring_ptr<float, true>(NB) : ring_ptr<float, false>(NB);
+  pl.B = dbl || ff || pl.keep ? 16 : 8;   // (both sides: xring.cuh)
+  pl.kernel = dbl           ? ring_ptr<double, false, 16>(NB)
+              : ff          ? ring_ptr<float, true, 16>(NB)
+              : pl.B == 16 ? ring_ptr<float, false, 16>(NB)
+                            : ring_ptr<float, false, 8>(NB);
   int dev = 0, nsm = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const int64_t nvec = (p + vec - 1) / vec, cap = 32 * XF_TV;
-  pl.B = dbl ? XF<double, false>::B : ff ? XF<float, true>::B : XF<float, false>::B;
   pl.nblk = (int)((n + pl.B - 1) / pl.B);
   const int64_t most = std::max<int64_t>(1, ((n + 15) / 16 + 1) / 2);
   double best = 0.0;
@@ -57,7 +61,7 @@ cudaError_t xring_plan(XSPlan& pl, int xk, bool f64acc, int NB, int64_t n, int64
   }
   if (best == 0.0) return cudaErrorNotSupported;   // p wider than nsm strips
   pl.boxb = (pl.B * pl.inner * es + 127) / 128 * 128;
-  pl.SA = ff ? XF<float, true>::SA : XF<float, false>::SA;
+  pl.SA = ff ? XF<float, true, 16>::SA : dbl ? XF<double, false, 16>::SA : XF<float, false, 8>::SA;
   pl.SB = XF_TV;
   pl.grid = pl.Gc * pl.Gr;
   pl.threads = XF_T;

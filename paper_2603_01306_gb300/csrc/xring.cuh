@@ -14,10 +14,14 @@
 // pair would take as long as the sums.
 //
 // FP32: bound by how much of X the rings hold (32 MB) against the round trip
-// from HBM to the end of a block's agreement, 5.2 TB/s for 20000 x 50000
-// (862 us on xstrip.cuh's kernel, which sent X through L2 twice, 772 now); small
-// designs by the fill of that pipeline (4000 x 4000 logistic 42 -> 29 us,
-// 1000 x 1000 24 -> 14.5).  Blocks of 8 rows: with 16 rows 817, 28 and 14.9 us.
+// from HBM to the end of a block's agreement.  20000 x 50000: 862 us on
+// xstrip.cuh's kernel, which sent X through L2 twice, 718 now (5.57 TB/s).
+// Eight rows per dot warp: its butterfly takes 9 exchanges of pairs instead of 12
+// for two times four (776 us; two rows 1204).  5 + 4 dot and link warps; 6 + 3
+// 725, 5 + 3 722, 6 + 4 740, 7 + 2 740, and with four rows 4 + 5 776, 6 + 5 741,
+// 4 + 9 788.  Blocks of 8 rows, of 16 where X stays in L2 (ROWS): 20000 x 50000
+// 718 and 764, 4000 x 4000 logistic 28.9 and 25.0 (42.5 before), 1000 x 1000 14.3
+// and 14.2 (24.5).  Prefetching the blocks after the ring into L2 lost: 920.
 //
 // FP64: latency in small designs (500 x 1000: 30.4 -> 16.4 us; a dependent FP64
 // operation takes 64 cycles), the FP64 pipe in large ones (16 cycles per warp
@@ -39,16 +43,18 @@
 
 namespace relax {
 
-template <typename TX, bool FF> struct XF {
-  static constexpr int SA = FF ? 6 : 4, SB = 6, NL = FF ? 3 : 5;   // dot, axpy and link warps
-  static constexpr int B = FF || sizeof(TX) == 8 ? 16 : 8;     // rows of a block
-  static constexpr int R = FF ? 2 : 4;      // rows a dot warp takes at a time
+template <typename TX, bool FF, int ROWS> struct XF {
+  static constexpr bool LOOP = !FF && sizeof(TX) == 4;
+  static constexpr int SA = FF ? 6 : LOOP ? 5 : 4, SB = 6, NL = FF ? 3 : LOOP ? 4 : 5;   // dot, axpy and link warps
+  static constexpr int B = ROWS;            // rows of a block
+  static constexpr int R = FF ? 2 : LOOP ? 8 : 4;   // rows a dot warp takes at a time
   static constexpr int RW = 4 * NL;         // blocks of weights in shared memory
   static constexpr int WF = FF ? 8 : 2;     // words of 32 bits of a weight there
 };
 constexpr int XF_T = 512;
-static_assert(32 * (1 + XF<float, true>::SA + XF<float, true>::SB + XF<float, true>::NL) == XF_T &&
-              32 * (1 + XF<float, false>::SA + XF<float, false>::SB + XF<float, false>::NL) == XF_T);
+static_assert(1 + XF<float, true, 16>::SA + XF<float, true, 16>::SB + XF<float, true, 16>::NL == XF_T / 32 &&
+              1 + XF<float, false, 8>::SA + XF<float, false, 8>::SB + XF<float, false, 8>::NL == XF_T / 32 &&
+              1 + XF<double, false, 16>::SA + XF<double, false, 16>::SB + XF<double, false, 16>::NL == XF_T / 32);
 constexpr int XF_TV = 6;                    // vectors of the strip per lane of a dot warp = axpy warps
 constexpr int XF_MAXR = 16;                 // ring stages at most
 constexpr int XF_LO = 44;                   // bits of the second word below the first's unit
@@ -91,9 +97,9 @@ __device__ __forceinline__ bool wait_row2(const unsigned long long* p, unsigned 
   }
 }
 
-template <typename TX, int NB, bool FF>
+template <typename TX, int NB, bool FF, int ROWS>
 __global__ void __launch_bounds__(XF_T, 1) xring_kernel(const __grid_constant__ XSArgs a) {
-  using K = XF<TX, FF>;
+  using K = XF<TX, FF, ROWS>;
   constexpr int XF_SA = K::SA, XF_SB = K::SB, XF_NL = K::NL, XF_B = K::B, XF_RW = K::RW, R = K::R;
   constexpr bool D = sizeof(TX) == 8;            // FP64 throughout
   constexpr int VEC = 16 / (int)sizeof(TX), WORDS = FF || D ? 2 : 1;
