@@ -178,15 +178,14 @@ relax_status relax_solve(relax_handle* h, const int8_t* fixings, const void* war
  * Per iteration the active nodes' points are the rows of a matrix B;
  * Z = X B' and G = X' R run as two products (FP32 X: the library's
  * tensor-core kernel on BF16 planes of X, X', B and R, FP32-accurate products
- * summed over K chunks in FP64; FP64 X: FP64 products), and each node's
+ * whose partial tiles are summed in a fixed order; FP64 X: FP64 products), and each node's
  * prox / g / g* / gap / restart step runs in its own segment of one launch.
  * Nodes converge after uneven iteration counts and leave the batch every 16
  * iterations (each round of 16 is one CUDA graph per active-set size); the
  * stall rule's window is at most 200 inside a batch, and a node that stalls
  * above gap_tol is finished by relax_solve's loop from its best point
  * (out[j].polish_iters).  The first batched call of a FP32 handle builds the
- * BF16 planes of X and X' (six bytes per element of X each) and times a few
- * K-chunk choices per product, keeping the fastest for the handle.  Each node's bound is
+ * BF16 planes of X and X' (six bytes per element of X each).  Each node's bound is
  * certified in FP64 as in relax_solve (without resuming).  Needs FP32 or
  * FP64 storage of X (RELAX_ENOTSUP for BF16/FP8).  Returns RELAX_OK when every
  * node certified gap_tol, else the first failing node's status (out[j].status
@@ -202,8 +201,8 @@ relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int8_t* fixing
  * dominate the method, Sec. 5.2; stacked as matrix products for many nodes).
  *   points: device [nb][p] of the handle's dtype.
  *   z_out: device double [nb][n]; g_out: device double [nb][p].
- * FP32 X: tensor-core products on BF16 planes (FP32-accurate products, FP64
- * sums of the K chunks); FP64 X: FP64 products.  Needs FP32 or FP64 storage
+ * FP32 X: tensor-core products on BF16 planes (FP32-accurate products, the
+ * partial tiles summed in a fixed order); FP64 X: FP64 products.  Needs FP32 or FP64 storage
  * (RELAX_ENOTSUP otherwise).
  *   products_ms: host double[2] or NULL: FP32 X, the device time of the two
  *      tensor-core launches (z, then g), from CUDA events on the handle's stream.
@@ -268,7 +267,8 @@ relax_status relax_destroy(relax_handle* h);
  *   counts_out: device int32[2] or NULL: {n_top, n_nz} = free coordinates with
  *      z_j = 1 (placed before the pooled block of Algorithm 2) and nonzero free
  *      outputs.
- * Uses stream-ordered scratch (cudaMallocAsync) on `stream`; does not synchronize,
+ * Takes no scratch where p fits one thread-block cluster (stream-ordered scratch
+ * on `stream` beyond that); does not synchronize,
  * so a failure inside the kernel cannot change the returned status.  It shows
  * in the outputs instead: a NaN or Inf in beta_in, or a bounded device wait
  * that expired, makes beta_out all NaN (every coordinate the failing blocks
