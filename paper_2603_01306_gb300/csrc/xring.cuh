@@ -34,8 +34,9 @@
 // the FP32 pipes per product of 5000 x 10000 at two cycles each, against 30 us
 // for X from HBM.  Hence six warps per product, three of the twelve on each
 // scheduler.  96 certificates at 2000 x 5000: 45 us each on xstrip.cuh's kernel
-// (six summing warps, two per scheduler at most), 27.5 here; 5000 x 10000, two
-// right-hand sides: 171 and 99 us.  What is left is the depth of the ring (four
+// (six summing warps, two per scheduler at most), 27.0 here; 5000 x 10000, two
+// right-hand sides: 171 and 96 us.  Four rows per dot warp (two: 2.68 ms for the
+// 96, 45.9 for 256 nodes of 5000 x 10000; four 2.60, 45.0; eight 2.46, 45.9).  What is left is the depth of the ring (four
 // blocks of 46 KB) and, in small problems, filling it.  Blocks of 8 rows: 3%
 // slower.
 #pragma once
@@ -47,7 +48,7 @@ template <typename TX, bool FF, int ROWS> struct XF {
   static constexpr bool LOOP = !FF && sizeof(TX) == 4;
   static constexpr int SA = FF ? 6 : LOOP ? 5 : 4, SB = 6, NL = FF ? 3 : LOOP ? 4 : 5;   // dot, axpy and link warps
   static constexpr int B = ROWS;            // rows of a block
-  static constexpr int R = FF ? 2 : LOOP ? 8 : 4;   // rows a dot warp takes at a time
+  static constexpr int R = LOOP ? 8 : 4;   // rows a dot warp takes at a time
   static constexpr int RW = 4 * NL;         // blocks of weights in shared memory
   static constexpr int WF = FF ? 8 : 2;     // words of 32 bits of a weight there
 };
