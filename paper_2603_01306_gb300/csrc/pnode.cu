@@ -589,8 +589,10 @@ __device__ __noinline__ void pn_finish3(int nx, int n3) {
   if (lane == 0) {
     s.c = z.cc;
     s.ccd = __double2float_rd(z.cc);
-    // a root at the bracket's very end: the bracket missed it
-    s.miss3 = !(z.cc > (double)__uint_as_float(lok) && z.cc < (double)__uint_as_float(hik));
+    // no root, or one at the bracket's very end (up to where a bisection towards
+    // that end stops): the bracket missed it
+    s.miss3 = !(done && z.cc > (double)__uint_as_float(lok) * (1.0 + 0x1p-40) &&
+                z.cc < (double)__uint_as_float(hik) * (1.0 - 0x1p-40));
   }
 }
 // S3 by cluster-wide classifications (ties that no bracket separates)
@@ -602,7 +604,7 @@ __device__ __noinline__ int pn_fallback3(int nx) {
   const int w0 = (warp - 1) * s.a.wch, w1 = warp ? min(s.cnt, w0 + s.a.wch) : w0, nw = s.nw[warp];
   C3 z;
   z.cl = 0.0;
-  z.ch = 3.0e38;
+  z.ch = F64 ? 1.7e308 : 3.4e38;
   z.cc = (double)__uint_as_float(min(s.hi3, kInfKey - 1));
   z.np = z.mp = -1.0;
   z.first = true;

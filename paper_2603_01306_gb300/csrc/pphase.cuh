@@ -232,14 +232,17 @@ __device__ __forceinline__ KT warm_cand(KT kc, KT lo, KT hi, int q, int shift) {
 // One multisection decision, taken by every warp on its own: lane q holds
 // candidate x (non-decreasing in q) and `ge`, whether its field reaches the
 // target, which holds on a prefix of the lanes (the fields do not increase
-// with the candidate).  The bracket's new lower end is the largest candidate
-// with ge, its upper end the smallest without; qlo / qhi are their lanes (-1 /
-// 32: none).
+// with the candidate).  The bracket's new upper end is the smallest candidate
+// without ge, its lower end the one before it; qlo / qhi are their lanes (-1 /
+// 32: none).  A field that is a rounded sum (pnode.cu's S3: one |v_j| far above
+// c n, or a sum beyond FP32's range) can reach the target again further on:
+// only the prefix counts, or the bracket would turn over and the rounds need
+// not end.
 template <typename KT>
 __device__ __forceinline__ void bracket_step(KT x, bool ge, KT& lo, KT& hi, int& qlo, int& qhi) {
   const unsigned b = __ballot_sync(0xffffffffu, ge);
-  qlo = b ? 31 - __clz(b) : -1;
   qhi = ~b ? __ffs(~b) - 1 : 32;
+  qlo = qhi - 1;
   const KT xlo = __shfl_sync(0xffffffffu, x, qlo >= 0 ? qlo : 0);
   const KT xhi = __shfl_sync(0xffffffffu, x, qhi < 32 ? qhi : 0);
   if (qlo >= 0 && xlo > lo) lo = xlo; else qlo = -1;
