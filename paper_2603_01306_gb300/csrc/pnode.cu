@@ -455,8 +455,10 @@ __device__ __noinline__ bool pn_step3(C3& z, double Nt, double Nm, double Sm) {
   z.first = false;
   z.np = Nt;
   z.mp = Nm;
-  if (stable) {
-    z.cc = (isfinite(cn) && cn > 0.0) ? cn : z.cc;
+  // the piece's root is the answer only where it lies on the piece (a search
+  // that began on the wrong side can meet one piece twice on its way)
+  if (stable && fabs(cn - z.cc) <= 0x1p-40 * z.cc) {
+    z.cc = cn;
     return true;
   }
   if (!(cn >= z.cl && cn <= z.ch) || !(cn > 0.0)) {
