@@ -1568,16 +1568,18 @@ relax_status relax_certify(relax_handle* h, const int8_t* fixings, const void* b
 
 // ------------------------------------------------- standalone regularizer ops
 // One thread-block cluster where p fits its shared memory (pnode_plan), else the
-// cooperative grid.  p = 1000 FP32, prox, g and g*: 210 us on the grid (seven or
-// more grid barriers each, a scratch area zeroed per call), 119 on a cluster;
-// waited for after every round of the three, 421 and 138 (see pool.cu).
+// cooperative grid.  Sums are FP64 for either type: the squares of FP32 values
+// leave FP32's range (a pair of FP32 sums gave NaN above 1.8e19 and 0 below
+// 1e-23).  p = 1000 FP32, prox, g and g*: 210 us on the grid (seven or more grid
+// barriers each, a scratch area zeroed per call), 131 on a cluster with pairs,
+// 140 with FP64 sums.
 static relax_status standalone(int mode, const void* vin, void* vout, int64_t p, double rho, int32_t k,
                                double lambda2, double M, const int8_t* fix, int32_t dtype, int32_t* counts,
                                double* out_host, cudaStream_t st) {
   if (!vin || p <= 0 || k < 0 || !(M > 0.0) || (dtype != RELAX_F64 && dtype != RELAX_F32)) return RELAX_EINVAL;
   const bool dbl = dtype == RELAX_F64;
   NPlan np;
-  const bool cluster = pnode_plan(np, dbl, p, 1) == cudaSuccess;
+  const bool cluster = pnode_plan(np, true, p, 1) == cudaSuccess;
   PPlan pl;
   if (!cluster) {
     (void)cudaGetLastError();
@@ -1604,6 +1606,7 @@ static relax_status standalone(int mode, const void* vin, void* vout, int64_t p,
     a.rho = rho;
     a.kc = pconst_make(lambda2, M, 0.0, rho);
     a.fix = fix;
+    a.vf32 = dbl ? 0 : 1;
     a.vin = vin;
     a.vout = vout;
     a.counts = counts;

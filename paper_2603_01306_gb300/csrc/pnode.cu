@@ -1,5 +1,6 @@
 // The node p-phase (pnode.cuh): kernel, plan and launch.
 #include <algorithm>
+#include <cfloat>
 #include <cstdlib>
 
 #include "launch.cuh"
@@ -255,14 +256,13 @@ __device__ __forceinline__ double pn_G64(int64_t j) {
   const float2 v = static_cast<const float2*>(pn().Gcur)[j];
   return (double)v.x + (double)v.y;
 }
-template <bool F64>
 __device__ __forceinline__ double pn_vin(int64_t j) {   // the standalone operations' input
   const void* v = pn().a.vin;
-  return F64 ? static_cast<const double*>(v)[j] : (double)static_cast<const float*>(v)[j];
+  return pn().a.vf32 ? (double)static_cast<const float*>(v)[j] : static_cast<const double*>(v)[j];
 }
 template <bool F64>
 __device__ __forceinline__ double pn_a64(int64_t j) {
-  if (pn().a.mode == PM_GSTAR) return fabs(pn_vin<F64>(j));
+  if (F64 && pn().a.mode == PM_GSTAR) return fabs(pn_vin(j));
   return fabs(pn_G64<F64>(j)) * pn().a.kc.inv2l;
 }
 
@@ -767,7 +767,7 @@ __device__ __noinline__ void pn_stage2(int nx, bool d1, bool d3) {
       const uint32_t mk = key_of(m);
       if (mk > a3 || a3 == 0) {
         if (mk > b3 && m > Th) ++ntop;
-        else if (mk > b3 && m < Tl) {
+        else if (mk > b3 && m < Tl && m < FLT_MAX) {   // (FLT_MAX: a magnitude beyond FP32)
           ++nmid;
           v3.add(md);
         } else pn_list(&s.n3, s.loc3, md);
@@ -1059,8 +1059,7 @@ __device__ __noinline__ void pn_decisions() {
 }
 
 // Stage 1 of the standalone operations over this warp's coordinates
-template <bool F64>
-__device__ __noinline__ void pn_load(Acc<F64> (&sum)[XS_NSUM], unsigned& nnz, unsigned& dom, unsigned& bad, unsigned& nzv,
+__device__ __noinline__ void pn_load(Acc<true> (&sum)[XS_NSUM], unsigned& nnz, unsigned& dom, unsigned& bad, unsigned& nzv,
                                      unsigned& j1, unsigned& jf) {
   PnSh& s = pn();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, mode = s.a.mode;
@@ -1077,13 +1076,13 @@ __device__ __noinline__ void pn_load(Acc<F64> (&sum)[XS_NSUM], unsigned& nnz, un
     if (i < w1) {
       const int64_t j = s.cb + i;
       const int8_t f = s.fix ? s.fix[j] : (int8_t)0;
-      x = pn_vin<F64>(j);
+      x = pn_vin(j);
       f8 = f == 0 ? 4 : f > 0 ? 8 : 0;
       j1 += f > 0;
       jf += f == 0;
       // (an FP64 value beyond FP32's range is finite all the same)
       const bool inf_nan = (((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ffu) == 0x7ffu;
-      const float ax = fminf(fabsf((float)x), 3.4e38f);
+      const float ax = fminf(fabsf((float)x), FLT_MAX);
       if (inf_nan && (mode == PM_PROX || (x != x && f >= 0))) ++bad;
       if (mode == PM_GSTAR) {   // an infinite value: dom on Jf, nnz on J1
         if (f == 0) key = key_of(ax);
@@ -1093,7 +1092,7 @@ __device__ __noinline__ void pn_load(Acc<F64> (&sum)[XS_NSUM], unsigned& nnz, un
           else sum[XS_J1H].add(huber_d<double>(fabs(x), s.a.M));
         }
       } else if (mode == PM_PROX) {
-        wide = F64 ? f >= 0 : f > 0;
+        wide = f >= 0;
         if (__double_as_longlong(x) < 0) f8 |= 1;
         if (f == 0) {
           m = ax;
@@ -1131,26 +1130,25 @@ __device__ __noinline__ void pn_load(Acc<F64> (&sum)[XS_NSUM], unsigned& nnz, un
 
 // The standalone prox's output and counts.  A non-finite input poisons them:
 // beta all NaN, counts -1.
-template <bool F64>
 __device__ __noinline__ void pn_prox_out(int nx, int kb, bool s3, unsigned bad) {
   PnSh& s = pn();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w0 = (warp - 1) * s.a.wch, w1 = warp ? min(s.cnt, w0 + s.a.wch) : w0, nw = s.nw[warp];
   const double c = kb <= 0 ? INFINITY : s3 ? s.c : 0.0, T = pn_T(c), inv1r = s.a.kc.inv1r, M = s.a.M;
-  const float ccd = kb <= 0 ? INFINITY : s3 ? s.ccd : 0.f;   // an FP32 m exceeds c iff it exceeds c rounded down
   unsigned ntop = 0, nnz = 0;
 #pragma unroll 1
   for (int u = lane; u < (w1 - w0) + nw; u += 32) {
-    const bool narrow = u < w1 - w0;
-    const int e = w0 + u - (narrow ? 0 : w1 - w0);
-    const int i = narrow ? e : s.wl[e];
+    // the coordinates fixed out, then the others from the list
+    const bool out = u < w1 - w0;
+    const int e = w0 + u - (out ? 0 : w1 - w0);
+    const int i = out ? e : s.wl[e];
     const uint8_t f8 = s.fl[i];
-    if (narrow && (f8 & 2)) continue;
+    if (out && (f8 & 2)) continue;
     double b = 0.0;
     if (bad) b = __longlong_as_double(0x7ff8000000000000ll);
     else if (f8 & 8) b = fmin(fmax(s.vw[e] * inv1r, -M), M);
-    else if ((f8 & 4) && (!narrow || s.mv[i] > ccd)) {
-      const double m = narrow ? (double)s.mv[i] : fabs(s.vw[e]);
+    else if (f8 & 4) {
+      const double m = fabs(s.vw[e]);
       const double r = fmax(0.0, fmin(fmin(m - c, m * inv1r), M));
       if (r > 0.0) {
         ++nnz;
@@ -1158,12 +1156,12 @@ __device__ __noinline__ void pn_prox_out(int nx, int kb, bool s3, unsigned bad) 
         b = (f8 & 1) ? -r : r;
       }
     }
-    if (F64) static_cast<double*>(s.a.vout)[s.cb + i] = b;
-    else static_cast<float*>(s.a.vout)[s.cb + i] = (float)b;
+    if (s.a.vf32) static_cast<float*>(s.a.vout)[s.cb + i] = (float)b;
+    else static_cast<double*>(s.a.vout)[s.cb + i] = b;
   }
   if (s.a.counts) {
-    const unsigned long long zero = Acc<F64>().word();
-    pn_small_sum<F64>(nx, zero, zero, ntop, nnz);
+    const unsigned long long zero = Acc<true>().word();
+    pn_small_sum<true>(nx, zero, zero, ntop, nnz);
     if (s.rank == 0 && threadIdx.x == 0) {
       s.a.counts[0] = bad ? -1 : (int)s.cnt0;
       s.a.counts[1] = bad ? -1 : (int)s.cnt1;
@@ -1267,7 +1265,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
     }
   }
   const int mode = s.a.mode;
-  const bool iter = mode == PM_ITER, alone = mode >= PM_PROX;
+  const bool iter = mode == PM_ITER, alone = F64 && mode >= PM_PROX;
   const int64_t cb = s.cb;
   const int wch = s.a.wch, w0 = (warp - 1) * wch, w1 = warp ? min(s.cnt, w0 + wch) : w0;
   const PConst& kc = s.a.kc;
@@ -1283,7 +1281,8 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
   A sum[XS_NSUM];
   unsigned c_nnz = 0, c_dom = 0, c_bad = 0, c_nab = 0, c_nzv = 0, c_j1 = 0, c_jf = 0;
   if (alone) {
-    if (warp) pn_load<F64>(sum, c_nnz, c_dom, c_bad, c_nzv, c_j1, c_jf);
+    if constexpr (F64)
+      if (warp) pn_load(sum, c_nnz, c_dom, c_bad, c_nzv, c_j1, c_jf);
   } else if (warp == 0) {   // the loss sums of the pass, in FP64
     const double* ls = s.a.lsum + (size_t)(iter ? s.prob : s.item) * s.a.lsum_stride;
     double f = 0.0, d = 0.0;
@@ -1533,7 +1532,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
 
   // ---------------------------------------------------------------------- D
   if (!iter) {
-    if (mode == PM_PROX) pn_prox_out<F64>(nx, kb, s3, bad);
+    if (alone && mode == PM_PROX) pn_prox_out(nx, kb, s3, bad);
     else if (tid == 0) pn_decisions();
     return;   // (every push to this CTA has been received: no exchange follows)
   }

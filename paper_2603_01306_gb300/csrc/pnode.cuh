@@ -27,8 +27,10 @@
 // arithmetic only, gradients travel as FP32 pairs (hi + lo) and sums are
 // float-float; the others ("wide") are collected per warp and take FP64 with
 // full warps.  (A dependent FP64 operation takes 64 cycles here, a division
-// about 580: thread 0 decides while the other warps write the next point.)  F64 = true (FP64 data, and the last rung of the precision
-// ladder): every coordinate is wide and sums are FP64.
+// about 580: thread 0 decides while the other warps write the next point.)
+// F64 = true (FP64 data, the last rungs of the precision ladder, and the
+// standalone operations of either type): every coordinate is wide and sums are
+// FP64.
 //
 // Measured per iteration, against the cooperative grid of pphase.cuh that ran
 // before (seven or more grid barriers): p = 1000 45 -> 29 us, p = 4000
@@ -89,8 +91,9 @@ struct NArgs {
   const int* cnt;               // [items][3] fixing counts {|J1|, |Jf|, .}; NULL: root
   double* out;                  // item's values at out_stride item + 2 (s % nq); PM_GVAL, PM_GSTAR: one value
   int64_t out_stride;
-  // the standalone operations, one problem on vectors of the kernel's type
-  // (F64: double, else float)
+  // the standalone operations, one problem, F64 kernel: sums and products of
+  // FP32 vectors (vf32) need FP64's range and precision too
+  int vf32;
   const void* vin;              // PM_PROX: v, PM_GVAL: beta, PM_GSTAR: alpha
   void* vout;                   // PM_PROX
   int* counts;                  // PM_PROX: {n_top, n_nz} or NULL

@@ -1,10 +1,14 @@
-"""The standalone prox where the candidates' rounded sums cross the target more
-than once: sums beyond FP32's largest value, one magnitude far above many equal
-ones.
+"""The standalone prox, g and g* over the range of their inputs' type: magnitudes
+whose squares leave FP32's range at either end, sums beyond FP32's largest
+value, one magnitude far above many equal ones (the candidates' rounded sums
+then cross the target more than once), M = inf.
 
-Tolerances are those of the ordinary magnitudes: 1e-12 relative (FP64) or one
-rounding to FP32 (2^-22 relative).
+Tolerances are those of the ordinary magnitudes: the sums run in FP64, so g and
+g* agree with the FP64 oracle to 1e-12 relative, the prox to 1e-12 (FP64) or one
+rounding to FP32 (2^-22 relative; subnormal outputs 2^-149 absolute).
 """
+import math
+
 import numpy as np
 import pytest
 
@@ -12,6 +16,7 @@ from oracle import regularizer as R
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
+SCALES = [1e-38, 1e-24, 1e-17, 1.0, 1e20, 3e37]
 
 
 def _dev(a, dtype):
@@ -37,7 +42,31 @@ def _check_prox(lib, v, rho, k, M, dtype):
     assert counts.cpu().tolist() == [ntop, nnz]
 
 
-@pytest.mark.parametrize("dtype", [torch.float64])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("scale", SCALES)
+@pytest.mark.parametrize("p,k,rho,box", [(40, 3, 0.5, 2.0), (700, 10, 0.05, math.inf), (3001, 30, 3.0, 0.3)])
+def test_prox_over_the_range(lib, p, k, rho, box, scale, dtype):
+    v = _as(scale * np.clip(np.random.default_rng(p).standard_normal(p) * 3.0, -9.0, 9.0), dtype)
+    _check_prox(lib, v, rho, k, box * scale, dtype)
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("scale", SCALES)
+@pytest.mark.parametrize("p,k,box", [(40, 3, 2.0), (700, 10, math.inf), (3001, 30, 0.3)])
+def test_g_and_gstar_over_the_range(lib, p, k, box, scale, dtype):
+    rng = np.random.default_rng(p + 1)
+    b = np.zeros(p)
+    at = rng.permutation(p)[:2 * k]
+    b[at] = 0.25 * min(box, 1.0) * rng.uniform(-1, 1, at.size) * scale
+    b = _as(b, dtype)
+    M = box * scale
+    # the squares themselves leave FP64's normal range at the lowest scale: 2^-1074 absolute
+    assert lib.gval_persp(_dev(b, dtype), k, M) == pytest.approx(R.g_alg1(b, None, k, M, domain_rtol=1e-6), rel=1e-12, abs=1e-320)
+    a = _as(scale * np.clip(rng.standard_normal(p) * 2.0, -9.0, 9.0), dtype)
+    assert lib.gstar_persp(_dev(a, dtype), k, M) == pytest.approx(R.gstar(a, None, k, M), rel=1e-12, abs=1e-320)
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
 def test_sums_beyond_fp32(lib, dtype):
     rng = np.random.default_rng(5)
     for t in range(8):
@@ -45,7 +74,7 @@ def test_sums_beyond_fp32(lib, dtype):
         _check_prox(lib, v, 10.0 ** rng.uniform(-6, 2), int(rng.integers(2, 40)), 10.0 ** rng.uniform(36, 39), dtype)
 
 
-@pytest.mark.parametrize("dtype", [torch.float64])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
 @pytest.mark.parametrize("big", [1e6, 1e10, 1e14])
 def test_one_magnitude_far_above_ties(lib, big, dtype):
     # counts are left out: on ties they depend on the rounding of the threshold
