@@ -435,15 +435,7 @@ cudaError_t bgemm_plan(BGPlan& pl, int M, int N, int K) {
   pl.stages = std::min(BG_MAXS, (optin - fixed) / (int)sb);
   if (pl.stages < 2) return cudaErrorNotSupported;
   pl.smem = (size_t)pl.stages * sb + 1024;
-  cudaFuncAttributes fa{};
-  cudaError_t e = cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(&bgemm_kernel));
-  if (e != cudaSuccess) return e;
-  if (fa.maxDynamicSharedSizeBytes < (int)pl.smem) {
-    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(&bgemm_kernel),
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  return raise_smem(reinterpret_cast<const void*>(&bgemm_kernel), pl.smem);
 }
 
 cudaError_t bgemm_encode(CUtensorMap* tm, const void* planes, int64_t K, int64_t rows, int64_t ld, int64_t plane_rows,

@@ -184,6 +184,9 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long* counter, unsign
 // device (pool.cu); returned with cudaFreeAsync.
 cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t st);
 void pool_trim();   // gives what the current device's pool holds unused back to the driver
+// At least `bytes` of dynamic shared memory for the kernel on the current device
+// (attr.cu); never lowered, safe from several threads.
+cudaError_t raise_smem(const void* kernel, size_t bytes);
 
 // ------------------------------------------------------------ misc helpers
 template <typename T>

@@ -1775,12 +1775,7 @@ cudaError_t pnode_plan(NPlan& pl, bool f64, int64_t p, int nprob) {
     if (!sized(pl, p, cl, (size_t)optin)) continue;
     if (cl > 8 && (e = cudaFuncSetAttribute(pl.kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
       return e;
-    // the attribute belongs to the kernel, shared by every plan and handle: only raise it
-    cudaFuncAttributes fa{};
-    if ((e = cudaFuncGetAttributes(&fa, pl.kernel)) != cudaSuccess) return e;
-    if (fa.maxDynamicSharedSizeBytes < (int)pl.smem &&
-        (e = cudaFuncSetAttribute(pl.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem)) != cudaSuccess)
-      return e;
+    if ((e = raise_smem(pl.kernel, pl.smem)) != cudaSuccess) return e;
     if (cl <= 8) return cudaSuccess;
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = config(pl, 1, attr, nullptr);
@@ -1788,10 +1783,7 @@ cudaError_t pnode_plan(NPlan& pl, bool f64, int64_t p, int nprob) {
     if (cudaOccupancyMaxActiveClusters(&n, pl.kernel, &cfg) == cudaSuccess && n >= 1) return cudaSuccess;
     (void)cudaGetLastError();
     // no 16 SMs to place one: the largest portable size, if the share fits it
-    if (sized(pl, p, 8, (size_t)optin))
-      return fa.maxDynamicSharedSizeBytes < (int)pl.smem
-                 ? cudaFuncSetAttribute(pl.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem)
-                 : cudaSuccess;
+    if (sized(pl, p, 8, (size_t)optin)) return raise_smem(pl.kernel, pl.smem);
   }
   return cudaErrorNotSupported;
 }

@@ -83,13 +83,8 @@ cudaError_t xmma_plan(XSPlan& pl, int xk, int NB, int64_t n, int64_t p) {
   pl.RB = 0;
   if (pl.RA < 2) return cudaErrorNotSupported;
   pl.smem = (size_t)pl.RA * stage + extra;
-  cudaFuncAttributes fa{};
-  cudaError_t e = cudaFuncGetAttributes(&fa, pl.kernel);
+  cudaError_t e = raise_smem(pl.kernel, pl.smem);
   if (e != cudaSuccess) return e;
-  if (fa.maxDynamicSharedSizeBytes < (int)pl.smem) {
-    e = cudaFuncSetAttribute(pl.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
-    if (e != cudaSuccess) return e;
-  }
   int per = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, pl.kernel, pl.threads, pl.smem);
   if (e != cudaSuccess) return e;

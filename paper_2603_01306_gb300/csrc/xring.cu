@@ -73,10 +73,7 @@ cudaError_t xring_plan(XSPlan& pl, int xk, bool f64acc, int NB, int64_t n, int64
   pl.RB = 0;
   if (pl.RA < 2) return cudaErrorNotSupported;
   pl.smem = (size_t)pl.RA * stage + 128;
-  if (fa.maxDynamicSharedSizeBytes < (int)pl.smem) {
-    e = cudaFuncSetAttribute(pl.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
-    if (e != cudaSuccess) return e;
-  }
+  if ((e = raise_smem(pl.kernel, pl.smem)) != cudaSuccess) return e;
   int per = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, pl.kernel, pl.threads, pl.smem);
   if (e != cudaSuccess) return e;

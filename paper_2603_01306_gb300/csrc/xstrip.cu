@@ -135,14 +135,8 @@ cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t
   const size_t comb = (size_t)SB * NB * pl.sw * 8;
   pl.smem = std::max(ring, comb) + 128;
   if (pl.smem + 2048 > (size_t)optin) return cudaErrorNotSupported;
-  // the attribute belongs to the kernel, shared by every plan and handle: only raise it
-  cudaFuncAttributes fa{};
-  cudaError_t e = cudaFuncGetAttributes(&fa, pl.kernel);
+  cudaError_t e = raise_smem(pl.kernel, pl.smem);
   if (e != cudaSuccess) return e;
-  if (fa.maxDynamicSharedSizeBytes < (int)pl.smem) {
-    e = cudaFuncSetAttribute(pl.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
-    if (e != cudaSuccess) return e;
-  }
   int per = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, pl.kernel, pl.threads, pl.smem);
   if (e != cudaSuccess) return e;
