@@ -965,7 +965,7 @@ __device__ __noinline__ unsigned pn_again() {
     s.vw[w0 + e] = v;
     s.fl[i] = (f8 & ~1) | (v < 0.0 ? 1 : 0);
     if (f8 & 4) {
-      s.mv[i] = (float)fabs(v);
+      s.mv[i] = fminf((float)fabs(v), FLT_MAX);
       nzv += !is_zero_bits(v);
     }
   }
@@ -1325,7 +1325,9 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
           const double G = pn_gdbl(j, 0);
           static_cast<double*>(s.Gcur)[j] = G;
           gf = (float)G;
-          aa = (float)(fabs(G) * kc.inv2l);
+          const double ad = fabs(G) * kc.inv2l;
+          // an FP64 value beyond FP32 is finite all the same: its key is the largest one's
+          aa = ad < INFINITY ? fminf((float)ad, FLT_MAX) : INFINITY;
         } else {
           const ffs g = pn_gpair(j, 0);
           static_cast<float2*>(s.Gcur)[j] = make_float2(g.hi, g.lo);
@@ -1399,7 +1401,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
         s.vw[w0 + e] = v;
         if (__double_as_longlong(v) < 0) s.fl[i] = f8 | 1;
         if (f8 & 4) {
-          s.mv[i] = (float)fabs(v);
+          s.mv[i] = fminf((float)fabs(v), FLT_MAX);
           if (!is_zero_bits(v)) ++c_nzv;
         }
       }
