@@ -34,6 +34,7 @@ cudaError_t xmma_plan(XSPlan& pl, int xk, int NB, int64_t n, int64_t p) {
   pl.xk = xk;
   pl.NF = 1;
   pl.NB = NB;
+  pl.words = 2;
   pl.mma = true;
   pl.keep = x_fits_l2(xk, n, p);
   if ((xk != XK_BF16 && xk != XK_FP8) || NB < 1 || NB > 2 || n < 1 || p < 1 || n > INT32_MAX || p > INT32_MAX)

@@ -7,9 +7,12 @@
 //    ring holds the blocks of one agreement's round trip, X crosses from L2
 //    to the SMs once (the second crossing of xstrip.cuh was what its narrow
 //    instantiations came to be bound by next to issue).
-//  * The row's word of z carries its own arrival count in the low eight bits,
-//    so a block is agreed on by polling its sixteen words: no release, no
-//    counter, one round trip through L2.
+//  * A row's z takes two words, 54 bits and 44 further ones, that carry their
+//    own arrival counts in the low eight bits: a block is agreed on by polling
+//    its rows' words, no release, no counter, one round trip through L2.  The
+//    unit follows from the largest row and the largest |beta_j|, so a row far
+//    below that bound needs the second word (with one, a row 10^6 times lighter
+//    than the heaviest was off by 9e-5 of itself, by 5e-3 at 10^8).
 //  * On the CUDA cores a narrow element costs a conversion and up to three
 //    FMAs (BF16 0.37, FP8 0.22 of the copy bandwidth, DRAM 31% busy).  Here a
 //    tile of 16 rows x 16 columns costs one ldmatrix and one mma.sync m16n8k16
@@ -100,23 +103,42 @@ __device__ __forceinline__ int plane_scale(float mx) {
   return min(126, 5 - e);
 }
 
-// bounded wait until the low eight bits of *p count `want` arrivals; the word in w
-__device__ __forceinline__ bool wait_row(const unsigned long long* p, unsigned want, unsigned long long& w, uint64_t limit_ns,
-                                         int* status) {
-  auto load = [&]() {
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-  };
-  w = load();
-  if ((unsigned)(w & 255ull) == want) return true;
-  const uint64_t t0 = globaltimer_ns();
-  for (uint32_t it = 1;; ++it) {
-    w = load();
-    if ((unsigned)(w & 255ull) == want) return true;
-    if ((it & 15u) == 0u && globaltimer_ns() - t0 > limit_ns) {
-      atomicCAS(status, ST_OK, ST_TIMEOUT);
-      return false;
+constexpr int Z_LO = 44;   // bits of z's second word below the first one's unit
+
+// m 2^sh as hi + lo 2^-Z_LO, in two's complement (|m 2^sh| < 2^54)
+__device__ __forceinline__ void fixed_words(float m, int sh, long long& hi, long long& lo) {
+  const uint32_t b = __float_as_uint(m);
+  const int ex = (int)((b >> 23) & 255u);
+  const unsigned long long mant = ex ? (b & 0x7fffffu) | 0x800000u : b & 0x7fffffu;
+  const int k = min((ex ? ex : 1) - 150 + sh, 38);   // |m| 2^sh = mant 2^k
+  long long h = 0, l = 0;
+  if (k >= 0) {
+    h = (long long)(mant << k);
+  } else {
+    const unsigned long long rem = k > -24 ? mant & ((1ull << -k) - 1ull) : mant;
+    if (k > -24) h = (long long)(mant >> -k);
+    const int s = k + Z_LO;
+    l = s >= 0 ? (long long)(rem << s) : s > -32 ? (long long)((rem + (1ull << (-s - 1))) >> -s) : 0ll;
+  }
+  const bool neg = (b >> 31) != 0u;
+  hi += neg ? -h : h;
+  lo += neg ? -l : l;
+}
+
+// bounded wait until the low eight bits of both words of a row count `want` arrivals
+__device__ __forceinline__ bool wait_row(const unsigned long long* p, unsigned want, unsigned long long& h, unsigned long long& l,
+                                          uint64_t limit_ns, int* status) {
+  uint64_t t0 = 0;
+  for (uint32_t it = 0;; ++it) {
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(h), "=l"(l) : "l"(p) : "memory");
+    if ((unsigned)(h & 255ull) == want && (unsigned)(l & 255ull) == want) return true;
+    if ((it & 15u) == 0u) {
+      const uint64_t t = globaltimer_ns();
+      if (it == 0) t0 = t;
+      else if (t - t0 > limit_ns) {
+        atomicCAS(status, ST_OK, ST_TIMEOUT);
+        return false;
+      }
     }
   }
 }
@@ -256,7 +278,6 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
     named_sync(1, DT);
     const uint32_t* fl = frag + lane * 2 * MM;
     int zs = 0;
-    double zf = 0.0;
     bool have_scale = false;
     // this lane's row of the four matrices: rows 0-7, 8-15 of vector v0, then of v0 + 1
     const uint32_t rowoff = (uint32_t)(lane & 15) * pitch + (uint32_t)(lane >> 4) * 16;
@@ -314,21 +335,26 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
         zr = ff_add(zr, ffs{__shfl_xor_sync(0xffffffffu, zr.hi, o), __shfl_xor_sync(0xffffffffu, zr.lo, o)});
         yr = ff_add(yr, ffs{__shfl_xor_sync(0xffffffffu, yr.hi, o), __shfl_xor_sync(0xffffffffu, yr.lo, o)});
       }
-      // row g on lanes t = 0, row g + 8 on lanes t = 1
-      const int row = (lane >> 2) + ((lane & 3) ? 8 : 0);
-      const float zh = (lane & 3) ? yr.hi : zr.hi, zl = (lane & 3) ? yr.lo : zr.lo;
+      // row g on lanes t = 0, 1, row g + 8 on lanes t = 2, 3, its first word on
+      // the even lane, the second on the odd one
+      const int row = (lane >> 2) + ((lane & 2) ? 8 : 0), word = lane & 1;
+      const float zh = (lane & 2) ? yr.hi : zr.hi, zl = (lane & 2) ? yr.lo : zr.lo;
       if (!have_scale) {
         if (!__all_sync(0xffffffffu, wait_count(a.zcnt, gridDim.x, a.limit_ns, a.status))) {
           tmo = 1;
           break;
         }
         zs = fixed_scale(a.rowl1 * __longlong_as_double((long long)__ldcg(&a.zmax[0])));
-        zf = zs == INT_MIN ? 0.0 : ldexp(1.0, zs - be - (BF ? 8 : 0));   // eight bits for the count (FP8: X is times 2^-8)
         have_scale = true;
       }
-      if ((lane & 3) < 2 && row < rows) {
-        const long long q = zs == INT_MIN ? 0ll : __double2ll_rn((double)zh * zf) + __double2ll_rn((double)zl * zf);
-        atomicAdd(&a.zfix[r0 + row], ((unsigned long long)q << 8) + 1ull);
+      if (row < rows) {
+        long long qh = 0, ql = 0;
+        if (zs != INT_MIN) {
+          const int sh = zs - be - (BF ? 8 : 0);   // eight bits for the count (FP8: X is times 2^-8)
+          fixed_words(zh, sh, qh, ql);
+          fixed_words(zl, sh, qh, ql);
+        }
+        atomicAdd(&a.zfix[2 * (r0 + row) + word], ((unsigned long long)(word ? ql : qh) << 8) + 1ull);
       }
     }
   } else if (warp < 1 + XM_SA + XM_NL) {
@@ -339,7 +365,7 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
     double* zout = static_cast<double*>(a.ps->zout);
     const double mom = a.ps->mom;
     const int jl = lane & 15, hb = lane >> 4;
-    double zinv = 0.0;
+    double uh = 0.0, ul = 0.0;   // values of the words' units
     bool have_scale = false;
     double lsum[3] = {0.0, 0.0, 0.0};
     // two blocks at a time, one per half warp
@@ -355,9 +381,9 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
       const double zp = need_zp ? zprev[rowj] : 0.0;
       const int ws = k % XM_RW;
       bool ok = !on || k < XM_RW || mbar_wait<false>(&wempty[ws], ((k / XM_RW) - 1) & 1, a.limit_ns, a.status);
-      // the row's word, complete once its low bits count every strip
-      unsigned long long zw = 0ull;
-      ok = ok && wait_row(&a.zfix[rowj], (unsigned)a.Gc, zw, a.limit_ns, a.status);
+      // the row's words, complete once their low bits count every strip
+      unsigned long long wh = 0ull, wl = 0ull;
+      ok = ok && wait_row(&a.zfix[2 * rowj], (unsigned)a.Gc, wh, wl, a.limit_ns, a.status);
       if (!__all_sync(0xffffffffu, ok)) {
         tmo = 1;
         break;
@@ -368,11 +394,12 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
           break;
         }
         const int zs = fixed_scale(a.rowl1 * __longlong_as_double((long long)__ldcg(&a.zmax[0])));
-        zinv = zs == INT_MIN ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, 8 - zs);
+        uh = zs == INT_MIN ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, 8 - zs);
+        ul = ldexp(uh, -Z_LO);
         have_scale = true;
       }
       double z[1];
-      z[0] = (double)((long long)zw >> 8) * zinv;
+      z[0] = fma((double)((long long)wl >> 8), ul, (double)((long long)wh >> 8) * uh);
       double rv[NB];
       link_of<1, NB, true>(a.link, z, yd, zp, mom, rv);
       float w[NB];

@@ -27,7 +27,7 @@ cudaError_t xring_plan(XSPlan& pl, int xk, bool f64acc, int NB, int64_t n, int64
   pl.cert = f64acc;
   pl.NF = 1;
   pl.NB = NB;
-  pl.words = ff || dbl ? 2 : 1;
+  pl.words = 2;
   pl.keep = x_fits_l2(xk, n, p);
   if (NB < 1 || NB > 2 || n < 1 || p < 1 || n > INT32_MAX || p > INT32_MAX) return cudaErrorNotSupported;
   pl.B = dbl || ff || pl.keep ? 16 : 8;   // (both sides: xring.cuh)

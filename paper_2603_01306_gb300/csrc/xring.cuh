@@ -9,9 +9,10 @@
 //  * a dot warp holds the strip of beta and takes R rows of a block at a time;
 //  * an axpy warp owns 32 vectors of the strip and takes all rows, the weights
 //    read as ready operand pairs from shared memory.
-// z in fixed point, 64-bit words with 8 bits of count (FF, FP64: a second word
-// holds 44 further bits), converted by shifts: FP64 conversions of two lanes per row
-// pair would take as long as the sums.
+// z in two words of fixed point (xmma.cuh), converted by shifts: FP64
+// conversions of two lanes per row pair would take as long as the sums.  A
+// block's words go out in one instruction: 40 iterations of 20000 x 50000 FP32
+// took 33.4 ms with one word, 35.6 with two in two instructions, 33.3 so.
 //
 // FP32: bound by how much of X the rings hold (32 MB) against the round trip
 // from HBM to the end of a block's agreement.  20000 x 50000: 862 us on
@@ -58,52 +59,13 @@ static_assert(1 + XF<float, true, 16>::SA + XF<float, true, 16>::SB + XF<float, 
               1 + XF<double, false, 16>::SA + XF<double, false, 16>::SB + XF<double, false, 16>::NL == XF_T / 32);
 constexpr int XF_TV = 6;                    // vectors of the strip per lane of a dot warp = axpy warps
 constexpr int XF_MAXR = 16;                 // ring stages at most
-constexpr int XF_LO = 44;                   // bits of the second word below the first's unit
-
-// m 2^sh as hi + lo 2^-XF_LO, in two's complement (|m 2^sh| < 2^54)
-__device__ __forceinline__ void fixed_words(float m, int sh, long long& hi, long long& lo) {
-  const uint32_t b = __float_as_uint(m);
-  const int ex = (int)((b >> 23) & 255u);
-  const unsigned long long mant = ex ? (b & 0x7fffffu) | 0x800000u : b & 0x7fffffu;
-  const int k = min((ex ? ex : 1) - 150 + sh, 38);   // |m| 2^sh = mant 2^k
-  long long h = 0, l = 0;
-  if (k >= 0) {
-    h = (long long)(mant << k);
-  } else {
-    const unsigned long long rem = k > -24 ? mant & ((1ull << -k) - 1ull) : mant;
-    if (k > -24) h = (long long)(mant >> -k);
-    const int s = k + XF_LO;
-    l = s >= 0 ? (long long)(rem << s) : s > -32 ? (long long)((rem + (1ull << (-s - 1))) >> -s) : 0ll;
-  }
-  const bool neg = (b >> 31) != 0u;
-  hi += neg ? -h : h;
-  lo += neg ? -l : l;
-}
-
-// bounded wait until the low eight bits of both words of a row count `want` arrivals
-__device__ __forceinline__ bool wait_row2(const unsigned long long* p, unsigned want, unsigned long long& h, unsigned long long& l,
-                                          uint64_t limit_ns, int* status) {
-  uint64_t t0 = 0;
-  for (uint32_t it = 0;; ++it) {
-    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(h), "=l"(l) : "l"(p) : "memory");
-    if ((unsigned)(h & 255ull) == want && (unsigned)(l & 255ull) == want) return true;
-    if ((it & 15u) == 0u) {
-      const uint64_t t = globaltimer_ns();
-      if (it == 0) t0 = t;
-      else if (t - t0 > limit_ns) {
-        atomicCAS(status, ST_OK, ST_TIMEOUT);
-        return false;
-      }
-    }
-  }
-}
 
 template <typename TX, int NB, bool FF, int ROWS>
 __global__ void __launch_bounds__(XF_T, 1) xring_kernel(const __grid_constant__ XSArgs a) {
   using K = XF<TX, FF, ROWS>;
   constexpr int XF_SA = K::SA, XF_SB = K::SB, XF_NL = K::NL, XF_B = K::B, XF_RW = K::RW, R = K::R;
   constexpr bool D = sizeof(TX) == 8;            // FP64 throughout
-  constexpr int VEC = 16 / (int)sizeof(TX), WORDS = FF || D ? 2 : 1;
+  constexpr int VEC = 16 / (int)sizeof(TX);
   static_assert(!(FF && D), "float-float: FP32 X");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t full[XF_MAXR], empty[XF_MAXR], wfull[XF_RW], wempty[XF_RW];
@@ -319,21 +281,23 @@ __global__ void __launch_bounds__(XF_T, 1) xring_kernel(const __grid_constant__ 
         zf = zs == INT_MIN ? 0.0 : ldexp(1.0, zs - 8);
         have_scale = true;
       }
+      // (a row's lanes hold the same sum: the first adds its first word, the
+      // second its second one, the block's words in one instruction)
       const int64_t row = r0 + lane / (32 / R);
-      if (lane % (32 / R) == 0 && row < n) {
+      const int word = lane % (32 / R);
+      if (word < 2 && row < n) {
         long long qh = 0, ql = 0;
         if (zs != INT_MIN) {
           if constexpr (D) {
             const double v = zd[0] * zf, vi = rint(v);
             qh = (long long)vi;
-            ql = __double2ll_rn((v - vi) * (double)(1ll << XF_LO));
+            ql = __double2ll_rn((v - vi) * (double)(1ll << Z_LO));
           } else {
             fixed_words(h[0], zs - 8, qh, ql);
             fixed_words(l[0], zs - 8, qh, ql);
           }
         }
-        atomicAdd(&a.zfix[WORDS * row], ((unsigned long long)qh << 8) + 1ull);
-        if constexpr (WORDS == 2) atomicAdd(&a.zfix[WORDS * row + 1], ((unsigned long long)ql << 8) + 1ull);
+        atomicAdd(&a.zfix[2 * row + word], ((unsigned long long)(word ? ql : qh) << 8) + 1ull);
       }
     }
   } else if (warp < 1 + XF_SA + XF_SB) {
@@ -461,8 +425,7 @@ __global__ void __launch_bounds__(XF_T, 1) xring_kernel(const __grid_constant__ 
       const int ws = k % XF_RW;
       unsigned long long wh = 0ull, wl = 0ull;
       bool ok = k < XF_RW || mbar_wait<false>(&wempty[ws], ((k / XF_RW) - 1) & 1, a.limit_ns, a.status);
-      if constexpr (WORDS == 2) ok = ok && wait_row2(&a.zfix[2 * rowj], (unsigned)a.Gc, wh, wl, a.limit_ns, a.status);
-      else ok = ok && wait_row(&a.zfix[rowj], (unsigned)a.Gc, wh, a.limit_ns, a.status);
+      ok = ok && wait_row(&a.zfix[2 * rowj], (unsigned)a.Gc, wh, wl, a.limit_ns, a.status);
       if (!__all_sync(0xffffffffu, ok)) {
         tmo = 1;
         break;
@@ -474,12 +437,11 @@ __global__ void __launch_bounds__(XF_T, 1) xring_kernel(const __grid_constant__ 
         }
         const int zs = fixed_scale(a.rowl1 * __longlong_as_double((long long)__ldcg(&a.zmax[0])));
         uh = zs == INT_MIN ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, 8 - zs);
-        ul = ldexp(uh, -XF_LO);
+        ul = ldexp(uh, -Z_LO);
         have_scale = true;
       }
       double z[1];
-      z[0] = (double)((long long)wh >> 8) * uh;
-      if constexpr (WORDS == 2) z[0] = fma((double)((long long)wl >> 8), ul, z[0]);
+      z[0] = fma((double)((long long)wl >> 8), ul, (double)((long long)wh >> 8) * uh);
       double rv[NB];
       link_of<1, NB, !FF && !D>(a.link, z, yd, zp, mom, rv);
       if (on) {
