@@ -21,10 +21,13 @@
 //    either way, and fragments in registers need no round trip through TMEM.)
 //  * The small operand (beta, a block's row weights) is split into four
 //    planes, one per column of the MMA's N = 8, so that products are exact and
-//    sums FP32.  On a common scale the first two planes are integers of at
-//    most six bits, whose sums over the MMA's K come out exactly: the tensor
-//    cores truncate, a bias that no later sum removes (with three planes of 8
-//    bits g of 30000 rows was off by 3e-8).  The sums of one or two MMAs are
+//    sums FP32.  On a common scale (the largest in [2^4, 2^5)) the first two
+//    planes of a value from 1 on are integers of at most six bits, whose sums
+//    over the MMA's K come out exactly: the tensor cores truncate, a bias that
+//    no later sum removes (with three planes of 8 bits g of 30000 rows was off
+//    by 3e-8).  A smaller value takes the last three planes with all their
+//    bits: the four hold every FP32 value exactly, FP16 planes (scaled up one
+//    by one) down to 2^-34 of the largest.  The sums of one or two MMAs are
 //    folded into compensated FP32 pairs.
 //  * The link has warps of its own, two blocks each at a time, which leave the
 //    weights' fragments in shared memory; an axpy warp owns every SB-th step
@@ -78,20 +81,31 @@ __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1
 // bytes 0 and 2 (ev), 1 and 3 (od) of four e4m3 values, as FP16 times 2^-8
 __device__ __forceinline__ uint32_t e4m3_ev(uint32_t w) { return ((w << 8) & 0x80008000u) | ((w << 7) & 0x3f803f80u); }
 __device__ __forceinline__ uint32_t e4m3_od(uint32_t w) { return (w & 0x80008000u) | ((w >> 1) & 0x3f803f80u); }
+// Plane q holds its part times 2^plane_exp (FP16 has five bits of exponent; the
+// parts are at most 2^5, 1, 2^-6 and 2^-18, or 0, 1, 2^-12 and 2^-24 of an |x| < 1)
+template <bool BF>
+__device__ __forceinline__ constexpr int plane_exp(int q) {
+  return BF || q == 0 ? 0 : q == 1 ? 15 : q == 2 ? 21 : 33;
+}
+template <bool BF>
+__device__ __forceinline__ float plane_inv(int q) {   // 2^-plane_exp
+  return BF ? 1.f : q == 0 ? 1.f : q == 1 ? 0x1p-15f : q == 2 ? 0x1p-21f : 0x1p-33f;
+}
 // the four planes of x (on the common scale, |x| < 2^5) as the MMA's 16-bit operand
 template <bool BF>
 __device__ __forceinline__ void planes16(float x, uint16_t (&u)[4]) {
+  const bool whole = fabsf(x) >= 1.f;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const float v = q == 0 ? rintf(x) : q == 1 ? rintf(x * 32.f) * 0.03125f : x;
+    const float v = q == 0 ? (whole ? rintf(x) : 0.f) : q == 1 && whole ? rintf(x * 32.f) * 0.03125f : x;
     if constexpr (BF) {
       const __nv_bfloat16 h = __float2bfloat16_rn(v);
       u[q] = __bfloat16_as_ushort(h);
       x -= __bfloat162float(h);   // exact
     } else {
-      const __half h = __float2half_rn(v);
+      const __half h = __float2half_rn(v * (float)(1ull << plane_exp<BF>(q)));
       u[q] = __half_as_ushort(h);
-      x -= __half2float(h);
+      x -= __half2float(h) * plane_inv<BF>(q);
     }
   }
 }
@@ -329,7 +343,8 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
       two_sum_acc2(hi0, lo0, hi1);
       lo0 = add2(lo0, lo1);
       // the planes (lanes t = 0 .. 3) together
-      ffs zr = ff_add(ffs{hi0.x, lo0.x}, ffs{0.f, 0.f}), yr = ff_add(ffs{hi0.y, lo0.y}, ffs{0.f, 0.f});
+      const float ps = plane_inv<BF>(lane & 3);
+      ffs zr = ff_add(ffs{hi0.x * ps, lo0.x * ps}, ffs{0.f, 0.f}), yr = ff_add(ffs{hi0.y * ps, lo0.y * ps}, ffs{0.f, 0.f});
 #pragma unroll
       for (int o = 1; o < 4; o <<= 1) {
         zr = ff_add(zr, ffs{__shfl_xor_sync(0xffffffffu, zr.hi, o), __shfl_xor_sync(0xffffffffu, zr.lo, o)});
@@ -454,6 +469,8 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
     const uint32_t rowoff = (uint32_t)((lane & 7) + ((lane >> 4) << 3)) * pitch;
     const int vsel = (lane >> 3) & 1;
     const int bn = lane >> 2, bt = lane & 3;
+    const float2 pinv = NB == 2 ? make_float2(plane_inv<BF>(bt), plane_inv<BF>(bt))
+                                : make_float2(plane_inv<BF>((2 * bt) & 3), plane_inv<BF>((2 * bt + 1) & 3));
     uint32_t off[MS];
 #pragma unroll
     for (int i = 0; i < MS; ++i) off[i] = rowoff + (uint32_t)vsel * 16 + (e + XM_SB * i < STEPS ? toff[e + XM_SB * i] : 0u);
@@ -469,8 +486,9 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
       }
       const uint32_t* wf = reinterpret_cast<const uint32_t*>(&wfrag[ws][bn][0]);
       const uint32_t b0 = wf[bt], b1 = wf[bt + 4];
-      float2 sc = make_float2(1.f, 1.f);
-      sc.x = sc.y = wscale[ws];
+      // (two right-hand sides: this lane's columns are of plane bt; one: of planes 2 bt, 2 bt + 1)
+      const float wsc = wscale[ws];
+      const float2 sc = make_float2(wsc * pinv.x, wsc * pinv.y);
       const uint32_t base = smem_u32(smem + sb * stage);
       constexpr int GS = BF ? 4 : 2;   // steps in flight
 #pragma unroll
