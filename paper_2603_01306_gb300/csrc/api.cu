@@ -1382,7 +1382,7 @@ relax_status relax_solve(relax_handle* h, const int8_t* fixings, const void* war
   // pass's precision (the loop stalled on its arithmetic's floor, or the
   // loop's problem is the BF16 / FP8 copy of X), the loop goes on from
   // beta_best on the FP32 master X, then with float-float products on it,
-  // with the FP64 p-phase.
+  // with the FP64 p-phase and FP64 loss terms.
   for (int rung = 0; err == cudaSuccess && ladder_ok && h->certify;) {
     if (rung == 0 && h->has_acc32) { rung = 1; cur_pl = &h->pl_acc32; }
     else if (rung < 2 && h->has_ff) { rung = 2; cur_pl = &h->pl_ff; }
@@ -1390,6 +1390,7 @@ relax_status relax_solve(relax_handle* h, const int8_t* fixings, const void* war
     cur_np = &h->np_exact;
     cur_xa = pass_args(h, *cur_pl, h->loss == RELAX_LS ? LINK_LS : LINK_LOGISTIC, &h->st->ps);
     cur_xa.lsum = h->backtrack ? nullptr : h->lsum;
+    cur_xa.loss64 = 1;
     pa.ncl = cur_pl->Gr;
     na.ncl = cur_pl->Gr;
     na.nl = cur_pl->grid;

@@ -464,7 +464,10 @@ __global__ void __launch_bounds__(XF_T, 1) xring_kernel(const __grid_constant__ 
       if (jl == 0 && on) mbar_arrive(&wfull[ws]);
       if (on && cc == k % a.Gc && jl < rows) {   // this CTA records the block
         if (zout) zout[r0 + jl] = z[0];
-        if (a.lsum) loss_of<1, !FF && !D>(a.link, z, yd, zp, lsum);
+        if (a.lsum) {
+          if (a.loss64) loss_of<1, false>(a.link, z, yd, zp, lsum);
+          else loss_of<1, !FF && !D>(a.link, z, yd, zp, lsum);
+        }
       }
     }
     if (a.lsum) {

@@ -84,6 +84,7 @@ struct XSArgs {
   void* g;               // [Gr][NB][p] X' r per row group: FP32 pairs (float2), FP64 for FP64 X
   double* lsum;          // [CTA][4] sums over the rows the CTA records: F at z, -F*(-zeta) at the
                          // dual point, the same at the second one (LINK_CERT2_*), 0; or NULL
+  int loss64;            // the logistic loss terms in FP64 from an FP32 pass too (the precision ladder)
   unsigned* cnt;         // [nblk] CTAs done with the block's dots (zeroed before the launch)
   int* status;
   uint64_t limit_ns;
