@@ -1403,6 +1403,7 @@ relax_status relax_solve(relax_handle* h, const int8_t* fixings, const void* war
                                                   (double*)h->vb[3], h->p, (double*)h->vb[6], (double*)h->vb[7],
                                                   h->n);
     CU(cudaGetLastError());
+    out->launches += 1;
     IterState s2 = s;
     s2.iter = it0;
     s2.tol = tol_exact;
@@ -2095,7 +2096,7 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
   std::vector<int> active(nb), hdone(nb);
   for (int j = 0; j < nb; ++j) active[j] = j;
   const int max_rounds = h->max_iters / kRetire + 2;
-  int launches = 0;
+  int launches = 2 + (fixings ? 1 : 0);   // the starts, the results, the fixings' count
   for (int round = 0; round < max_rounds && !active.empty(); ++round) {
     const int m = (int)active.size();
     BTRYC(cudaMemcpyAsync(active_d, active.data(), sizeof(int) * (size_t)m, cudaMemcpyHostToDevice, h->stream));
@@ -2140,9 +2141,10 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
     const dim3 gn((unsigned)std::min<int64_t>(64, (n + 255) / 256), (unsigned)m);
     const dim3 gz((unsigned)((n + 63) / 64), (unsigned)((m + 15) / 16));
     const dim3 gg((unsigned)((p + 63) / 64), (unsigned)((NB * m + 15) / 16));
-    int round_launches = 0;
+    // (a graph kept from an earlier round is launched without being enqueued here)
+    const int per_iter = (f64 || bt ? 5 : 3) + (bt && !clustered ? (m + wave - 1) / wave : 1);
+    const int round_launches = kRetire * per_iter + (f64 || bt ? 0 : 1);
     auto enqueue_round = [&](cudaStream_t cs) -> cudaError_t {
-      round_launches = 0;
       for (int it = 0; it < kRetire; ++it) {
         cudaError_t e;
         if (f64) {
@@ -2163,16 +2165,13 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
           if ((e = bgemm_launch(pl2, a2, cs)) != cudaSuccess) return e;
           if (bt && (e = batch_reduce_grad(io, cs)) != cudaSuccess) return e;
         }
-        round_launches += 5;
         if (!bt) {
           if ((e = pnode_launch(np, na, m, cs)) != cudaSuccess) return e;
-          ++round_launches;
         } else if (clustered) {
           PArgs pw = pa;
           pw.seg_node = active_d;
           pw.cluster = 1;
           if ((e = pphase_launch_clusters(pc, pw, m, cs)) != cudaSuccess) return e;
-          ++round_launches;
         } else {
           for (int w0 = 0; w0 < m; w0 += wave) {
             PArgs pw = pa;
@@ -2180,7 +2179,6 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
             pw.part = part + (size_t)w0 * NB * p;
             const int cnt = std::min(wave, m - w0);
             if ((e = pphase_launch_grid(pp, pw, cnt * segb, cs)) != cudaSuccess) return e;
-            ++round_launches;
           }
         }
       }
@@ -2210,7 +2208,7 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
     } else {
       BTRYC(enqueue_round(h->stream));
     }
-    launches += round_launches;
+    launches += round_launches + 1;
     batch_done_kernel<<<1, 256, 0, h->stream>>>(dst, active_d, m, done_d);
     BTRYC(cudaGetLastError());
     BTRYC(cudaMemcpyAsync(hdone.data(), done_d, sizeof(int) * (size_t)m, cudaMemcpyDeviceToHost, h->stream));
@@ -2266,7 +2264,7 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
     o.lipschitz = S.Lk;
     o.primal_loop = S.phi_best;
     o.dual_loop = S.psi_best;
-    o.launches = launches + (h->certify ? nb + 2 * ((nb + kCertGroup - 1) / kCertGroup) : 0) + 1;
+    o.launches = launches + (h->certify ? nb + (nb + kCertGroup - 1) / kCertGroup : 0);
     relax_status st_j = map_dev_status(dstat);
     if (h->certify && st_j == RELAX_OK) {
       const double phi = cert[4 * (size_t)j];
