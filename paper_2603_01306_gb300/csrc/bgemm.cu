@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bgemm_kernel(const __grid_const
         const int nt = g.t % a.NT, mt = g.t / a.NT;
         for (int kb = g.kb0; kb < g.kb1; ++kb) {
           const int s = it % S;
-          if (it >= S && !mbar_wait<false>(&empty[s], ((it / S) - 1) & 1, a.limit_ns, a.status)) {
+          if (it >= S && !mbar_wait(&empty[s], ((it / S) - 1) & 1, a.limit_ns, a.status)) {
             tmo = 1;
             break;
           }
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bgemm_kernel(const __grid_const
         }
       }
       // the copies in flight land before the CTA may exit
-      for (int k = max(0, it - S); k < it; ++k) mbar_wait<false>(&full[k % S], (k / S) & 1, a.limit_ns, a.status);
+      for (int k = max(0, it - S); k < it; ++k) mbar_wait(&full[k % S], (k / S) & 1, a.limit_ns, a.status);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bgemm_kernel(const __grid_const
         const int kb1 = g.kb1;
         for (int pb = g.kb0; pb < kb1 && !tmo; pb += BG_DRAIN, ++gp) {
           const int b = gp % BG_NBUF;
-          if (gp >= BG_NBUF && !mbar_wait<false>(&tempty[b], ((gp / BG_NBUF) - 1) & 1, a.limit_ns, a.status)) {
+          if (gp >= BG_NBUF && !mbar_wait(&tempty[b], ((gp / BG_NBUF) - 1) & 1, a.limit_ns, a.status)) {
             tmo = 1;
             break;
           }
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bgemm_kernel(const __grid_const
           const int pe = min(kb1, pb + BG_DRAIN);
           for (int kb = pb; kb < pe; ++kb, ++it) {
             const int s = it % S;
-            if (!mbar_wait<false>(&full[s], (it / S) & 1, a.limit_ns, a.status)) {
+            if (!mbar_wait(&full[s], (it / S) & 1, a.limit_ns, a.status)) {
               tmo = 1;
               break;
             }
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bgemm_kernel(const __grid_const
       }
       // no MMA may be in flight when the TMEM is freed
       umma_commit(&drain);
-      mbar_wait<false>(&drain, 0, a.limit_ns, a.status);
+      mbar_wait(&drain, 0, a.limit_ns, a.status);
     }
     __syncwarp();
   } else {
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bgemm_kernel(const __grid_const
       bool ok = true;
       for (int pb = kb0; pb < kb1; pb += BG_DRAIN, ++gp) {
         const int b = gp % BG_NBUF;
-        ok = __all_sync(0xffffffffu, mbar_wait<false>(&tfull[b], (gp / BG_NBUF) & 1, a.limit_ns, a.status));
+        ok = __all_sync(0xffffffffu, mbar_wait(&tfull[b], (gp / BG_NBUF) & 1, a.limit_ns, a.status));
         if (!ok) break;
         tc_fence_after();
         const uint32_t col = (uint32_t)(2 * b * BG_MAXN + c0);

@@ -232,7 +232,6 @@ struct GradSm {
   alignas(16) float H1[TILE * W2P];       // [row][h]
   alignas(16) float DA2[TILE * W2P];      // [row][o] dL/da2
   float XS[TILE * 8];         // [row] standardised inputs
-  float sq[TILE], d[TILE];    // squared residuals, dL/dout
   float comb[16][NH * (NIN + 3)];
 };
 

@@ -1,7 +1,6 @@
 // The node p-phase (pnode.cuh): kernel, plan and launch.
 #include <algorithm>
 #include <cfloat>
-#include <cstdlib>
 
 #include "launch.cuh"
 
@@ -1755,7 +1754,6 @@ cudaLaunchConfig_t config(const NPlan& pl, int nprob, cudaLaunchAttribute* attr,
 // problem where the sizes allow (256 problems of p = 10000, whole call: 1 / 2 /
 // 4 / 8 CTAs 62.8 / 63.1 / 60.7 / 63.7 ms; 48 of p = 5000: 2 / 4 / 8 CTAs 7.59 /
 // 6.97 / 7.62 ms).  A CTA's coordinates must fit its shared memory either way.
-// RELAX_PN=c sets the cluster size for tuning runs.
 cudaError_t pnode_plan(NPlan& pl, bool f64, int64_t p, int nprob) {
   pl = NPlan{};
   pl.f64 = f64;
@@ -1768,8 +1766,7 @@ cudaError_t pnode_plan(NPlan& pl, bool f64, int64_t p, int nprob) {
   const int64_t target = f64 ? 64 : 224;
   int share = 4;
   while (share < PN_MAXCL && 2 * share * nprob <= 2 * nsm) share *= 2;
-  int64_t want = std::min<int64_t>((p + target - 1) / target, share);
-  if (const char* ov = std::getenv("RELAX_PN")) want = std::max(1, std::min(PN_MAXCL, std::atoi(ov)));
+  const int64_t want = std::min<int64_t>((p + target - 1) / target, share);
   int cl = 1;
   while (cl < want) cl *= 2;
   cudaError_t e;

@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
       for (int k = 0; k < kloc; ++k) {
         const int s = k % a.RA;
         if (tmo) break;
-        if (k >= a.RA && !mbar_wait<false>(&empty[s], ((k / a.RA) - 1) & 1, a.limit_ns, a.status)) { tmo = 1; break; }
+        if (k >= a.RA && !mbar_wait(&empty[s], ((k / a.RA) - 1) & 1, a.limit_ns, a.status)) { tmo = 1; break; }
         const int y0 = (cr + k * a.Gr) * 16;
         mbar_arrive_expect_tx(&full[s], tilebytes);
         for (int i = 0; i < a.nbox; ++i)
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
       }
       // let every copy in flight land before the CTA may exit
       for (int k = (issued > a.RA ? issued - a.RA : 0); k < issued; ++k)
-        mbar_wait<false>(&full[k % a.RA], (k / a.RA) & 1, a.limit_ns, a.status);
+        mbar_wait(&full[k % a.RA], (k / a.RA) & 1, a.limit_ns, a.status);
     }
     __syncwarp();
   } else if (warp < 1 + XM_SA) {
@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
     for (int k = st; k < kloc; k += XM_SA) {
       if (tmo) break;
       const int sa = k % a.RA;
-      if (!__all_sync(0xffffffffu, mbar_wait<false>(&full[sa], (k / a.RA) & 1, a.limit_ns, a.status))) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&full[sa], (k / a.RA) & 1, a.limit_ns, a.status))) {
         tmo = 1;
         break;
       }
@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
       const double yd = a.y[rowj];
       const double zp = need_zp ? zprev[rowj] : 0.0;
       const int ws = k % XM_RW;
-      bool ok = !on || k < XM_RW || mbar_wait<false>(&wempty[ws], ((k / XM_RW) - 1) & 1, a.limit_ns, a.status);
+      bool ok = !on || k < XM_RW || mbar_wait(&wempty[ws], ((k / XM_RW) - 1) & 1, a.limit_ns, a.status);
       // the row's words, complete once their low bits count every strip
       unsigned long long wh = 0ull, wl = 0ull;
       ok = ok && wait_row(&a.zfix[2 * rowj], (unsigned)a.Gc, wh, wl, a.limit_ns, a.status);
@@ -478,8 +478,8 @@ __global__ void __launch_bounds__(XM_T, 1) xmma_kernel(const __grid_constant__ X
       if (tmo) break;
       // (the block's tile is there: its own dot products are part of the agreed z)
       const int ws = k % XM_RW, sb = k % a.RA;
-      const bool ok = mbar_wait<false>(&full[sb], (k / a.RA) & 1, a.limit_ns, a.status) &&
-                      mbar_wait<false>(&wfull[ws], (k / XM_RW) & 1, a.limit_ns, a.status);
+      const bool ok = mbar_wait(&full[sb], (k / a.RA) & 1, a.limit_ns, a.status) &&
+                      mbar_wait(&wfull[ws], (k / XM_RW) & 1, a.limit_ns, a.status);
       if (!__all_sync(0xffffffffu, ok)) {
         tmo = 1;
         break;

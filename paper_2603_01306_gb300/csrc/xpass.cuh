@@ -15,14 +15,12 @@ enum Link : int {
   LINK_IDENT = 2,      // NF=1 NB=1: r = z             (power iteration on X'X)
   LINK_CERT_LS = 3,    // NF=2 NB=1: F at z0, r = 2(z1 - y)
   LINK_CERT_LOGI = 4,  // NF=2 NB=1: F at z0, r = grad at z1
-  LINK_CERTZ_LS = 5,   // NF=1 NB=1: F at z0, r = 2(zd - y) with zd = ps.zprev (given dual point)
-  LINK_CERTZ_LOGI = 6, // NF=1 NB=1: F at z0, r = grad at zd
   // both dual points of a certificate in one pass: NF=1 NB=2, F at z0,
   // r0 = the link at zd = ps.zprev (the loop's best dual point), r1 = the link
-  // at z0 (zeta = -grad F(X beta)); lterm gets {F, dual term at zd}, lterm2
-  // {F, dual term at z0}
-  LINK_CERT2_LS = 7,
-  LINK_CERT2_LOGI = 8,
+  // at z0 (zeta = -grad F(X beta)); the loss sums are F, the dual terms at zd
+  // and those at z0
+  LINK_CERT2_LS = 5,
+  LINK_CERT2_LOGI = 6,
 };
 
 // Device-resident solver state that the pass reads (pointers rotate between
@@ -37,15 +35,11 @@ struct PassState {
 };
 
 template <typename TX> struct XTraits;
-// 16-byte vectors of X: load from shared memory (load), from global memory
-// keeping the line in L2 for a later re-read (load_global: ld.global.cg), or
-// from global memory as its last use (load_global_last: ld.global.cs).
+// 16-byte vectors of X from shared memory
 template <> struct XTraits<double> {
   static constexpr int VEC = 2;
   template <typename TA> __device__ static void cvt(const double2 v, TA* o) { o[0] = (TA)v.x; o[1] = (TA)v.y; }
   template <typename TA> __device__ static void load(const double* p, TA* o) { cvt(*reinterpret_cast<const double2*>(p), o); }
-  template <typename TA> __device__ static void load_global(const double* p, TA* o) { cvt(__ldcg(reinterpret_cast<const double2*>(p)), o); }
-  template <typename TA> __device__ static void load_global_last(const double* p, TA* o) { cvt(__ldcs(reinterpret_cast<const double2*>(p)), o); }
 };
 template <> struct XTraits<float> {
   static constexpr int VEC = 4;
@@ -53,8 +47,6 @@ template <> struct XTraits<float> {
     o[0] = (TA)v.x; o[1] = (TA)v.y; o[2] = (TA)v.z; o[3] = (TA)v.w;
   }
   template <typename TA> __device__ static void load(const float* p, TA* o) { cvt(*reinterpret_cast<const float4*>(p), o); }
-  template <typename TA> __device__ static void load_global(const float* p, TA* o) { cvt(__ldcg(reinterpret_cast<const float4*>(p)), o); }
-  template <typename TA> __device__ static void load_global_last(const float* p, TA* o) { cvt(__ldcs(reinterpret_cast<const float4*>(p)), o); }
 };
 // Float-float sums (Knuth's TwoSum; about 48 significant bits from FP32
 // instructions).  This GPU issues FP64 arithmetic, comparisons and
@@ -182,33 +174,6 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float a) {
   const float err = (hi - (s - bp)) + (a - bp);
   hi = s;
   lo += err;
-}
-
-// A (hi, lo) FP32 pair travels through the exchange as the bits of a double.
-__device__ __forceinline__ double pack_pair(float hi, float lo) {
-  return __hiloint2double(__float_as_int(hi), __float_as_int(lo));
-}
-__device__ __forceinline__ void add_pair(float& hi, float& lo, double packed) {
-  const float ph = __int_as_float(__double2hiint(packed));
-  const float pl = __int_as_float(__double2loint(packed));
-  two_sum_acc(hi, lo, ph);
-  lo += pl;
-}
-__device__ __forceinline__ float exp_t(float t) { return expf(t); }
-__device__ __forceinline__ double exp_t(double t) { return exp(t); }
-
-// Warp sum of (hi, lo) FP32 pairs: each butterfly step adds the partner's pair
-// with TwoSum, keeping about 44 bits; FP32 pipe only.
-__device__ __forceinline__ void warp_sum_pair(float& hi, float& lo) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float oh = __shfl_xor_sync(0xffffffffu, hi, o);
-    const float ol = __shfl_xor_sync(0xffffffffu, lo, o);
-    float h = hi, l = 0.f;
-    two_sum_acc(h, l, oh);
-    hi = h;
-    lo = lo + ol + l;
-  }
 }
 
 }  // namespace relax

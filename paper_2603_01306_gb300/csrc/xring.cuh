@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(XF_T, 1) xring_kernel(const __grid_constant__ 
       for (int k = 0; k < kloc; ++k) {
         const int s = k % a.RA;
         if (tmo) break;
-        if (k >= a.RA && !mbar_wait<false>(&empty[s], ((k / a.RA) - 1) & 1, a.limit_ns, a.status)) { tmo = 1; break; }
+        if (k >= a.RA && !mbar_wait(&empty[s], ((k / a.RA) - 1) & 1, a.limit_ns, a.status)) { tmo = 1; break; }
         const int y0 = (cr + k * a.Gr) * XF_B;
         mbar_arrive_expect_tx(&full[s], tilebytes);
         for (int i = 0; i < a.nbox; ++i)
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(XF_T, 1) xring_kernel(const __grid_constant__ 
       }
       // let every copy in flight land before the CTA may exit
       for (int k = (issued > a.RA ? issued - a.RA : 0); k < issued; ++k)
-        mbar_wait<false>(&full[k % a.RA], (k / a.RA) & 1, a.limit_ns, a.status);
+        mbar_wait(&full[k % a.RA], (k / a.RA) & 1, a.limit_ns, a.status);
     }
     __syncwarp();
   } else if (warp < 1 + XF_SA) {
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(XF_T, 1) xring_kernel(const __grid_constant__ 
       if (tmo) break;
       const int k = i / UB, pr = i % UB;
       const int sa = k % a.RA;
-      if (!__all_sync(0xffffffffu, mbar_wait<false>(&full[sa], (k / a.RA) & 1, a.limit_ns, a.status))) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&full[sa], (k / a.RA) & 1, a.limit_ns, a.status))) {
         tmo = 1;
         break;
       }
@@ -315,8 +315,8 @@ __global__ void __launch_bounds__(XF_T, 1) xring_kernel(const __grid_constant__ 
     for (int k = 0; k < kloc; ++k) {
       if (tmo) break;
       const int ws = k % XF_RW, sb = k % a.RA;
-      const bool ok = mbar_wait<false>(&full[sb], (k / a.RA) & 1, a.limit_ns, a.status) &&
-                      mbar_wait<false>(&wfull[ws], (k / XF_RW) & 1, a.limit_ns, a.status);
+      const bool ok = mbar_wait(&full[sb], (k / a.RA) & 1, a.limit_ns, a.status) &&
+                      mbar_wait(&wfull[ws], (k / XF_RW) & 1, a.limit_ns, a.status);
       if (!__all_sync(0xffffffffu, ok)) {
         tmo = 1;
         break;
@@ -405,8 +405,7 @@ __global__ void __launch_bounds__(XF_T, 1) xring_kernel(const __grid_constant__ 
   } else {
     // ------------------------------------------------ the link of the rows
     const int st = warp - 1 - XF_SA - XF_SB;
-    const bool need_zp = a.link == LINK_CERTZ_LS || a.link == LINK_CERTZ_LOGI || a.link == LINK_CERT2_LS ||
-                         a.link == LINK_CERT2_LOGI || (a.link == LINK_LOGISTIC && NB > 1);
+    const bool need_zp = a.link == LINK_CERT2_LS || a.link == LINK_CERT2_LOGI || (a.link == LINK_LOGISTIC && NB > 1);
     const double* zprev = static_cast<const double*>(a.ps->zprev);
     double* zout = static_cast<double*>(a.ps->zout);
     const double mom = a.ps->mom;
@@ -424,7 +423,7 @@ __global__ void __launch_bounds__(XF_T, 1) xring_kernel(const __grid_constant__ 
       const double zp = need_zp ? zprev[rowj] : 0.0;
       const int ws = k % XF_RW;
       unsigned long long wh = 0ull, wl = 0ull;
-      bool ok = k < XF_RW || mbar_wait<false>(&wempty[ws], ((k / XF_RW) - 1) & 1, a.limit_ns, a.status);
+      bool ok = k < XF_RW || mbar_wait(&wempty[ws], ((k / XF_RW) - 1) & 1, a.limit_ns, a.status);
       ok = ok && wait_row(&a.zfix[2 * rowj], (unsigned)a.Gc, wh, wl, a.limit_ns, a.status);
       if (!__all_sync(0xffffffffu, ok)) {
         tmo = 1;

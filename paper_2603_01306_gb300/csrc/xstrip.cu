@@ -1,9 +1,7 @@
 // Instantiations, plan and launch of the strip-stationary fused pass.
 #include <algorithm>
 #include <cmath>
-#include <cstdio>
 #include <cstdint>
-#include <cstdlib>
 
 #include "launch.cuh"
 
@@ -33,7 +31,8 @@ static int xs_tv(int vec) { return vec == 2 ? XSShape<2>::TV : XSShape<4>::TV; }
 //    as many stages per warp as shared memory holds (ring A first);
 //  * phase A may lead phase B by `lag` blocks: about 64 MB of X in L2 (at
 //    least 20 blocks with four or more row groups).
-// RELAX_XS="B,SA,SB,lag,vps,mA,mB,Gr" overrides for tuning runs (0 keeps a default).
+// Lags and row groups were measured on the loop's passes while this kernel ran
+// them; the certificate of two different vectors kept the choices.
 cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t n, int64_t p) {
   if ((xk == XK_BF16 || xk == XK_FP8) && !f64acc && NF == 1) return xmma_plan(pl, xk, NB, n, p);
   if ((xk == XK_F32 || xk == XK_F64) && NF == 1) return xring_plan(pl, xk, f64acc, NB, n, p);
@@ -50,9 +49,6 @@ cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const int es = xkind_esize(xk);
   const int vec = xkind_vec(xk);
-  int B_f = 0, SA_f = 0, SB_f = 0, lag_f = 0, vps_f = 0, mA_f = 0, mB_f = 0, gr_f = 0;
-  if (const char* ov = std::getenv("RELAX_XS"))
-    std::sscanf(ov, "%d,%d,%d,%d,%d,%d,%d,%d", &B_f, &SA_f, &SB_f, &lag_f, &vps_f, &mA_f, &mB_f, &gr_f);
   // strips: over the number of row groups Gr, the strip width (at most `cap`
   // vectors) that keeps the most SMs busy, strips under 2 KB counted as
   // streaming less efficiently
@@ -70,7 +66,6 @@ cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t
     const double score = (double)(gc * gr) * std::sqrt(std::min(1.0, (double)(v * 16) / 2048.0));
     if (score > best * 1.0001) { best = score; vps = v; }
   }
-  if (vps_f > 0) vps = vps_f;
   if (vps <= 0 || vps > cap) return cudaErrorNotSupported;   // p wider than nsm strips of one lane row
   const int64_t cols = vps * vec;
   const int64_t nbox = (cols + 255) / 256;
@@ -83,7 +78,6 @@ cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t
   pl.Gc = (int)Gc;
   // blocks
   int64_t B = std::max<int64_t>(1, std::min<int64_t>(XS_MAXB, 40960 / (pl.sw * es)));
-  if (B_f > 0) B = std::min<int64_t>(B_f, XS_MAXB);
   B = std::min<int64_t>(B, n);
   auto boxb = [&](int64_t b) { return (b * inner * es + 127) / 128 * 128; };
   const size_t fixed = 2048 + 128;   // static shared memory, alignment slack
@@ -91,22 +85,16 @@ cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t
     return (size_t)(sa + sb) * (size_t)(nbox * boxb(b)) + fixed <= (size_t)optin;
   };
   while (B > 1 && !fits(B, 3, 3)) --B;
-  int SA = 3, SB = 3;   // 2 + SA + SB warps <= 8
-  if (SA_f > 0) SA = std::min(SA_f, XS_MAXS);
-  if (SB_f > 0) SB = std::min(SB_f, XS_MAXS);
-  if (2 + SA + SB > XS_MAXT / 32 || !fits(B, SA, SB)) return cudaErrorNotSupported;
+  const int SA = 3, SB = 3;   // 2 + SA + SB warps <= 8
+  static_assert(2 + 3 + 3 <= XS_MAXT / 32);
+  if (!fits(B, SA, SB)) return cudaErrorNotSupported;
   // ring depths: stages per warp.  A stage is held from its TMA issue until
   // its warp has read the block, so small blocks (narrow element types) need
   // more of them to keep enough of X in flight; ring A (HBM) first, then
   // ring B (L2), while shared memory allows
   int mA = 1, mB = 1;
-  if (mA_f > 0 || mB_f > 0) {
-    mA = std::max(1, mA_f);
-    mB = std::max(1, mB_f);
-  } else {
-    while ((mA + 1) * SA <= XS_MAXR && fits(B, (mA + 1) * SA, mB * SB)) ++mA;
-    if (mA > 1 && (mB + 1) * SB <= XS_MAXR && fits(B, mA * SA, (mB + 1) * SB)) ++mB;
-  }
+  while ((mA + 1) * SA <= XS_MAXR && fits(B, (mA + 1) * SA, mB * SB)) ++mA;
+  if (mA > 1 && (mB + 1) * SB <= XS_MAXR && fits(B, mA * SA, (mB + 1) * SB)) ++mB;
   if (mA * SA > XS_MAXR || mB * SB > XS_MAXR || !fits(B, mA * SA, mB * SB)) return cudaErrorNotSupported;
   pl.RA = mA * SA;
   pl.RB = mB * SB;
@@ -117,17 +105,16 @@ cudaError_t xstrip_plan(XSPlan& pl, int xk, bool f64acc, int NF, int NB, int64_t
   pl.SB = SB;
   pl.Gr = (int)std::max<int64_t>(1, std::min<int64_t>(nsm / Gc, pl.nblk));
   // at least two blocks per CTA: a row group costs the p-phase one partial of
-  // X'r per column, and the pass little (1000 x 1000 FP32, 63 -> 32 groups:
-  // pass 21.7 -> 20.8 us, p-phase 31.6 -> 29.2; 500 x 1000 FP64, 30 -> 16:
-  // 30.9 -> 30.6, 33.7 -> 29.7; fewer still and the pass loses more)
+  // X'r per column, and the pass little (loop passes, 1000 x 1000 FP32, 63 -> 32
+  // groups: pass 21.7 -> 20.8 us, p-phase 31.6 -> 29.2; 500 x 1000 FP64, 30 ->
+  // 16: 30.9 -> 30.6, 33.7 -> 29.7; fewer still and the pass loses more)
   pl.Gr = std::max(1, std::min(pl.Gr, (pl.nblk + 1) / 2));
-  if (gr_f > 0) pl.Gr = std::min(pl.Gr, gr_f);
   const double row_bytes = (double)p * es;
-  pl.lag = lag_f > 0 ? lag_f : (int)std::max(4.0, std::min(64.0, 64.0e6 / (B * row_bytes * pl.Gr)));
+  pl.lag = (int)std::max(4.0, std::min(64.0, 64.0e6 / (B * row_bytes * pl.Gr)));
   // tall designs (four or more row groups): a deeper lead measured faster
-  // (100000 x 20000 logistic: lag 12 -> 20 took the pass from 0.28 to 0.43 of
-  // the copy bandwidth) although it holds more of X than L2 does
-  if (lag_f <= 0 && pl.Gr >= 4) pl.lag = std::max(pl.lag, 20);
+  // (100000 x 20000 logistic loop pass: lag 12 -> 20, 0.28 -> 0.43 of the copy
+  // bandwidth) although it holds more of X than L2 does
+  if (pl.Gr >= 4) pl.lag = std::max(pl.lag, 20);
   pl.grid = pl.Gc * pl.Gr;
   pl.threads = 32 * (2 + SA + SB);   // two producers, SA dot, SB axpy
   // the combine of the axpy warps' strip sums reuses the rings

@@ -95,9 +95,6 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
   asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ void st_release_u32(unsigned* p, unsigned v) {
-  asm volatile("st.release.gpu.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 
 // bounded wait until *ctr >= target; false (and ST_TIMEOUT) after limit_ns
 __device__ __forceinline__ bool wait_count(const unsigned* ctr, unsigned target, uint64_t limit_ns, int* status) {
@@ -139,11 +136,6 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
-__device__ __forceinline__ uint64_t policy_evict_last() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
 __device__ __forceinline__ uint64_t policy_evict_normal() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
@@ -240,12 +232,10 @@ __device__ __forceinline__ void link_of(int link, const double* z, double yd, do
       w[0] = z[0];
       break;
     case LINK_CERT_LS:
-    case LINK_CERTZ_LS:
-      w[0] = 2.0 * ((link == LINK_CERT_LS ? z[NF - 1] : zp) - yd);
+      w[0] = 2.0 * (z[NF - 1] - yd);
       break;
     case LINK_CERT_LOGI:
-    case LINK_CERTZ_LOGI:
-      w[0] = -yd / (1.0 + exp(yd * (link == LINK_CERT_LOGI ? z[NF - 1] : zp)));
+      w[0] = -yd / (1.0 + exp(yd * z[NF - 1]));
       break;
     case LINK_CERT2_LS:
       w[0] = 2.0 * (zp - yd);
@@ -265,7 +255,7 @@ __device__ __forceinline__ void link_of(int link, const double* z, double yd, do
 template <int NF, bool LOWP>
 __device__ __forceinline__ void loss_of(int link, const double* z, double yd, double zp, double (&s)[3]) {
   if (link == LINK_IDENT) return;
-  const bool ls = link == LINK_LS || link == LINK_CERT_LS || link == LINK_CERTZ_LS || link == LINK_CERT2_LS;
+  const bool ls = link == LINK_LS || link == LINK_CERT_LS || link == LINK_CERT2_LS;
   const bool loop = link == LINK_LS || link == LINK_LOGISTIC;
   const bool two = link == LINK_CERT2_LS || link == LINK_CERT2_LOGI;
   const double zd = loop ? z[0] : (link == LINK_CERT_LS || link == LINK_CERT_LOGI) ? z[NF - 1] : zp;
@@ -365,7 +355,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
       for (int k = 0; k < kloc; ++k) {
         const int s = k % a.RA;
         if (tmo) break;
-        if (k >= a.RA && !mbar_wait<false>(&emptyA[s], ((k / a.RA) - 1) & 1, a.limit_ns, a.status)) { tmo = 1; break; }
+        if (k >= a.RA && !mbar_wait(&emptyA[s], ((k / a.RA) - 1) & 1, a.limit_ns, a.status)) { tmo = 1; break; }
         if (k > a.lag && !wait_smem(&bcnt, (unsigned)(k - a.lag), a.limit_ns, a.status)) { tmo = 1; break; }
         const int y0 = (cr + k * a.Gr) * a.B;
         mbar_arrive_expect_tx(&fullA[s], tilebytes);
@@ -375,7 +365,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
       }
       // let every copy in flight land before the CTA may exit
       for (int k = (issued > a.RA ? issued - a.RA : 0); k < issued; ++k)
-        mbar_wait<false>(&fullA[k % a.RA], (k / a.RA) & 1, a.limit_ns, a.status);
+        mbar_wait(&fullA[k % a.RA], (k / a.RA) & 1, a.limit_ns, a.status);
     }
   } else if (warp == 1) {
     // ---------------------------------- producer B: L2 -> ring B (its own warp,
@@ -386,7 +376,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
       for (int k = 0; k < kloc; ++k) {
         const int s = k % a.RB;
         if (tmo) break;
-        if (k >= a.RB && !mbar_wait<false>(&emptyB[s], ((k / a.RB) - 1) & 1, a.limit_ns, a.status)) { tmo = 1; break; }
+        if (k >= a.RB && !mbar_wait(&emptyB[s], ((k / a.RB) - 1) & 1, a.limit_ns, a.status)) { tmo = 1; break; }
         const int y0 = (cr + k * a.Gr) * a.B;
         mbar_arrive_expect_tx(&fullB[s], tilebytes);
         for (int i = 0; i < a.nbox; ++i)
@@ -394,7 +384,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
         issued = k + 1;
       }
       for (int k = (issued > a.RB ? issued - a.RB : 0); k < issued; ++k)
-        mbar_wait<false>(&fullB[k % a.RB], (k / a.RB) & 1, a.limit_ns, a.status);
+        mbar_wait(&fullB[k % a.RB], (k / a.RB) & 1, a.limit_ns, a.status);
     }
   } else if (warp < 2 + a.SA) {
     // ------------------------------------------------ phase A: strip dot products
@@ -447,7 +437,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
     for (int k = st; k < kloc; k += a.SA) {
       if (tmo) break;
       const int sa = k % a.RA;   // one of this warp's stages
-      if (!__all_sync(0xffffffffu, mbar_wait<false>(&fullA[sa], (k / a.RA) & 1, a.limit_ns, a.status))) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&fullA[sa], (k / a.RA) & 1, a.limit_ns, a.status))) {
         tmo = 1;
         break;
       }
@@ -574,8 +564,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
           acc[q][t][l] = (TA)0;
           if constexpr (FF) accl[q][t][l] = 0.f;
         }
-    const bool need_zp = a.link == LINK_CERTZ_LS || a.link == LINK_CERTZ_LOGI || a.link == LINK_CERT2_LS ||
-                         a.link == LINK_CERT2_LOGI || (a.link == LINK_LOGISTIC && NB > 1);
+    const bool need_zp = a.link == LINK_CERT2_LS || a.link == LINK_CERT2_LOGI || (a.link == LINK_LOGISTIC && NB > 1);
     const double* zprev = static_cast<const double*>(a.ps->zprev);
     double* zout = static_cast<double*>(a.ps->zout);
     const double mom = a.ps->mom;
@@ -625,7 +614,7 @@ __global__ void __launch_bounds__(XS_MAXT, 1) xstrip_kernel(const __grid_constan
         if (a.lsum) loss_of<NF, false>(a.link, z, yd, zp, lsum);
       }
       const int sb = k % a.RB;   // one of this warp's stages
-      if (!__all_sync(0xffffffffu, mbar_wait<false>(&fullB[sb], (k / a.RB) & 1, a.limit_ns, a.status))) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&fullB[sb], (k / a.RB) & 1, a.limit_ns, a.status))) {
         tmo = 1;
         break;
       }
