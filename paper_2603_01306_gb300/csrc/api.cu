@@ -808,7 +808,7 @@ relax_status cert_eval(relax_handle* h, int dual, int items, const int8_t* fix, 
   na.out = out;
   na.out_stride = ostride;
   NPlan np = h->np_eval;
-  if (items * na.nq > 2) CU(pnode_plan(np, h->dtype == RELAX_F64, h->p, items * na.nq));
+  if (items * na.nq > 2) CU(pnode_plan(np, h->f64() ? PK_F64 : PK_PAIR64, h->p, items * na.nq));
   CU(pnode_launch(np, na, items * na.nq, h->stream));
   return RELAX_OK;
 }
@@ -1048,11 +1048,12 @@ relax_status relax_create(relax_handle** out, const void* X, const void* y, int6
     // FP32, BF16 and FP8 data: the loop's per-coordinate arithmetic in FP32
     // (FP64 at a small fraction of the FP32 rate on this GPU); FP64 data keeps
     // FP64 throughout
-    TRYC(pnode_plan(h->np_iter, h->xk_loop == XK_F64, p, 1));
+    TRYC(pnode_plan(h->np_iter, h->xk_loop == XK_F64 ? PK_F64 : PK_PAIR, p, 1));
     // the certificate's evaluation: FP32 per coordinate and FP64 wherever a
-    // term of Phi or Psi is nonzero (FP32 data); FP64 throughout for FP64 data
-    TRYC(pnode_plan(h->np_eval, vd, p, 2));
-    TRYC(pnode_plan(h->np_exact, true, p, 1));
+    // term of Phi or Psi is nonzero, its sums FP64 (FP32 data); FP64 throughout
+    // for FP64 data
+    TRYC(pnode_plan(h->np_eval, vd ? PK_F64 : PK_PAIR64, p, 2));
+    TRYC(pnode_plan(h->np_exact, PK_F64, p, 1));
     if (h->backtrack) TRYC(pphase_plan(h->pp_iter, true, p, true));
     {
       const XSPlan* pls[7] = {&h->pl_loop, &h->pl_ident, &h->pl_cert, &h->pl_certz, &h->pl_cert2,
@@ -1581,7 +1582,7 @@ static relax_status standalone(int mode, const void* vin, void* vout, int64_t p,
   if (!vin || p <= 0 || k < 0 || !(M > 0.0) || (dtype != RELAX_F64 && dtype != RELAX_F32)) return RELAX_EINVAL;
   const bool dbl = dtype == RELAX_F64;
   NPlan np;
-  const bool cluster = pnode_plan(np, true, p, 1) == cudaSuccess;
+  const bool cluster = pnode_plan(np, PK_F64, p, 1) == cudaSuccess;
   PPlan pl;
   if (!cluster) {
     (void)cudaGetLastError();
@@ -2134,7 +2135,7 @@ extern "C" relax_status relax_solve_batch(relax_handle* h, int32_t nb, const int
       io.lsum = bt ? nullptr : W.lsum;
     }
     NPlan np;
-    if (!bt) BTRYC(pnode_plan(np, f64, p, m));
+    if (!bt) BTRYC(pnode_plan(np, f64 ? PK_F64 : PK_PAIR, p, m));
     na.m = m;
     na.s2 = pl2.split();
     const dim3 gp((unsigned)std::min<int64_t>(64, (p + 255) / 256), (unsigned)m);

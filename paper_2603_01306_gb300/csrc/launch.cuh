@@ -55,12 +55,12 @@ cudaError_t xstrip_launch(const XSPlan& pl, const XSArgs& a, bool clear, cudaStr
 // evaluation of `nprob` problems of length p, one cluster each.
 struct NPlan {
   const void* kernel = nullptr;
-  bool f64 = false;
   int cl = 1, cpc = 32, lc = 64;   // CTAs per problem, coordinates per CTA, list entries per CTA
   int warps = 8, wch = 32;         // warps per CTA (the first takes no coordinates), coordinates per warp
   size_t smem = 0;
 };
-cudaError_t pnode_plan(NPlan& pl, bool f64, int64_t p, int nprob);
+// kind: PNKind (pnode.cuh)
+cudaError_t pnode_plan(NPlan& pl, int kind, int64_t p, int nprob);
 // fills the plan's fields of `a`; grid = nprob clusters
 cudaError_t pnode_launch(const NPlan& pl, NArgs a, int nprob, cudaStream_t st);
 

@@ -53,7 +53,7 @@ extern __shared__ __align__(16) unsigned char pn_raw[];
 __device__ __forceinline__ PnSh& pn() { return *reinterpret_cast<PnSh*>(pn_raw); }
 
 // a sum in the data's working precision: float-float, or FP64
-template <bool F64> struct Acc;
+template <bool S64> struct Acc;
 template <> struct Acc<false> {
   ffs s;
   __device__ Acc() : s{0.f, 0.f} {}
@@ -74,10 +74,10 @@ template <> struct Acc<true> {
   __device__ unsigned long long word() const { return (unsigned long long)__double_as_longlong(s); }
   __device__ double val() const { return s; }
 };
-template <bool F64>
-__device__ __forceinline__ void warp_merge(Acc<F64>& a) {
+template <bool S64>
+__device__ __forceinline__ void warp_merge(Acc<S64>& a) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a.merge(Acc<F64>(__shfl_xor_sync(0xffffffffu, a.word(), o)));
+  for (int o = 16; o > 0; o >>= 1) a.merge(Acc<S64>(__shfl_xor_sync(0xffffffffu, a.word(), o)));
 }
 __device__ __forceinline__ unsigned long long pack2(unsigned lo, unsigned hi) { return ((unsigned long long)hi << 32) | lo; }
 __device__ __forceinline__ void st_cluster_u64(uint32_t addr, unsigned long long v) {
@@ -132,9 +132,9 @@ __device__ __forceinline__ A xacc(int nx, int w) {   // over the CTAs in rank or
 // Every warp's words of `red` are in place: sum them over the warps, push the
 // sums into every CTA's shared memory, and wait until every CTA has pushed.
 // Words below na0 are float-float, below na1 A sums, the others counts.
-template <bool F64>
+template <int K>
 __device__ __noinline__ void pn_exchange(int nx, int na0, int na1, int words) {
-  using A = Acc<F64>;
+  using A = Acc<(K != PK_PAIR)>;
   PnSh& s = pn();
   __syncthreads();
   const int W = blockDim.x >> 5, S = s.a.cl;
@@ -166,14 +166,14 @@ __device__ __noinline__ void pn_exchange(int nx, int na0, int na1, int words) {
 }
 // A small cluster-wide sum of two A sums and two counts per lane -> red_,
 // cnt0, cnt1; returns the next exchange's number
-template <bool F64>
+template <int K>
 __device__ __noinline__ int pn_small_sum(int nx, unsigned long long w0, unsigned long long w1, unsigned c0, unsigned c1) {
-  using A = Acc<F64>;
+  using A = Acc<(K != PK_PAIR)>;
   PnSh& s = pn();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   A v0(w0), v1(w1);
-  warp_merge<F64>(v0);
-  warp_merge<F64>(v1);
+  warp_merge<(K != PK_PAIR)>(v0);
+  warp_merge<(K != PK_PAIR)>(v1);
   c0 = __reduce_add_sync(0xffffffffu, c0);
   c1 = __reduce_add_sync(0xffffffffu, c1);
   if (lane == 0) {
@@ -182,7 +182,7 @@ __device__ __noinline__ int pn_small_sum(int nx, unsigned long long w0, unsigned
     rw[1] = v1.word();
     rw[2] = pack2(c0, c1);
   }
-  pn_exchange<F64>(nx, 0, 2, 3);
+  pn_exchange<K>(nx, 0, 2, 3);
   if (warp == 0) {
     if (lane < 2) s.red_[lane] = xacc<A>(nx, lane).val();
     else if (lane == 2) {
@@ -236,11 +236,23 @@ __device__ __noinline__ float2 pn_gpair_call(int64_t j, int q) {
   const ffs v = pn_gpair(j, q);
   return make_float2(v.hi, v.lo);
 }
+// the same in FP64 (sums of pairs too, but in the loop on FP32 data)
+template <int K>
 __device__ __noinline__ double pn_gdbl(int64_t j, int q) {
   const PnSh& s = pn();
-  if (s.a.gpair || s.a.tiles) {
+  if (K == PK_PAIR) {
     const float2 v = pn_gpair_call(j, q);
     return (double)v.x + (double)v.y;
+  }
+  if (s.a.gpair) {
+    const float2* src = static_cast<const float2*>(s.part) + (size_t)q * s.a.p + j;
+    double v = 0.0;
+#pragma unroll 8
+    for (int c = 0; c < s.a.ncl; ++c) {
+      const float2 y = __ldcg(src + (size_t)c * s.a.NB * s.a.p);
+      v += (double)y.x + (double)y.y;
+    }
+    return v;
   }
   const double* src = static_cast<const double*>(s.part) + (size_t)q * s.a.p + j;
   double v = 0.0;
@@ -249,9 +261,9 @@ __device__ __noinline__ double pn_gdbl(int64_t j, int q) {
   return v;
 }
 // FP64 G^t_j, as stage 1 stored it
-template <bool F64>
+template <int K>
 __device__ __forceinline__ double pn_G64(int64_t j) {
-  if (F64) return static_cast<const double*>(pn().Gcur)[j];
+  if (K == PK_F64) return static_cast<const double*>(pn().Gcur)[j];
   const float2 v = static_cast<const float2*>(pn().Gcur)[j];
   return (double)v.x + (double)v.y;
 }
@@ -259,24 +271,25 @@ __device__ __forceinline__ double pn_vin(int64_t j) {   // the standalone operat
   const void* v = pn().a.vin;
   return pn().a.vf32 ? (double)static_cast<const float*>(v)[j] : static_cast<const double*>(v)[j];
 }
-template <bool F64>
+template <int K>
 __device__ __forceinline__ double pn_a64(int64_t j) {
-  if (F64 && pn().a.mode == PM_GSTAR) return fabs(pn_vin(j));
-  return fabs(pn_G64<F64>(j)) * pn().a.kc.inv2l;
+  if (K == PK_F64 && pn().a.mode == PM_GSTAR) return fabs(pn_vin(j));
+  if (K == PK_PAIR64) return fabs(pn_gdbl<K>(j, 0)) * pn().a.kc.inv2l;   // (the stored pair only ranks the coordinates)
+  return fabs(pn_G64<K>(j)) * pn().a.kc.inv2l;
 }
 
 // v_j of a wide coordinate, FP64 (on FP32 data the gradient at y, whose terms
 // are FP32 pairs, in float-float)
-template <bool F64>
+template <int K>
 __device__ __forceinline__ double pn_v_wide(int64_t j, double b, double mu) {
   const PnSh& s = pn();
   const double bp = s.bprev[j];
   double gy;
   if (is_zero_bits(mu)) {
-    gy = pn_G64<F64>(j);
+    gy = pn_G64<K>(j);
   } else if (s.a.loss == 0) {
-    if (F64) {
-      gy = (1.0 + mu) * pn_G64<F64>(j) - mu * static_cast<const double*>(s.Gprev)[j];
+    if (K == PK_F64) {
+      gy = (1.0 + mu) * pn_G64<K>(j) - mu * static_cast<const double*>(s.Gprev)[j];
     } else {
       const float2 g = static_cast<const float2*>(s.Gcur)[j], gp = static_cast<const float2*>(s.Gprev)[j];
       // G + mu (G - Gprev)
@@ -287,7 +300,7 @@ __device__ __forceinline__ double pn_v_wide(int64_t j, double b, double mu) {
       gy = (double)r.hi + (double)r.lo;
     }
   } else {
-    gy = pn_gdbl(j, 1);
+    gy = pn_gdbl<K>(j, 1);
   }
   return (b + mu * (b - bp)) - s.a.step * gy;
 }
@@ -411,7 +424,7 @@ __device__ __noinline__ void pn_decide(int nx, bool do1, bool do3, uint32_t x1, 
 }
 // further rounds while a bracket holds too many entries (no prediction yet, or
 // one that was far off)
-template <bool F64>
+template <int K>
 __device__ __noinline__ int pn_more_rounds(int nx) {
   PnSh& s = pn();
   const int lane = threadIdx.x & 31;
@@ -420,8 +433,8 @@ __device__ __noinline__ int pn_more_rounds(int nx) {
     const uint32_t x1 = d1 ? cand<uint32_t>(s.lo1, s.hi1, lane) : 0u;
     const uint32_t x3 = d3 ? cand<uint32_t>(s.lo3, s.hi3, lane) : 0u;
     pn_count(d1, d3, x1, x3);
-    if (lane < XS_NSUM) s.red[(threadIdx.x >> 5) * XW_WORDS + XW_SUM + lane] = Acc<F64>().word();
-    pn_exchange<F64>(nx, XW_SUM, XW_SUM + XS_NSUM, XW_INT);
+    if (lane < XS_NSUM) s.red[(threadIdx.x >> 5) * XW_WORDS + XW_SUM + lane] = Acc<(K != PK_PAIR)>().word();
+    pn_exchange<K>(nx, XW_SUM, XW_SUM + XS_NSUM, XW_INT);
     pn_decide(nx, d1, d3, x1, x3);
     __syncthreads();
     ++nx;
@@ -475,9 +488,9 @@ __device__ __forceinline__ double pn_T(double c) {
 // is searched in FP32 arithmetic (sums float-float), then the closed form
 // taken once in FP64 and the classification checked against the exact values;
 // where it does not stand the search goes on in FP64.
-template <bool F64>
+template <int K>
 __device__ __noinline__ void pn_finish3(int nx, int n3) {
-  using A = Acc<F64>;
+  using A = Acc<(K != PK_PAIR)>;
   PnSh& s = pn();
   const int lane = threadIdx.x & 31;
   const PConst& kc = s.a.kc;
@@ -492,7 +505,7 @@ __device__ __noinline__ void pn_finish3(int nx, int n3) {
   // nothing beyond the bracket: c lies below the list's largest entry
   if (nt0 + nm0 == 0 && n3 > 0) c = fminf(c, s.f3[0] * 0.9999f);
   const double smd = sm0.val();
-  const ffs sm0f = F64 ? ff_of(smd) : ffs{__uint_as_float((unsigned)sm0.word()), __uint_as_float((unsigned)(sm0.word() >> 32))};
+  const ffs sm0f = K != PK_PAIR ? ff_of(smd) : ffs{__uint_as_float((unsigned)sm0.word()), __uint_as_float((unsigned)(sm0.word() >> 32))};
   unsigned pt = ~0u, pm = ~0u, nt = 0, nm = 0;
   ffs Sm = sm0f;
 #pragma unroll 1
@@ -540,7 +553,7 @@ __device__ __noinline__ void pn_finish3(int nx, int n3) {
       const float x = s.f3[i];
       if (x > c && !(x >= T)) v.add(__longlong_as_double((long long)s.srt3[i]));
     }
-    if (nm > nm0) warp_merge<F64>(v);
+    if (nm > nm0) warp_merge<(K != PK_PAIR)>(v);
     const bool low = key_of(c) < kc.krho;
     const double Se = smd + v.val(), kr = (double)(s.kb - (int)nt), n = (double)nm;
     const double cn = (low ? s.a.rho * Se : Se - s.a.M * kr) / (low ? kr + s.a.rho * n : n);
@@ -584,7 +597,7 @@ __device__ __noinline__ void pn_finish3(int nx, int n3) {
     }
     mt = __reduce_add_sync(0xffffffffu, mt);
     mm = __reduce_add_sync(0xffffffffu, mm);
-    warp_merge<F64>(v);
+    warp_merge<(K != PK_PAIR)>(v);
     done = pn_step3(z, (double)(nt0 + mt), (double)(nm0 + mm), smd + v.val());
   }
   if (lane == 0) {
@@ -597,15 +610,15 @@ __device__ __noinline__ void pn_finish3(int nx, int n3) {
   }
 }
 // S3 by cluster-wide classifications (ties that no bracket separates)
-template <bool F64>
+template <int K>
 __device__ __noinline__ int pn_fallback3(int nx) {
-  using A = Acc<F64>;
+  using A = Acc<(K != PK_PAIR)>;
   PnSh& s = pn();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w0 = (warp - 1) * s.a.wch, w1 = warp ? min(s.cnt, w0 + s.a.wch) : w0, nw = s.nw[warp];
   C3 z;
   z.cl = 0.0;
-  z.ch = F64 ? 1.7e308 : 3.4e38;
+  z.ch = K == PK_F64 ? 1.7e308 : 3.4e38;
   z.cc = (double)__uint_as_float(min(s.hi3, kInfKey - 1));
   z.np = z.mp = -1.0;
   z.first = true;
@@ -626,7 +639,7 @@ __device__ __noinline__ int pn_fallback3(int nx) {
         v.add(m);
       }
     }
-    nx = pn_small_sum<F64>(nx, v.word(), A().word(), nt, nm);
+    nx = pn_small_sum<K>(nx, v.word(), A().word(), nt, nm);
     const bool done = pn_step3(z, (double)s.cnt0, (double)s.cnt1, s.red_[0]);   // the same on every thread
     __syncthreads();
     if (done) break;
@@ -644,15 +657,15 @@ __device__ __noinline__ int pn_fallback3(int nx) {
 // kbar H(t*) + sum (H(|a_j|) - H(t*))_+.  On FP32 data, where FP32 cannot
 // tell the kbar-th and the next |a_j| apart, t* is their common FP32 value: an
 // upper bound of TopSum, so that Psi stays a lower bound.  (warp 0)
-template <bool F64>
+template <int K>
 __device__ __noinline__ void pn_finish1(int nx, int n1) {
-  using A = Acc<F64>;
+  using A = Acc<(K != PK_PAIR)>;
   PnSh& s = pn();
   const int lane = threadIdx.x & 31;
   const double sumH = xacc<A>(nx, 0).val();
   const int r = s.kb - (int)xcnt(nx, 2);
   double ts = r >= 1 && r <= n1 ? __longlong_as_double((long long)s.srt1[r - 1]) : 0.0;
-  if (!F64 && r >= 1 && r < n1 && (float)__longlong_as_double((long long)s.srt1[r]) == (float)ts) ts = (double)(float)ts;
+  if (K != PK_F64 && r >= 1 && r < n1 && (float)__longlong_as_double((long long)s.srt1[r]) == (float)ts) ts = (double)(float)ts;
   const double ht = huber_d<double>(ts, s.a.M);
   A v;
 #pragma unroll 1
@@ -660,7 +673,7 @@ __device__ __noinline__ void pn_finish1(int nx, int n1) {
     const double hv = huber_d<double>(__longlong_as_double((long long)s.srt1[i]), s.a.M) - ht;
     if (hv > 0.0) v.add(hv);
   }
-  warp_merge<F64>(v);
+  warp_merge<(K != PK_PAIR)>(v);
   if (lane == 0) {
     s.top = (double)r * ht + sumH + v.val();
     s.t1 = ts;
@@ -668,9 +681,9 @@ __device__ __noinline__ void pn_finish1(int nx, int n1) {
   }
 }
 // S1 by bisection over the FP64 bits of |a|
-template <bool F64>
+template <int K>
 __device__ __noinline__ int pn_fallback1(int nx) {
-  using A = Acc<F64>;
+  using A = Acc<(K != PK_PAIR)>;
   PnSh& s = pn();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w0 = (warp - 1) * s.a.wch, w1 = warp ? min(s.cnt, w0 + s.a.wch) : w0;
@@ -682,23 +695,23 @@ __device__ __noinline__ int pn_fallback1(int nx) {
     unsigned n = 0;
 #pragma unroll 1
     for (int i = w0 + lane; i < w1; i += 32)
-      if (s.fl[i] & 4) n += (unsigned long long)__double_as_longlong(pn_a64<F64>(s.cb + i)) >= mid ? 1u : 0u;
-    nx = pn_small_sum<F64>(nx, zero, zero, n, 0u);
+      if (s.fl[i] & 4) n += (unsigned long long)__double_as_longlong(pn_a64<K>(s.cb + i)) >= mid ? 1u : 0u;
+    nx = pn_small_sum<K>(nx, zero, zero, n, 0u);
     if (s.cnt0 >= (unsigned)s.kb) lo = mid;
     else hi = mid;
     __syncthreads();
   }
   double ts = __longlong_as_double((long long)lo);
-  if (!F64) ts = (double)(float)ts;   // (ties in FP32 brought the search here)
+  if (K != PK_F64) ts = (double)(float)ts;   // (ties in FP32 brought the search here)
   const double ht = huber_d<double>(ts, s.a.M);
   A v;
 #pragma unroll 1
   for (int i = w0 + lane; i < w1; i += 32)
     if (s.fl[i] & 4) {
-      const double ad = pn_a64<F64>(s.cb + i);
+      const double ad = pn_a64<K>(s.cb + i);
       if (ad > ts) v.add(huber_d<double>(ad, s.a.M) - ht);
     }
-  nx = pn_small_sum<F64>(nx, v.word(), zero, 0u, 0u);
+  nx = pn_small_sum<K>(nx, v.word(), zero, 0u, 0u);
   if (threadIdx.x == 0) {
     s.top = (double)s.kb * ht + s.red_[0];
     s.t1 = ts;
@@ -714,9 +727,9 @@ __device__ __forceinline__ void pn_list(int* n, unsigned long long* l, double x)
 }
 // Exact sums over the coordinates beyond the brackets (margins cover the FP32
 // rounding of the keys), the others into lists, to every CTA
-template <bool F64>
+template <int K>
 __device__ __noinline__ void pn_stage2(int nx, bool d1, bool d3) {
-  using A = Acc<F64>;
+  using A = Acc<(K != PK_PAIR)>;
   PnSh& s = pn();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int w0 = (warp - 1) * s.a.wch, w1 = warp ? min(s.cnt, w0 + s.a.wch) : w0, nw = s.nw[warp];
@@ -736,7 +749,7 @@ __device__ __noinline__ void pn_stage2(int nx, bool d1, bool d3) {
     if (d1) {
       const uint32_t key = s.ka[i];
       if (key >= a1) {
-        const double ad = pn_a64<F64>(s.cb + i);
+        const double ad = pn_a64<K>(s.cb + i);
         if (key >= b1) {
           ++ndef;
           v1.add(huber_d<double>(ad, s.a.M));
@@ -776,8 +789,8 @@ __device__ __noinline__ void pn_stage2(int nx, bool d1, bool d3) {
   ndef = __reduce_add_sync(0xffffffffu, ndef);
   ntop = __reduce_add_sync(0xffffffffu, ntop);
   nmid = __reduce_add_sync(0xffffffffu, nmid);
-  if (ndef) warp_merge<F64>(v1);
-  if (nmid) warp_merge<F64>(v3);
+  if (ndef) warp_merge<(K != PK_PAIR)>(v1);
+  if (nmid) warp_merge<(K != PK_PAIR)>(v3);
   if (lane == 0) {
     unsigned long long* rw = s.red + warp * XW_WORDS;
     rw[0] = v1.word();
@@ -797,7 +810,7 @@ __device__ __noinline__ void pn_stage2(int nx, bool d1, bool d3) {
     for (int r = 0; r < S; ++r) st_cluster_u64(pn_remote(dst, r), x);
   }
   if (tid == 0) s.red[4] = pack2((unsigned)s.n1, (unsigned)s.n3);
-  pn_exchange<F64>(nx, 0, 2, 5);
+  pn_exchange<K>(nx, 0, 2, 5);
 }
 
 // The lists of the cluster, flat in CTA order and then sorted (descending) by
@@ -853,14 +866,14 @@ __device__ __noinline__ unsigned long long pn_sort(int nx, bool d1, bool d3) {
 
 // Both searches to their ends once the brackets are narrow; the searches of a
 // list that overflowed go on by rounds, or without lists
-template <bool F64>
+template <int K>
 __device__ __noinline__ int pn_repair(int nx, bool d1, bool d3, bool o1, bool o3) {
   PnSh& s = pn();
   for (;;) {
     const bool again1 = d1 && o1 && s.hi1 - s.lo1 > 1, again3 = d3 && o3 && s.hi3 - s.lo3 > 1;
     __syncthreads();
-    if (d1 && !again1) nx = pn_fallback1<F64>(nx);
-    if (d3 && !again3) nx = pn_fallback3<F64>(nx);
+    if (d1 && !again1) nx = pn_fallback1<K>(nx);
+    if (d3 && !again3) nx = pn_fallback3<K>(nx);
     d1 = again1;
     d3 = again3;
     if (!d1 && !d3) return nx;
@@ -871,13 +884,13 @@ __device__ __noinline__ int pn_repair(int nx, bool d1, bool d3, bool o1, bool o3
       s.n1 = s.n3 = 0;
     }
     __syncthreads();
-    nx = pn_more_rounds<F64>(nx);
-    pn_stage2<F64>(nx, d1, d3);
+    nx = pn_more_rounds<K>(nx);
+    pn_stage2<K>(nx, d1, d3);
     const unsigned long long t = pn_sort(nx, d1, d3);
     o1 = (unsigned)t == ~0u;
     o3 = (unsigned)(t >> 32) == ~0u;
-    if (threadIdx.x < 32 && d1 && !o1) pn_finish1<F64>(nx, (int)(unsigned)t);
-    if (threadIdx.x >= 32 && threadIdx.x < 64 && d3 && !o3) pn_finish3<F64>(nx, (int)(t >> 32));
+    if (threadIdx.x < 32 && d1 && !o1) pn_finish1<K>(nx, (int)(unsigned)t);
+    if (threadIdx.x >= 32 && threadIdx.x < 64 && d3 && !o3) pn_finish3<K>(nx, (int)(t >> 32));
     __syncthreads();
     ++nx;
     d1 = d1 && (o1 || s.miss1);
@@ -890,9 +903,9 @@ __device__ __noinline__ int pn_repair(int nx, bool d1, bool d3, bool o1, bool o3
 // Newton's method on the concave sum_j min(|beta_j|, w) - kbar w from the right
 // of its root (w <= S / kbar there): w <- S_below / (kbar - N_above) decreases
 // to the root and ends when the classification stands.
-template <bool F64>
+template <int K>
 __device__ __noinline__ int pn_level(int nx) {
-  using A = Acc<F64>;
+  using A = Acc<(K != PK_PAIR)>;
   PnSh& s = pn();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w0 = (warp - 1) * s.a.wch, nw = s.nw[warp];
@@ -917,7 +930,7 @@ __device__ __noinline__ int pn_level(int nx) {
         v1.add(ab * ab);
       }
     }
-    nx = pn_small_sum<F64>(nx, v0.word(), v1.word(), na, 0u);
+    nx = pn_small_sum<K>(nx, v0.word(), v1.word(), na, 0u);
     if (threadIdx.x == 0) {
       const double Nab = (double)s.cnt0, Sbel = s.tot[XS_B] - s.red_[0];
       if ((double)s.kb - Nab <= 0.5) {   // the budget is filled by the coordinates above
@@ -939,7 +952,7 @@ __device__ __noinline__ int pn_level(int nx) {
 }
 
 // Stage 1 of this warp's coordinates again with momentum 0 (after a restart)
-template <bool F64>
+template <int K>
 __device__ __noinline__ unsigned pn_again() {
   PnSh& s = pn();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -960,7 +973,7 @@ __device__ __noinline__ unsigned pn_again() {
     const int i = s.wl[w0 + e];
     const uint8_t f8 = s.fl[i];
     if (!(f8 & 12)) continue;
-    const double v = pn_v_wide<F64>(s.cb + i, s.bcur[s.cb + i], 0.0);
+    const double v = pn_v_wide<K>(s.cb + i, s.bcur[s.cb + i], 0.0);
     s.vw[w0 + e] = v;
     s.fl[i] = (f8 & ~1) | (v < 0.0 ? 1 : 0);
     if (f8 & 4) {
@@ -1160,7 +1173,7 @@ __device__ __noinline__ void pn_prox_out(int nx, int kb, bool s3, unsigned bad) 
   }
   if (s.a.counts) {
     const unsigned long long zero = Acc<true>().word();
-    pn_small_sum<true>(nx, zero, zero, ntop, nnz);
+    pn_small_sum<PK_F64>(nx, zero, zero, ntop, nnz);
     if (s.rank == 0 && threadIdx.x == 0) {
       s.a.counts[0] = bad ? -1 : (int)s.cnt0;
       s.a.counts[1] = bad ? -1 : (int)s.cnt1;
@@ -1169,9 +1182,10 @@ __device__ __noinline__ void pn_prox_out(int nx, int kb, bool s3, unsigned bad) 
 }
 
 // ==================================================================== kernel
-template <bool F64>
-__global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const __grid_constant__ NArgs args) {
-  using A = Acc<F64>;
+template <int K>
+__global__ void __launch_bounds__(32 * PN_MAXW, K == PK_F64 ? 1 : 2) pnode_kernel(const __grid_constant__ NArgs args) {
+  using A = Acc<(K != PK_PAIR)>;
+  constexpr bool F64 = K == PK_F64;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W = blockDim.x >> 5;
   PnSh& s = pn();
   {
@@ -1321,7 +1335,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
         wide = F64 || f > 0 || !is_zero_bits(b) || !is_zero_bits(bp);
         float aa, gf;
         if constexpr (F64) {
-          const double G = pn_gdbl(j, 0);
+          const double G = pn_gdbl<K>(j, 0);
           static_cast<double*>(s.Gcur)[j] = G;
           gf = (float)G;
           const double ad = fabs(G) * kc.inv2l;
@@ -1360,13 +1374,13 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
       const int64_t j = cb + i;
       const double b = s.bcur[j];
       const uint8_t f8 = s.fl[i];
-      if (f8 & 8) sum[XS_J1H].add(huber_d<double>(pn_a64<F64>(j), s.a.M));
+      if (f8 & 8) sum[XS_J1H].add(huber_d<double>(pn_a64<K>(j), s.a.M));
       if (!iter) s.vw[w0 + e] = b;
       if (!is_zero_bits(b)) {
         const double ab = fabs(b);
         A a1, a2;   // |b| and b^2 (FP32 data: as pairs, one conversion for both)
         bool above;
-        if constexpr (F64) {
+        if constexpr (K != PK_PAIR) {
           a1.s = ab;
           a2.s = ab * ab;
           above = w_known && ab > w_closed;
@@ -1396,7 +1410,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
         }
       }
       if (iter && (f8 & 12)) {
-        const double v = pn_v_wide<F64>(j, b, mu);
+        const double v = pn_v_wide<K>(j, b, mu);
         s.vw[w0 + e] = v;
         if (__double_as_longlong(v) < 0) s.fl[i] = f8 | 1;
         if (f8 & 4) {
@@ -1437,7 +1451,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
   }
   cluster_wait();   // every CTA of the cluster runs
   int nx = 0;
-  pn_exchange<F64>(nx, XW_SUM, XW_SUM + XS_NSUM, XW_WORDS);
+  pn_exchange<K>(nx, XW_SUM, XW_SUM + XS_NSUM, XW_WORDS);
   // S3 has a threshold to find when more coordinates of v are nonzero than the
   // budget holds
   const unsigned long long bz = xcnt(nx, XW_INT + 1);
@@ -1472,14 +1486,14 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
   pn_decide(nx, s1, s3, x1, x3);
   __syncthreads();
   ++nx;
-  if (s.more1 || s.more3) nx = pn_more_rounds<F64>(nx);
+  if (s.more1 || s.more3) nx = pn_more_rounds<K>(nx);
 
   const bool need_b = iter || mode == PM_EVAL || mode == PM_GVAL;
   const bool check_dom = !iter || t == 0;
   const bool g_inf = check_dom && (s.dom > 0 || (kb > 0 && s.tot[XS_B] > s.a.M * (double)kb * (1.0 + 1e-6)) ||
                                    (kb <= 0 && s.tot[XS_B] > 0.0));
   const bool level = need_b && !g_inf && kb > 0 && s.nnz > (unsigned)kb;   // a water level to find
-  if (level && !w_known) nx = pn_level<F64>(nx);
+  if (level && !w_known) nx = pn_level<K>(nx);
   // g, and FISTA's next t_k and momentum should this iteration not restart:
   // by warps that have nothing else to do while the searches end
   auto g_closed = [&]() {   // one lane
@@ -1503,25 +1517,25 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
   // ------------------------------------------------------ stage 2, exchange 2
   bool o1 = false, o3 = false;
   if (s1 || s3) {
-    pn_stage2<F64>(nx, s1, s3);
+    pn_stage2<K>(nx, s1, s3);
     const unsigned long long n = pn_sort(nx, s1, s3);
     o1 = s1 && (unsigned)n == ~0u;
     o3 = s3 && (unsigned)(n >> 32) == ~0u;
-    if (warp == 0 && s1 && !o1) pn_finish1<F64>(nx, (int)(unsigned)n);
-    if (warp == 1 && s3 && !o3) pn_finish3<F64>(nx, (int)(n >> 32));
+    if (warp == 0 && s1 && !o1) pn_finish1<K>(nx, (int)(unsigned)n);
+    if (warp == 1 && s3 && !o3) pn_finish3<K>(nx, (int)(n >> 32));
   }
   if (warp == 2 && lane == 0) g_closed();
   if (warp == 3 && lane == 0) next_tau();
   __syncthreads();
   ++nx;
   if ((s1 && (o1 || s.miss1)) || (s3 && (o3 || s.miss3)))
-    nx = pn_repair<F64>(nx, s1 && (o1 || s.miss1), s3 && (o3 || s.miss3), o1, o3);
+    nx = pn_repair<K>(nx, s1 && (o1 || s.miss1), s3 && (o3 || s.miss3), o1, o3);
   if (kb > 0 && s.pb <= kb && mode != PM_PROX && mode != PM_GVAL) {   // a slack budget: the whole free set (at most kbar coordinates)
     A v;
 #pragma unroll 1
     for (int i = w0 + lane; i < w1; i += 32)
-      if (s.fl[i] & 4) v.add(huber_d<double>(pn_a64<F64>(cb + i), s.a.M));
-    nx = pn_small_sum<F64>(nx, v.word(), A().word(), 0u, 0u);
+      if (s.fl[i] & 4) v.add(huber_d<double>(pn_a64<K>(cb + i), s.a.M));
+    nx = pn_small_sum<K>(nx, v.word(), A().word(), 0u, 0u);
     if (tid == 0) {
       s.top = s.red_[0];
       s.t1 = 0.0;
@@ -1588,7 +1602,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
   const bool stop = flags & 1, restart = (flags & 8) != 0 && !stop;
   if (restart && !is_zero_bits(mu)) {
     unsigned nz = 0;
-    if (warp) nz = pn_again<F64>();
+    if (warp) nz = pn_again<K>();
     if (tid == 0) {
       s.lo3 = 0;
       s.hi3 = kInfKey;
@@ -1604,7 +1618,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
       if (lane < XS_NSUM) rw[XW_SUM + lane] = A().word();
       if (lane < 3) rw[XW_INT + lane] = lane == 1 ? pack2(0u, nz) : 0ull;
     }
-    pn_exchange<F64>(nx, XW_SUM, XW_SUM + XS_NSUM, XW_WORDS);
+    pn_exchange<K>(nx, XW_SUM, XW_SUM + XS_NSUM, XW_WORDS);
     const unsigned nzv2 = (unsigned)(xcnt(nx, XW_INT + 1) >> 32);
     s3 = can3 && (int)nzv2 > kb;
     if (tid == 0 && s3) s.cmlo = s.ctlo = nzv2;
@@ -1613,14 +1627,14 @@ __global__ void __launch_bounds__(32 * PN_MAXW, F64 ? 1 : 2) pnode_kernel(const 
     __syncthreads();
     ++nx;
     if (s3) {
-      if (s.more3) nx = pn_more_rounds<F64>(nx);
-      pn_stage2<F64>(nx, false, true);
+      if (s.more3) nx = pn_more_rounds<K>(nx);
+      pn_stage2<K>(nx, false, true);
       const unsigned long long n = pn_sort(nx, false, true);
       o3 = (unsigned)(n >> 32) == ~0u;
-      if (warp == 1 && !o3) pn_finish3<F64>(nx, (int)(n >> 32));
+      if (warp == 1 && !o3) pn_finish3<K>(nx, (int)(n >> 32));
       __syncthreads();
       ++nx;
-      if (o3 || s.miss3) nx = pn_repair<F64>(nx, false, true, false, o3);
+      if (o3 || s.miss3) nx = pn_repair<K>(nx, false, true, false, o3);
     }
     if (warp) write_next();
   }
@@ -1754,16 +1768,17 @@ cudaLaunchConfig_t config(const NPlan& pl, int nprob, cudaLaunchAttribute* attr,
 // problem where the sizes allow (256 problems of p = 10000, whole call: 1 / 2 /
 // 4 / 8 CTAs 62.8 / 63.1 / 60.7 / 63.7 ms; 48 of p = 5000: 2 / 4 / 8 CTAs 7.59 /
 // 6.97 / 7.62 ms).  A CTA's coordinates must fit its shared memory either way.
-cudaError_t pnode_plan(NPlan& pl, bool f64, int64_t p, int nprob) {
+cudaError_t pnode_plan(NPlan& pl, int kind, int64_t p, int nprob) {
   pl = NPlan{};
-  pl.f64 = f64;
-  pl.kernel = f64 ? reinterpret_cast<const void*>(&pnode_kernel<true>) : reinterpret_cast<const void*>(&pnode_kernel<false>);
+  pl.kernel = kind == PK_F64      ? reinterpret_cast<const void*>(&pnode_kernel<PK_F64>)
+              : kind == PK_PAIR64 ? reinterpret_cast<const void*>(&pnode_kernel<PK_PAIR64>)
+                                  : reinterpret_cast<const void*>(&pnode_kernel<PK_PAIR>);
   if (p < 1 || nprob < 1) return cudaErrorInvalidValue;
   int dev = 0, nsm = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const int64_t target = f64 ? 64 : 224;
+  const int64_t target = kind == PK_F64 ? 64 : 224;
   int share = 4;
   while (share < PN_MAXCL && 2 * share * nprob <= 2 * nsm) share *= 2;
   const int64_t want = std::min<int64_t>((p + target - 1) / target, share);

@@ -43,6 +43,10 @@
 
 namespace relax {
 
+// the kernel's instantiations: FP32 data with float-float sums (the loop), FP64,
+// FP32 data with FP64 sums (the certificate)
+enum PNKind : int { PK_PAIR = 0, PK_F64 = 1, PK_PAIR64 = 2 };
+
 constexpr int PN_MAXW = 16;          // warps per CTA at most (warp 0 takes the decisions, the others coordinates)
 constexpr int PN_MAXCL = 16;         // CTAs per cluster at most (16: a non-portable size)
 constexpr int PN_CAP = 256;          // bracket entries finished in place, per search
