@@ -690,12 +690,16 @@ __device__ __noinline__ int pn_fallback1(int nx) {
   unsigned long long lo = s.lo1 > 4 ? (unsigned long long)__double_as_longlong((double)__uint_as_float(s.lo1 - 4)) : 0ull;
   unsigned long long hi = (unsigned long long)__double_as_longlong((double)__uint_as_float(min(s.hi1 + 4, kInfKey))) + 1;
   const unsigned long long zero = A().word();
+  // (the certificate of FP32 data ranks by the stored pairs: t* may be any value
+  // near the kbar-th, and near an optimum, where the pooled block ties, the
+  // search comes here often)
+  auto rank = [&](int64_t j) { return K == PK_PAIR64 ? fabs(pn_G64<K>(j)) * s.a.kc.inv2l : pn_a64<K>(j); };
   while (hi - lo > 1) {
     const unsigned long long mid = lo + (hi - lo) / 2;
     unsigned n = 0;
 #pragma unroll 1
     for (int i = w0 + lane; i < w1; i += 32)
-      if (s.fl[i] & 4) n += (unsigned long long)__double_as_longlong(pn_a64<K>(s.cb + i)) >= mid ? 1u : 0u;
+      if (s.fl[i] & 4) n += (unsigned long long)__double_as_longlong(rank(s.cb + i)) >= mid ? 1u : 0u;
     nx = pn_small_sum<K>(nx, zero, zero, n, 0u);
     if (s.cnt0 >= (unsigned)s.kb) lo = mid;
     else hi = mid;
@@ -707,7 +711,7 @@ __device__ __noinline__ int pn_fallback1(int nx) {
   A v;
 #pragma unroll 1
   for (int i = w0 + lane; i < w1; i += 32)
-    if (s.fl[i] & 4) {
+    if ((s.fl[i] & 4) && rank(s.cb + i) > ts * (1.0 - 0x1p-40)) {
       const double ad = pn_a64<K>(s.cb + i);
       if (ad > ts) v.add(huber_d<double>(ad, s.a.M) - ht);
     }
