@@ -1575,14 +1575,14 @@ relax_status relax_certify(relax_handle* h, const int8_t* fixings, const void* b
 // leave FP32's range (a pair of FP32 sums gave NaN above 1.8e19 and 0 below
 // 1e-23).  p = 1000 FP32, prox, g and g*: 210 us on the grid (seven or more grid
 // barriers each, a scratch area zeroed per call), 131 on a cluster with pairs,
-// 140 with FP64 sums.
+// 137 with FP64 sums (140 with FP64 throughout); p = 102400, prox: 107, 111 (125).
 static relax_status standalone(int mode, const void* vin, void* vout, int64_t p, double rho, int32_t k,
                                double lambda2, double M, const int8_t* fix, int32_t dtype, int32_t* counts,
                                double* out_host, cudaStream_t st) {
   if (!vin || p <= 0 || k < 0 || !(M > 0.0) || (dtype != RELAX_F64 && dtype != RELAX_F32)) return RELAX_EINVAL;
   const bool dbl = dtype == RELAX_F64;
   NPlan np;
-  const bool cluster = pnode_plan(np, PK_F64, p, 1) == cudaSuccess;
+  const bool cluster = pnode_plan(np, dbl ? PK_F64 : PK_PAIR64, p, 1) == cudaSuccess;
   PPlan pl;
   if (!cluster) {
     (void)cudaGetLastError();
@@ -1609,7 +1609,6 @@ static relax_status standalone(int mode, const void* vin, void* vout, int64_t p,
     a.rho = rho;
     a.kc = pconst_make(lambda2, M, 0.0, rho);
     a.fix = fix;
-    a.vf32 = dbl ? 0 : 1;
     a.vin = vin;
     a.vout = vout;
     a.counts = counts;

@@ -267,13 +267,14 @@ __device__ __forceinline__ double pn_G64(int64_t j) {
   const float2 v = static_cast<const float2*>(pn().Gcur)[j];
   return (double)v.x + (double)v.y;
 }
+template <int K>
 __device__ __forceinline__ double pn_vin(int64_t j) {   // the standalone operations' input
   const void* v = pn().a.vin;
-  return pn().a.vf32 ? (double)static_cast<const float*>(v)[j] : static_cast<const double*>(v)[j];
+  return K == PK_F64 ? static_cast<const double*>(v)[j] : (double)static_cast<const float*>(v)[j];
 }
 template <int K>
 __device__ __forceinline__ double pn_a64(int64_t j) {
-  if (K == PK_F64 && pn().a.mode == PM_GSTAR) return fabs(pn_vin(j));
+  if (K != PK_PAIR && pn().a.mode == PM_GSTAR) return fabs(pn_vin<K>(j));
   if (K == PK_PAIR64) return fabs(pn_gdbl<K>(j, 0)) * pn().a.kc.inv2l;   // (the stored pair only ranks the coordinates)
   return fabs(pn_G64<K>(j)) * pn().a.kc.inv2l;
 }
@@ -618,7 +619,7 @@ __device__ __noinline__ int pn_fallback3(int nx) {
   const int w0 = (warp - 1) * s.a.wch, w1 = warp ? min(s.cnt, w0 + s.a.wch) : w0, nw = s.nw[warp];
   C3 z;
   z.cl = 0.0;
-  z.ch = K == PK_F64 ? 1.7e308 : 3.4e38;
+  z.ch = K == PK_F64 ? DBL_MAX : (double)FLT_MAX;
   z.cc = (double)__uint_as_float(min(s.hi3, kInfKey - 1));
   z.np = z.mp = -1.0;
   z.first = true;
@@ -693,7 +694,7 @@ __device__ __noinline__ int pn_fallback1(int nx) {
   // (the certificate of FP32 data ranks by the stored pairs: t* may be any value
   // near the kbar-th, and near an optimum, where the pooled block ties, the
   // search comes here often)
-  auto rank = [&](int64_t j) { return K == PK_PAIR64 ? fabs(pn_G64<K>(j)) * s.a.kc.inv2l : pn_a64<K>(j); };
+  auto rank = [&](int64_t j) { return K == PK_PAIR64 && s.a.mode == PM_EVAL ? fabs(pn_G64<K>(j)) * s.a.kc.inv2l : pn_a64<K>(j); };
   while (hi - lo > 1) {
     const unsigned long long mid = lo + (hi - lo) / 2;
     unsigned n = 0;
@@ -1075,6 +1076,7 @@ __device__ __noinline__ void pn_decisions() {
 }
 
 // Stage 1 of the standalone operations over this warp's coordinates
+template <int K>
 __device__ __noinline__ void pn_load(Acc<true> (&sum)[XS_NSUM], unsigned& nnz, unsigned& dom, unsigned& bad, unsigned& nzv,
                                      unsigned& j1, unsigned& jf) {
   PnSh& s = pn();
@@ -1092,7 +1094,7 @@ __device__ __noinline__ void pn_load(Acc<true> (&sum)[XS_NSUM], unsigned& nnz, u
     if (i < w1) {
       const int64_t j = s.cb + i;
       const int8_t f = s.fix ? s.fix[j] : (int8_t)0;
-      x = pn_vin(j);
+      x = pn_vin<K>(j);
       f8 = f == 0 ? 4 : f > 0 ? 8 : 0;
       j1 += f > 0;
       jf += f == 0;
@@ -1108,7 +1110,7 @@ __device__ __noinline__ void pn_load(Acc<true> (&sum)[XS_NSUM], unsigned& nnz, u
           else sum[XS_J1H].add(huber_d<double>(fabs(x), s.a.M));
         }
       } else if (mode == PM_PROX) {
-        wide = f >= 0;
+        wide = K == PK_F64 ? f >= 0 : f > 0;   // (an FP32 |v_j| is exact in its FP32 word)
         if (__double_as_longlong(x) < 0) f8 |= 1;
         if (f == 0) {
           m = ax;
@@ -1146,25 +1148,27 @@ __device__ __noinline__ void pn_load(Acc<true> (&sum)[XS_NSUM], unsigned& nnz, u
 
 // The standalone prox's output and counts.  A non-finite input poisons them:
 // beta all NaN, counts -1.
+template <int K>
 __device__ __noinline__ void pn_prox_out(int nx, int kb, bool s3, unsigned bad) {
   PnSh& s = pn();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w0 = (warp - 1) * s.a.wch, w1 = warp ? min(s.cnt, w0 + s.a.wch) : w0, nw = s.nw[warp];
   const double c = kb <= 0 ? INFINITY : s3 ? s.c : 0.0, T = pn_T(c), inv1r = s.a.kc.inv1r, M = s.a.M;
+  const float ccd = kb <= 0 ? INFINITY : s3 ? s.ccd : 0.f;   // an FP32 m exceeds c iff it exceeds c rounded down
   unsigned ntop = 0, nnz = 0;
 #pragma unroll 1
   for (int u = lane; u < (w1 - w0) + nw; u += 32) {
-    // the coordinates fixed out, then the others from the list
-    const bool out = u < w1 - w0;
-    const int e = w0 + u - (out ? 0 : w1 - w0);
-    const int i = out ? e : s.wl[e];
+    // the coordinates with FP32 words (FP64: those fixed out), then the others from the list
+    const bool narrow = u < w1 - w0;
+    const int e = w0 + u - (narrow ? 0 : w1 - w0);
+    const int i = narrow ? e : s.wl[e];
     const uint8_t f8 = s.fl[i];
-    if (out && (f8 & 2)) continue;
+    if (narrow && (f8 & 2)) continue;
     double b = 0.0;
     if (bad) b = __longlong_as_double(0x7ff8000000000000ll);
     else if (f8 & 8) b = fmin(fmax(s.vw[e] * inv1r, -M), M);
-    else if (f8 & 4) {
-      const double m = fabs(s.vw[e]);
+    else if ((f8 & 4) && (!narrow || s.mv[i] > ccd)) {
+      const double m = narrow ? (double)s.mv[i] : fabs(s.vw[e]);
       const double r = fmax(0.0, fmin(fmin(m - c, m * inv1r), M));
       if (r > 0.0) {
         ++nnz;
@@ -1172,12 +1176,12 @@ __device__ __noinline__ void pn_prox_out(int nx, int kb, bool s3, unsigned bad) 
         b = (f8 & 1) ? -r : r;
       }
     }
-    if (s.a.vf32) static_cast<float*>(s.a.vout)[s.cb + i] = (float)b;
-    else static_cast<double*>(s.a.vout)[s.cb + i] = b;
+    if (K == PK_F64) static_cast<double*>(s.a.vout)[s.cb + i] = b;
+    else static_cast<float*>(s.a.vout)[s.cb + i] = (float)b;
   }
   if (s.a.counts) {
     const unsigned long long zero = Acc<true>().word();
-    pn_small_sum<PK_F64>(nx, zero, zero, ntop, nnz);
+    pn_small_sum<K>(nx, zero, zero, ntop, nnz);
     if (s.rank == 0 && threadIdx.x == 0) {
       s.a.counts[0] = bad ? -1 : (int)s.cnt0;
       s.a.counts[1] = bad ? -1 : (int)s.cnt1;
@@ -1282,7 +1286,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, K == PK_F64 ? 1 : 2) pnode_kerne
     }
   }
   const int mode = s.a.mode;
-  const bool iter = mode == PM_ITER, alone = F64 && mode >= PM_PROX;
+  const bool iter = mode == PM_ITER, alone = K != PK_PAIR && mode >= PM_PROX;
   const int64_t cb = s.cb;
   const int wch = s.a.wch, w0 = (warp - 1) * wch, w1 = warp ? min(s.cnt, w0 + wch) : w0;
   const PConst& kc = s.a.kc;
@@ -1298,8 +1302,8 @@ __global__ void __launch_bounds__(32 * PN_MAXW, K == PK_F64 ? 1 : 2) pnode_kerne
   A sum[XS_NSUM];
   unsigned c_nnz = 0, c_dom = 0, c_bad = 0, c_nab = 0, c_nzv = 0, c_j1 = 0, c_jf = 0;
   if (alone) {
-    if constexpr (F64)
-      if (warp) pn_load(sum, c_nnz, c_dom, c_bad, c_nzv, c_j1, c_jf);
+    if constexpr (K != PK_PAIR)
+      if (warp) pn_load<K>(sum, c_nnz, c_dom, c_bad, c_nzv, c_j1, c_jf);
   } else if (warp == 0) {   // the loss sums of the pass, in FP64
     const double* ls = s.a.lsum + (size_t)(iter ? s.prob : s.item) * s.a.lsum_stride;
     double f = 0.0, d = 0.0;
@@ -1551,7 +1555,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, K == PK_F64 ? 1 : 2) pnode_kerne
 
   // ---------------------------------------------------------------------- D
   if (!iter) {
-    if (alone && mode == PM_PROX) pn_prox_out(nx, kb, s3, bad);
+    if (alone && mode == PM_PROX) pn_prox_out<K>(nx, kb, s3, bad);
     else if (tid == 0) pn_decisions();
     return;   // (every push to this CTA has been received: no exchange follows)
   }
@@ -1766,7 +1770,7 @@ cudaLaunchConfig_t config(const NPlan& pl, int nprob, cudaLaunchAttribute* attr,
 
 // Cluster size.  One problem: latency counts, so a CTA gets few coordinates
 // (the FP64 pipe is the narrowest: 64 per CTA where all of them take FP64,
-// else 224, one per lane), on up to 16 CTAs (measured at 1000 x 1000 FP32:
+// else 224, one per lane), on up to 16 CTAs (measured when the kernel came in, at 1000 x 1000 FP32:
 // 1 / 2 / 4 / 8 / 16 CTAs 50 / 41 / 38 / 31 / 34 us; p = 20000: 4 / 8 / 16 CTAs
 // 110 / 76 / 59 us).  Many problems: about two CTAs per SM, but four per
 // problem where the sizes allow (256 problems of p = 10000, whole call: 1 / 2 /

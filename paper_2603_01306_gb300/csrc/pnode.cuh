@@ -22,21 +22,22 @@
 // latency is one way; sums run over the CTAs in rank order (deterministic).
 //
 // FP64 arithmetic, comparisons and conversions issue at about 1.6 lanes per
-// clock per SM here (FP32: about 112), so on FP32 data (F64 = false) the
+// clock per SM here (FP32: about 112), so on FP32 data (PK_PAIR) the
 // coordinates with beta^t_j = beta^{t-1}_j = 0 that are not fixed in take FP32
 // arithmetic only, gradients travel as FP32 pairs (hi + lo) and sums are
 // float-float; the others ("wide") are collected per warp and take FP64 with
 // full warps.  (A dependent FP64 operation takes 64 cycles here, a division
 // about 580: thread 0 decides while the other warps write the next point.)
-// F64 = true (FP64 data, the last rungs of the precision ladder, and the
-// standalone operations of either type): every coordinate is wide and sums are
-// FP64.
+// PK_F64 (FP64 data, the last rungs of the precision ladder): every coordinate is
+// wide and sums are FP64.  PK_PAIR64 (FP32 data: the certificate, the standalone
+// operations): FP32 per coordinate, FP64 sums.
 //
 // Measured per iteration, against the cooperative grid of pphase.cuh that ran
 // before (seven or more grid barriers): p = 1000 45 -> 29 us, p = 4000
-// (logistic) 53 -> 38 us, p = 20000 81 -> 59 us, p = 50000 85 -> 70 us, FP64 p =
-// 1000 66 -> 30 us; whole calls: 256 nodes of 5000 x 10000 110 -> 61 ms (with
-// the certificates evaluated together), 48 of 2000 x 5000 14.5 -> 7.0 ms.
+// (logistic) 53 -> 39 us, p = 20000 81 -> 44 us, p = 50000 85 -> 58 us (47 over a
+// solve of 577 iterations), FP64 p = 1000 66 -> 32 us; whole calls at this step:
+// 256 nodes of 5000 x 10000 110 -> 61 ms (with the certificates evaluated
+// together), 48 of 2000 x 5000 14.5 -> 7.0 ms.
 #pragma once
 #include "bgemm.cuh"
 #include "pphase.cuh"
@@ -44,7 +45,7 @@
 namespace relax {
 
 // the kernel's instantiations: FP32 data with float-float sums (the loop), FP64,
-// FP32 data with FP64 sums (the certificate)
+// FP32 data with FP64 sums (the certificate, the standalone operations)
 enum PNKind : int { PK_PAIR = 0, PK_F64 = 1, PK_PAIR64 = 2 };
 
 constexpr int PN_MAXW = 16;          // warps per CTA at most (warp 0 takes the decisions, the others coordinates)
@@ -95,9 +96,8 @@ struct NArgs {
   const int* cnt;               // [items][3] fixing counts {|J1|, |Jf|, .}; NULL: root
   double* out;                  // item's values at out_stride item + 2 (s % nq); PM_GVAL, PM_GSTAR: one value
   int64_t out_stride;
-  // the standalone operations, one problem, F64 kernel: sums and products of
-  // FP32 vectors (vf32) need FP64's range and precision too
-  int vf32;
+  // the standalone operations, one problem, FP64 vectors (PK_F64) or FP32 ones
+  // (PK_PAIR64: their sums and products need FP64's range and precision too)
   const void* vin;              // PM_PROX: v, PM_GVAL: beta, PM_GSTAR: alpha
   void* vout;                   // PM_PROX
   int* counts;                  // PM_PROX: {n_top, n_nz} or NULL

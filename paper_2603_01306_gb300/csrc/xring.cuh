@@ -15,8 +15,8 @@
 // took 33.4 ms with one word, 35.6 with two in two instructions, 33.3 so.
 //
 // FP32: bound by how much of X the rings hold (32 MB) against the round trip
-// from HBM to the end of a block's agreement.  20000 x 50000: 862 us on
-// xstrip.cuh's kernel, which sent X through L2 twice, 718 now (5.57 TB/s).
+// from HBM to the end of a block's agreement.  20000 x 50000: 852 us on
+// xstrip.cuh's kernel, which sent X through L2 twice, 718 to 723 now (5.55 TB/s).
 // Eight rows per dot warp: its butterfly takes 9 exchanges of pairs instead of 12
 // for two times four (776 us; two rows 1204).  5 + 4 dot and link warps; 6 + 3
 // 725, 5 + 3 722, 6 + 4 740, 7 + 2 740, and with four rows 4 + 5 776, 6 + 5 741,

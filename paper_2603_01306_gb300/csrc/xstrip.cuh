@@ -77,7 +77,8 @@ struct XSArgs {
   const float* colscale; // FP8 storage (xmma.cuh): the columns' scales
   int keep;              // single-crossing passes: X stays in L2 from pass to pass
   PassState* ps;
-  unsigned long long* zfix;   // [NF][n] z in fixed point (two's complement)   } zeroed
+  unsigned long long* zfix;   // [NF][n] z in fixed point (two's complement;   } zeroed
+                              // one-ring passes: [n][2] words with counts)
   unsigned long long* zmax;   // [NF] max_j |beta_j| (bits of a nonnegative double) } before
   unsigned* zcnt;             // CTAs that have added to zmax                   } the launch
   double rowl1;               // max_i ||x_i||_1 of the stored X (NaN when X holds a NaN)
