@@ -6,6 +6,10 @@
 // Allocation and release are ordered on the caller's stream, so the pool
 // serves several threads and streams; it holds at most kKeep bytes beyond what
 // is in use and gives them back when a handle is closed.
+//
+// On a stream that is being captured the allocation becomes a node whose memory
+// the graph owns, so it is left to the default pool (making a pool there would
+// also invalidate the capture).
 #include <mutex>
 
 #include "common.cuh"
@@ -24,6 +28,9 @@ cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t st) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing != cudaStreamCaptureStatusNone)
+    return cudaMallocAsync(p, bytes, st);
   cudaMemPool_t pool = nullptr;
   {
     std::lock_guard<std::mutex> lock(g_mu);
