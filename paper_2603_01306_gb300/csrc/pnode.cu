@@ -448,9 +448,17 @@ __device__ __noinline__ int pn_more_rounds(int nx) {
 // in between, the sum of the latter): the closed form on the piece, the
 // bracket [cl, ch] tightened by the sign at cc; true when it stands
 struct C3 {
-  double cc, cl, ch, np, mp;
-  bool first;
+  double cc, cl, ch;
+  int n;
 };
+// A root at the end of a flat stretch of the sum is moved onto it: all `nm`
+// coordinates in between at z = 1 (kr of them wanted), or all at z = 0.  Any
+// point of the stretch is a root; on it n_top and n_nz count as Algorithm 2's block does.
+__device__ __forceinline__ double pn_flat(double c, double kr, double nm, double sm) {
+  if (nm == 0.0) return c;
+  if (kr == nm) return c - fmin(0x1p-50 * (sm / nm), 0x1p-10 * c);
+  return kr == 0.0 ? c * (1.0 + 0x1p-50) : c;
+}
 __device__ __noinline__ bool pn_step3(C3& z, double Nt, double Nm, double Sm) {
   const PnSh& s = pn();
   const double rho = s.a.rho, rhoM = s.a.kc.rhoM, M = s.a.M;
@@ -464,20 +472,19 @@ __device__ __noinline__ bool pn_step3(C3& z, double Nt, double Nm, double Sm) {
   // Ntop == kbar, none when not
   const bool none = Nm == 0.0 && kr != 0.0;
   double cn = none ? -1.0 : Nm == 0.0 ? z.cc : num / den;
-  const bool stable = !none && !z.first && Nt == z.np && Nm == z.mp;
-  z.first = false;
-  z.np = Nt;
-  z.mp = Nm;
-  // the piece's root is the answer only where it lies on the piece (a search
-  // that began on the wrong side can meet one piece twice on its way)
-  if (stable && fabs(cn - z.cc) <= 0x1p-40 * z.cc) {
-    z.cc = cn;
+  // a root that reproduces the point it was formed at lies on its piece
+  if (fabs(cn - z.cc) <= 0x1p-50 * z.cc) {
+    z.cc = pn_flat(cn, kr, Nm, Sm);
     return true;
   }
-  if (!(cn >= z.cl && cn <= z.ch) || !(cn > 0.0)) {
+  // else on to it, where it narrows the bracket (the sum bends both ways, and the
+  // roots of two pieces can name each other: the end of the bracket is no
+  // progress, and every fourth step bisects)
+  if (!(cn > z.cl && cn < z.ch) || (z.n & 3) == 3) {
     cn = z.cl > 0.0 ? sqrt(z.cl) * sqrt(z.ch) : z.ch * 0x1p-20;
     if (!(cn > z.cl && cn < z.ch)) return true;   // the bracket is one value
   }
+  ++z.n;
   z.cc = cn;
   return false;
 }
@@ -508,6 +515,7 @@ __device__ __noinline__ void pn_finish3(int nx, int n3) {
   const double smd = sm0.val();
   const ffs sm0f = K != PK_PAIR ? ff_of(smd) : ffs{__uint_as_float((unsigned)sm0.word()), __uint_as_float((unsigned)(sm0.word() >> 32))};
   unsigned pt = ~0u, pm = ~0u, nt = 0, nm = 0;
+  bool settled = false;
   ffs Sm = sm0f;
 #pragma unroll 1
   for (int it = 0; it < 32; ++it) {
@@ -525,7 +533,10 @@ __device__ __noinline__ void pn_finish3(int nx, int n3) {
     }
     nt = nt0 + __reduce_add_sync(0xffffffffu, nt);
     nm = nm0 + __reduce_add_sync(0xffffffffu, nm);
-    if (nt == pt && nm == pm && nm > 0) break;
+    if (nt == pt && nm == pm && (nm > 0 || nt == (unsigned)s.kb)) {   // (c is the one that these counts belong to)
+      settled = true;
+      break;
+    }
     pt = nt;
     pm = nm;
     warp_merge<false>(v);
@@ -546,7 +557,7 @@ __device__ __noinline__ void pn_finish3(int nx, int n3) {
   C3 z;
   z.cc = (double)c;
   bool done = false;
-  if (nm > 0) {
+  if (settled && nm > 0) {
     A v;
     const float T = key_of(c) < kc.krho ? c * kc.kTc_f : c + kc.M;
 #pragma unroll 1
@@ -572,13 +583,12 @@ __device__ __noinline__ void pn_finish3(int nx, int n3) {
     const float cf = (float)cn;
     // (positive and finite; on the side of rho M that the form assumed)
     done = mt == nt && mm == nm && cf > 0.f && cf < 3e38f && (low ? key_of(cf) < kc.krho : key_of(cf) > kc.krho);
-    z.cc = cn;
+    z.cc = pn_flat(cn, kr, n, Se);
   }
   if (!done) {   // search on in FP64
     z.cl = (double)__uint_as_float(lok);
     z.ch = (double)__uint_as_float(hik);
-    z.np = z.mp = -1.0;
-    z.first = true;
+    z.n = 0;
     z.cc = (double)c;
   }
 #pragma unroll 1
@@ -621,8 +631,7 @@ __device__ __noinline__ int pn_fallback3(int nx) {
   z.cl = 0.0;
   z.ch = K == PK_F64 ? DBL_MAX : (double)FLT_MAX;
   z.cc = (double)__uint_as_float(min(s.hi3, kInfKey - 1));
-  z.np = z.mp = -1.0;
-  z.first = true;
+  z.n = 0;
 #pragma unroll 1
   for (int it = 0; it < 200; ++it) {
     const double T = pn_T(z.cc);
