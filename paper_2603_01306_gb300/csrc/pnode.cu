@@ -916,7 +916,8 @@ __device__ __noinline__ int pn_repair(int nx, bool d1, bool d3, bool o1, bool o3
 // --------------------------------------------------------------- g(beta), S2
 // Newton's method on the concave sum_j min(|beta_j|, w) - kbar w from the right
 // of its root (w <= S / kbar there): w <- S_below / (kbar - N_above) decreases
-// to the root and ends when the classification stands.
+// to the root and ends when the classification stands, or w does not fall any
+// more (values equal to the level to rounding can fall on either side of it in turn).
 template <int K>
 __device__ __noinline__ int pn_level(int nx) {
   using A = Acc<(K != PK_PAIR)>;
@@ -952,7 +953,7 @@ __device__ __noinline__ int pn_level(int nx) {
         s.go = 0;
       } else {
         const double wn = Sbel / ((double)s.kb - Nab);
-        if (s.mu == Nab) {
+        if (s.mu == Nab || !(wn < s.w)) {
           s.g = 0.5 * (s.tot[XS_J1B2] + s.red_[1] + wn * Sbel);
           s.go = 0;
         }
