@@ -232,32 +232,31 @@ __device__ __forceinline__ ffs pn_gpair(int64_t j, int q) {
   }
   return ff_add(v, u);
 }
-__device__ __noinline__ float2 pn_gpair_call(int64_t j, int q) {
-  const ffs v = pn_gpair(j, q);
-  return make_float2(v.hi, v.lo);
-}
-// the same in FP64 (sums of pairs too, but in the loop on FP32 data)
+// the same in FP64 (sums of pairs too, but in the loop on FP32 data).  Inlined:
+// lanes call it on their own, and as a function of its own with an unrolled
+// loop it came out wrong (by whole partials) for lanes that a branch had split
+// from their warp.
 template <int K>
-__device__ __noinline__ double pn_gdbl(int64_t j, int q) {
+__device__ __forceinline__ double pn_gdbl(int64_t j, int q) {
   const PnSh& s = pn();
   if (K == PK_PAIR) {
-    const float2 v = pn_gpair_call(j, q);
-    return (double)v.x + (double)v.y;
+    const ffs v = pn_gpair(j, q);
+    return (double)v.hi + (double)v.lo;
   }
-  if (s.a.gpair) {
+  const size_t stride = (size_t)s.a.NB * s.a.p;
+  double v = 0.0;
+  if (K == PK_PAIR64 || s.a.gpair) {
     const float2* src = static_cast<const float2*>(s.part) + (size_t)q * s.a.p + j;
-    double v = 0.0;
-#pragma unroll 8
+#pragma unroll 4
     for (int c = 0; c < s.a.ncl; ++c) {
-      const float2 y = __ldcg(src + (size_t)c * s.a.NB * s.a.p);
+      const float2 y = __ldcg(src + c * stride);
       v += (double)y.x + (double)y.y;
     }
     return v;
   }
   const double* src = static_cast<const double*>(s.part) + (size_t)q * s.a.p + j;
-  double v = 0.0;
-#pragma unroll 8
-  for (int c = 0; c < s.a.ncl; ++c) v += __ldcg(src + (size_t)c * s.a.NB * s.a.p);
+#pragma unroll 4
+  for (int c = 0; c < s.a.ncl; ++c) v += __ldcg(src + c * stride);
   return v;
 }
 // FP64 G^t_j, as stage 1 stored it
@@ -1369,7 +1368,7 @@ __global__ void __launch_bounds__(32 * PN_MAXW, K == PK_F64 ? 1 : 2) pnode_kerne
         if (f == 0) key = key_of(aa);
         if (!F64 && iter && !wide && f == 0) {   // y_j = 0: v_j = -s gy_j in FP32
           float gy = gf;
-          if (!mu0) gy = ls ? opm32 * gf - mu32 * gp : pn_gpair_call(j, 1).x;
+          if (!mu0) gy = ls ? opm32 * gf - mu32 * gp : pn_gpair(j, 1).hi;
           const float v = -(kc.s_f * gy);
           if (v < 0.f) f8 |= 1;
           m = fabsf(v);
