@@ -41,7 +41,7 @@ GAP_TOL = 1e-6
 # GB300 by this script's own arm; used by --impl reference to extrapolate).
 GPU_ITERS_TO_GAP = {"ls_20000x50000_f32": 576}
 METRIC = "node relaxations/s to rel. gap 1e-6 on 1 GB300; fused X-pass HBM GB/s vs peak"
-PROFILE = os.path.join(ROOT, "profiles", "xstrip_ls_20000x50000_f32.md")
+PROFILE = os.path.join(ROOT, "profiles", "xring_ls_20000x50000_f32.md")
 
 
 def max_over_ranks(ms, world, device="cpu"):
@@ -396,7 +396,7 @@ def run_batch(device, workload=BATCH_WORKLOAD, reps=2, singles=16):
                          "peak_source": "MEASURED_PEAKS.json bf16_tflops, burst (of measured)" if peaks
                          else "fallback 1900 TFLOP/s (of fallback)"},
             "products": "the library's tcgen05 kernel on BF16 planes of X, X' and the node operands "
-                        "(FP32-accurate products, TMEM sums drained every 128 terms, FP64 sums of the K chunks); "
+                        "(FP32-accurate products, TMEM sums drained every 128 terms, partial tiles summed in a fixed order); "
                         "each round of 16 iterations is one CUDA graph"}
 
 

@@ -179,7 +179,8 @@ relax_status relax_solve(relax_handle* h, const int8_t* fixings, const void* war
  * Z = X B' and G = X' R run as two products (FP32 X: the library's
  * tensor-core kernel on BF16 planes of X, X', B and R, FP32-accurate products
  * whose partial tiles are summed in a fixed order; FP64 X: FP64 products), and each node's
- * prox / g / g* / gap / restart step runs in its own segment of one launch.
+ * prox / g / g* / gap / restart step runs on a thread-block cluster of its own,
+ * all nodes in one launch.
  * Nodes converge after uneven iteration counts and leave the batch every 16
  * iterations (each round of 16 is one CUDA graph per active-set size); the
  * stall rule's window is at most 200 inside a batch, and a node that stalls

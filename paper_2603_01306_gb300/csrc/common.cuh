@@ -8,7 +8,7 @@
 
 namespace relax {
 
-enum : int { ST_OK = 0, ST_TIMEOUT = 5, ST_NUMERIC = 6, ST_INTERNAL = 7 };   // ST_INTERNAL: a kernel launched outside its plan (reported as RELAX_ECUDA)
+enum : int { ST_OK = 0, ST_TIMEOUT = 5, ST_NUMERIC = 6 };
 
 __device__ __forceinline__ uint64_t globaltimer_ns() {
   uint64_t t;
